@@ -20,20 +20,19 @@ __device__ __forceinline__ uint32_t eq4(uint32_t a, uint32_t b) {
   return (z * 0x00204081u) >> 21 & 0xFu;
 }
 
-// Bonds of 32 consecutive sites of one row, and the observables of the
-// spins read (bonds joining equal spins; sites per state for q <= QREG).
-struct RowBonds {
-  uint32_t east, north;     // bit i: east / north bond of site i (rule of Eq. 7)
-  int n_eq;                 // equal east and north neighbours among the sites
-  int cnt[8];               // sites per state (q <= 8)
-};
-
 constexpr int QREG_MAX = 8;
 
-template <class Keys>
-__device__ __forceinline__ void row_bonds(const int8_t* __restrict__ spins, int L, int y, int x, int nvalid,
-                                          uint64_t T, const Keys& keys, uint32_t sw_lo, uint32_t sw_hi,
-                                          int q, RowBonds& rb) {
+// Which of 32 consecutive sites of one row equal their east and north
+// neighbours, and the observables of the spins read (bonds joining equal
+// spins; sites per state for q <= QREG).
+struct RowEqual {
+  uint32_t east, north;     // bit i: site i equals its east / north neighbour
+  int n_eq;                 // equal east and north neighbours among the sites
+  int cnt[QREG_MAX];        // sites per state (q <= 8)
+};
+
+__device__ __forceinline__ void row_equal(const int8_t* __restrict__ spins, int L, int y, int x, int nvalid, int q,
+                                          RowEqual& rb) {
   const int yn = (y + 1 == L) ? 0 : y + 1;
   const int64_t row = (int64_t)y * L, rown = (int64_t)yn * L;
   uint32_t s[8], n[8];
@@ -100,26 +99,44 @@ __device__ __forceinline__ void row_bonds(const int8_t* __restrict__ spins, int 
       }
     }
   }
-  // bonds: one Philox call per pair of sites i, i+1 (words: east i, north i,
-  // east i+1, north i+1)
-  if (T >= (1ull << 32)) {
-    rb.east = eq_e;                      // p = 1: every bond between equal spins opens
-    rb.north = eq_n;
-  } else if (T == 0) {
-    rb.east = rb.north = 0u;
-  } else {
-    const uint32_t thr = (uint32_t)T;
-    uint32_t e = 0u, n = 0u;
+  rb.east = eq_e;
+  rb.north = eq_n;
+}
+
+// e |= bit if r < thr: a compare and one predicated add.
+__device__ __forceinline__ void set_if_below(uint32_t& e, uint32_t r, uint32_t thr, uint32_t bit) {
+  asm("{ .reg .pred p; setp.lt.u32 p, %1, %2; @p add.u32 %0, %0, %3; }" : "+r"(e) : "r"(r), "r"(thr), "r"(bit));
+}
+
+// Open bonds of 32 consecutive sites from site index `site0` on (even; rule
+// of Eq. 7): the bits of east / north (equal neighbours) whose draw is below
+// T.  One Philox call per pair of sites i, i+1 (words: east i, north i, east
+// i+1, north i+1).  Draws past the last valid site are dropped by the masks.
+template <class Keys>
+__device__ __forceinline__ void draw_bonds(uint32_t site0, int nvalid, uint64_t T, const Keys& keys, uint32_t sw_lo,
+                                           uint32_t sw_hi, uint32_t& east, uint32_t& north) {
+  if (T >= (1ull << 32)) return;         // p = 1: every bond between equal spins opens
+  uint32_t e = 0u, n = 0u;
+  if (T != 0) {
+    const uint32_t thr = (uint32_t)T, c0 = site0 >> 1;
+    constexpr int U = 16;   // sites per loop body (8: 5 % longer, 32: 4 %, its code misses the instruction cache)
+#pragma unroll 1
+    for (int i0 = 0; i0 < nvalid; i0 += U) {
+      uint32_t eb = 0u, nb = 0u;
 #pragma unroll
-    for (int i = 0; i < 32; i += 2) {
-      if (i >= nvalid) break;
-      const uint4 r = philox_draw(make_uint4((uint32_t)((row + x + i) >> 1), sw_lo, sw_hi, TAG_BOND), keys);
-      e |= ((uint32_t)(r.x < thr) | ((uint32_t)(r.z < thr) << 1)) << i;
-      n |= ((uint32_t)(r.y < thr) | ((uint32_t)(r.w < thr) << 1)) << i;
+      for (int i = 0; i < U; i += 2) {
+        const uint4 r = philox_draw(make_uint4(c0 + (uint32_t)((i0 + i) >> 1), sw_lo, sw_hi, TAG_BOND), keys);
+        set_if_below(eb, r.x, thr, 1u << i);
+        set_if_below(eb, r.z, thr, 2u << i);
+        set_if_below(nb, r.y, thr, 1u << i);
+        set_if_below(nb, r.w, thr, 2u << i);
+      }
+      e |= eb << i0;
+      n |= nb << i0;
     }
-    rb.east = e & eq_e;
-    rb.north = n & eq_n;
   }
+  east &= e;
+  north &= n;
 }
 
 // Block-wide sums of n_eq and the state counts, added to the observable slot.
@@ -152,33 +169,31 @@ __device__ __forceinline__ void add_observables(long long n_eq, const int* cnt, 
 }
 
 // The two halves of add_observables, for a kernel that has a __syncthreads()
-// between them anyway: every warp leaves its sums in `red` ...
+// between them anyway: every warp leaves its sums in `red` (at most 64 bonds
+// and 32 sites per lane, so 32-bit sums are exact) ...
 template <int NTHREADS>
-__device__ __forceinline__ void observables_warp_sums(long long n_eq, const int* cnt, int qreg,
-                                                      unsigned long long* red) {
+__device__ __forceinline__ void observables_warp_sums(unsigned n_eq, const int* cnt, int qreg, unsigned* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int NW = NTHREADS / 32;
-  unsigned long long v = (unsigned long long)n_eq;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
+  const unsigned v = __reduce_add_sync(FULL, n_eq);
   if (lane == 0) red[warp] = v;
 #pragma unroll
   for (int k = 0; k < QREG_MAX; ++k) {
     if (k >= qreg) break;
-    unsigned long long c = (unsigned long long)cnt[k];
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(FULL, c, o);
+    const unsigned c = __reduce_add_sync(FULL, (unsigned)cnt[k]);
     if (lane == 0) red[(1 + k) * NW + warp] = c;
   }
 }
 
 // ... and, after a barrier, the block's totals are added to the slot.
 template <int NTHREADS>
-__device__ __forceinline__ void observables_commit(int q, int qreg, unsigned long long* slot,
-                                                   const unsigned long long* red, const int* hist) {
+__device__ __forceinline__ void observables_commit(int q, int qreg, unsigned long long* slot, const unsigned* red,
+                                                   const int* hist) {
   constexpr int NW = NTHREADS / 32;
   if (threadIdx.x <= qreg) {
-    unsigned long long tot = 0;
+    unsigned tot = 0;
     for (int w = 0; w < NW; ++w) tot += red[threadIdx.x * NW + w];
-    if (tot && (threadIdx.x == 0 || threadIdx.x - 1 < q)) atomicAdd(slot + threadIdx.x, tot);
+    if (tot && (threadIdx.x == 0 || threadIdx.x - 1 < q)) atomicAdd(slot + threadIdx.x, (unsigned long long)tot);
   }
   if (qreg == 0) {
     for (int k = threadIdx.x; k < q; k += NTHREADS)
@@ -192,8 +207,7 @@ constexpr int QREG = QREG_MAX;   // state counts kept in registers for q <= QREG
 using namespace fused;
 
 // After the labeling kernel, the first TILE_SITES / 32 words of a tile's
-// pair-list slot (no longer needed once the tile is labeled) hold its
-// edge-root bits: bit r set iff local root r's component touches the tile
+// root-list slot hold its edge-root bits: bit r set iff local root r's component touches the tile
 // edge, so that its cluster may continue in other tiles.  The flip and the
 // few-cluster seed selection read them.
 constexpr int EDGE_WORDS = TILE_SITES / 32;
@@ -206,7 +220,6 @@ static_assert(TILE_SITES <= ROOT_MASK + 1, "local index fits below the flag");
 struct LabelTileSmem {
   TileSmem tile;
   uint32_t edge_bits[EDGE_WORDS];                   // local roots on the tile edge
-  uint32_t e_last;                                  // raw east bit of column w-1, bit = row
   unsigned long long red[(1 + QREG) * (LABEL_THREADS / 32)];
   int hist[128];
 };
@@ -224,8 +237,7 @@ template <class Keys>
 __device__ __forceinline__ void sw_label_tile(const SwRep& R, int t, uint64_t sweep, bool do_obs, int obs_cap,
                                               LabelTileSmem& ls, const Keys& keys) {
   TileSmem& sm = ls.tile;
-  uint32_t& e_last = ls.e_last;
-  unsigned long long* red = ls.red;
+  unsigned* red = reinterpret_cast<unsigned*>(ls.red);
   int* hist = ls.hist;
   const int8_t* __restrict__ spins = R.spins;
   uint16_t* __restrict__ lroot = R.lroot;
@@ -240,110 +252,83 @@ __device__ __forceinline__ void sw_label_tile(const SwRep& R, int t, uint64_t sw
   const int h = min(TILE_H, L - y0), w = min(TILE_W, L - x0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int32_t* slot = s.roots + (int64_t)t * TILE_SITES;
-  int32_t* hook_log = s.work + (int64_t)t * TILE_SITES;
-  if (threadIdx.x == 0) {
-    sm.n_hooked = 0;
-    e_last = 0u;
+  uint32_t* edge_bits = ls.edge_bits;
+  edge_bits[threadIdx.x] = 0u;        // the engine's barriers order it before the marks
+  if (q > QREG) {
+    for (int k = threadIdx.x; k < 128; k += LABEL_THREADS) hist[k] = 0;
+    __syncthreads();
   }
-  for (int k = threadIdx.x; k < 128; k += LABEL_THREADS) hist[k] = 0;
-  ls.edge_bits[threadIdx.x] = 0u;
-  __syncthreads();
 
-  // 1. bonds: warp c draws strip c, lane ly row ly
-  long long n_eq = 0;
-  int cnt[QREG];
-#pragma unroll
-  for (int k = 0; k < QREG; ++k) cnt[k] = 0;
-  uint32_t we = 0u, wn = 0u;
+  // 1. bonds: warp c draws strip c, lane ly row ly; the observables are
+  //    summed before the draws, so that their counters hold no registers
+  //    across them
+  const int nvalid = min(max(w - 32 * warp, 0), 32);
+  const bool last_strip = nvalid > 0 && 32 * warp + nvalid == w;
+  uint32_t we = 0u, wn = 0u, e_last = 0u;   // e_last: raw east bits of column w-1, bit = row
   {
-    const int ly = lane, c = warp;
-    const int nvalid = min(max(w - 32 * c, 0), 32);
-    if (ly < h && nvalid > 0) {
-      const int y = y0 + ly, x = x0 + 32 * c;
-      RowBonds rb;
-      row_bonds(spins, L, y, x, nvalid, T, keys, (uint32_t)sweep, (uint32_t)(sweep >> 32), q, rb);
-      we = rb.east;
-      wn = rb.north;
-      if (32 * c + nvalid == w) {                 // east bond leaving the tile
-        const uint32_t bit = 1u << (nvalid - 1);
-        if (we & bit) atomicOr(&e_last, 1u << ly);
-        we &= ~bit;
-      }
-      if (do_obs) {
-        n_eq = rb.n_eq;
-        if (q <= QREG) {
+    const bool in = lane < h && nvalid > 0;
+    const int y = y0 + lane, x = x0 + 32 * warp;
+    {
+      RowEqual rb;
+      rb.n_eq = 0;
 #pragma unroll
-          for (int k = 0; k < QREG; ++k) cnt[k] = rb.cnt[k];
-        } else {
+      for (int k = 0; k < QREG; ++k) rb.cnt[k] = 0;
+      if (in) {
+        row_equal(spins, L, y, x, nvalid, q, rb);
+        we = rb.east;
+        wn = rb.north;
+        if (do_obs && q > QREG) {
           const int8_t* p = spins + (int64_t)y * L + x;
           for (int j = 0; j < nvalid; ++j) atomicAdd(&hist[p[j]], 1);
         }
       }
+      if (do_obs) observables_warp_sums<LABEL_THREADS>((unsigned)rb.n_eq, rb.cnt, q <= QREG ? q : 0, red);
     }
-    sm.be[ly * STRIPS + c] = we;
-    sm.bn[ly * STRIPS + c] = wn;
+    if (in)
+      draw_bonds((uint32_t)((int64_t)y * L + x), nvalid, T, keys, (uint32_t)sweep, (uint32_t)(sweep >> 32), we, wn);
+    if (last_strip) {                 // east bonds leaving the tile
+      const uint32_t bit = 1u << (nvalid - 1);
+      e_last = __ballot_sync(FULL, (we & bit) != 0u);
+      we &= ~bit;
+    }
   }
-  if (do_obs) observables_warp_sums<LABEL_THREADS>(n_eq, cnt, q <= QREG ? q : 0, red);
-  __syncthreads();
 
-  // 2. label the tile (the engine ends with a barrier)
-  tile_engine_regs(sm, we, wn, h, slot, hook_log, s.err);
+  // 2. label the tile
+  tile_engine(sm, we, wn, h, w, s.err);
   if (do_obs) {   // observables of the spins read (the previous sweep's result)
     unsigned long long* oslot =
         reinterpret_cast<unsigned long long*>(R.obs + (int64_t)((sweep - 1) % (uint64_t)obs_cap) * (q + 1));
     observables_commit<LABEL_THREADS>(q, q <= QREG ? q : 0, oslot, red, hist);
   }
 
-  // 3. tile roots as 16-bit local indices: per step a thread takes four
-  //    consecutive sites (consecutive lanes, consecutive 16-byte words of
-  //    par: no bank conflicts) and stores 8 bytes (L % 4 == 0; w is a
-  //    multiple of 4, so four sites are all inside or all outside)
-  auto entry = [&](int p) -> uint32_t { return (uint32_t)sm.par[p]; };   // p = par[site]
+  // 3. tile roots of my strip as 16-bit local indices: per step a thread
+  //    takes eight consecutive sites (four threads a row) and stores 16
+  //    bytes, or two halves where rows start only 8-byte aligned (L % 4 == 0;
+  //    w is a multiple of 4, so four sites are all inside or all outside)
+  {
+    const int lx = 32 * warp + 8 * (lane & 3);
 #pragma unroll 2
-  for (int k = threadIdx.x; k < TILE_SITES / 4; k += LABEL_THREADS) {
-    const int sidx = 4 * k;
-    const int ly = sidx >> TILE_W_LOG2, lx = sidx & (TILE_W - 1);
-    if (ly >= h || lx >= w) continue;
-    const int4 pa = *reinterpret_cast<const int4*>(&sm.par[sidx]);
-    uint16_t* dst = lroot + (int64_t)(y0 + ly) * L + x0 + lx;
-    *reinterpret_cast<uint2*>(dst) = make_uint2(entry(pa.x) | (entry(pa.y) << 16), entry(pa.z) | (entry(pa.w) << 16));
+    for (int ly = lane >> 2; ly < h; ly += 8) {
+      if (lx >= w) break;
+      const uint4 r = roots_of(sm.par, local_of(ly, lx));
+      uint16_t* dst = lroot + (int64_t)(y0 + ly) * L + x0 + lx;
+      if ((L & 7) == 0) {   // then w is a multiple of 8 too
+        *reinterpret_cast<uint4*>(dst) = r;
+      } else {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(r.x, r.y);
+        if (lx + 8 <= w) *reinterpret_cast<uint2*>(dst + 4) = make_uint2(r.z, r.w);
+      }
+    }
   }
 
-  // 4. seam record; parent entries of edge roots; edge roots marked
-  int32_t* rec = s.seams + (int64_t)t * SeamLayout::INTS;
-  uint32_t* edge_bits = ls.edge_bits;
-  auto root_at = [&](int ly, int lx) -> int { return sm.par[sm.par[ly * TILE_W + lx]]; };
-  auto edge_root = [&](bool ok, int r) -> int32_t {
-    // global index of local root r; the first of a run of equal roots among
-    // consecutive lanes writes its parent entry and its edge mark
-    const int left = __shfl_up_sync(FULL, ok ? r : -1, 1);
-    if (!ok) return -1;
-    const int32_t gr = tile_global(r, y0, x0, L);
-    if (lane == 0 || left != r) {
-      gpar[gr] = gr;
-      atomicOr(&edge_bits[r >> 5], 1u << (r & 31));
-    }
-    return gr;
-  };
-  for (int k = threadIdx.x; k < TILE_H; k += LABEL_THREADS) {
-    const bool ok = k < h;
-    rec[SeamLayout::COL_L + k] = edge_root(ok, ok ? root_at(k, 0) : 0);
-    rec[SeamLayout::COL_R + k] = edge_root(ok, ok ? root_at(k, w - 1) : 0);
-    if (lane == 0) rec[SeamLayout::E_BITS + (k >> 5)] = (int32_t)e_last;
-  }
-  for (int k = threadIdx.x; k < TILE_W; k += LABEL_THREADS) {
-    const bool ok = k < w;
-    rec[SeamLayout::ROW_B + k] = edge_root(ok, ok ? root_at(0, k) : 0);
-    rec[SeamLayout::ROW_T + k] = edge_root(ok, ok ? root_at(h - 1, k) : 0);
-    const bool n = ok && ((sm.bn[(h - 1) * STRIPS + (k >> 5)] >> (k & 31)) & 1u);
-    const uint32_t nb = __ballot_sync(FULL, n);
-    if (lane == 0) rec[SeamLayout::N_BITS + (k >> 5)] = (int32_t)nb;
-  }
+  // 4. my strip's part of the seam record; parent entries of edge roots; edge
+  //    roots marked
+  seam_strip(sm, s.seams + (int64_t)t * SeamLayout::INTS, gpar, edge_bits, wn, e_last, h, w, y0, x0, L);
 
   __syncthreads();
-  // 5. edge-root bits into the (now free) pair-list slot; each thread reads
+  // 5. edge-root bits into the tile's root-list slot; each thread reads
   //    and next clears only its own word
-  slot[threadIdx.x] = (int32_t)ls.edge_bits[threadIdx.x];
+  slot[threadIdx.x] = (int32_t)edge_bits[threadIdx.x];
 }
 
 // One tile of the fused flip step (see k_fused.cu).  All threads of the CTA
@@ -397,23 +382,20 @@ __device__ __forceinline__ void flip_tile_core(const SwRep& R, int t, uint64_t s
   fs.edge_bits[threadIdx.x] = (uint32_t)__ldcg(R.s.roots + (int64_t)t * TILE_SITES + threadIdx.x);
 
   // 2. my roots: a site is a tile root iff its entry is its own local index.
-  //    Word k of pass j holds sites 2k and 2k + 1; both are compared at once
-  //    (a half-word is zero iff its low 15 bits plus 0x7FFF stay below bit
-  //    15 and its bit 15 is clear).  Sites outside the tile hold 0xFFFF and
-  //    never match.  Bit 4j + k of `mine` flags site 2k of pass j, bit
+  //    Word k of pass j holds sites 2k and 2k + 1; both are compared at once.
+  //    Sites outside the tile hold 0xFFFF and never match.  Bit 4j + k of `mine` flags site 2k of pass j, bit
   //    16 + 4j + k site 2k + 1.
   uint32_t mine = 0;
 #pragma unroll
   for (int j = 0; j < PASSES; ++j) {
     const uint4 rv = roots.get(j);
-    const uint32_t base = (uint32_t)((8 * j + orow) * TILE_W + lx0);
+    const uint32_t base = (uint32_t)local_of(8 * j + orow, lx0);
     const uint32_t own = base * 0x00010001u + 0x00010000u;   // (base, base + 1)
     const uint32_t wv[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t x = wv[k] ^ (own + (uint32_t)k * 0x00020002u);
-      const uint32_t nz = ((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x;
-      mine |= (~nz & 0x80008000u) >> (15 - (4 * j + k));
+      mine |= zero_halves(x) >> (15 - (4 * j + k));
     }
   }
   const int cnt = __popc(mine);
@@ -436,7 +418,7 @@ __device__ __forceinline__ void flip_tile_core(const SwRep& R, int t, uint64_t s
     const int b = __ffs(mine) - 1;
     mine &= mine - 1;
     const int jk = b & 15;
-    const int r = (8 * (jk >> 2) + orow) * TILE_W + lx0 + 2 * (jk & 3) + (b >> 4);
+    const int r = local_of(8 * (jk >> 2) + orow, lx0) + 2 * (jk & 3) + (b >> 4);
     rlist[base++] = (uint16_t)r | (((fs.edge_bits[r >> 5] >> (r & 31)) & 1u) ? EDGE_ROOT : (uint16_t)0);
   }
   __syncthreads();
@@ -462,7 +444,7 @@ __device__ __forceinline__ void flip_tile_core(const SwRep& R, int t, uint64_t s
       if (FEW) {
         // the cluster's current state, read at the tile root (this tile's own
         // site: step 5 rewrites it only after a barrier)
-        int v = spins[(int64_t)(y0 + (r[u] >> TILE_W_LOG2)) * L + x0 + (r[u] & (TILE_W - 1))];
+        int v = spins[(uint32_t)tile_global(r[u], y0, x0, L)];
         if ((__ldcg(sel + (Rg[u] >> 5)) >> (Rg[u] & 31)) & 1u) {
           const uint4 d =
               philox_draw(make_uint4((uint32_t)Rg[u], (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
@@ -614,14 +596,13 @@ __device__ __forceinline__ void sw_flip_whole_tile(const SwRep& R, int t, uint64
 #pragma unroll
     for (int j = 0; j < PASSES; ++j) {
       const uint4 rv = held[j];
-      const uint32_t base = (uint32_t)((8 * j + orow) * TILE_W + lx0);
+      const uint32_t base = (uint32_t)local_of(8 * j + orow, lx0);
       const uint32_t own = base * 0x00010001u + 0x00010000u;
       const uint32_t wv[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const uint32_t x = wv[k] ^ (own + (uint32_t)k * 0x00020002u);
-        const uint32_t nz = ((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x;
-        mine |= (~nz & 0x80008000u) >> (15 - (4 * j + k));
+        mine |= zero_halves(x) >> (15 - (4 * j + k));
       }
     }
   }
@@ -645,7 +626,7 @@ __device__ __forceinline__ void sw_flip_whole_tile(const SwRep& R, int t, uint64
     const int b = __ffs(mine) - 1;
     mine &= mine - 1;
     const int jk = b & 15;
-    const int r = (8 * (jk >> 2) + orow) * TILE_W + lx0 + 2 * (jk & 3) + (b >> 4);
+    const int r = local_of(8 * (jk >> 2) + orow, lx0) + 2 * (jk & 3) + (b >> 4);
     rlist[base++] = (uint16_t)r | (((fs.edge_bits[r >> 5] >> (r & 31)) & 1u) ? EDGE_ROOT : (uint16_t)0);
   }
   __syncthreads();

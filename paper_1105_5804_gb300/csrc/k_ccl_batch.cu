@@ -21,8 +21,8 @@ __device__ __forceinline__ int job_of_tile(const CclBatchView& v, int gt) {
   return lo;
 }
 
-__global__ void __launch_bounds__(LABEL_THREADS) k_cclb_tile(const __grid_constant__ CclBatchView v) {
-  __shared__ TileSmem sm;
+__global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_cclb_tile(const __grid_constant__ CclBatchView v) {
+  __shared__ CclTileSmem sm;
   const int gt = blockIdx.x;
   const CclJob& J = v.jobs[job_of_tile(v, gt)];
   ccl_label_tile<true>(J.mask, J.labels, J.g, J.s, gt - J.tile0, sm);

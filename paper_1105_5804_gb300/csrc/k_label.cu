@@ -41,7 +41,7 @@ namespace swccl {
 
 __global__ void __launch_bounds__(LABEL_THREADS)
 k_tile_label(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid g, LabelScratch s) {
-  __shared__ TileSmem sm;
+  __shared__ CclTileSmem sm;
   ccl_label_tile(mask, labels, g, s, blockIdx.x, sm);
 }
 
@@ -53,9 +53,9 @@ cudaError_t launch_tile_label(const uint8_t* mask, int32_t* labels, const Grid& 
 
 // Stand-alone labeling: local labeling with local-root labels, then (after
 // the seam merge) the final labels of every tile in one pass.
-__global__ void __launch_bounds__(LABEL_THREADS)
+__global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
 k_ccl_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid g, LabelScratch s) {
-  __shared__ TileSmem sm;
+  __shared__ CclTileSmem sm;
   ccl_label_tile<true>(mask, labels, g, s, blockIdx.x, sm);
 }
 

@@ -19,26 +19,58 @@ __device__ __forceinline__ uint32_t even_bits(unsigned long long x) {
   return (uint32_t)x;
 }
 
-// Local labeling of one tile for the stand-alone labeling path: the tile's
-// bond bits are copied from the packed mask into shared memory (bits of
+// Mask bits of `nvalid` (1..32) consecutive sites from site0 on, site i in bits
+// 2i (east) and 2i + 1 (north), the rest zero.  One 64-bit load where the
+// sites start on a 32-site word; else three 32-bit words shifted into place
+// (rows of any width start anywhere in a byte); single bytes only for a mask
+// that is not 4-byte aligned and in its last word.
+__device__ __forceinline__ unsigned long long mask_word(const uint8_t* __restrict__ mask, int64_t n_bytes,
+                                                        int64_t site0, int nvalid) {
+  const int64_t b0 = site0 >> 2;
+  unsigned long long wd = 0ull;
+  if ((site0 & 31) == 0 && (reinterpret_cast<uintptr_t>(mask) & 7) == 0 && b0 + 8 <= n_bytes) {
+    wd = *reinterpret_cast<const unsigned long long*>(mask + b0);
+  } else {
+    const int off = 2 * (int)(site0 & 15);                  // first bit in its 32-bit word
+    const int n_words = (off + 2 * nvalid + 31) >> 5;       // 1..3
+    const int64_t w0 = site0 >> 4;
+    if ((reinterpret_cast<uintptr_t>(mask) & 3) == 0 && 4 * (w0 + n_words) <= n_bytes) {
+      const uint32_t* p = reinterpret_cast<const uint32_t*>(mask) + w0;
+      const uint32_t a = p[0], b = n_words > 1 ? p[1] : 0u, c = n_words > 2 ? p[2] : 0u;
+      wd = (unsigned long long)__funnelshift_r(a, b, off) | (unsigned long long)__funnelshift_r(b, c, off) << 32;
+    } else {
+      for (int i = 0; i < nvalid; ++i) wd |= (unsigned long long)site_bits(mask, site0 + i) << (2 * i);
+    }
+  }
+  return nvalid < 32 ? wd & ((1ull << (2 * nvalid)) - 1ull) : wd;
+}
+
+// Local labeling of one tile for the stand-alone labeling path: every thread
+// takes the bond bits of its row of its strip from the packed mask (bits of
 // sites outside the grid and the east bond of the tile's last column
-// cleared), the engine of tile_engine.cuh labels the tile, and the kernel
-// writes every site's label (global index of its tile root, the minimum
+// cleared), the engine of tile_engine.cuh labels the tile, and the warps
+// write their strips' labels (global index of the tile root, the minimum
 // site index of its tile component), the tile's root list, and the seam
 // record (labels and outgoing bond bits of the four tile edges).
 // LOCAL (the stand-alone labeling path, finished by final_labels_tile): the
 // label array receives only the parent entries of the tile roots whose
 // component reaches the tile edge (label = own global index), which the
 // seam merge and the final root walks use; every site's tile root goes, as
-// a 16-bit local index, to the tile's hook-log slot (free once the engine
-// has ended), in tile row-major order; the root list holds local indices,
-// with CCL_EDGE_ROOT set on the edge roots.  final_labels_tile writes every
-// site's label.
+// a 16-bit local index, to the tile's slot of `work`, in tile row-major order;
+// the root list holds local indices, with CCL_EDGE_ROOT set on the edge
+// roots.  final_labels_tile writes every site's label.
 constexpr int CCL_EDGE_ROOT = 1 << 30;
+struct CclTileSmem {
+  TileSmem tile;
+  uint32_t edge_bits[TILE_SITES / 32];   // local roots on the tile edge
+};
+static_assert(TILE_SITES / 32 == LABEL_THREADS, "one edge word per thread");
+
 template <bool LOCAL = false>
 __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels,
-                                               const Grid& g, const LabelScratch& s, int t, TileSmem& sm) {
-  int* par = sm.par;
+                                               const Grid& g, const LabelScratch& s, int t, CclTileSmem& cs) {
+  TileSmem& sm = cs.tile;
+  const uint16_t* par = sm.par;
   int* warp_roots = sm.warp_roots;
 
   const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
@@ -46,93 +78,62 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
   const int h = min(TILE_H, g.H - y0), w = min(TILE_W, g.W - x0);
   const int W = g.W;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int32_t* slot = s.roots + (int64_t)t * TILE_SITES;     // pair lists, later the root list
-  int32_t* hook_log = s.work + (int64_t)t * TILE_SITES;
-  if (threadIdx.x == 0) sm.n_hooked = 0;
+  int32_t* slot = s.roots + (int64_t)t * TILE_SITES;     // the root list
+  cs.edge_bits[threadIdx.x] = 0u;                        // the engine's barriers order it before the marks
 
-  // 1. bond bits
-  for (int k = threadIdx.x; k < TILE_H * STRIPS; k += LABEL_THREADS) {
-    const int ly = k / STRIPS, c = k - ly * STRIPS;
-    const int nvalid = min(max(w - 32 * c, 0), 32);
-    unsigned long long wd = 0ull;
-    if (ly < h && nvalid > 0) {
-      const int64_t site0 = (int64_t)(y0 + ly) * W + x0 + 32 * c;
-      if ((W & 31) == 0 && (reinterpret_cast<uintptr_t>(mask) & 7) == 0) {
-        wd = reinterpret_cast<const unsigned long long*>(mask)[site0 >> 5];
-      } else {
-        for (int i = 0; i < nvalid; ++i) wd |= (unsigned long long)site_bits(mask, site0 + i) << (2 * i);
-      }
-      if (nvalid < 32) wd &= (1ull << (2 * nvalid)) - 1ull;
-      if (32 * c + nvalid == w) wd &= ~(1ull << (2 * (nvalid - 1)));   // east bond leaving the tile
-    }
-    sm.be[k] = even_bits(wd);        // the mask interleaves east (even) and north (odd) bits
-    sm.bn[k] = even_bits(wd >> 1);
+  // 1. bond bits of row `lane` of strip `warp`
+  const int nvalid = min(max(w - 32 * warp, 0), 32);
+  uint32_t we = 0u, wn = 0u, e_last = 0u;
+  if (lane < h && nvalid > 0) {
+    const unsigned long long wd =
+        mask_word(mask, (g.n_sites() + 3) >> 2, (int64_t)(y0 + lane) * W + x0 + 32 * warp, nvalid);
+    we = even_bits(wd);        // the mask interleaves east (even) and north (odd) bits
+    wn = even_bits(wd >> 1);
   }
-  __syncthreads();
+  if (nvalid > 0 && 32 * warp + nvalid == w) {   // east bonds leaving the tile
+    const uint32_t bit = 1u << (nvalid - 1);
+    e_last = __ballot_sync(FULL, (we & bit) != 0u);
+    we &= ~bit;
+  }
 
   // 2-4a. label the tile
-  tile_engine(sm, h, slot, hook_log, s.err);
+  tile_engine(sm, we, wn, h, w, s.err);
 
-  // LOCAL: mark the tile roots whose component reaches the tile edge (only
-  // they can belong to clusters that continue in other tiles); the marks go
-  // to the shared words the engine no longer needs
-  uint32_t* edge = reinterpret_cast<uint32_t*>(sm.pairs);
-  if (LOCAL) {
-    static_assert(TILE_SITES / 32 <= STRIPS * PAIR_FAST, "edge marks fit");
-    for (int k = threadIdx.x; k < TILE_SITES / 32; k += LABEL_THREADS) edge[k] = 0u;
-    __syncthreads();
-    auto mark = [&](int ly, int lx) {
-      const int r = par[par[ly * TILE_W + lx]];
-      atomicOr(&edge[r >> 5], 1u << (r & 31));
-    };
-    for (int k = threadIdx.x; k < h; k += LABEL_THREADS) {
-      mark(k, 0);
-      mark(k, w - 1);
-    }
-    for (int k = threadIdx.x; k < w; k += LABEL_THREADS) {
-      mark(0, k);
-      mark(h - 1, k);
-    }
-    __syncthreads();
-  }
-
-  // 4b. every site's root; root list.  LOCAL: the roots as 16-bit local
-  //     indices into the tile's hook-log slot (free since the engine ended),
-  //     four consecutive sites per thread and step (lane-consecutive words of
-  //     par); mine bit j: site 4 (threadIdx.x + (j / 4) LABEL_THREADS) + j % 4.
-  //     Otherwise global labels; mine bit j: site threadIdx.x + j LABEL_THREADS.
-  constexpr int PER_T = TILE_SITES / LABEL_THREADS;
+  // 4b. the roots of my strip's sites, eight consecutive sites per thread and
+  //     step, four threads a row.  LOCAL: as 16-bit local indices into the
+  //     tile's slot of `work`.  Otherwise as global labels.  Bit 4j + k of mine
+  //     flags site 2k of step j as a root, bit 16 + 4j + k site 2k + 1.
+  const int lx0 = 32 * warp + 8 * (lane & 3);
+  const int in = min(max(w - lx0, 0), 8);   // columns past the grid are no roots of the tile
+  const uint32_t in_mask = ((1u << ((in + 1) >> 1)) - 1u) | ((1u << (in >> 1)) - 1u) << 16;
+  uint16_t* lr = reinterpret_cast<uint16_t*>(s.work + (int64_t)t * TILE_SITES);
   uint32_t mine = 0;
-  if (LOCAL) {
-    uint16_t* lr = reinterpret_cast<uint16_t*>(hook_log);
-#pragma unroll 2
-    for (int j = 0; j < PER_T / 4; ++j) {
-      const int sidx = 4 * ((int)threadIdx.x + j * LABEL_THREADS);
-      const int ly = sidx >> TILE_W_LOG2, lx = sidx & (TILE_W - 1);
-      if (ly >= h) continue;   // rows past the grid: the engine wrote no entries there
-      const int4 pv = *reinterpret_cast<const int4*>(&par[sidx]);
-      const int r0 = par[pv.x], r1 = par[pv.y], r2 = par[pv.z], r3 = par[pv.w];
-      *reinterpret_cast<uint2*>(lr + sidx) =
-          make_uint2((uint32_t)r0 | ((uint32_t)r1 << 16), (uint32_t)r2 | ((uint32_t)r3 << 16));
-      // columns past the grid (bondless, each its own root) are no roots of the tile
-      const uint32_t in = lx + 4 <= w ? 0xFu : (lx < w ? (1u << (w - lx)) - 1u : 0u);
-      const uint32_t is_root = (uint32_t)(r0 == sidx) | ((uint32_t)(r1 == sidx + 1) << 1) |
-                               ((uint32_t)(r2 == sidx + 2) << 2) | ((uint32_t)(r3 == sidx + 3) << 3);
-      mine |= (is_root & in) << (4 * j);
-    }
-  } else {
-#pragma unroll 4
-    for (int j = 0; j < PER_T; ++j) {
-      const int sidx = threadIdx.x + j * LABEL_THREADS;
-      const int ly = sidx >> TILE_W_LOG2, lx = sidx & (TILE_W - 1);
-      if (ly < h && lx < w) {
-        const int p = par[sidx];
-        const int r = par[p];
-        labels[(int64_t)(y0 + ly) * W + x0 + lx] = (y0 + (r >> TILE_W_LOG2)) * W + x0 + (r & (TILE_W - 1));
-        if (r == sidx) mine |= 1u << j;
-      }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int ly = (lane >> 2) + 8 * j;
+    if (ly >= h || in == 0) continue;   // the engine wrote no entries there
+    const int sidx = local_of(ly, lx0);
+    const uint4 r = roots_of(par, sidx);
+    if (LOCAL) *reinterpret_cast<uint4*>(lr + ly * TILE_W + lx0) = r;
+    const uint32_t own = (uint32_t)sidx * 0x00010001u + 0x00010000u;   // (sidx, sidx + 1)
+    const uint32_t wv[4] = {r.x, r.y, r.z, r.w};
+    uint32_t m = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m |= zero_halves(wv[k] ^ (own + (uint32_t)k * 0x00020002u)) >> (15 - k);
+    mine |= (m & in_mask) << (4 * j);
+    if (!LOCAL) {
+      int32_t* dst = labels + (int64_t)(y0 + ly) * W + x0 + lx0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < in) dst[k] = tile_global((int)(wv[k >> 1] >> (16 * (k & 1)) & 0xFFFFu), y0, x0, W);
     }
   }
+
+  // 5. my strip's part of the seam record; parent entries of edge roots; edge
+  //    roots marked
+  seam_strip(sm, s.seams + (int64_t)t * SeamLayout::INTS, labels, cs.edge_bits, wn, e_last, h, w, y0, x0, W);
+
+  // 6. root list
   int cnt = __popc(mine), incl = cnt;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -150,44 +151,12 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
   }
   base += incl - cnt;
   while (mine) {
-    const int j = __ffs(mine) - 1;
+    const int b = __ffs(mine) - 1;
     mine &= mine - 1;
-    if (LOCAL) {
-      // an edge root's label entry is its parent entry for the seam merge
-      const int sidx = 4 * ((int)threadIdx.x + (j >> 2) * LABEL_THREADS) + (j & 3);
-      const bool on_edge = (edge[sidx >> 5] >> (sidx & 31)) & 1u;
-      if (on_edge) {
-        const int32_t gr = (y0 + (sidx >> TILE_W_LOG2)) * W + x0 + (sidx & (TILE_W - 1));
-        labels[gr] = gr;
-      }
-      slot[base++] = sidx | (on_edge ? CCL_EDGE_ROOT : 0);
-    } else {
-      const int sidx = threadIdx.x + j * LABEL_THREADS;
-      slot[base++] = (y0 + (sidx >> TILE_W_LOG2)) * W + x0 + (sidx & (TILE_W - 1));
-    }
-  }
-
-  // 5. seam record
-  int32_t* rec = s.seams + (int64_t)t * SeamLayout::INTS;
-  auto glabel = [&](int ly, int lx) -> int32_t {
-    const int r = par[par[ly * TILE_W + lx]];
-    return (y0 + (r >> TILE_W_LOG2)) * W + x0 + (r & (TILE_W - 1));
-  };
-  for (int k = threadIdx.x; k < TILE_H; k += LABEL_THREADS) {
-    const bool ok = k < h;
-    rec[SeamLayout::COL_L + k] = ok ? glabel(k, 0) : -1;
-    rec[SeamLayout::COL_R + k] = ok ? glabel(k, w - 1) : -1;
-    const bool e = ok && (site_bits(mask, (int64_t)(y0 + k) * W + x0 + w - 1) & 1u);
-    const uint32_t eb = __ballot_sync(FULL, e);
-    if (lane == 0) rec[SeamLayout::E_BITS + (k >> 5)] = (int32_t)eb;
-  }
-  for (int k = threadIdx.x; k < TILE_W; k += LABEL_THREADS) {
-    const bool ok = k < w;
-    rec[SeamLayout::ROW_B + k] = ok ? glabel(0, k) : -1;
-    rec[SeamLayout::ROW_T + k] = ok ? glabel(h - 1, k) : -1;
-    const bool n = ok && ((sm.bn[(h - 1) * STRIPS + (k >> 5)] >> (k & 31)) & 1u);
-    const uint32_t nb = __ballot_sync(FULL, n);
-    if (lane == 0) rec[SeamLayout::N_BITS + (k >> 5)] = (int32_t)nb;
+    const int jk = b & 15;
+    const int sidx = local_of((lane >> 2) + 8 * (jk >> 2), lx0) + 2 * (jk & 3) + (b >> 4);
+    if (LOCAL) slot[base++] = sidx | (((cs.edge_bits[sidx >> 5] >> (sidx & 31)) & 1u) ? CCL_EDGE_ROOT : 0);
+    else slot[base++] = tile_global(sidx, y0, x0, W);
   }
   if (threadIdx.x == 0) s.root_counts[t] = total;
   __syncthreads();
@@ -262,8 +231,8 @@ __device__ __forceinline__ void final_labels_tile(int32_t* labels, const Grid& g
   }
   __syncthreads();
   // 2. every site takes its tile root's cluster root; the tile roots are the
-  //    16-bit local indices ccl_label_tile<true> left in the tile's hook-log
-  //    slot, eight sites per 16-byte word, in tile row-major order; labels go
+  //    16-bit local indices ccl_label_tile<true> left in the tile's slot
+  //    of `work`, eight sites per 16-byte word, in tile row-major order; labels go
   //    out four sites per 16-byte store when rows start 16-byte aligned (a
   //    16-byte aligned array and W % 4 == 0; x0 is a multiple of TILE_W, so w
   //    is a multiple of 4 too)

@@ -36,8 +36,7 @@ struct sw3_handle {
   int8_t* spins = nullptr;
   uint16_t* lroot = nullptr;      // brick root of every site (16-bit local index)
   int32_t* gpar = nullptr;        // parents of edge roots; also staging for host spins
-  uint32_t* edge_words = nullptr; // edge-root bits of every brick
-  int32_t* scratch = nullptr;     // labeling scratch of every brick
+  uint32_t* words = nullptr;      // edge-root bits and face bonds of every brick
   SwCtl* ctl = nullptr;
   int* chk = nullptr;             // spin-check flag of sw3_set_spins
   int64_t* obs = nullptr;
@@ -63,8 +62,7 @@ void free3(sw3_handle* h) {
   cudaFree(h->spins);
   cudaFree(h->lroot);
   cudaFree(h->gpar);
-  cudaFree(h->edge_words);
-  cudaFree(h->scratch);
+  cudaFree(h->words);
   cudaFree(h->ctl);
   cudaFree(h->chk);
   cudaFree(h->obs);
@@ -127,8 +125,7 @@ sw3_handle* sw3_create(int X, int Y, int Z, int q, uint64_t T, uint64_t seed, in
   }
   if (cudaMalloc(&h->spins, (size_t)n) != cudaSuccess || cudaMalloc(&h->gpar, (size_t)n * 4) != cudaSuccess ||
       cudaMalloc(&h->lroot, (size_t)n * 2) != cudaSuccess ||
-      cudaMalloc(&h->edge_words, (size_t)edge_words3(h->box) * 4) != cudaSuccess ||
-      cudaMalloc(&h->scratch, (size_t)scratch_ints3(h->box) * 4) != cudaSuccess ||
+      cudaMalloc(&h->words, (size_t)brick_words3(h->box) * 4) != cudaSuccess ||
       cudaMalloc(&h->ctl, sizeof(SwCtl)) != cudaSuccess || cudaMalloc(&h->chk, sizeof(int)) != cudaSuccess ||
       cudaMalloc(&h->obs, (size_t)OBS3_CAP * (q + 1) * 8) != cudaSuccess) {
     cudaGetLastError();
@@ -173,14 +170,14 @@ int sw3_sweep(sw3_handle* h, int n) {
         }
         h->ev_pending.push_back(e);
       }
-      CK3(launch_sweep3(h->spins, h->lroot, h->gpar, h->edge_words, h->scratch, h->box, h->q, h->T, h->seed, h->ctl,
+      CK3(launch_sweep3(h->spins, h->lroot, h->gpar, h->words, h->box, h->q, h->T, h->seed, h->ctl,
                         h->obs, OBS3_CAP, h->stream, ev));
       h->sweeps++;
     }
   } else {
     if (!h->exec) {
       CK3(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-      cudaError_t e = launch_sweep3(h->spins, h->lroot, h->gpar, h->edge_words, h->scratch, h->box, h->q, h->T,
+      cudaError_t e = launch_sweep3(h->spins, h->lroot, h->gpar, h->words, h->box, h->q, h->T,
                                     h->seed, h->ctl, h->obs, OBS3_CAP, h->stream, nullptr);
       cudaGraph_t gr = nullptr;
       cudaError_t e2 = cudaStreamEndCapture(h->stream, &gr);
@@ -271,7 +268,7 @@ int sw3_labels(sw3_handle* h, int32_t* out, int is_device) {
   const int64_t n = h->box.n();
   int32_t* dst = out;
   if (!is_device) CK3(cudaMalloc(&dst, (size_t)n * 4));
-  cudaError_t e = launch_labels3(h->lroot, h->gpar, h->edge_words, h->box, dst, &h->ctl->err, h->stream);
+  cudaError_t e = launch_labels3(h->lroot, h->gpar, h->words, h->box, dst, &h->ctl->err, h->stream);
   if (e == cudaSuccess && !is_device) e = cudaMemcpyAsync(out, dst, (size_t)n * 4, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (!is_device) cudaFree(dst);

@@ -101,81 +101,162 @@ __device__ __forceinline__ void set_error(int* err, int code) {
 }
 
 // ---------------------------------------------------------------------------
-// Union-find in shared memory.  par[x] <= x always; roots satisfy par[r] == r.
+// Local indices.  A tile's sites are numbered row by row, with neighbouring
+// 32-column strips swapped in odd rows: a strip's 16-bit entries (64 bytes a
+// row) then alternate between the two halves of the 32 shared-memory banks
+// instead of all falling into one.  Within a strip, and between different
+// rows, local indices order like site indices; sites of one row compare by
+// node_key.
 // ---------------------------------------------------------------------------
-// Path halving writes with atomicMin, never with a plain store: a plain
-// store of a grandparent read earlier could overwrite a smaller pointer that
-// another thread has written since (for instance the final root), undoing
-// its compression.  With atomicMin every entry only ever decreases, and a
-// root, the minimum of its tree, once written stays.  Walks at most `limit`
-// steps (a tile tree has fewer nodes); on overrun the error word is set.
-__device__ __forceinline__ int sm_find(volatile int* par, int x, int limit, int* err) {
-  int p = par[x];
-  int steps = 0;
-  while (p != x) {
-    const int gp = par[p];
-    if (gp != p) atomicMin((int*)&par[x], gp);   // path halving
-    x = p;
-    p = gp;
-    if (++steps > limit) { set_error(err, SW_ERR_STATE); return x; }
-  }
-  return x;
-}
+__host__ __device__ constexpr int local_of(int ly, int lx) { return ly * TILE_W + (lx ^ ((ly & 1) << 5)); }
+__device__ __forceinline__ int local_y(int r) { return r >> TILE_W_LOG2; }
+__device__ __forceinline__ int local_x(int r) { return (r & (TILE_W - 1)) ^ ((r >> (TILE_W_LOG2 - 5)) & 32); }
 
-// The roots of two nodes at once: the walks run in lock step, so that their
-// shared-memory loads overlap.  No path compression: inside a tile the
-// unions keep trees shallow, and the atomics that compression needs cost
-// more than the steps they save; the hooked roots are resolved at the end.
-// Same step limit as sm_find.
-__device__ __forceinline__ void sm_find2(volatile int* par, int& a, int& b, int limit, int* err) {
-  int pa = par[a], pb = par[b];
-  for (int steps = 0; pa != a || pb != b; ++steps) {
-    if (pa != a) { a = pa; pa = par[a]; }
-    if (pb != b) { b = pb; pb = par[b]; }
-    if (steps > limit) { set_error(err, SW_ERR_STATE); return; }
-  }
+// ---------------------------------------------------------------------------
+// Union-find in shared memory on 16-bit entries.  A node id and an entry are
+// byte offsets of entries (2 x local index), so that a walk step is one load
+// with no address arithmetic.  A node's entry is the node itself (a root) or a
+// node of a smaller site index in its component, so every walk ends.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int sm_at(const uint16_t* par, int x) {
+  return *reinterpret_cast<const volatile uint16_t*>(reinterpret_cast<const char*>(par) + x);
 }
-
-// Join the sets of a and b.  atomicMin hooks the larger root under the
-// smaller; when the target was hooked meanwhile, the returned old parent is
-// joined in the next round, so no link is lost.  Every round strictly lowers
-// the larger operand, so at most `limit` rounds run.
-__device__ __forceinline__ void sm_union(int* par, int a, int b, int limit, int* err) {
-  volatile int* vp = par;
-  for (int rounds = 0; rounds <= limit; ++rounds) {
-    a = sm_find(vp, a, limit, err);
-    b = sm_find(vp, b, limit, err);
-    if (a == b) return;
-    if (a > b) { const int t = a; a = b; b = t; }
-    const int old = atomicMin(&par[b], a);
-    if (old == b) return;
-    b = old;
-  }
-  set_error(err, SW_ERR_STATE);
+__device__ __forceinline__ void sm_set(uint16_t* par, int x, int v) {
+  *reinterpret_cast<volatile uint16_t*>(reinterpret_cast<char*>(par) + x) = (uint16_t)v;
 }
+// Orders nodes like their sites: twice the row-major index.
+__device__ __forceinline__ int node_key(int x) { return x ^ ((x >> (TILE_W_LOG2 - 5)) & 64); }
 
-// As sm_union; a root that gets hooked is appended to a log of the hooked
-// roots (count in *n_hooked), so that only hooked nodes need resolving
-// later.  Entry k goes to hooked_fast[k] (shared memory) for k < fast_cap,
-// else to hooked[k - fast_cap] (capacity cap).
-__device__ __forceinline__ void sm_union_log(int* par, int a, int b, int limit, int* err, int* hooked_fast,
-                                             int fast_cap, int* hooked, int* n_hooked, int cap) {
-  volatile int* vp = par;
-  for (int rounds = 0; rounds <= limit; ++rounds) {
-    sm_find2(vp, a, b, limit, err);
-    if (a == b) return;
-    if (a > b) { const int t = a; a = b; b = t; }
-    const int old = atomicMin(&par[b], a);
-    if (old == b) {
-      const int k = atomicAdd(n_hooked, 1);
-      if (k < fast_cap) hooked_fast[k] = b;
-      else if (k - fast_cap < cap) hooked[k - fast_cap] = b;
-      else set_error(err, SW_ERR_STATE);
-      return;
+// The functions below are called by all 32 lanes of a warp together, each lane
+// with valid nodes (one that has nothing to join or find passes any written
+// node), and loop until every lane is done (a lane that is done reads its root
+// again): uniform branches cost fewer instructions than 32 divergent walks,
+// whose trees are shallow (0.8 steps per find at criticality).  No path
+// compression; hooked roots are resolved at the end.
+
+// The roots of N nodes of every lane, loads in flight together, two steps per
+// vote.  Inside one strip node ids order like sites, so a walk that goes on
+// only while entries decrease ends by itself; across strips the steps are
+// counted, and on overrun (corrupted state) the error word is set and the walk
+// stops.
+constexpr int WALK_LIMIT = TILE_H * TILE_W;   // a tree has fewer nodes
+template <int N>
+__device__ __forceinline__ void sm_find_strip(const uint16_t* par, int (&x)[N]) {
+  bool more;
+  do {
+    int p[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) p[u] = sm_at(par, x[u]);
+    more = false;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      x[u] = sm_at(par, p[u]);
+      more |= x[u] < p[u];
     }
-    b = old;
+  } while (__any_sync(0xFFFFFFFFu, more));
+}
+template <int N>
+__device__ __forceinline__ void sm_find_tile(const uint16_t* par, int (&x)[N], int* err) {
+  for (int steps = 0; steps <= WALK_LIMIT; ++steps) {
+    int p[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) p[u] = sm_at(par, x[u]);
+    bool more = false;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      x[u] = sm_at(par, p[u]);
+      more |= x[u] != p[u];
+    }
+    if (!__any_sync(0xFFFFFFFFu, more)) return;
   }
   set_error(err, SW_ERR_STATE);
+}
+
+// Join every lane's pair (a, b) (a == b: none) where other warps may join
+// theirs at the same time.  The root of the larger site is hooked under the
+// other by a compare-and-swap of the 32-bit word that holds its entry,
+// repeated while only the entry beside it changed (it can be hooked once, so
+// twice at most); if the root itself was hooked meanwhile, its new parent is
+// joined in the next round, so no link is lost.  Every round lowers the larger
+// operand, so at most WALK_LIMIT rounds run.
+__device__ __forceinline__ void sm_union_tile(uint16_t* par, int a, int b, int* err) {
+  for (int rounds = 0; rounds <= WALK_LIMIT; ++rounds) {
+    int x[2] = {a, b};
+    sm_find_tile(par, x, err);
+    a = x[0];
+    b = x[1];
+    if (a != b) {
+      const bool a_first = node_key(a) < node_key(b);
+      const int lo = a_first ? a : b, hi = a_first ? b : a;
+      unsigned* word = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(par) + (hi & ~3));
+      const int sh = 8 * (hi & 2);
+      unsigned old = *reinterpret_cast<volatile unsigned*>(word);
+      a = b = lo;
+      for (;;) {
+        const int cur = (int)((old >> sh) & 0xFFFFu);
+        if (cur != hi) {   // hooked meanwhile
+          b = cur;
+          break;
+        }
+        const unsigned seen = atomicCAS(word, old, old ^ ((unsigned)(lo ^ hi) << sh));
+        if (seen == old) break;
+        old = seen;
+      }
+    }
+    if (!__any_sync(0xFFFFFFFFu, a != b)) return;
+  }
+  set_error(err, SW_ERR_STATE);
+}
+
+// Join every lane's pair (a, b) (a == b: none) in one strip, whose trees no
+// other warp changes meanwhile: no atomics.  In a round every lane finds the
+// roots of its pair, then hooks the larger under the smaller with a plain
+// store, then reads the entry back: of several lanes hooking one root a single
+// one finds its own value and is done, the others go on to join their smaller
+// root with the one that won (1.9 rounds of 1.6 steps on average at
+// criticality).  Returns the root that the lane hooked, or -1 (lanes that
+// stored the same value all name it).
+__device__ __forceinline__ int sm_union_strip(uint16_t* par, int a, int b) {
+  int hooked = -1;
+  do {
+    int x[2] = {a, b};
+    sm_find_strip(par, x);
+    a = min(x[0], x[1]);
+    b = max(x[0], x[1]);
+    __syncwarp();
+    if (a != b) sm_set(par, b, a);
+    __syncwarp();
+    if (a != b) {
+      const int won = sm_at(par, b);
+      if (won == a) hooked = b;
+      b = won;
+    }
+  } while (__any_sync(0xFFFFFFFFu, a != b));
+  return hooked;
+}
+
+// sm_union_strip for pairs whose trees lie in several strips that no other
+// warp touches meanwhile.
+__device__ __forceinline__ int sm_union_strips(uint16_t* par, int a, int b, int* err) {
+  int hooked = -1;
+  for (int rounds = 0; rounds <= WALK_LIMIT; ++rounds) {
+    int x[2] = {a, b};
+    sm_find_tile(par, x, err);
+    const bool first = node_key(x[0]) < node_key(x[1]);
+    a = first ? x[0] : x[1];
+    b = first ? x[1] : x[0];
+    __syncwarp();
+    if (a != b) sm_set(par, b, a);
+    __syncwarp();
+    if (a != b) {
+      const int won = sm_at(par, b);
+      if (won == a) hooked = b;
+      b = won;
+    }
+    if (!__any_sync(0xFFFFFFFFu, a != b)) return hooked;
+  }
+  set_error(err, SW_ERR_STATE);
+  return hooked;
 }
 
 // ---------------------------------------------------------------------------

@@ -28,8 +28,9 @@ static_assert(TILE_W == 64 || TILE_W == 128 || TILE_W == 256, "tile width");
 constexpr int TILE_W_LOG2 = TILE_W == 64 ? 6 : TILE_W == 128 ? 7 : 8;
 constexpr int LABEL_THREADS = TILE_W;
 // Resident CTAs per SM the labeling and flip kernels are built for (the same
-// threads per SM at every tile width).
-constexpr int LABEL_CTAS_PER_SM = 5 * 256 / TILE_W;
+// threads per SM at every tile width).  Labeling: 40 registers a thread; at 5
+// (48 registers) it takes 5 % longer, at 7 it spills.
+constexpr int LABEL_CTAS_PER_SM = 6 * 256 / TILE_W;
 constexpr int FLIP_CTAS_PER_SM = 6 * 256 / TILE_W;
 
 // Per-tile seam record written by the local labeling phase and read by the
@@ -74,8 +75,8 @@ inline Grid make_grid(int H, int W, int periodic) {
 
 // Scratch of one labeling problem.
 struct LabelScratch {
-  int32_t* roots;        // n_tiles * TILE_H * TILE_W: pair lists, then tile-root lists
-  int32_t* work;         // n_tiles * TILE_H * TILE_W: per-tile log of hooked roots
+  int32_t* roots;        // n_tiles * TILE_H * TILE_W: tile-root lists (sweeps: a tile's edge-root bits)
+  int32_t* work;         // n_tiles * TILE_H * TILE_W: stand-alone labeling: 16-bit tile roots
   int32_t* root_counts;  // n_tiles
   int32_t* seams;        // n_tiles * SeamLayout::INTS
   int* err;              // device status word
@@ -95,7 +96,7 @@ struct SwRep {
   uint16_t* lroot;    // L*L tile roots (local index)
   int32_t* gpar;      // L*L parent entries (only edge roots are used)
   int64_t* obs;       // observable ring: obs_cap x (1 + q)
-  LabelScratch s;     // per-tile pair lists, hook logs, seam records, status word
+  LabelScratch s;     // per-tile edge-root bits, seam records, status word
   Grid g;             // L x L, periodic
   uint64_t T, seed;
   int q;
@@ -170,14 +171,13 @@ cudaError_t launch_init_spins_n(int8_t* spins, int64_t n, int q, uint64_t seed, 
 // observables of a sweep are counted by the next sweep's local step, or by
 // launch_observe3 (the last sweep, when they are read).
 Box3 make_box3(int X, int Y, int Z);
-int64_t edge_words3(const Box3& b);     // uint32 words of edge-root bits
-int64_t scratch_ints3(const Box3& b);   // int32 words of labeling scratch (pair lists, hook logs)
-cudaError_t launch_sweep3(int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* edge_words, int32_t* scratch,
-                          const Box3& b, int q, uint64_t T, uint64_t seed, SwCtl* ctl, int64_t* obs, int obs_cap,
-                          cudaStream_t st, cudaEvent_t* ev);
+int64_t brick_words3(const Box3& b);    // uint32 words of edge-root bits and face bonds
+cudaError_t launch_sweep3(int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, const Box3& b, int q,
+                          uint64_t T, uint64_t seed, SwCtl* ctl, int64_t* obs, int obs_cap, cudaStream_t st,
+                          cudaEvent_t* ev);
 cudaError_t launch_observe3(const int8_t* spins, const Box3& b, int q, SwCtl* ctl, int64_t* obs, int obs_cap,
                             cudaStream_t st);
-cudaError_t launch_labels3(const uint16_t* lroot, int32_t* gpar, const uint32_t* edge_words, const Box3& b,
+cudaError_t launch_labels3(const uint16_t* lroot, int32_t* gpar, const uint32_t* words, const Box3& b,
                            int32_t* out, int* err, cudaStream_t st);
 
 cudaError_t launch_tile_label(const uint8_t* mask, int32_t* labels, const Grid& g,

@@ -2,13 +2,12 @@
 // stand-alone labeling kernel (bond mask in memory), the fused
 // Swendsen-Wang kernel (bonds drawn on the fly) and the simple-cubic kernel.
 //
-// Input: the tile's bond bits as 32-bit words, one per row and 32-column
-// strip (be: bit i = east bond of site i of the strip; bn: bit i = its north
-// bond), with bits of sites outside the grid and the east bond of the tile's
-// last column cleared.  Thread (lane, warp) holds the words of row `lane` of
-// strip `warp`.  Output: par[] such that every site's tile root is
-// par[par[site]], the root being the smallest local index of the site's tile
-// component.
+// Input: thread (lane, warp) holds the bond bits of row `lane` of the 32-column
+// strip `warp` (we: bit i = east bond of site i of the strip; wn: bit i = its
+// north bond), with bits of sites outside the grid and the east bond of the
+// tile's last column cleared.  Output: par[] such that a site's tile root is
+// the entry its entry names (root_of), the root being the smallest local index
+// of the site's tile component.
 //
 // A row word is cut into runs of east-joined sites.  Every run is labelled by
 // a union-find node: a run that no north bond from the row below reaches
@@ -24,17 +23,33 @@
 //     pair of runs.
 //  2. warp c sweeps strip c from row 0 upwards, one site per lane, with the
 //     labels of the row below in registers.  A lane finds its run's start
-//     (the highest bit of S at or below it) and its run's anchor (the lowest
-//     bit of F | U from the start on: the first contact, or the start of an
-//     unreached run); the anchor lane's candidate -- the label below it if it
-//     is a first contact, else its own index -- is the run's label (one
-//     shuffle).  No union-find work happens in the sweep.
-//  3. the extra contacts whose two labels differ, and the east bonds from
-//     strip c into strip c + 1, are listed per warp and joined with the
-//     shared-memory union-find (larger root hooked under the smaller);
-//     hooked roots are logged;
-//  4. logged roots resolve their final roots, so every node points at its
-//     root and every site's label (a node) is one step from it.
+//     (the highest bit of S at or below it) and its run's anchor (the one
+//     bit of F | U in the run: the first contact, or the start of an
+//     unreached run; searched in the reversed word, where the lowest bit from
+//     the start on is the highest of the remaining ones); the anchor lane's
+//     candidate -- the label below it if it is a first contact, else its own
+//     index -- is the run's label (one shuffle).  No union-find work happens
+//     in the sweep.
+//  3. the extra contacts are listed per warp and joined with a union-find in
+//     shared memory (larger root hooked under the smaller), 32 at a time;
+//     only the strip's own warp touches its nodes, so plain stores do;
+//  4. after a barrier the east bonds from strip c into strip c + 1 are joined
+//     (at most 32 per strip; compare-and-swap hooks);
+//  5. after a barrier every hooked root takes its final root: the warp's list
+//     and the strip roots of the strip's first and last column (only those can
+//     have been hooked in step 4) cover the strip's nodes, so a warp goes on to
+//     its own strip's sites without another barrier.
+// What bounds the engine is instruction issue (about 70 % of the slots in the
+// fused sweep) and the shared-memory pipe, so: 16-bit entries (six CTAs per SM
+// instead of the five of 32-bit ones) laid out over all 32 banks (local_of;
+// with plain rows the 64-byte strips fall into half of them: 37 against 23
+// million conflicts at L = 8192), no shared atomics inside a strip, find loops
+// with uniform branches and two steps per vote (the divergent form took twice
+// the instructions), and only two barriers where the warps of a tile meet, so
+// that their serial stretches overlap with other warps' arithmetic.  Fused
+// sweep, critical Ising, L = 8192 (8192 tiles): 226 us for the whole labeling
+// kernel against 259 us with 32-bit entries, atomicMin hooks, logged roots and
+// four barriers; 95 us of it are the bond draws.
 // The root is the smallest index of the tile component: the component's
 // smallest site starts a run nothing reaches from below, so it is a node,
 // and a smaller root never hooks under a larger one.
@@ -50,30 +65,51 @@ constexpr int STRIPS = TILE_W / 32;
 static_assert(LABEL_THREADS == TILE_W, "one warp per 32-column strip");
 static_assert(TILE_H == 32, "one lane per row of a strip");
 constexpr unsigned FULL = 0xFFFFFFFFu;
-// Per warp at most 32 pairs per row word: a run's first contact is no extra
-// contact, so a row word of r runs has at most 32 - r <= 31, plus the
-// strip join.
-constexpr int PAIR_CAP = TILE_SITES / STRIPS;
-// Lists kept in shared memory up to these lengths, the rest in global scratch.
-constexpr int PAIR_FAST = 4 * TILE_H;           // per warp (the space of the sweep inputs)
-constexpr int HOOK_FAST = 512;
+constexpr int SWEEP_UNROLL = 16;                // rows of the sweep per loop body (32: no faster, twice the code)
 
-struct TileSmem {
-  alignas(16) int par[TILE_SITES];   // 16-byte aligned: read as int4 when the tile roots are written
-  uint32_t be[TILE_H * STRIPS];   // east bonds, bit = lane of the strip
-  uint32_t bn[TILE_H * STRIPS];   // north bonds
+// ROWS: rows of the tile (32; the simple-cubic bricks have 16).
+template <int ROWS>
+struct TileSmemT {
+  static constexpr int LIST_CAP = 8 * ROWS;     // contacts per warp and pass (the space of the sweep inputs)
+  alignas(16) uint16_t par[ROWS * TILE_W];      // byte offsets (2 x local index); read eight sites at a time
+  uint32_t be[ROWS * STRIPS];                   // east bonds, bit = lane of the strip
+  uint32_t bn[ROWS * STRIPS];                   // north bonds
   union {
-    alignas(16) uint4 rowinfo[STRIPS * TILE_H];   // per row word, strip-major: S, F | U, F (sweep inputs)
-    int pairs[STRIPS * PAIR_FAST];                // then: the warps' first contacts to join
+    alignas(16) uint4 rowinfo[STRIPS * ROWS];   // per row word, strip-major: S, F | U reversed, F (sweep inputs)
+    uint16_t list[STRIPS * LIST_CAP];           // then: the warps' extra contacts to join
   };
-  int hooks[HOOK_FAST];                           // the first hooked roots
   int warp_roots[LABEL_THREADS / 32];
-  int n_hooked;
 };
+using TileSmem = TileSmemT<TILE_H>;
 
 // Global index of local index r of the tile at (y0, x0) of a W-wide grid.
 __device__ __forceinline__ int tile_global(int r, int y0, int x0, int W) {
-  return (y0 + (r >> TILE_W_LOG2)) * W + x0 + (r & (TILE_W - 1));
+  return (y0 + local_y(r)) * W + x0 + local_x(r);
+}
+
+// Halves (16 bits) of x that are zero: bit 15 / bit 31 of the result.  A
+// half is zero iff its low 15 bits plus 0x7FFF stay below bit 15 and its bit
+// 15 is clear.
+__device__ __forceinline__ uint32_t zero_halves(uint32_t x) {
+  return ~(((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x) & 0x80008000u;
+}
+
+// Tile root (local index) of the site with local index i.
+__device__ __forceinline__ int root_of(const uint16_t* par, int i) { return sm_at(par, par[i]) >> 1; }
+
+// The tile roots of eight consecutive sites from local index `sidx` on (a
+// multiple of 8), two per word.
+__device__ __forceinline__ uint4 roots_of(const uint16_t* par, int sidx) {
+  const uint4 v = *reinterpret_cast<const uint4*>(par + sidx);
+  auto two = [&](uint32_t w) { return (uint32_t)sm_at(par, w & 0xFFFFu) >> 1 | (uint32_t)sm_at(par, w >> 16) << 15; };
+  return make_uint4(two(v.x), two(v.y), two(v.z), two(v.w));
+}
+
+// Position of the highest set bit (x != 0).
+__device__ __forceinline__ int high_bit(uint32_t x) {
+  int p;
+  asm("bfind.u32 %0, %1;" : "=r"(p) : "r"(x));
+  return p;
 }
 
 // Inclusive OR of the bits of x towards higher bits inside segments: bit i
@@ -108,16 +144,26 @@ __device__ __forceinline__ uint32_t seg_or_down(uint32_t x, uint32_t j) {
 }
 
 // Runs the engine.  we, wn: the calling thread's row word (row = lane, strip =
-// warp), zero for rows >= h.  sm.be and sm.bn must hold every row word and
-// sm.n_hooked must be zero, followed by a __syncthreads().  `pairs` and
-// `hook_log` (TILE_SITES ints of global scratch each) hold what does not fit
-// in shared memory of the warps' lists of contacts to join and of the hooked
-// roots.  Ends with a __syncthreads().
-__device__ __forceinline__ void tile_engine_regs(TileSmem& sm, uint32_t we, uint32_t wn, int h, int32_t* pairs,
-                                                 int32_t* hook_log, int* err) {
+// warp), zero for rows >= h; w: columns of the tile (strips past them hold no
+// sites and are skipped); rows past h are swept as rows of single sites.  All
+// threads call it.  On return the calling warp's strip is
+// resolved: other strips' roots may be read after a __syncthreads().
+template <int ROWS>
+__device__ __forceinline__ void tile_engine(TileSmemT<ROWS>& sm, uint32_t we, uint32_t wn, int h, int w, int* err) {
+  constexpr int LIST_CAP = TileSmemT<ROWS>::LIST_CAP;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int* par = sm.par;
+  uint16_t* par = sm.par;
   const int colbase = warp * 32;
+  const bool strip = colbase < w;   // same for the whole warp
+  const int row = local_of(lane, colbase);   // my row's first site in the strip
+  uint16_t* list = sm.list + warp * LIST_CAP;
+  int n_list = 0;
+  int ends[2] = {0, 0};             // strip roots of my row's first and last site
+  if (lane < ROWS) {
+    sm.be[lane * STRIPS + warp] = we;
+    sm.bn[lane * STRIPS + warp] = wn;
+  }
+  if (strip) {
   // 1. run structure of my row word against the row below
   uint32_t X;
   {
@@ -131,105 +177,139 @@ __device__ __forceinline__ void tile_engine_regs(TileSmem& sm, uint32_t we, uint
     const uint32_t j2 = we & e_below;                               // joined east in both rows
     const uint32_t before2 = (seg_or_up(c, j2) << 1) & (j2 << 1);
     X = c & ~before2 & ~F;
-    sm.rowinfo[warp * TILE_H + lane] = make_uint4(S, F | U, F, 0u);
+    if (lane < ROWS) sm.rowinfo[warp * ROWS + lane] = make_uint4(S, __brev(F | U), F, 0u);
   }
   __syncwarp();
-  // 2. strip sweep (lane = column)
+  // 2. strip sweep.  Lane l takes column 31 - l: the anchor's column comes out
+  //    as 31 - anchor, the lane to read from.
   {
-    const uint32_t upto = (2u << lane) - 1u;     // bits 0..lane
-    const uint32_t me = 1u << lane;
+    const int col = 31 - lane;
+    const uint32_t upto = FULL >> lane;          // bits 0..col
+    const uint32_t me = 1u << col;
     int lab_below = 0;
-#pragma unroll
-    for (int ly = 0; ly < TILE_H; ++ly) {
-      if (ly < h) {
-        const uint4 ri = sm.rowinfo[warp * TILE_H + ly];
-        const int start = 31 - __clz(ri.x & upto);
-        const int anchor = start + __ffs(ri.y >> start) - 1;
-        const int site = ly * TILE_W + colbase + lane;
-        const int cand = (ri.z & me) ? lab_below : site;
-        const int label = __shfl_sync(FULL, cand, anchor);
-        par[site] = label;
-        lab_below = label;
-      }
+#pragma unroll SWEEP_UNROLL
+    for (int ly = 0; ly < ROWS; ++ly) {
+      const uint4 ri = sm.rowinfo[warp * ROWS + ly];
+      const int start = high_bit(ri.x & upto);
+      const int from = high_bit(ri.y & (FULL >> start));
+      const int site = local_of(ly, colbase) + col;
+      const int cand = (ri.z & me) ? lab_below : 2 * site;
+      const int label = __shfl_sync(FULL, cand, from);
+      par[site] = (uint16_t)label;
+      lab_below = label;
     }
   }
-  __syncthreads();
+  __syncwarp();
 
-  // 3. joins.  The extra contacts of my row (lane = row) whose two labels
-  //    differ (a contact whose runs already carry one label joins nothing
-  //    new), and the east bond of my row from strip c into strip c + 1, are
-  //    listed in the warp's part of `pairs`; then the warp joins its list 32
-  //    pairs at a time.
+  // 3. joins inside the strip: list the sites of the extra contacts of my row
+  //    (lane = row), join the labels on both ends 32 at a time, and leave the
+  //    root that each join hooked in the contact's place.  A strip with more
+  //    contacts than the list holds takes them in several passes.
   {
-    const uint32_t* be = sm.be;
-    const uint32_t* bn = sm.bn;
-    const int row = lane * TILE_W + colbase;
-    uint32_t D = 0u;
-    for (uint32_t x = X; x; x &= x - 1) {
-      const int b = __ffs(x) - 1;
-      if (par[row + b] != par[row - TILE_W + b]) D |= 1u << b;
-    }
-    bool join = false;   // east bond into the next strip, unless joined below
-    if (warp < STRIPS - 1 && lane < h) {
-      const int ly = lane, c = warp;
-      join = (be[ly * STRIPS + c] >> 31) & 1u;
-      if (join && ly > 0) {
-        const int k0 = (ly - 1) * STRIPS + c;
-        if (((be[k0] >> 31) & 1u) && ((bn[k0] >> 31) & 1u) && (bn[k0 + 1] & 1u)) join = false;
-      }
-    }
-    const int cnt = __popc(D) + (join ? 1 : 0);
+    const int cnt = __popc(X);
     int incl = cnt;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const int v = __shfl_up_sync(FULL, incl, d);
       if (lane >= d) incl += v;
     }
-    const int total = __shfl_sync(FULL, incl, 31);   // at most PAIR_CAP
-    int* fast = sm.pairs + warp * PAIR_FAST;
-    int32_t* slow = pairs + warp * PAIR_CAP;
-    __syncwarp();                                 // the warp's sweep inputs are read
-    int k = incl - cnt;
-    for (; D; D &= D - 1, ++k) {
-      const int b = __ffs(D) - 1;
-      const int v = (par[row + b] << 16) | par[row - TILE_W + b];
-      if (k < PAIR_FAST) fast[k] = v;
-      else slow[k - PAIR_FAST] = v;
+    n_list = __shfl_sync(FULL, incl, 31);
+    for (int first = 0; first < n_list; first += LIST_CAP) {
+      int k = incl - cnt - first;
+      for (uint32_t x = X; x; x &= x - 1, ++k)
+        if ((unsigned)k < LIST_CAP) list[k] = (uint16_t)(row + high_bit(x & -x));
+      __syncwarp();
+      const int n = min(n_list - first, LIST_CAP);
+      for (int j = lane; j - lane < n; j += 32) {
+        int a = 2 * colbase, b = a;   // no contact: a node of the own strip (other strips' entries may not be written yet)
+        if (j < n) {
+          const int site = list[j];
+          a = par[site];
+          b = par[(site - TILE_W) ^ 32];   // the site below
+        }
+        const int hooked = sm_union_strip(par, a, b);
+        if (j < n) list[j] = (uint16_t)hooked;   // -1: 0xFFFF, not an offset
+      }
+      __syncwarp();
     }
-    if (join) {
-      const int a = row + 31;   // last column of strip c, row `lane`
-      const int v = (par[a] << 16) | par[a + 1];
-      if (k < PAIR_FAST) fast[k] = v;
-      else slow[k - PAIR_FAST] = v;
-    }
-    __syncwarp();
-    for (int j = lane; j < total; j += 32) {
-      const int v = j < PAIR_FAST ? fast[j] : slow[j - PAIR_FAST];
-      sm_union_log(par, v >> 16, v & 0xFFFF, TILE_SITES, err, sm.hooks, HOOK_FAST, hook_log, &sm.n_hooked,
-                   TILE_SITES);
-    }
+  }
+  // strip roots of my row's ends (lanes past the tile's rows go along with row 0)
+  ends[0] = par[lane < h ? row : colbase];
+  ends[1] = par[lane < h ? row + 31 : colbase];
+  sm_find_strip(par, ends);
   }
   __syncthreads();
 
-  // 4. hooked roots resolve their final roots (every other node is a root)
-  {
-    const int nh = min(sm.n_hooked, TILE_SITES + HOOK_FAST);
-    for (int k = threadIdx.x; k < nh; k += LABEL_THREADS) {
-      const int x = k < HOOK_FAST ? sm.hooks[k] : hook_log[k - HOOK_FAST];
-      const int r = sm_find(par, x, TILE_SITES, err);
-      atomicMin(&par[x], r);
+  // 4. joins between strips: the east bond of my row into the next strip,
+  //    unless the rows below join the same two runs
+  if (warp < STRIPS - 1 && colbase + 32 < w) {
+    bool join = lane < h && (we >> 31);
+    if (join && lane > 0) {
+      const int k0 = (lane - 1) * STRIPS + warp;
+      if ((sm.be[k0] >> 31) && (sm.bn[k0] >> 31) && (sm.bn[k0 + 1] & 1u)) join = false;
     }
+    if (__any_sync(FULL, join))
+      sm_union_tile(par, ends[1], join ? (int)par[local_of(lane, colbase + 32)] : ends[1], err);
   }
   __syncthreads();
+
+  // 5. final roots of the strip's hooked roots; a parent is replaced by an
+  //    ancestor, so other walks through it stay valid
+  if (strip) {
+    int r[2] = {ends[0], ends[1]};
+    sm_find_tile(par, r, err);
+    sm_set(par, ends[0], r[0]);
+    sm_set(par, ends[1], r[1]);
+    if (n_list <= LIST_CAP) {
+      for (int j = lane; j - lane < n_list; j += 32) {
+        const int x = j < n_list ? (int)list[j] : 0xFFFF;
+        int f[1] = {x != 0xFFFF ? x : r[0]};
+        sm_find_tile(par, f, err);
+        if (x != 0xFFFF) sm_set(par, x, f[0]);
+      }
+    } else {   // the list holds the last pass only: every site takes its root
+      for (int ly = 0; ly < h; ++ly) {
+        const int x = 2 * (local_of(ly, colbase) + lane);
+        int f[1] = {x};
+        sm_find_tile(par, f, err);
+        sm_set(par, x, f[0]);
+      }
+    }
+  }
+  __syncwarp();
 }
 
-// The engine with the row words read from sm.be / sm.bn (rows < h filled,
-// and sm.n_hooked zero, before a __syncthreads()).
-__device__ __forceinline__ void tile_engine(TileSmem& sm, int h, int32_t* pairs, int32_t* hook_log, int* err) {
+// The calling warp's part of the tile's seam record after the engine (tile
+// roots on the tile edge, bonds leaving the tile), with the parent entries
+// gpar[g] = g of those roots and their marks in edge_bits (TILE_SITES / 32
+// words, zeroed before the engine).  wn: my row's north bonds; e_last: raw
+// east bits of column w - 1 (bit = row) in the warp that holds that column.
+__device__ __forceinline__ void seam_strip(const TileSmem& sm, int32_t* rec, int32_t* gpar, uint32_t* edge_bits,
+                                           uint32_t wn, uint32_t e_last, int h, int w, int y0, int x0, int W) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool in = lane < h;
-  tile_engine_regs(sm, in ? sm.be[lane * STRIPS + warp] : 0u, in ? sm.bn[lane * STRIPS + warp] : 0u, h, pairs,
-                   hook_log, err);
+  auto edge_root = [&](bool ok, int i) -> int32_t {
+    // global index of the tile root of local site i; the first of a run of
+    // equal roots among consecutive lanes writes its parent entry and its mark
+    const int r = ok ? root_of(sm.par, i) : -1;
+    const int left = __shfl_up_sync(FULL, r, 1);
+    if (!ok) return -1;
+    const int32_t gr = tile_global(r, y0, x0, W);
+    if (lane == 0 || left != r) {
+      gpar[gr] = gr;
+      atomicOr(&edge_bits[r >> 5], 1u << (r & 31));
+    }
+    return gr;
+  };
+  if (warp == 0) rec[SeamLayout::COL_L + lane] = edge_root(lane < h, local_of(lane, 0));
+  if (warp == (w - 1) >> 5) {
+    rec[SeamLayout::COL_R + lane] = edge_root(lane < h, local_of(lane, w - 1));
+    if (lane == 0) rec[SeamLayout::E_BITS] = (int32_t)e_last;
+  }
+  const int lx = 32 * warp + lane;
+  rec[SeamLayout::ROW_B + lx] = edge_root(lx < w, local_of(0, lx));
+  rec[SeamLayout::ROW_T + lx] = edge_root(lx < w, local_of(h - 1, lx));
+  const uint32_t nb = __shfl_sync(FULL, wn, h - 1);
+  if (lane == 0) rec[SeamLayout::N_BITS + warp] = (int32_t)nb;
 }
 
 // ---------------------------------------------------------------------------

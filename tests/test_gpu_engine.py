@@ -1,0 +1,63 @@
+"""GPU parity of the tile engine where its strips are densest: masks whose
+strips have more extra contacts than the engine's list holds (several passes,
+every site resolved), contacts of every row at once, and joins across every
+strip boundary, on whole and ragged tiles of every tile width."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1105_5804_gb300 as sw
+
+pytestmark = pytest.mark.gpu
+
+
+def _mask(kind, H, W, seed):
+    """Bond arrays: `rungs` -- every second row fully joined east, all north
+    bonds open but one in eight (31 contacts in a joined row's strip word, 496
+    in a strip); `dense` -- every bond open with probability 0.9; `stairs` --
+    two-site runs shifted by one from row to row, so that every run touches two
+    runs below."""
+    rng = np.random.default_rng(seed)
+    y, x = np.mgrid[0:H, 0:W]
+    if kind == "rungs":
+        east, north = (y % 2 == 0), rng.random((H, W)) < 0.875
+    elif kind == "dense":
+        east, north = rng.random((H, W)) < 0.9, rng.random((H, W)) < 0.9
+    else:
+        east, north = (x + y) % 2 == 0, rng.random((H, W)) < 0.95
+    return oracle.pack_mask(east.astype(np.uint8).reshape(-1), north.astype(np.uint8).reshape(-1))
+
+
+@pytest.mark.parametrize("tile_w", sw.TILE_WIDTHS)
+@pytest.mark.parametrize("H,W", [(32, 32), (33, 64), (64, 256), (97, 290), (160, 513)])
+@pytest.mark.parametrize("kind", ["rungs", "dense", "stairs"])
+def test_labels_of_dense_strips(tile_w, H, W, kind):
+    L = sw.lib(tile_w)
+    mask = _mask(kind, H, W, H * 1000 + W)
+    dev = torch.from_numpy(mask).cuda()
+    for periodic in (0, 1):
+        ref, _ = oracle.label(mask, H, W, bool(periodic))
+        lab = torch.full((H * W,), -7, dtype=torch.int32, device="cuda")
+        rc = L.ccl_label(ctypes.c_void_p(dev.data_ptr()), ctypes.c_void_p(lab.data_ptr()), H, W, periodic, None)
+        assert rc == 0, L.sw_last_error()
+        torch.cuda.synchronize()
+        sw.ccl_status()
+        assert np.array_equal(lab.cpu().numpy(), ref), periodic
+
+
+@pytest.mark.parametrize("off", [1, 2, 4])
+def test_labels_of_an_unaligned_mask(off):
+    """A mask that starts 1, 2 or 4 bytes past an aligned address (byte loads,
+    and 32-bit loads that are not 64-bit aligned), rows of odd and even width."""
+    for H, W in [(40, 96), (37, 131), (5, 257)]:
+        mask = oracle.perc_mask(H, W, 3)
+        buf = torch.zeros(mask.size + 8, dtype=torch.uint8, device="cuda")
+        buf[off:off + mask.size] = torch.from_numpy(mask).cuda()
+        lab = torch.full((H * W,), -7, dtype=torch.int32, device="cuda")
+        sw.ccl_label(buf[off:off + mask.size], lab, H, W, True)
+        sw.ccl_status()
+        ref, _ = oracle.label(mask, H, W, True)
+        assert np.array_equal(lab.cpu().numpy(), ref), (H, W)
