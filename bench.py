@@ -39,20 +39,20 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "b5eab634facdf9da"
+SWEEP_COUNTER_HASH = "043e07cc93a5365b"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
-    "k_sw_label": ((89.068544 + 135.476224) * 1e6 / 67108864, 183656856 / 67108864),
-    "k_merge": ((68.810496 + 1.408512) * 1e6 / 67108864, 20486034 / 67108864),
-    "k_sw_flip": ((203.594752 + 51.161600) * 1e6 / 67108864, 89248935 / 67108864),
+    "k_sw_label": ((88.869888 + 130.657024) * 1e6 / 67108864, 183791414 / 67108864),
+    "k_merge": ((56.285952 + 0.717568) * 1e6 / 67108864, 14835682 / 67108864),
+    "k_sw_flip": ((203.558400 + 47.656192) * 1e6 / 67108864, 70964935 / 67108864),
 }
 # The stand-alone labeling call (k_ccl_tile, k_merge, k_ccl_final), one ncu
 # capture per kernel of a 4096^2 critical percolation mask: DRAM bytes per site,
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "affc40caa765774f"
+CCL_COUNTER_HASH = "2a92a73c54077569"
 CCL_COUNTER_TILE_W = 128
-CCL_TRAFFIC_BYTES_PER_SITE = ((7.892992 + 6.620416) + (19.919616 + 0.000256) + (59.143424 + 10.010368)) * 1e6 / 16777216
+CCL_TRAFFIC_BYTES_PER_SITE = ((7.877632 + 6.576640) + (16.628992 + 0.000256) + (59.144704 + 10.124800)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8
 # spins once (2 B, the minimum of any sweep); the kernel split adds the
 # 16-bit tile roots written by k_sw_label and read by k_sw_flip (6 B).

@@ -250,8 +250,8 @@ uint64_t sw_prob_threshold(double p);
  * F_q of word 0) and the observables (n_eq over the 3N bonds, then n_k) are
  * as on the square lattice.  Hot start: INIT draw of site i as in 2D.
  * Requires X, Y, Z >= 1 with X*Y*Z <= 2^30, 2 <= q <= 127, T <= 2^32.  The
- * library owns the device memory: about 23 bytes per site (spins, brick
- * roots, parent array, labeling scratch) plus the observable ring.  NULL on failure (see sw_last_error).  Each sweep is
+ * library owns the device memory: about 7.2 bytes per site (spins, brick
+ * roots, parent array, edge and face bits) plus the observable ring.  NULL on failure (see sw_last_error).  Each sweep is
  * three kernels (brick-local union-find with the previous sweep's
  * observables, face merge, flip) and a counter advance, replayed as a
  * captured CUDA graph unless timing is on. */

@@ -224,10 +224,12 @@ struct LabelTileSmem {
   int hist[128];
 };
 
+constexpr int FLIP_LIST = TILE_SITES / 4;           // roots listed per pass (at criticality a tile has 0.14 per site)
+
 struct FlipTileSmem {
-  uint16_t rlist[TILE_SITES];   // the tile's roots (EDGE_ROOT flag on edge roots)
+  uint4 roots[TILE_SITES / 8];  // the tile roots of every thread's sites (pass-major, thread by thread)
   uint8_t ns[TILE_SITES];       // new state, indexed by local root
-  uint32_t edge_bits[EDGE_WORDS];
+  uint16_t rlist[FLIP_LIST];    // the tile's roots, edge roots first
   int warp_cnt[LABEL_THREADS / 32];
 };
 
@@ -304,7 +306,10 @@ __device__ __forceinline__ void sw_label_tile(const SwRep& R, int t, uint64_t sw
   // 3. tile roots of my strip as 16-bit local indices: per step a thread
   //    takes eight consecutive sites (four threads a row) and stores 16
   //    bytes, or two halves where rows start only 8-byte aligned (L % 4 == 0;
-  //    w is a multiple of 4, so four sites are all inside or all outside)
+  //    w is a multiple of 4, so four sites are all inside or all outside).
+  //    Streaming stores: the roots are read once, after the merge, and leave
+  //    L2 to spins, seam records and parents (L = 16384: this kernel 0.892 ->
+  //    0.858 ms)
   {
     const int lx = 32 * warp + 8 * (lane & 3);
 #pragma unroll 2
@@ -313,7 +318,7 @@ __device__ __forceinline__ void sw_label_tile(const SwRep& R, int t, uint64_t sw
       const uint4 r = roots_of(sm.par, local_of(ly, lx));
       uint16_t* dst = lroot + (int64_t)(y0 + ly) * L + x0 + lx;
       if ((L & 7) == 0) {   // then w is a multiple of 8 too
-        *reinterpret_cast<uint4*>(dst) = r;
+        __stcs(reinterpret_cast<uint4*>(dst), r);
       } else {
         *reinterpret_cast<uint2*>(dst) = make_uint2(r.x, r.y);
         if (lx + 8 <= w) *reinterpret_cast<uint2*>(dst + 4) = make_uint2(r.z, r.w);
@@ -347,134 +352,203 @@ __device__ __forceinline__ int root_in(const uint4& v, int i) {
   return (int)((wv >> (16 * (i & 1))) & 0xFFFFu);
 }
 
-// The pass words of the calling thread.
-struct RootsInRegs {
-  uint4 r4[FLIP_PASSES];
-  __device__ __forceinline__ uint4 get(int j) const { return r4[j]; }
-};
-// Steps 2-5 of the flip of tile t (see k_fused.cu) given the tile roots of
-// the calling thread's sites.  All threads of the CTA call it; it ends with a
-// barrier.
+// 16 bytes from global memory (through L2) to shared memory, asynchronously.
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Bit i of x (i < 16) to bit 2i.
+__device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
+  x = (x | (x << 8)) & 0x00FF00FFu;
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  return (x | (x << 1)) & 0x55555555u;
+}
+
+// The flip of tile t (see k_fused.cu).  All threads of the CTA call it; it
+// ends with a barrier.
 // FEW: the few-cluster update (Sec. III, variant (c)).  Only clusters whose
 // global root has its bit set in `sel` (seeded clusters) move: with FLIP draw
 // w of the root, iff (uint64)w.y < P, to state (s + 1 + F_{q-1}(w.x)) mod q,
 // s being the cluster's current state (read at the tile root).
-template <bool FEW, class Roots, class Keys>
-__device__ __forceinline__ void flip_tile_core(const SwRep& R, int t, uint64_t sweep, int limit, FlipTileSmem& fs,
-                                               const Roots& roots, const uint32_t* __restrict__ sel, uint64_t P,
-                                               const Keys& keys) {
+// The tile roots wait in shared memory for the site pass (held in registers
+// across the draws they spill at six CTAs per SM, read again through L2 they
+// cost its traffic twice).  Edge roots, whose cluster root has to be found on
+// gpar, come first in the list, so that each of the first threads has one walk
+// whose first load is in flight while the thread draws its interior roots.
+// Bound by instruction issue (74 % of the slots, 1.03 warp instructions per
+// site, a third of them the draws); critical Ising, L = 16384: 0.298 ms against
+// 0.389 ms with the roots read twice, flags looked up root by root and four
+// walks per thread in step.
+template <bool FEW = false, class Keys = SeedKey>
+__device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t sweep, int limit, FlipTileSmem& fs,
+                                             const Keys& keys, const uint32_t* __restrict__ sel = nullptr,
+                                             uint64_t P = 0) {
   constexpr int PASSES = FLIP_PASSES;
-  uint16_t* rlist = fs.rlist;
   uint8_t* ns = fs.ns;
-  int* warp_cnt = fs.warp_cnt;
   int8_t* __restrict__ spins = R.spins;
   int32_t* __restrict__ gpar = R.gpar;
-  const Grid& g = R.g;
   const int q = R.q;
   int* err = R.s.err;
-  const int L = g.W;
-  const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
+  const int L = R.g.W;
+  const int ty = t / R.g.tiles_x, tx = t - ty * R.g.tiles_x;
   const int y0 = ty * TILE_H, x0 = tx * TILE_W;
   const int h = min(TILE_H, L - y0), w = min(TILE_W, L - x0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int orow = threadIdx.x / FLIP_GROUPS, lx0 = 8 * (threadIdx.x % FLIP_GROUPS);   // my sites
-  // the tile's edge-root bits, left by the labeling kernel
-  fs.edge_bits[threadIdx.x] = (uint32_t)__ldcg(R.s.roots + (int64_t)t * TILE_SITES + threadIdx.x);
+
+  // 1. tile roots of my sites into shared memory (0xFFFF outside the tile; w
+  //    is a multiple of 4: a group of eight sites is wholly inside, or its
+  //    first four are; 16-byte loads need L % 8 == 0, 8-byte ones L % 4 == 0).
+  //    Read through L2 because a persistent kernel wrote them on other SMs.
+  uint4* const my_roots = fs.roots + threadIdx.x;   // pass j: my_roots[j LABEL_THREADS]
+  const int id0 = local_of(orow, lx0);              // local index of my first site; pass j: id0 + 8 j TILE_W
+  uint32_t edges = 0u;   // bit 8j + i: edge-root bit of site i of pass j
+  {
+    const uint8_t* eb = reinterpret_cast<const uint8_t*>(R.s.roots + (int64_t)t * TILE_SITES) + (id0 >> 3);
+    const uint16_t* src = R.lroot + (int64_t)(y0 + orow) * L + x0 + lx0;
+    const int64_t step = (int64_t)8 * L;
+#pragma unroll
+    for (int j = 0; j < PASSES; ++j) edges |= (uint32_t)__ldcg(eb + j * TILE_W) << (8 * j);
+    if ((L & 7) == 0 && h == TILE_H && lx0 < w) {   // w is a multiple of 8
+#pragma unroll
+      for (int j = 0; j < PASSES; ++j) copy16_async(my_roots + j * LABEL_THREADS, src + j * step);
+      copies_wait();   // a thread reads back only what it copied itself
+    } else {
+#pragma unroll
+      for (int j = 0; j < PASSES; ++j) {
+        uint4 v = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+        if (8 * j + orow < h && lx0 < w) {
+          const uint2 a = __ldcg(reinterpret_cast<const uint2*>(src + j * step));
+          v.x = a.x;
+          v.y = a.y;
+          if (lx0 + 8 <= w) {
+            const uint2 c = __ldcg(reinterpret_cast<const uint2*>(src + j * step + 4));
+            v.z = c.x;
+            v.w = c.y;
+          }
+        }
+        my_roots[j * LABEL_THREADS] = v;
+      }
+    }
+  }
 
   // 2. my roots: a site is a tile root iff its entry is its own local index.
   //    Word k of pass j holds sites 2k and 2k + 1; both are compared at once.
-  //    Sites outside the tile hold 0xFFFF and never match.  Bit 4j + k of `mine` flags site 2k of pass j, bit
-  //    16 + 4j + k site 2k + 1.
-  uint32_t mine = 0;
+  //    Bit 8j + i of mine flags site i of pass j.
+  uint32_t mine;
+  {
+    uint32_t m = 0;   // bit 4j + k: site 2k of pass j, bit 16 + 4j + k: site 2k + 1
 #pragma unroll
-  for (int j = 0; j < PASSES; ++j) {
-    const uint4 rv = roots.get(j);
-    const uint32_t base = (uint32_t)local_of(8 * j + orow, lx0);
-    const uint32_t own = base * 0x00010001u + 0x00010000u;   // (base, base + 1)
-    const uint32_t wv[4] = {rv.x, rv.y, rv.z, rv.w};
+    for (int j = 0; j < PASSES; ++j) {
+      const uint4 rv = my_roots[j * LABEL_THREADS];
+      const uint32_t own = (uint32_t)(id0 + 8 * j * TILE_W) * 0x00010001u + 0x00010000u;   // (site, site + 1)
+      const uint32_t wv[4] = {rv.x, rv.y, rv.z, rv.w};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint32_t x = wv[k] ^ (own + (uint32_t)k * 0x00020002u);
-      mine |= zero_halves(x) >> (15 - (4 * j + k));
+      for (int k = 0; k < 4; ++k) m |= zero_halves(wv[k] ^ (own + (uint32_t)k * 0x00020002u)) >> (15 - (4 * j + k));
     }
+    mine = spread_bits(m & 0xFFFFu) | spread_bits(m >> 16) << 1;
   }
-  const int cnt = __popc(mine);
+  const uint32_t on_edge = mine & edges;
+  const uint32_t inner = mine & ~edges;
+
+  // 3. the tile's root list: edge roots, then the others (counts of both in
+  //    one scan; a tile with more roots than the list holds takes several
+  //    passes)
+  const int cnt = __popc(on_edge) << 16 | __popc(inner);
   int incl = cnt;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const int v = __shfl_up_sync(FULL, incl, d);
     if (lane >= d) incl += v;
   }
-  if (lane == 31) warp_cnt[warp] = incl;
+  if (lane == 31) fs.warp_cnt[warp] = incl;
   __syncthreads();
-  int base = 0, n_roots = 0;
+  int before = incl - cnt, total = 0;
 #pragma unroll
   for (int k = 0; k < LABEL_THREADS / 32; ++k) {
-    base += (k < warp) ? warp_cnt[k] : 0;
-    n_roots += warp_cnt[k];
+    before += (k < warp) ? fs.warp_cnt[k] : 0;
+    total += fs.warp_cnt[k];
   }
-  base += incl - cnt;
-  while (mine) {   // the tile's root list, edge roots flagged
-    const int b = __ffs(mine) - 1;
-    mine &= mine - 1;
-    const int jk = b & 15;
-    const int r = local_of(8 * (jk >> 2) + orow, lx0) + 2 * (jk & 3) + (b >> 4);
-    rlist[base++] = (uint16_t)r | (((fs.edge_bits[r >> 5] >> (r & 31)) & 1u) ? EDGE_ROOT : (uint16_t)0);
-  }
-  __syncthreads();
+  const int n_edge = total >> 16, n_roots = n_edge + (total & 0xFFFF);
+  const int at_edge = before >> 16, at_inner = n_edge + (before & 0xFFFF);
 
-  // 4. one draw per tile root, keyed by its cluster's final root; a thread
-  //    takes its roots two at a time, their parent walks in lock step
-  constexpr int U = 2;
-  for (int k0 = threadIdx.x; k0 < n_roots; k0 += U * LABEL_THREADS) {
-    int r[U], Rg[U];
-    bool act[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int k = k0 + u * LABEL_THREADS;
-      const int raw = k < n_roots ? (int)rlist[k] : 0;
-      r[u] = raw & ROOT_MASK;
-      Rg[u] = tile_global(r[u], y0, x0, L);
-      act[u] = k < n_roots && (raw & EDGE_ROOT);
-    }
-    g_find_multi<U>(gpar, Rg, act, limit, err);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (k0 + u * LABEL_THREADS >= n_roots) break;
-      if (FEW) {
-        // the cluster's current state, read at the tile root (this tile's own
-        // site: step 5 rewrites it only after a barrier)
-        int v = spins[(uint32_t)tile_global(r[u], y0, x0, L)];
-        if ((__ldcg(sel + (Rg[u] >> 5)) >> (Rg[u] & 31)) & 1u) {
-          const uint4 d =
-              philox_draw(make_uint4((uint32_t)Rg[u], (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
-          if ((uint64_t)d.y < P) v = (v + 1 + state_of(d.x, q - 1)) % q;
-        }
-        ns[r[u]] = (uint8_t)v;
-      } else {
-        const uint4 d =
-            philox_draw(make_uint4((uint32_t)Rg[u], (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
-        ns[r[u]] = (uint8_t)state_of(d.x, q);
+  auto set_state = [&](int r, int G) {   // new state of the component with local root r and cluster root G
+    if (FEW) {
+      // the cluster's current state, read at the tile root (this tile's own
+      // site: the site pass rewrites it only after a barrier)
+      int v = spins[(uint32_t)tile_global(r, y0, x0, L)];
+      if ((__ldcg(sel + (G >> 5)) >> (G & 31)) & 1u) {
+        const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
+        if ((uint64_t)d.y < P) v = (v + 1 + state_of(d.x, q - 1)) % q;
       }
+      ns[r] = (uint8_t)v;
+    } else {
+      const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
+      ns[r] = (uint8_t)state_of(d.x, q);
     }
+  };
+
+  for (int first = 0; first < n_roots; first += FLIP_LIST) {
+    // my roots as local indices id0 + (site of a pass) + 8 (pass) TILE_W
+    auto list = [&](uint32_t bits, int at, bool fits) {
+      while (bits) {
+        const int n = high_bit(bits);
+        bits ^= 1u << n;
+        if (fits || (unsigned)at < FLIP_LIST) fs.rlist[at] = (uint16_t)(id0 + n + (n & 24) * (TILE_W - 1));
+        ++at;
+      }
+    };
+    if (n_roots <= FLIP_LIST) {
+      list(on_edge, at_edge, true);
+      list(inner, at_inner, true);
+    } else {
+      list(on_edge, at_edge - first, false);
+      list(inner, at_inner - first, false);
+    }
+    __syncthreads();
+
+    // 4. one draw per tile root, keyed by its cluster's final root
+    const int n = min(n_roots - first, FLIP_LIST), ne = min(max(n_edge - first, 0), n);
+    const int k0 = threadIdx.x;
+    int r0 = 0, x = 0, p = 0;
+    if (k0 < n) {
+      r0 = fs.rlist[k0];
+      p = x = tile_global(r0, y0, x0, L);
+      if (k0 < ne) p = g_load(gpar + x);
+    }
+    for (int k = k0 + LABEL_THREADS; k < n; k += LABEL_THREADS) {
+      const int r = fs.rlist[k];
+      int G = tile_global(r, y0, x0, L);
+      if (k < ne) G = g_find(gpar, G, limit, err);
+      set_state(r, G);
+    }
+    if (k0 < n) set_state(r0, p == x ? x : g_find_from(gpar, x, p, limit, err));
+    __syncthreads();
   }
-  __syncthreads();
 
   // 5. every site takes its tile root's state
+  int8_t* dst = spins + (int64_t)(y0 + orow) * L + x0 + lx0;
+  if (lx0 < w) {
 #pragma unroll
-  for (int j = 0; j < PASSES; ++j) {
-    const int ly = 8 * j + orow;
-    if (ly >= h || lx0 + 4 > w) continue;
-    const uint4 rv = roots.get(j);
-    uint32_t lo = 0, hi = 0;
+    for (int j = 0; j < PASSES; ++j, dst += (int64_t)8 * L) {
+      if (8 * j + orow >= h) break;
+      const uint4 rv = my_roots[j * LABEL_THREADS];
+      uint32_t lo = 0, hi = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) lo |= (uint32_t)ns[root_in(rv, i)] << (8 * i);
-    int8_t* dst = spins + (int64_t)(y0 + ly) * L + x0 + lx0;
-    *reinterpret_cast<uint32_t*>(dst) = lo;   // 4-byte aligned: L % 4 == 0
-    if (lx0 + 8 <= w) {
+      for (int i = 0; i < 4; ++i) lo |= (uint32_t)ns[root_in(rv, i)] << (8 * i);
+      if ((L & 7) == 0 || lx0 + 8 <= w) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) hi |= (uint32_t)ns[root_in(rv, 4 + i)] << (8 * i);
-      *reinterpret_cast<uint32_t*>(dst + 4) = hi;
+        for (int i = 0; i < 4; ++i) hi |= (uint32_t)ns[root_in(rv, 4 + i)] << (8 * i);
+      }
+      if ((L & 7) == 0) {
+        *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);
+      } else {
+        *reinterpret_cast<uint32_t*>(dst) = lo;   // 4-byte aligned: L % 4 == 0
+        if (lx0 + 8 <= w) *reinterpret_cast<uint32_t*>(dst + 4) = hi;
+      }
     }
   }
   __syncthreads();
@@ -526,149 +600,6 @@ __device__ __forceinline__ void observe_tile(const SwRep& R, int t, uint64_t don
   __syncthreads();
 }
 
-
-// The flip of tile t with the tile roots loaded into registers (one CTA per
-// tile; also the batch kernels).
-template <bool FEW = false, class Keys = SeedKey>
-__device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t sweep, int limit, FlipTileSmem& fs,
-                                             const Keys& keys, const uint32_t* __restrict__ sel = nullptr,
-                                             uint64_t P = 0) {
-  const uint16_t* __restrict__ lroot = R.lroot;
-  const int L = R.g.W;
-  const int ty = t / R.g.tiles_x, tx = t - ty * R.g.tiles_x;
-  const int y0 = ty * TILE_H, x0 = tx * TILE_W;
-  const int h = min(TILE_H, L - y0), w = min(TILE_W, L - x0);
-  const int orow = threadIdx.x / FLIP_GROUPS, lx0 = 8 * (threadIdx.x % FLIP_GROUPS);   // my sites
-  // 1. tile roots of my sites (w is a multiple of 4: a group of eight sites is
-  //    either wholly inside, or its first four are); read through L2 because a
-  //    persistent kernel wrote them on other SMs
-  RootsInRegs roots;
-#pragma unroll
-  for (int j = 0; j < FLIP_PASSES; ++j) {
-    const int ly = 8 * j + orow;
-    const uint16_t* src = lroot + (int64_t)(y0 + ly) * L + x0 + lx0;
-    uint4 v = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
-    // 16-byte loads need L % 8 == 0; L % 4 == 0 always allows 8-byte loads
-    if (ly < h && lx0 + 8 <= w) {
-      if ((L & 7) == 0) {
-        v = __ldcg(reinterpret_cast<const uint4*>(src));
-      } else {
-        const uint2 a = __ldcg(reinterpret_cast<const uint2*>(src)), b = __ldcg(reinterpret_cast<const uint2*>(src + 4));
-        v = make_uint4(a.x, a.y, b.x, b.y);
-      }
-    } else if (ly < h && lx0 + 4 <= w) {
-      const uint2 a = __ldcg(reinterpret_cast<const uint2*>(src));
-      v.x = a.x;
-      v.y = a.y;
-    }
-    roots.r4[j] = v;
-  }
-  flip_tile_core<FEW>(R, t, sweep, limit, fs, roots, sel, P, keys);
-}
-
-// The flip of tile t when every tile of the lattice is whole (L a multiple
-// of TILE_W, TILE_H and 8): the steps of flip_tile_core with no bounds
-// checks, and the tile roots of the calling thread's sites read through L2
-// twice (root discovery, site pass) instead of held in registers across
-// the draws, which would not fit the register budget of six CTAs per SM.
-template <class Keys>
-__device__ __forceinline__ void sw_flip_whole_tile(const SwRep& R, int t, uint64_t sweep, int limit,
-                                                   FlipTileSmem& fs, const Keys& keys) {
-  constexpr int PASSES = FLIP_PASSES;
-  const int L = R.g.W;
-  const int ty = t / R.g.tiles_x, tx = t - ty * R.g.tiles_x;
-  const int y0 = ty * TILE_H, x0 = tx * TILE_W;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int orow = threadIdx.x / FLIP_GROUPS, lx0 = 8 * (threadIdx.x % FLIP_GROUPS);   // my sites
-  const uint16_t* src0 = R.lroot + (int64_t)(y0 + orow) * L + x0 + lx0;   // pass 0; 16-byte aligned
-  const int64_t pass_stride = (int64_t)8 * L;
-  uint16_t* rlist = fs.rlist;
-  uint8_t* ns = fs.ns;
-  int* warp_cnt = fs.warp_cnt;
-  fs.edge_bits[threadIdx.x] = (uint32_t)__ldcg(R.s.roots + (int64_t)t * TILE_SITES + threadIdx.x);
-
-  // 2. my roots (as in flip_tile_core)
-  uint32_t mine = 0;
-  {
-    uint4 held[PASSES];
-#pragma unroll
-    for (int j = 0; j < PASSES; ++j) held[j] = __ldcg(reinterpret_cast<const uint4*>(src0 + j * pass_stride));
-#pragma unroll
-    for (int j = 0; j < PASSES; ++j) {
-      const uint4 rv = held[j];
-      const uint32_t base = (uint32_t)local_of(8 * j + orow, lx0);
-      const uint32_t own = base * 0x00010001u + 0x00010000u;
-      const uint32_t wv[4] = {rv.x, rv.y, rv.z, rv.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t x = wv[k] ^ (own + (uint32_t)k * 0x00020002u);
-        mine |= zero_halves(x) >> (15 - (4 * j + k));
-      }
-    }
-  }
-  const int cnt = __popc(mine);
-  int incl = cnt;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const int v = __shfl_up_sync(FULL, incl, d);
-    if (lane >= d) incl += v;
-  }
-  if (lane == 31) warp_cnt[warp] = incl;
-  __syncthreads();
-  int base = 0, n_roots = 0;
-#pragma unroll
-  for (int k = 0; k < LABEL_THREADS / 32; ++k) {
-    base += (k < warp) ? warp_cnt[k] : 0;
-    n_roots += warp_cnt[k];
-  }
-  base += incl - cnt;
-  while (mine) {   // 3. the tile's root list, edge roots flagged
-    const int b = __ffs(mine) - 1;
-    mine &= mine - 1;
-    const int jk = b & 15;
-    const int r = local_of(8 * (jk >> 2) + orow, lx0) + 2 * (jk & 3) + (b >> 4);
-    rlist[base++] = (uint16_t)r | (((fs.edge_bits[r >> 5] >> (r & 31)) & 1u) ? EDGE_ROOT : (uint16_t)0);
-  }
-  __syncthreads();
-
-  // 4. one draw per tile root, keyed by its cluster's final root
-  constexpr int U = 4;   // four walks of a thread in flight (flip_tile_core, with the roots in registers, keeps two)
-  for (int k0 = threadIdx.x; k0 < n_roots; k0 += U * LABEL_THREADS) {
-    int r[U], Rg[U];
-    bool act[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int k = k0 + u * LABEL_THREADS;
-      const int raw = k < n_roots ? (int)rlist[k] : 0;
-      r[u] = raw & ROOT_MASK;
-      Rg[u] = tile_global(r[u], y0, x0, L);
-      act[u] = k < n_roots && (raw & EDGE_ROOT);
-    }
-    g_find_multi<U>(R.gpar, Rg, act, limit, R.s.err);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (k0 + u * LABEL_THREADS >= n_roots) break;
-      const uint4 d =
-          philox_draw(make_uint4((uint32_t)Rg[u], (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
-      ns[r[u]] = (uint8_t)state_of(d.x, R.q);
-    }
-  }
-  __syncthreads();
-
-  // 5. every site takes its tile root's state (tile roots read again)
-#pragma unroll
-  for (int j = 0; j < PASSES; ++j) {
-    const int ly = 8 * j + orow;
-    const uint4 rv = __ldcg(reinterpret_cast<const uint4*>(src0 + j * pass_stride));
-    uint32_t lo = 0, hi = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) lo |= (uint32_t)ns[root_in(rv, i)] << (8 * i);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) hi |= (uint32_t)ns[root_in(rv, 4 + i)] << (8 * i);
-    int8_t* dst = R.spins + (int64_t)(y0 + ly) * L + x0 + lx0;
-    *reinterpret_cast<uint2*>(dst) = make_uint2(lo, hi);   // 8-byte aligned: L % 8 == 0
-  }
-}
 
 // ---------------------------------------------------------------------------
 // Few-cluster seed selection (Sec. III, variant (c)): the seed of block b of

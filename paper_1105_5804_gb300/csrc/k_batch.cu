@@ -79,7 +79,7 @@ __device__ __forceinline__ bool grid_barrier(BatchCtl* ctl, unsigned nblocks, lo
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// Phase kernels: one CTA per global tile (merge: one thread per seam bond).
+// Phase kernels: one CTA per global tile (merge: per few tiles).
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_batch_label(BatchView b, const BatchCtl* __restrict__ ctl) {
   __shared__ LabelTileSmem ls;
   const uint64_t sweep = ctl->sweep;
@@ -89,12 +89,15 @@ __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_batch_labe
   sw_label_tile(R, gt - R.tile0, sweep, do_obs, b.obs_cap, ls, SeedKey{(uint32_t)R.seed, (uint32_t)(R.seed >> 32)});
 }
 
-constexpr int BATCH_MERGE_THREADS = MERGE_PER_TILE;   // one CTA per tile
-
-__global__ void __launch_bounds__(BATCH_MERGE_THREADS) k_batch_merge(BatchView b) {
-  const int gt = blockIdx.x;
-  const SwRep& R = b.reps[b.tile_rep[gt]];
-  merge_seam_bond(R.gpar, R.g, R.s, gt - R.tile0, threadIdx.x, true, b.limit);
+__global__ void __launch_bounds__(MERGE_PER_TILE) k_batch_merge(BatchView b, int per) {
+  __shared__ MergeSmem ms;
+  const int gt0 = blockIdx.x * per;
+  merge_tiles(ms, min(per, b.n_tiles - gt0),
+              [&](int u) {
+                const SwRep& R = b.reps[b.tile_rep[gt0 + u]];
+                return MergeTile{&R.g, R.gpar, R.s.seams, R.s.err, gt0 + u - R.tile0};
+              },
+              b.limit);
 }
 
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM) k_batch_flip(BatchView b, const BatchCtl* __restrict__ ctl) {
@@ -142,7 +145,7 @@ __global__ void __launch_bounds__(LABEL_THREADS, 4 * 256 / TILE_W) k_batch_persi
          unit += (int64_t)nb * WARPS) {
       const int gt = (int)(unit / WPT), part = (int)(unit - (int64_t)gt * WPT);
       const SwRep& R = b.reps[b.tile_rep[gt]];
-      merge_seam_bond(R.gpar, R.g, R.s, gt - R.tile0, part * 32 + (threadIdx.x & 31), true, b.limit);
+      merge_seam_bond(R.gpar, R.g, R.s, gt - R.tile0, part * 32 + (threadIdx.x & 31), b.limit);
     }
   }
   if (!grid_barrier(ctl, nb, limit_cycles)) return;
@@ -162,7 +165,8 @@ cudaError_t launch_batch_label(const BatchView& b, BatchCtl* ctl, cudaStream_t s
 }
 
 cudaError_t launch_batch_merge(const BatchView& b, cudaStream_t st) {
-  k_batch_merge<<<b.n_tiles, BATCH_MERGE_THREADS, 0, st>>>(b);
+  const int per = merge_tiles_per_cta(b.n_tiles);
+  k_batch_merge<<<(b.n_tiles + per - 1) / per, MERGE_PER_TILE, 0, st>>>(b, per);
   return cudaGetLastError();
 }
 

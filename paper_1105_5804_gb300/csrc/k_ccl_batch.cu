@@ -28,10 +28,15 @@ __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_cclb_tile(
   ccl_label_tile<true>(J.mask, J.labels, J.g, J.s, gt - J.tile0, sm);
 }
 
-__global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_constant__ CclBatchView v) {
-  const int gt = blockIdx.x;
-  const CclJob& J = v.jobs[job_of_tile(v, gt)];
-  merge_seam_bond(J.labels, J.g, J.s, gt - J.tile0, threadIdx.x, true, v.limit);
+__global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_constant__ CclBatchView v, int per) {
+  __shared__ MergeSmem ms;
+  const int gt0 = blockIdx.x * per;
+  merge_tiles(ms, min(per, v.n_tiles - gt0),
+              [&](int u) {
+                const CclJob& J = v.jobs[job_of_tile(v, gt0 + u)];
+                return MergeTile{&J.g, J.labels, J.s.seams, J.s.err, gt0 + u - J.tile0};
+              },
+              v.limit);
 }
 
 __global__ void __launch_bounds__(256) k_cclb_final(const __grid_constant__ CclBatchView v) {
@@ -44,7 +49,8 @@ __global__ void __launch_bounds__(256) k_cclb_final(const __grid_constant__ CclB
 cudaError_t launch_ccl_batch(const CclBatchView& v, cudaStream_t st) {
   if (v.n_tiles == 0) return cudaSuccess;
   k_cclb_tile<<<v.n_tiles, LABEL_THREADS, 0, st>>>(v);
-  k_cclb_merge<<<v.n_tiles, MERGE_PER_TILE, 0, st>>>(v);
+  const int per = merge_tiles_per_cta(v.n_tiles);
+  k_cclb_merge<<<(v.n_tiles + per - 1) / per, MERGE_PER_TILE, 0, st>>>(v, per);
   k_cclb_final<<<v.n_tiles, 256, 0, st>>>(v);
   return cudaGetLastError();
 }

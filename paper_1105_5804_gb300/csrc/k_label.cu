@@ -16,8 +16,8 @@
 //                 minimum site index); roots are appended to a per-tile list,
 //                 and the labels and bond bits of the four tile edges go to a
 //                 compact seam record.
-//  k_merge        one thread per bond leaving a tile (the periodic wrap
-//                 included, Sec. II.C): union of the two tile roots on the
+//  k_merge        the bonds leaving a tile (the periodic wrap included,
+//                 Sec. II.C): union of the two tile roots on the
 //                 global label array with atomicMin hooking.  A lane whose
 //                 root pair equals its left neighbour's skips the union, so
 //                 consecutive seam bonds of one cluster cost one union.
@@ -78,25 +78,20 @@ cudaError_t launch_ccl(const uint8_t* mask, int32_t* labels, const Grid& g, cons
 }
 
 // ---------------------------------------------------------------------------
-// Seam merge: thread k of tile t handles east seam bond k (k < TILE_H) or
-// north seam bond k - TILE_H.
+// Seam merge: one CTA per `per` consecutive tiles (merge_tiles).
 // ---------------------------------------------------------------------------
-constexpr int MERGE_THREADS = 256;
-
-__global__ void __launch_bounds__(MERGE_THREADS)
-k_merge(int32_t* __restrict__ labels, Grid g, LabelScratch s, int limit) {
-  const int64_t gid = blockIdx.x * (int64_t)MERGE_THREADS + threadIdx.x;
-  const int64_t total = (int64_t)g.n_tiles() * MERGE_PER_TILE;
-  if (gid - (threadIdx.x & 31) >= total) return;   // whole warp past the end
-  const int t = (int)(gid / MERGE_PER_TILE);
-  merge_seam_bond(labels, g, s, t, (int)(gid - (int64_t)t * MERGE_PER_TILE), gid < total, limit);
+__global__ void __launch_bounds__(MERGE_PER_TILE)
+k_merge(int32_t* __restrict__ labels, const __grid_constant__ Grid g, LabelScratch s, int per, int limit) {
+  __shared__ MergeSmem ms;
+  const int t0 = blockIdx.x * per;
+  merge_tiles(ms, min(per, g.n_tiles() - t0), [&](int u) { return MergeTile{&g, labels, s.seams, s.err, t0 + u}; },
+              limit);
 }
 
 cudaError_t launch_merge(int32_t* labels, const Grid& g, const LabelScratch& s, cudaStream_t st) {
-  const int64_t total = (int64_t)g.n_tiles() * MERGE_PER_TILE;
-  const int64_t blocks = (total + MERGE_THREADS - 1) / MERGE_THREADS;
+  const int per = merge_tiles_per_cta(g.n_tiles());
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
-  k_merge<<<(unsigned)blocks, MERGE_THREADS, 0, st>>>(labels, g, s, limit);
+  k_merge<<<(unsigned)((g.n_tiles() + per - 1) / per), MERGE_PER_TILE, 0, st>>>(labels, g, s, per, limit);
   return cudaGetLastError();
 }
 

@@ -267,17 +267,20 @@ __device__ __forceinline__ int sm_union_strips(uint16_t* par, int a, int b, int*
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int g_load(const int* p) { return __ldcg(p); }
 
-__device__ __forceinline__ int g_find(int* lab, int x, int limit, int* err) {
-  int p = g_load(lab + x);
+__device__ __forceinline__ int g_find_from(int* lab, int x, int p, int limit, int* err) {   // p: the loaded parent of x
   int steps = 0;
   while (p != x) {
     const int gp = g_load(lab + p);
-    if (gp != p) atomicMin(lab + x, gp);   // path halving, decreasing only (see sm_find)
+    if (gp != p) atomicMin(lab + x, gp);   // path halving; entries only ever decrease
     x = p;
     p = gp;
     if (++steps > limit) { set_error(err, SW_ERR_STATE); return x; }
   }
   return x;
+}
+
+__device__ __forceinline__ int g_find(int* lab, int x, int limit, int* err) {
+  return g_find_from(lab, x, g_load(lab + x), limit, err);
 }
 
 // g_find of up to U nodes at once (those with act[u] set): the walks run in

@@ -29,9 +29,10 @@ constexpr int TILE_W_LOG2 = TILE_W == 64 ? 6 : TILE_W == 128 ? 7 : 8;
 constexpr int LABEL_THREADS = TILE_W;
 // Resident CTAs per SM the labeling and flip kernels are built for (the same
 // threads per SM at every tile width).  Labeling: 40 registers a thread; at 5
-// (48 registers) it takes 5 % longer, at 7 it spills.
+// (48 registers) it takes 5 % longer, at 7 it spills.  Flip: 36 registers and
+// 29 KB of shared memory (6 CTAs: equal at L = 8192, q = 2, 1 % slower at q = 4).
 constexpr int LABEL_CTAS_PER_SM = 6 * 256 / TILE_W;
-constexpr int FLIP_CTAS_PER_SM = 6 * 256 / TILE_W;
+constexpr int FLIP_CTAS_PER_SM = 7 * 256 / TILE_W;
 
 // Per-tile seam record written by the local labeling phase and read by the
 // merge: labels of the four tile edges and the raw bond bits leaving the

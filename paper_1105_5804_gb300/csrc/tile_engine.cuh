@@ -318,56 +318,133 @@ __device__ __forceinline__ void seam_strip(const TileSmem& sm, int32_t* rec, int
 // included.  If it is open, the two tile roots on its ends are joined on the
 // global array `gpar` (atomicMin hooking, larger root under the smaller).  A
 // lane whose root pair equals its left neighbour's skips the union, so runs
-// of seam bonds of one cluster cost one union.  All 32 lanes of a warp must
-// call together (active == false for lanes past the end); MERGE_PER_TILE is
-// a multiple of 32, so a warp never spans two tiles.  Seam records are read
-// through L2 (ld.cg): in a persistent kernel they were written by other SMs.
+// of seam bonds of one cluster cost one union.  MERGE_PER_TILE is a multiple of
+// 32, so a warp never spans two tiles.
 constexpr int MERGE_PER_TILE = TILE_H + TILE_W;
 static_assert(MERGE_PER_TILE % 32 == 0, "warps must not straddle tiles");
 
+// The bond's bit and the roots at both ends, loaded together (the neighbour
+// index wraps, so the loads stay inside the records even where the bond does
+// not exist; then has is false).  Seam records are read through L2 (ld.cg): in
+// a persistent kernel they were written by other SMs.
+struct SeamBond {
+  uint32_t bits;
+  int a, b;
+  bool has;
+};
+__device__ __forceinline__ SeamBond load_seam_bond(const Grid& g, const int32_t* seams, int t, int k) {
+  const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
+  const int32_t* rec = seams + (int64_t)t * SeamLayout::INTS;
+  SeamBond s;
+  int tn, i_bits, i_a, i_b;
+  if (k < TILE_H) {
+    s.has = g.periodic || tx + 1 < g.tiles_x;
+    tn = ty * g.tiles_x + (tx + 1 == g.tiles_x ? 0 : tx + 1);
+    i_bits = SeamLayout::E_BITS;
+    i_a = SeamLayout::COL_R + k;
+    i_b = SeamLayout::COL_L + k;
+  } else {
+    const int lx = k - TILE_H;
+    s.has = g.periodic || ty + 1 < g.tiles_y;
+    tn = (ty + 1 == g.tiles_y ? 0 : ty + 1) * g.tiles_x + tx;
+    i_bits = SeamLayout::N_BITS + (lx >> 5);
+    i_a = SeamLayout::ROW_T + lx;
+    i_b = SeamLayout::ROW_B + lx;
+  }
+  s.bits = (uint32_t)__ldcg(rec + i_bits);
+  s.a = __ldcg(rec + i_a);
+  s.b = __ldcg(seams + (int64_t)tn * SeamLayout::INTS + i_b);
+  return s;
+}
+static_assert(TILE_H == 32, "bond k's bit is bit k % 32 of its word");
+
+// Whether the calling lane has to join (lo, hi); all 32 lanes call together.
+__device__ __forceinline__ bool seam_pair(const SeamBond& s, int k, int& lo, int& hi) {
+  const bool valid = s.has && ((s.bits >> (k & 31)) & 1u) && s.a != s.b;
+  lo = min(s.a, s.b);
+  hi = max(s.a, s.b);
+  const unsigned long long key = valid ? ((unsigned long long)(unsigned)lo << 32) | (unsigned)hi : ~0ull;
+  const unsigned long long left = __shfl_up_sync(FULL, key, 1);
+  return valid && ((threadIdx.x & 31) == 0 || left != key);
+}
+
+// Join lo < hi on gpar, trying the hook before any walk: most larger roots are
+// still roots, and an entry that was hooked already is lowered if lo is
+// smaller, its old parent then joined with lo as after a lost race.
+__device__ __forceinline__ void seam_join(int32_t* gpar, int lo, int hi, int limit, int* err) {
+  const int old = atomicMin(gpar + hi, lo);
+  if (old != hi && old != lo) g_union(gpar, lo, old, limit, err);
+}
+
+// One bond per lane (the persistent batch kernel; all 32 lanes call together).
 __device__ __forceinline__ void merge_seam_bond(int32_t* gpar, const Grid& g, const LabelScratch& s, int t, int k,
-                                                bool active, int limit) {
-  int a = -1, b = -1;
-  bool valid = false;
-  if (active) {
-    // the bond's bit and the roots at both ends are loaded together (the
-    // neighbour index wraps, so the loads stay inside the records even
-    // where the bond does not exist), then the bit decides
-    const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-    const int32_t* rec = s.seams + (int64_t)t * SeamLayout::INTS;
-    bool has;
-    int tn, i_bits, i_a, i_b, bit;
-    if (k < TILE_H) {
-      has = g.periodic || tx + 1 < g.tiles_x;
-      tn = ty * g.tiles_x + (tx + 1 == g.tiles_x ? 0 : tx + 1);
-      i_bits = SeamLayout::E_BITS + (k >> 5);
-      i_a = SeamLayout::COL_R + k;
-      i_b = SeamLayout::COL_L + k;
-      bit = k & 31;
-    } else {
-      const int lx = k - TILE_H;
-      has = g.periodic || ty + 1 < g.tiles_y;
-      tn = (ty + 1 == g.tiles_y ? 0 : ty + 1) * g.tiles_x + tx;
-      i_bits = SeamLayout::N_BITS + (lx >> 5);
-      i_a = SeamLayout::ROW_T + lx;
-      i_b = SeamLayout::ROW_B + lx;
-      bit = lx & 31;
-    }
-    const uint32_t bits = (uint32_t)__ldcg(rec + i_bits);
-    const int ra = __ldcg(rec + i_a);
-    const int rb = __ldcg(s.seams + (int64_t)tn * SeamLayout::INTS + i_b);
-    if (has && ((bits >> bit) & 1u)) {
-      a = ra;
-      b = rb;
-      valid = true;
+                                                int limit) {
+  int lo, hi;
+  if (seam_pair(load_seam_bond(g, s.seams, t, k), k, lo, hi)) seam_join(gpar, lo, hi, limit, s.err);
+}
+
+// The seam bonds of n <= MERGE_TILES consecutive tiles by one CTA of
+// MERGE_PER_TILE threads (thread = bond): every thread loads its bond of all
+// the tiles at once, the pairs to join (about one bond in six at criticality)
+// go to a list, and the list is joined with all lanes busy.  With a union per
+// lane where it stands, a warp ran its divergent walks for five lanes of 32:
+// bound by the latency of the parent loads and by issue, 157 us at L = 16384
+// against XXX us.  tile_of(u): grid, parents and scratch of tile u.
+constexpr int MERGE_TILES = 2;
+struct MergeSmem {
+  int2 pairs[MERGE_TILES * MERGE_PER_TILE];
+  uint8_t tile[MERGE_TILES * MERGE_PER_TILE];
+  int n;
+};
+struct MergeTile {
+  const Grid* g;
+  int32_t* gpar;
+  const int32_t* seams;
+  int* err;
+  int t;
+};
+template <class TileOf>
+__device__ __forceinline__ void merge_tiles(MergeSmem& ms, int n, const TileOf& tile_of, int limit) {
+  const int k = threadIdx.x, lane = threadIdx.x & 31;
+  if (k == 0) ms.n = 0;
+  SeamBond bond[MERGE_TILES];
+#pragma unroll
+  for (int u = 0; u < MERGE_TILES; ++u) {
+    bond[u].has = false;
+    if (u < n) {
+      const MergeTile m = tile_of(u);
+      bond[u] = load_seam_bond(*m.g, m.seams, m.t, k);
     }
   }
-  valid = valid && a != b;
-  const unsigned long long key =
-      valid ? ((unsigned long long)(unsigned)min(a, b) << 32) | (unsigned)max(a, b) : ~0ull;
-  const unsigned long long prev = __shfl_up_sync(FULL, key, 1);
-  const bool leader = (threadIdx.x & 31) == 0 || prev != key;
-  if (valid && leader) g_union(gpar, a, b, limit, s.err);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < MERGE_TILES; ++u) {
+    if (u >= n) break;
+    int lo, hi;
+    const bool join = seam_pair(bond[u], k, lo, hi);
+    const uint32_t m = __ballot_sync(FULL, join);
+    if (m == 0u) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(&ms.n, __popc(m));
+    at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
+    if (join) {
+      ms.pairs[at] = make_int2(lo, hi);
+      ms.tile[at] = (uint8_t)u;
+    }
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < ms.n; j += MERGE_PER_TILE) {
+    const MergeTile m = tile_of(ms.tile[j]);
+    seam_join(m.gpar, ms.pairs[j].x, ms.pairs[j].y, limit, m.err);
+  }
+}
+
+// Tiles per CTA of a merge over n_tiles tiles: two where their bonds fill the
+// GPU's 152 x 2048 threads more than once, one below (latency of one wave:
+// L = 2048 13.2 against 13.9 us, L = 4096 19.4 against 16.6; three to six tiles
+// are 2 % better at L = 16384 and up to 60 % worse at 4096).
+inline int merge_tiles_per_cta(int64_t n_tiles) {
+  return n_tiles * MERGE_PER_TILE > (int64_t)152 * 2048 ? MERGE_TILES : 1;
 }
 
 }  // namespace swccl

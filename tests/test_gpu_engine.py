@@ -61,3 +61,24 @@ def test_labels_of_an_unaligned_mask(off):
         sw.ccl_status()
         ref, _ = oracle.label(mask, H, W, True)
         assert np.array_equal(lab.cpu().numpy(), ref), (H, W)
+
+
+@pytest.mark.parametrize("tile_w,W", [(256, 6801), (128, 6500), (64, 6410)])
+@pytest.mark.parametrize("rows", [41, 40])
+def test_merge_with_several_tiles_per_block(tile_w, W, rows):
+    """Grids just above the size where a merge block takes two tiles, with an
+    odd and an even number of tiles, ragged in both directions."""
+    H = rows * 32 - 5
+    n_tiles = rows * ((W + tile_w - 1) // tile_w)
+    assert n_tiles * (32 + tile_w) > 152 * 2048
+    L = sw.lib(tile_w)
+    mask = oracle.perc_mask(H, W, rows)
+    dev = torch.from_numpy(mask).cuda()
+    lab = torch.full((H * W,), -7, dtype=torch.int32, device="cuda")
+    for periodic in (0, 1):
+        rc = L.ccl_label(ctypes.c_void_p(dev.data_ptr()), ctypes.c_void_p(lab.data_ptr()), H, W, periodic, None)
+        assert rc == 0, L.sw_last_error()
+        torch.cuda.synchronize()
+        sw.ccl_status()
+        ref, _ = oracle.label(mask, H, W, bool(periodic))
+        assert np.array_equal(lab.cpu().numpy(), ref), periodic
