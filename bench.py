@@ -39,20 +39,20 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "043e07cc93a5365b"
+SWEEP_COUNTER_HASH = "5586470ab5ccf522"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
-    "k_sw_label": ((88.869888 + 130.657024) * 1e6 / 67108864, 183791414 / 67108864),
-    "k_merge": ((56.285952 + 0.717568) * 1e6 / 67108864, 14835682 / 67108864),
-    "k_sw_flip": ((203.558400 + 47.656192) * 1e6 / 67108864, 70964935 / 67108864),
+    "k_sw_label": ((88.865536 + 130.616064) * 1e6 / 67108864, 184025928 / 67108864),
+    "k_merge": ((56.335360 + 0.713984) * 1e6 / 67108864, 15158671 / 67108864),
+    "k_sw_flip": ((203.547392 + 48.124160) * 1e6 / 67108864, 71156542 / 67108864),
 }
 # The stand-alone labeling call (k_ccl_tile, k_merge, k_ccl_final), one ncu
 # capture per kernel of a 4096^2 critical percolation mask: DRAM bytes per site,
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "2a92a73c54077569"
+CCL_COUNTER_HASH = "f8a115ec97125295"
 CCL_COUNTER_TILE_W = 128
-CCL_TRAFFIC_BYTES_PER_SITE = ((7.877632 + 6.576640) + (16.628992 + 0.000256) + (59.144704 + 10.124800)) * 1e6 / 16777216
+CCL_TRAFFIC_BYTES_PER_SITE = ((7.881216 + 6.681856) + (16.647424 + 0.000000) + (59.144448 + 10.003456)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8
 # spins once (2 B, the minimum of any sweep); the kernel split adds the
 # 16-bit tile roots written by k_sw_label and read by k_sw_flip (6 B).
@@ -825,7 +825,7 @@ def run_ours(args):
                    "timed_path": "sw_sweep replaying one captured CUDA graph per sweep; the per-kernel split comes "
                                  "from a separate pass of %d eagerly launched sweeps with events" % PHASE_SWEEPS},
         "clocks": clk,
-        "gpu_launches": 4 * args.steps,
+        "gpu_launches": 3 * args.steps,
         "e2e": {"value": e2e_value, "unit": "site-updates/ns", "h2d_bytes_per_step": N,
                 "d2h_bytes_per_step": N + 8 * (q + 1), "steps": e2e_steps,
                 "synchronous_value": world * N * e2e_steps / (te_sync * 1e9) if e2e_steps else None,

@@ -6,7 +6,7 @@
 // sweep (draw + label, seam merge, flip) over all tiles of all chains:
 //
 //  * phases: one launch per step over the global tile list (CUDA graph of
-//    four kernels per sweep); kernel boundaries order the steps;
+//    three kernels per sweep); kernel boundaries order the steps;
 //  * persistent: one cooperative launch per sweep.  Each CTA walks the
 //    global tile list step by step; a grid barrier separates the steps.  The
 //    barrier's wait is bounded: if it does not complete within the time
@@ -27,7 +27,8 @@ __device__ __forceinline__ bool batch_do_obs(const BatchCtl* ctl, uint64_t sweep
 }
 
 // Zero the observable slot of sweep s of every chain (the next sweep's draw
-// step, or the observe kernel, fills it), then advance.  One CTA.
+// step, or the observe kernel, fills it), then advance.  One CTA; the steps after
+// it in the sweep count from the advanced counter.
 __device__ __forceinline__ void batch_advance_block(const BatchView& b, BatchCtl* ctl, uint64_t s) {
   for (int r = 0; r < b.n_reps; ++r) {
     const SwRep& R = b.reps[r];
@@ -82,6 +83,7 @@ __device__ __forceinline__ bool grid_barrier(BatchCtl* ctl, unsigned nblocks, lo
 // Phase kernels: one CTA per global tile (merge: per few tiles).
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_batch_label(BatchView b, const BatchCtl* __restrict__ ctl) {
   __shared__ LabelTileSmem ls;
+  wait_for_previous();
   const uint64_t sweep = ctl->sweep;
   const bool do_obs = batch_do_obs(ctl, sweep);
   const int gt = blockIdx.x;
@@ -89,8 +91,10 @@ __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_batch_labe
   sw_label_tile(R, gt - R.tile0, sweep, do_obs, b.obs_cap, ls, SeedKey{(uint32_t)R.seed, (uint32_t)(R.seed >> 32)});
 }
 
-__global__ void __launch_bounds__(MERGE_PER_TILE) k_batch_merge(BatchView b, int per) {
+__global__ void __launch_bounds__(MERGE_PER_TILE) k_batch_merge(BatchView b, BatchCtl* ctl, int per) {
   __shared__ MergeSmem ms;
+  wait_for_previous();
+  if (blockIdx.x == 0) batch_advance_block(b, ctl, ctl->sweep);   // the next draw step fills this sweep's slots
   const int gt0 = blockIdx.x * per;
   merge_tiles(ms, min(per, b.n_tiles - gt0),
               [&](int u) {
@@ -102,12 +106,11 @@ __global__ void __launch_bounds__(MERGE_PER_TILE) k_batch_merge(BatchView b, int
 
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM) k_batch_flip(BatchView b, const BatchCtl* __restrict__ ctl) {
   __shared__ FlipTileSmem fs;
+  wait_for_previous();
   const int gt = blockIdx.x;
   const SwRep& R = b.reps[b.tile_rep[gt]];
-  sw_flip_tile(R, gt - R.tile0, ctl->sweep, b.limit, fs, SeedKey{(uint32_t)R.seed, (uint32_t)(R.seed >> 32)});
+  sw_flip_tile(R, gt - R.tile0, ctl->sweep - 1, b.limit, fs, SeedKey{(uint32_t)R.seed, (uint32_t)(R.seed >> 32)});
 }
-
-__global__ void k_batch_advance(BatchView b, BatchCtl* ctl) { batch_advance_block(b, ctl, ctl->sweep); }
 
 __global__ void __launch_bounds__(LABEL_THREADS) k_batch_observe(BatchView b, BatchCtl* ctl) {
   __shared__ LabelTileSmem ls;
@@ -160,24 +163,16 @@ __global__ void __launch_bounds__(LABEL_THREADS, 4 * 256 / TILE_W) k_batch_persi
 
 // ---------------------------------------------------------------------------
 cudaError_t launch_batch_label(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
-  k_batch_label<<<b.n_tiles, LABEL_THREADS, 0, st>>>(b, ctl);
-  return cudaGetLastError();
+  return launch_after(k_batch_label, b.n_tiles, LABEL_THREADS, st, b, ctl);
 }
 
-cudaError_t launch_batch_merge(const BatchView& b, cudaStream_t st) {
+cudaError_t launch_batch_merge(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
   const int per = merge_tiles_per_cta(b.n_tiles);
-  k_batch_merge<<<(b.n_tiles + per - 1) / per, MERGE_PER_TILE, 0, st>>>(b, per);
-  return cudaGetLastError();
+  return launch_after(k_batch_merge, (unsigned)((b.n_tiles + per - 1) / per), MERGE_PER_TILE, st, b, ctl, per);
 }
 
 cudaError_t launch_batch_flip(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
-  k_batch_flip<<<b.n_tiles, LABEL_THREADS, 0, st>>>(b, ctl);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_batch_advance(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
-  k_batch_advance<<<1, 128, 0, st>>>(b, ctl);
-  return cudaGetLastError();
+  return launch_after(k_batch_flip, b.n_tiles, LABEL_THREADS, st, b, ctl);
 }
 
 cudaError_t launch_batch_observe(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {

@@ -23,6 +23,8 @@ __device__ __forceinline__ int job_of_tile(const CclBatchView& v, int gt) {
 
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_cclb_tile(const __grid_constant__ CclBatchView v) {
   __shared__ CclTileSmem sm;
+  wait_for_previous();
+  let_next_start();
   const int gt = blockIdx.x;
   const CclJob& J = v.jobs[job_of_tile(v, gt)];
   ccl_label_tile<true>(J.mask, J.labels, J.g, J.s, gt - J.tile0, sm);
@@ -30,6 +32,8 @@ __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_cclb_tile(
 
 __global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_constant__ CclBatchView v, int per) {
   __shared__ MergeSmem ms;
+  wait_for_previous();
+  let_next_start();
   const int gt0 = blockIdx.x * per;
   merge_tiles(ms, min(per, v.n_tiles - gt0),
               [&](int u) {
@@ -41,6 +45,7 @@ __global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_cons
 
 __global__ void __launch_bounds__(256) k_cclb_final(const __grid_constant__ CclBatchView v) {
   __shared__ int32_t table[TILE_SITES];
+  wait_for_previous();
   const int gt = blockIdx.x;
   const CclJob& J = v.jobs[job_of_tile(v, gt)];
   final_labels_tile(J.labels, J.g, J.s, gt - J.tile0, table, v.limit);
@@ -48,11 +53,12 @@ __global__ void __launch_bounds__(256) k_cclb_final(const __grid_constant__ CclB
 
 cudaError_t launch_ccl_batch(const CclBatchView& v, cudaStream_t st) {
   if (v.n_tiles == 0) return cudaSuccess;
-  k_cclb_tile<<<v.n_tiles, LABEL_THREADS, 0, st>>>(v);
+  cudaError_t e = launch_after(k_cclb_tile, v.n_tiles, LABEL_THREADS, st, v);
+  if (e != cudaSuccess) return e;
   const int per = merge_tiles_per_cta(v.n_tiles);
-  k_cclb_merge<<<(v.n_tiles + per - 1) / per, MERGE_PER_TILE, 0, st>>>(v, per);
-  k_cclb_final<<<v.n_tiles, 256, 0, st>>>(v);
-  return cudaGetLastError();
+  e = launch_after(k_cclb_merge, (unsigned)((v.n_tiles + per - 1) / per), MERGE_PER_TILE, st, v, per);
+  if (e != cudaSuccess) return e;
+  return launch_after(k_cclb_final, v.n_tiles, 256, st, v);
 }
 
 }  // namespace swccl

@@ -7,7 +7,7 @@
 // Philox call per site (tag BOND3, counter (i, sweep), word = direction) and
 // open iff the two spins are equal and the word is below T (Eq. 7).
 //
-// One sweep is three kernels and an advance, the structure of the fused
+// One sweep is three kernels, the structure of the fused
 // square-lattice sweep (k_fused.cu) carried to bricks of 32 x 8 x 16 sites:
 //  k3_local    one CTA per brick: draws the bonds of its sites, labels every
 //              (x, z) plane of the brick with the square-lattice tile engine
@@ -152,6 +152,7 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
   uint16_t* par = sm.par;
   const Brick k = brick_of(b, blockIdx.x);
   const int lane = threadIdx.x & 31, ly = threadIdx.x >> 5;
+  wait_for_previous();
   const uint64_t sweep = ctl->sweep;
   const bool do_obs = sweep > 0 && ctl->obs_done != (long long)(sweep - 1);
   const bool plane = ly < k.h;               // the warp has a plane
@@ -456,7 +457,15 @@ constexpr int MERGE3_THREADS = 256;
 
 __global__ void __launch_bounds__(MERGE3_THREADS)
 k3_merge(const uint16_t* __restrict__ lroot, int32_t* gpar, const uint32_t* __restrict__ words, Box3 b, int limit,
-         int* err) {
+         SwCtl* ctl, int64_t* obs, int obs_cap, int q) {
+  wait_for_previous();
+  int* err = &ctl->err;
+  if (blockIdx.x == 0) {   // the next sweep's local step fills this sweep's observable slot
+    const uint64_t s = ctl->sweep;
+    if ((int)threadIdx.x <= q) obs[(int64_t)(s % (uint64_t)obs_cap) * (q + 1) + threadIdx.x] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) ctl->sweep = s + 1;
+  }
   const int64_t unit = blockIdx.x * (int64_t)(MERGE3_THREADS / 32) + (threadIdx.x >> 5);
   if (unit >= b.n_bricks() * B3_MERGE_UNITS) return;
   const int t = (int)(unit / B3_MERGE_UNITS), u = (int)(unit - (int64_t)t * B3_MERGE_UNITS);
@@ -511,7 +520,8 @@ k3_flip(int8_t* __restrict__ spins, const uint16_t* __restrict__ lroot, int32_t*
   __shared__ uint32_t edge[B3_EDGE_WORDS];
   __shared__ int warp_cnt[B3_THREADS / 32];
   const Brick k = brick_of(b, blockIdx.x);
-  const uint64_t sweep = ctl->sweep;
+  wait_for_previous();
+  const uint64_t sweep = ctl->sweep - 1;   // the merge has advanced the counter
   const int lane = threadIdx.x & 31, ly = threadIdx.x >> 5, warp = ly;
   const int lx0 = 8 * (lane & 3);
   const int in = ly < k.h ? min(max(k.w - lx0, 0), 8) : 0;
@@ -669,15 +679,6 @@ k3_observe(const int8_t* __restrict__ spins, Box3 b, int q, SwCtl* __restrict__ 
   if (blockIdx.x == 0 && threadIdx.x == 0) ctl->obs_done = (long long)done;
 }
 
-// End of a sweep: clear the observable slot of the sweep just done (the next
-// sweep's k3_local, or k3_observe, fills it), then advance the counter.
-__global__ void k3_advance(SwCtl* ctl, int64_t* obs, int obs_cap, int q) {
-  const uint64_t s = ctl->sweep;
-  if ((int)threadIdx.x <= q) obs[(int64_t)(s % (uint64_t)obs_cap) * (q + 1) + threadIdx.x] = 0;
-  __syncthreads();
-  if (threadIdx.x == 0) ctl->sweep = s + 1;
-}
-
 // Canonical labels of the last sweep: the cluster root of every site's brick root.
 __global__ void k3_labels(const uint16_t* __restrict__ lroot, int32_t* gpar, const uint32_t* __restrict__ words,
                           Box3 b, int32_t* out, int limit, int* err) {
@@ -722,23 +723,23 @@ cudaError_t launch_sweep3(int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_
   int* err = &ctl->err;
   if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
   const PhiloxKeys keys = philox_keys(seed);
-  k3_local<<<(unsigned)b.n_bricks(), B3_THREADS, 0, st>>>(spins, lroot, gpar, words, b, q, T, keys, ctl, obs, obs_cap,
-                                                          err);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch_after(k3_local, (unsigned)b.n_bricks(), B3_THREADS, st, spins, lroot, gpar, words, b, q, T, keys, ctl, obs,
+                   obs_cap, err);
+  if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
-  if (b.bx > 1 || b.by > 1 || b.bz > 1) {
-    constexpr int WARPS = MERGE3_THREADS / 32;
-    const int64_t blocks = (b.n_bricks() * B3_MERGE_UNITS + WARPS - 1) / WARPS;
-    k3_merge<<<(unsigned)blocks, MERGE3_THREADS, 0, st>>>(lroot, gpar, words, b, limit3(b), err);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+  // a box of one brick has no face bonds: one block only advances the counter
+  constexpr int WARPS = MERGE3_THREADS / 32;
+  const bool faces = b.bx > 1 || b.by > 1 || b.bz > 1;
+  const int64_t blocks = faces ? (b.n_bricks() * B3_MERGE_UNITS + WARPS - 1) / WARPS : 1;
+  e = launch_after(k3_merge, (unsigned)blocks, MERGE3_THREADS, st, lroot, gpar, words, b, limit3(b), ctl, obs, obs_cap, q);
+  if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
-  k3_flip<<<(unsigned)b.n_bricks(), B3_THREADS, 0, st>>>(spins, lroot, gpar, words, b, q, keys, ctl, limit3(b), err);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
-  k3_advance<<<1, 128, 0, st>>>(ctl, obs, obs_cap, q);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (ev && (e = cudaEventRecord(ev[4], st)) != cudaSuccess) return e;
+  e = launch_after(k3_flip, (unsigned)b.n_bricks(), B3_THREADS, st, spins, lroot, gpar, words, b, q, keys, ctl, limit3(b),
+                   err);
+  if (e != cudaSuccess) return e;
+  // the advance is part of the merge: its phase is empty
+  if (ev && ((e = cudaEventRecord(ev[3], st)) != cudaSuccess || (e = cudaEventRecord(ev[4], st)) != cudaSuccess))
+    return e;
   return cudaSuccess;
 }
 

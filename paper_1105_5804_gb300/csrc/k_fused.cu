@@ -38,6 +38,7 @@ namespace swccl {
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
 k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys) {
   __shared__ LabelTileSmem ls;
+  wait_for_previous();
   const uint64_t sweep = ctl->sweep;
   const bool do_obs = sweep > 0 && ctl->obs_done != (long long)(sweep - 1);
   sw_label_tile(R, blockIdx.x, sweep, do_obs, obs_cap, ls, keys);
@@ -46,14 +47,16 @@ k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_con
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
 k_sw_flip(SwRep R, const SwCtl* __restrict__ ctl, int limit, const __grid_constant__ PhiloxKeys keys) {
   __shared__ FlipTileSmem fs;
-  sw_flip_tile(R, blockIdx.x, ctl->sweep, limit, fs, keys);
+  wait_for_previous();
+  sw_flip_tile(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys);   // the merge has advanced the counter
 }
 
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
 k_sw_flip_few(SwRep R, const SwCtl* __restrict__ ctl, int limit, const uint32_t* __restrict__ sel, uint64_t P,
               const __grid_constant__ PhiloxKeys keys) {
   __shared__ FlipTileSmem fs;
-  sw_flip_tile<true>(R, blockIdx.x, ctl->sweep, limit, fs, keys, sel, P);
+  wait_for_previous();
+  sw_flip_tile<true>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys, sel, P);
 }
 
 constexpr int SELECT_THREADS = 256;
@@ -61,7 +64,7 @@ constexpr int SELECT_THREADS = 256;
 __global__ void __launch_bounds__(SELECT_THREADS)
 k_few_select(SwRep R, const SwCtl* __restrict__ ctl, int ell, uint32_t* sel, int limit) {
   const int64_t b = blockIdx.x * (int64_t)SELECT_THREADS + threadIdx.x;   // one thread per seed
-  if (b < (int64_t)ell * ell) few_select_seed(R, ell, b, ctl->sweep, sel, limit);
+  if (b < (int64_t)ell * ell) few_select_seed(R, ell, b, ctl->sweep - 1, sel, limit);
 }
 
 // ---------------------------------------------------------------------------
@@ -110,15 +113,6 @@ k_observe(const int8_t* __restrict__ spins, int L, int q, SwCtl* __restrict__ ct
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) ctl->obs_done = (long long)done;
 }
 
-// End of a fused sweep: clear the observable slot of the sweep just done
-// (the next sweep's k_sw_label, or k_observe, fills it) and advance.
-__global__ void k_advance_fused(SwCtl* ctl, int64_t* obs, int obs_cap, int q) {
-  const uint64_t s = ctl->sweep;
-  if ((int)threadIdx.x <= q) obs[(int64_t)(s % (uint64_t)obs_cap) * (q + 1) + threadIdx.x] = 0;
-  __syncthreads();
-  if (threadIdx.x == 0) ctl->sweep = s + 1;
-}
-
 // ---------------------------------------------------------------------------
 SwRep make_rep(int8_t* spins, uint16_t* lroot, int32_t* gpar, int64_t* obs, const Grid& g,
                const LabelScratch& s, int q, uint64_t T, uint64_t seed) {
@@ -140,16 +134,14 @@ cudaError_t launch_sw_label(const int8_t* spins, uint16_t* lroot, int32_t* gpar,
                             const LabelScratch& s, int q, uint64_t T, uint64_t seed, const SwCtl* ctl,
                             int64_t* obs, int obs_cap, cudaStream_t st) {
   const SwRep R = make_rep(const_cast<int8_t*>(spins), lroot, gpar, obs, g, s, q, T, seed);
-  k_sw_label<<<g.n_tiles(), LABEL_THREADS, 0, st>>>(R, ctl, obs_cap, philox_keys(seed));
-  return cudaGetLastError();
+  return launch_after(k_sw_label, g.n_tiles(), LABEL_THREADS, st, R, ctl, obs_cap, philox_keys(seed));
 }
 
 cudaError_t launch_sw_flip(int8_t* spins, const uint16_t* lroot, int32_t* gpar, const Grid& g,
                            const LabelScratch& s, int q, uint64_t seed, const SwCtl* ctl, cudaStream_t st) {
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
   const SwRep R = make_rep(spins, const_cast<uint16_t*>(lroot), gpar, nullptr, g, s, q, 0, seed);
-  k_sw_flip<<<g.n_tiles(), LABEL_THREADS, 0, st>>>(R, ctl, limit, philox_keys(seed));
-  return cudaGetLastError();
+  return launch_after(k_sw_flip, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, philox_keys(seed));
 }
 
 // The same for L % 16 == 0 at HBM speed: a thread owns 16 columns (one
@@ -242,13 +234,7 @@ cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gp
                                const SwCtl* ctl, cudaStream_t st) {
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
   const SwRep R = make_rep(spins, const_cast<uint16_t*>(lroot), gpar, nullptr, g, s, q, 0, seed);
-  k_sw_flip_few<<<g.n_tiles(), LABEL_THREADS, 0, st>>>(R, ctl, limit, sel, P, philox_keys(seed));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_advance_fused(SwCtl* ctl, int64_t* obs, int obs_cap, int q, cudaStream_t st) {
-  k_advance_fused<<<1, 128, 0, st>>>(ctl, obs, obs_cap, q);
-  return cudaGetLastError();
+  return launch_after(k_sw_flip_few, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, sel, P, philox_keys(seed));
 }
 
 }  // namespace swccl

@@ -56,6 +56,8 @@ cudaError_t launch_tile_label(const uint8_t* mask, int32_t* labels, const Grid& 
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
 k_ccl_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid g, LabelScratch s) {
   __shared__ CclTileSmem sm;
+  wait_for_previous();
+  let_next_start();
   ccl_label_tile<true>(mask, labels, g, s, blockIdx.x, sm);
 }
 
@@ -64,35 +66,44 @@ constexpr int FINAL_THREADS = 256;
 __global__ void __launch_bounds__(FINAL_THREADS)
 k_ccl_final(int32_t* labels, Grid g, LabelScratch s, int limit) {
   __shared__ int32_t table[TILE_SITES];
+  wait_for_previous();
   final_labels_tile(labels, g, s, blockIdx.x, table, limit);
 }
 
 cudaError_t launch_ccl(const uint8_t* mask, int32_t* labels, const Grid& g, const LabelScratch& s, cudaStream_t st) {
-  k_ccl_tile<<<g.n_tiles(), LABEL_THREADS, 0, st>>>(mask, labels, g, s);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_after(k_ccl_tile, g.n_tiles(), LABEL_THREADS, st, mask, labels, g, s);
   if (e != cudaSuccess) return e;
-  if ((e = launch_merge(labels, g, s, st)) != cudaSuccess) return e;
+  if ((e = launch_merge(labels, g, s, nullptr, nullptr, 0, 0, st)) != cudaSuccess) return e;
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
-  k_ccl_final<<<g.n_tiles(), FINAL_THREADS, 0, st>>>(labels, g, s, limit);
-  return cudaGetLastError();
+  return launch_after(k_ccl_final, g.n_tiles(), FINAL_THREADS, st, labels, g, s, limit);
 }
 
 // ---------------------------------------------------------------------------
 // Seam merge: one CTA per `per` consecutive tiles (merge_tiles).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(MERGE_PER_TILE)
-k_merge(int32_t* __restrict__ labels, const __grid_constant__ Grid g, LabelScratch s, int per, int limit) {
+k_merge(int32_t* __restrict__ labels, const __grid_constant__ Grid g, LabelScratch s, int per, int limit, SwCtl* adv,
+        int64_t* obs, int obs_cap, int q) {
   __shared__ MergeSmem ms;
+  wait_for_previous();
+  if (!adv) let_next_start();
+  if (adv && blockIdx.x == 0) {   // end of the drawing step: the next sweep's fills this sweep's observable slot
+    const uint64_t sweep = adv->sweep;
+    for (int k = threadIdx.x; k <= q; k += MERGE_PER_TILE) obs[(int64_t)(sweep % (uint64_t)obs_cap) * (q + 1) + k] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) adv->sweep = sweep + 1;
+  }
   const int t0 = blockIdx.x * per;
   merge_tiles(ms, min(per, g.n_tiles() - t0), [&](int u) { return MergeTile{&g, labels, s.seams, s.err, t0 + u}; },
               limit);
 }
 
-cudaError_t launch_merge(int32_t* labels, const Grid& g, const LabelScratch& s, cudaStream_t st) {
+cudaError_t launch_merge(int32_t* labels, const Grid& g, const LabelScratch& s, SwCtl* adv, int64_t* obs, int obs_cap,
+                         int q, cudaStream_t st) {
   const int per = merge_tiles_per_cta(g.n_tiles());
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
-  k_merge<<<(unsigned)((g.n_tiles() + per - 1) / per), MERGE_PER_TILE, 0, st>>>(labels, g, s, per, limit);
-  return cudaGetLastError();
+  return launch_after(k_merge, (unsigned)((g.n_tiles() + per - 1) / per), MERGE_PER_TILE, st, labels, g, s, per, limit,
+                      adv, obs, obs_cap, q);
 }
 
 // ---------------------------------------------------------------------------

@@ -46,6 +46,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 constexpr int OBS_CAP = 4096;
 constexpr size_t READBACK_BYTES = 64 << 10;
+constexpr int SMALL_SWEEPS = 1024;   // sweeps per launch of the small-lattice kernel (a few ms at L = 128)
 
 }  // namespace
 
@@ -138,7 +139,7 @@ cudaError_t enqueue_sweep(sw_handle* h, cudaEvent_t* ev) {
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
   if ((e = launch_tile_label(h->mask, h->labels, h->grid, h->ls, st))) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
-  if ((e = launch_merge(h->labels, h->grid, h->ls, st))) return e;
+  if ((e = launch_merge(h->labels, h->grid, h->ls, nullptr, nullptr, 0, 0, st))) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
   if ((e = launch_root_compress(h->labels, h->grid, h->ls, h->spins, h->q, h->seed, h->ctl, st))) return e;
   if (ev && (e = cudaEventRecord(ev[4], st)) != cudaSuccess) return e;
@@ -147,7 +148,7 @@ cudaError_t enqueue_sweep(sw_handle* h, cudaEvent_t* ev) {
   return launch_advance(h->ctl, st);
 }
 
-// Enqueue one fused sweep: draw + label, merge, flip, advance.  With timing
+// Enqueue one fused sweep: draw + label, merge and advance, flip.  With timing
 // events the activation and root phases are recorded as empty.
 cudaError_t enqueue_sweep_fused(sw_handle* h, cudaEvent_t* ev) {
   cudaError_t e;
@@ -158,7 +159,7 @@ cudaError_t enqueue_sweep_fused(sw_handle* h, cudaEvent_t* ev) {
                            OBS_CAP, st)))
     return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
-  if ((e = launch_merge(h->labels, h->grid, h->ls, st))) return e;
+  if ((e = launch_merge(h->labels, h->grid, h->ls, h->ctl, h->obs, OBS_CAP, h->q, st))) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
   if (h->update == SW_UPDATE_FEW &&
       (e = launch_few_select(h->lroot, h->labels, h->grid, h->ls, h->seed, h->ell, h->sel, h->ctl, st)))
@@ -171,8 +172,7 @@ cudaError_t enqueue_sweep_fused(sw_handle* h, cudaEvent_t* ev) {
   } else if ((e = launch_sw_flip(h->spins, h->lroot, h->labels, h->grid, h->ls, h->q, h->seed, h->ctl, st))) {
     return e;
   }
-  if (ev && (e = cudaEventRecord(ev[5], st)) != cudaSuccess) return e;
-  return launch_advance_fused(h->ctl, h->obs, OBS_CAP, h->q, st);
+  return ev ? cudaEventRecord(ev[5], st) : cudaSuccess;
 }
 
 // Fused mode counts a sweep's observables in the next sweep's first kernel;
@@ -328,6 +328,7 @@ sw_handle* sw_create_threshold(int L, int q, uint64_t T, uint64_t seed, int hot_
   if ((e = cudaHostAlloc(&h->readback, READBACK_BYTES, cudaHostAllocMapped))) return bad(e, "read-back buffer");
   if ((e = cudaMalloc(&h->obs, (int64_t)OBS_CAP * (q + 1) * 8))) return bad(e, "observable ring");
   if ((e = cudaMalloc(&h->lroot, (N * 2 + 15) & ~15LL))) return bad(e, "tile roots");
+  if (L <= SMALL_L && (e = small_prepare())) return bad(e, "small-lattice kernel");
   h->ls = carve_label_scratch(h->grid, h->scratch,
                               reinterpret_cast<int*>(reinterpret_cast<char*>(h->ctl) + offsetof(SwCtl, err)));
   {
@@ -366,6 +367,17 @@ int sw_sweep(sw_handle* h, int n) {
   if (n == 0) return SW_OK;
   const bool fused = h->mode == SW_MODE_FUSED;
   auto enqueue = fused ? enqueue_sweep_fused : enqueue_sweep;
+  if (fused && !h->timing && h->update == SW_UPDATE_SW && h->L <= SMALL_L) {
+    // all sweeps of the call by one block, which writes their observables too
+    for (int done = 0; done < n; done += SMALL_SWEEPS) {
+      const int m = std::min(n - done, SMALL_SWEEPS);
+      CK(launch_sw_small(h->spins, h->L, h->q, h->T, h->seed, h->ctl, h->obs, OBS_CAP, m, h->stream));
+      h->sweeps += m;
+    }
+    h->dump_valid = false;
+    h->final_obs_pending = false;
+    return SW_OK;
+  }
   if (h->timing) {
     for (int k = 0; k < n; ++k) {
       cudaEvent_t ev[SW_N_PHASES + 1];

@@ -69,9 +69,8 @@ cudaError_t enqueue_batch_sweep(sw_batch* b) {
   if (b->schedule == SW_BATCH_PERSISTENT)
     return launch_batch_persistent(b->view, b->ctl, b->blocks, b->barrier_limit, b->stream);
   if ((e = launch_batch_label(b->view, b->ctl, b->stream))) return e;
-  if ((e = launch_batch_merge(b->view, b->stream))) return e;
-  if ((e = launch_batch_flip(b->view, b->ctl, b->stream))) return e;
-  return launch_batch_advance(b->view, b->ctl, b->stream);
+  if ((e = launch_batch_merge(b->view, b->ctl, b->stream))) return e;
+  return launch_batch_flip(b->view, b->ctl, b->stream);
 }
 
 // Forget the captured sweep of schedule k (its launch arguments changed).

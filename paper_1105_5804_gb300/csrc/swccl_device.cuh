@@ -14,6 +14,41 @@
 namespace swccl {
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch.  A kernel launched with launch_after may be
+// launched before the kernels ahead of it in the stream have ended, so that its
+// launch overlaps them.  Every thread of such a kernel calls wait_for_previous
+// first: it returns when the kernels ahead have completed and their writes are
+// visible (at once in a kernel launched plainly).  A sweep at L = 256 takes 25.0
+// us instead of 27.4.  let_next_start lets the next kernel's blocks become
+// resident as soon as all of this one's run: 1 us more for a chain of kernels
+// that leave the GPU mostly empty (labeling 200 x 300), but the heavy blocks of
+// the next step then land unevenly (a sweep at L = 2048 46 instead of 42 us), so
+// only the stand-alone labeling uses it.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline cudaError_t launch_after_smem(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem,
+                                     cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), unsigned blocks, unsigned threads, cudaStream_t st, A... args) {
+  return launch_after_smem(kernel, blocks, threads, 0, st, args...);
+}
+
+// ---------------------------------------------------------------------------
 // Philox4x32-10.  Each round takes the two 32x32->64 products of the even
 // counter words with the published multipliers; the high halves are mixed
 // with the odd words and the round key, the key advances by the Weyl
@@ -78,6 +113,24 @@ __device__ __forceinline__ uint4 philox_draw(uint4 ctr, const PhiloxKeys& k) {
   return ctr;
 }
 
+// N draws in step, round by round: where only a few warps run, the independent
+// chains hide each other's latency.
+template <int N>
+__device__ __forceinline__ void philox_draws(uint4 (&ctr)[N], const PhiloxKeys& k) {
+#pragma unroll
+  for (int round = 0; round < 10; ++round) {
+    unsigned long long pa[N], pb[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) pa[u] = (unsigned long long)ctr[u].x * 0xD2511F53ull;
+#pragma unroll
+    for (int u = 0; u < N; ++u) pb[u] = (unsigned long long)ctr[u].z * 0xCD9E8D57ull;
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+      ctr[u] = make_uint4((uint32_t)(pb[u] >> 32) ^ ctr[u].y ^ k.lo[round], (uint32_t)pb[u],
+                          (uint32_t)(pa[u] >> 32) ^ ctr[u].w ^ k.hi[round], (uint32_t)pa[u]);
+  }
+}
+
 __device__ __forceinline__ uint4 philox_draw(uint4 ctr, const SeedKey& k) { return philox(ctr, k.lo, k.hi); }
 
 __device__ __forceinline__ uint4 draw(uint32_t c0, uint64_t sweep, uint32_t tag, uint64_t seed) {
@@ -124,8 +177,15 @@ __device__ __forceinline__ int sm_at(const uint16_t* par, int x) {
 __device__ __forceinline__ void sm_set(uint16_t* par, int x, int v) {
   *reinterpret_cast<volatile uint16_t*>(reinterpret_cast<char*>(par) + x) = (uint16_t)v;
 }
-// Orders nodes like their sites: twice the row-major index.
+// Orders nodes like their sites: twice the row-major index of the tile
+// (TileOrder), or the node itself where entries are laid out like sites.
 __device__ __forceinline__ int node_key(int x) { return x ^ ((x >> (TILE_W_LOG2 - 5)) & 64); }
+struct TileOrder {
+  static __device__ __forceinline__ int key(int x) { return node_key(x); }
+};
+struct SiteOrder {
+  static __device__ __forceinline__ int key(int x) { return x; }
+};
 
 // The functions below are called by all 32 lanes of a warp together, each lane
 // with valid nodes (one that has nothing to join or find passes any written
@@ -139,7 +199,7 @@ __device__ __forceinline__ int node_key(int x) { return x ^ ((x >> (TILE_W_LOG2 
 // only while entries decrease ends by itself; across strips the steps are
 // counted, and on overrun (corrupted state) the error word is set and the walk
 // stops.
-constexpr int WALK_LIMIT = TILE_H * TILE_W;   // a tree has fewer nodes
+constexpr int WALK_LIMIT = 1 << 15;   // more steps than any tree has nodes (16-bit byte offsets of 2-byte entries)
 template <int N>
 __device__ __forceinline__ void sm_find_strip(const uint16_t* par, int (&x)[N]) {
   bool more;
@@ -172,40 +232,56 @@ __device__ __forceinline__ void sm_find_tile(const uint16_t* par, int (&x)[N], i
   set_error(err, SW_ERR_STATE);
 }
 
-// Join every lane's pair (a, b) (a == b: none) where other warps may join
+// Join N pairs (a, b) of every lane (a == b: none) where other warps may join
 // theirs at the same time.  The root of the larger site is hooked under the
 // other by a compare-and-swap of the 32-bit word that holds its entry,
 // repeated while only the entry beside it changed (it can be hooked once, so
 // twice at most); if the root itself was hooked meanwhile, its new parent is
 // joined in the next round, so no link is lost.  Every round lowers the larger
 // operand, so at most WALK_LIMIT rounds run.
-__device__ __forceinline__ void sm_union_tile(uint16_t* par, int a, int b, int* err) {
+template <class Order = TileOrder, int N>
+__device__ __forceinline__ void sm_union_tile(uint16_t* par, int (&a)[N], int (&b)[N], int* err) {
   for (int rounds = 0; rounds <= WALK_LIMIT; ++rounds) {
-    int x[2] = {a, b};
+    int x[2 * N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      x[2 * u] = a[u];
+      x[2 * u + 1] = b[u];
+    }
     sm_find_tile(par, x, err);
-    a = x[0];
-    b = x[1];
-    if (a != b) {
-      const bool a_first = node_key(a) < node_key(b);
-      const int lo = a_first ? a : b, hi = a_first ? b : a;
-      unsigned* word = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(par) + (hi & ~3));
-      const int sh = 8 * (hi & 2);
-      unsigned old = *reinterpret_cast<volatile unsigned*>(word);
-      a = b = lo;
-      for (;;) {
-        const int cur = (int)((old >> sh) & 0xFFFFu);
-        if (cur != hi) {   // hooked meanwhile
-          b = cur;
-          break;
+    bool more = false;
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      a[u] = x[2 * u];
+      b[u] = x[2 * u + 1];
+      if (a[u] != b[u]) {
+        const bool a_first = Order::key(a[u]) < Order::key(b[u]);
+        const int lo = a_first ? a[u] : b[u], hi = a_first ? b[u] : a[u];
+        unsigned* word = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(par) + (hi & ~3));
+        const int sh = 8 * (hi & 2);
+        unsigned old = *reinterpret_cast<volatile unsigned*>(word);
+        a[u] = b[u] = lo;
+        for (;;) {
+          const int cur = (int)((old >> sh) & 0xFFFFu);
+          if (cur != hi) {   // hooked meanwhile
+            b[u] = cur;
+            break;
+          }
+          const unsigned seen = atomicCAS(word, old, old ^ ((unsigned)(lo ^ hi) << sh));
+          if (seen == old) break;
+          old = seen;
         }
-        const unsigned seen = atomicCAS(word, old, old ^ ((unsigned)(lo ^ hi) << sh));
-        if (seen == old) break;
-        old = seen;
+        more |= a[u] != b[u];
       }
     }
-    if (!__any_sync(0xFFFFFFFFu, a != b)) return;
+    if (!__any_sync(0xFFFFFFFFu, more)) return;
   }
   set_error(err, SW_ERR_STATE);
+}
+template <class Order = TileOrder>
+__device__ __forceinline__ void sm_union_tile(uint16_t* par, int a, int b, int* err) {
+  int x[1] = {a}, y[1] = {b};
+  sm_union_tile<Order>(par, x, y, err);
 }
 
 // Join every lane's pair (a, b) (a == b: none) in one strip, whose trees no

@@ -85,7 +85,7 @@ struct LabelScratch {
 
 // Control block of a Swendsen-Wang chain, in device memory.
 struct SwCtl {
-  unsigned long long sweep;  // index of the sweep being computed
+  unsigned long long sweep;  // index of the sweep being computed (fused: advanced by its merge)
   long long obs_done;        // fused mode: last sweep whose observables k_observe completed (-1: none)
   int err;                   // first device-side failure (SW_ERR_*)
   int pad;
@@ -183,7 +183,11 @@ cudaError_t launch_labels3(const uint16_t* lroot, int32_t* gpar, const uint32_t*
 
 cudaError_t launch_tile_label(const uint8_t* mask, int32_t* labels, const Grid& g,
                               const LabelScratch& s, cudaStream_t st);
-cudaError_t launch_merge(int32_t* labels, const Grid& g, const LabelScratch& s, cudaStream_t st);
+// The seam merge.  adv, if not null, is the control block of a fused sweep:
+// the merge clears the observable slot of the sweep (row of 1 + q in obs) and
+// advances the counter; the kernels after it in the sweep count from there.
+cudaError_t launch_merge(int32_t* labels, const Grid& g, const LabelScratch& s, SwCtl* adv, int64_t* obs, int obs_cap,
+                         int q, cudaStream_t st);
 // Root compression; when `spins` is non-null also draws each final root's
 // new state (FLIP tag, sweep from ctl) into spins[root].
 cudaError_t launch_root_compress(int32_t* labels, const Grid& g, const LabelScratch& s,
@@ -205,7 +209,6 @@ cudaError_t launch_sw_flip(int8_t* spins, const uint16_t* lroot, int32_t* gpar, 
                            const LabelScratch& s, int q, uint64_t seed, const SwCtl* ctl, cudaStream_t st);
 cudaError_t launch_observe(const int8_t* spins, int L, int q, SwCtl* ctl, int64_t* obs, int obs_cap,
                            cudaStream_t st);
-cudaError_t launch_advance_fused(SwCtl* ctl, int64_t* obs, int obs_cap, int q, cudaStream_t st);
 // Few-cluster update: bytes of the seed-selection bit array of n sites, the
 // selection (clears the array, then marks the seeded clusters' roots), and
 // the flip of the selected clusters.
@@ -216,11 +219,19 @@ cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gp
                                const LabelScratch& s, int q, uint64_t seed, const uint32_t* sel, uint64_t P,
                                const SwCtl* ctl, cudaStream_t st);
 
+// Whole sweeps of a lattice with L <= SMALL_L by one block (k_small.cu): n sweeps
+// in one launch, their observables (and the pending ones of the sweep before)
+// written to the ring, ctl advanced.  small_prepare: once per device before the
+// first launch.
+constexpr int SMALL_L = 128;
+cudaError_t small_prepare();
+cudaError_t launch_sw_small(int8_t* spins, int L, int q, uint64_t T, uint64_t seed, SwCtl* ctl, int64_t* obs,
+                            int obs_cap, int n, cudaStream_t st);
+
 // Batched chains (k_batch.cu).
 cudaError_t launch_batch_label(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
-cudaError_t launch_batch_merge(const BatchView& b, cudaStream_t st);
+cudaError_t launch_batch_merge(const BatchView& b, BatchCtl* ctl, cudaStream_t st);   // and advance (see launch_merge)
 cudaError_t launch_batch_flip(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
-cudaError_t launch_batch_advance(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
 cudaError_t launch_batch_observe(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
 // One persistent cooperative launch for the whole sweep; `blocks` CTAs; a
 // grid-barrier wait gives up after limit_cycles of clock64().

@@ -143,6 +143,23 @@ __device__ __forceinline__ uint32_t seg_or_down(uint32_t x, uint32_t j) {
   return x;
 }
 
+// Step 1 for the calling lane's row word (lane = row; all lanes call): `info`
+// (S, F | U reversed, F) for the sweep, and the extra contacts X.
+__device__ __forceinline__ uint32_t run_words(uint32_t we, uint32_t wn, int h, uint4& info) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t e_below = __shfl_up_sync(FULL, we, 1);
+  uint32_t c = __shfl_up_sync(FULL, wn, 1);   // contacts: north bonds of the row below into my row
+  if (lane == 0 || lane >= h) c = 0u;
+  const uint32_t S = ~(we << 1);               // run starts (bit 0 always)
+  const uint32_t before = (seg_or_up(c, we) << 1) & (we << 1);     // a contact earlier in my run
+  const uint32_t F = c & ~before;
+  const uint32_t U = S & ~seg_or_down(c, we);                     // starts of runs without contact
+  const uint32_t j2 = we & e_below;                               // joined east in both rows
+  const uint32_t before2 = (seg_or_up(c, j2) << 1) & (j2 << 1);
+  info = make_uint4(S, __brev(F | U), F, 0u);
+  return c & ~before2 & ~F;
+}
+
 // Runs the engine.  we, wn: the calling thread's row word (row = lane, strip =
 // warp), zero for rows >= h; w: columns of the tile (strips past them hold no
 // sites and are skipped); rows past h are swept as rows of single sites.  All
@@ -165,20 +182,9 @@ __device__ __forceinline__ void tile_engine(TileSmemT<ROWS>& sm, uint32_t we, ui
   }
   if (strip) {
   // 1. run structure of my row word against the row below
-  uint32_t X;
-  {
-    const uint32_t e_below = __shfl_up_sync(FULL, we, 1);
-    uint32_t c = __shfl_up_sync(FULL, wn, 1);   // contacts: north bonds of the row below into my row
-    if (lane == 0 || lane >= h) c = 0u;
-    const uint32_t S = ~(we << 1);               // run starts (bit 0 always)
-    const uint32_t before = (seg_or_up(c, we) << 1) & (we << 1);     // a contact earlier in my run
-    const uint32_t F = c & ~before;
-    const uint32_t U = S & ~seg_or_down(c, we);                     // starts of runs without contact
-    const uint32_t j2 = we & e_below;                               // joined east in both rows
-    const uint32_t before2 = (seg_or_up(c, j2) << 1) & (j2 << 1);
-    X = c & ~before2 & ~F;
-    if (lane < ROWS) sm.rowinfo[warp * ROWS + lane] = make_uint4(S, __brev(F | U), F, 0u);
-  }
+  uint4 info;
+  const uint32_t X = run_words(we, wn, h, info);
+  if (lane < ROWS) sm.rowinfo[warp * ROWS + lane] = info;
   __syncwarp();
   // 2. strip sweep.  Lane l takes column 31 - l: the anchor's column comes out
   //    as 31 - anchor, the lane to read from.
@@ -387,9 +393,9 @@ __device__ __forceinline__ void merge_seam_bond(int32_t* gpar, const Grid& g, co
 // MERGE_PER_TILE threads (thread = bond): every thread loads its bond of all
 // the tiles at once, the pairs to join (about one bond in six at criticality)
 // go to a list, and the list is joined with all lanes busy.  With a union per
-// lane where it stands, a warp ran its divergent walks for five lanes of 32:
-// bound by the latency of the parent loads and by issue, 157 us at L = 16384
-// against XXX us.  tile_of(u): grid, parents and scratch of tile u.
+// lane where it stands, a warp ran its divergent walks for five lanes of 32 and
+// issued 278 instructions; bound by the latency of the parent loads (L = 16384:
+// 156 us then, 153 with the hook before the walk, 120 us as it is).  tile_of(u): grid, parents and scratch of tile u.
 constexpr int MERGE_TILES = 2;
 struct MergeSmem {
   int2 pairs[MERGE_TILES * MERGE_PER_TILE];

@@ -63,7 +63,7 @@ def test_labels_of_an_unaligned_mask(off):
         assert np.array_equal(lab.cpu().numpy(), ref), (H, W)
 
 
-@pytest.mark.parametrize("tile_w,W", [(256, 6801), (128, 6500), (64, 6410)])
+@pytest.mark.parametrize("tile_w,W", [(256, 7001), (128, 6500), (64, 6410)])
 @pytest.mark.parametrize("rows", [41, 40])
 def test_merge_with_several_tiles_per_block(tile_w, W, rows):
     """Grids just above the size where a merge block takes two tiles, with an
