@@ -9,17 +9,6 @@ namespace swccl {
 
 namespace fused {
 
-// Four byte lanes of a and b compared: bit k of the result is set iff byte k
-// of a equals byte k of b.  Exact zero-byte test of a ^ b (no carry crosses a
-// byte: each byte of (x & 0x7F..) + 0x7F.. is at most 0xFE), then the four
-// flag bits are gathered by one multiply.
-__device__ __forceinline__ uint32_t eq4(uint32_t a, uint32_t b) {
-  const uint32_t x = a ^ b;
-  const uint32_t y = ((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x;   // bit 7 of a byte set iff the byte is non-zero
-  const uint32_t z = (~y & 0x80808080u) >> 7;                  // bit 0 of a byte set iff equal
-  return (z * 0x00204081u) >> 21 & 0xFu;
-}
-
 constexpr int QREG_MAX = 8;
 
 // Which of 32 consecutive sites of one row equal their east and north
@@ -350,21 +339,6 @@ static_assert(FLIP_PASSES * 8 * LABEL_THREADS == TILE_SITES && LABEL_THREADS / F
 __device__ __forceinline__ int root_in(const uint4& v, int i) {
   const uint32_t wv = (i < 2) ? v.x : (i < 4) ? v.y : (i < 6) ? v.z : v.w;
   return (int)((wv >> (16 * (i & 1))) & 0xFFFFu);
-}
-
-// 16 bytes from global memory (through L2) to shared memory, asynchronously.
-__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Bit i of x (i < 16) to bit 2i.
-__device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
-  x = (x | (x << 8)) & 0x00FF00FFu;
-  x = (x | (x << 4)) & 0x0F0F0F0Fu;
-  x = (x | (x << 2)) & 0x33333333u;
-  return (x | (x << 1)) & 0x55555555u;
 }
 
 // The flip of tile t (see k_fused.cu).  All threads of the CTA call it; it

@@ -109,34 +109,73 @@ cudaError_t launch_perc_mask(uint8_t* mask, int H, int W, uint64_t k, cudaStream
 }
 
 // ---------------------------------------------------------------------------
-__global__ void k_pixel_bonds(const uint8_t* __restrict__ px, uint8_t* __restrict__ mask, int H,
-                              int W, int periodic) {
-  const int64_t n = (int64_t)H * W, nbytes = (n + 3) >> 2;
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nbytes;
-       b += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t out = 0;
+// Mask byte b of the image: four sites, one by one.
+__device__ __forceinline__ uint32_t pixel_bond_byte(const uint8_t* __restrict__ px, int64_t b, int H, int W, int periodic) {
+  const int64_t n = (int64_t)H * W;
+  uint32_t out = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int64_t i = 4 * b + k;
-      if (i >= n) break;
-      const int y = (int)(i / W), x = (int)(i - (int64_t)y * W);
-      const uint8_t v = px[i];
-      uint32_t bits = 0;
-      if (periodic || x + 1 < W) bits |= (v == px[(int64_t)y * W + (x + 1 == W ? 0 : x + 1)]) ? 1u : 0u;
-      if (periodic || y + 1 < H) bits |= (v == px[(int64_t)(y + 1 == H ? 0 : y + 1) * W + x]) ? 2u : 0u;
-      out |= bits << (2 * k);
-    }
-    mask[b] = (uint8_t)out;
+  for (int k = 0; k < 4; ++k) {
+    const int64_t i = 4 * b + k;
+    if (i >= n) break;
+    const int y = (int)(i / W), x = (int)(i - (int64_t)y * W);
+    const uint8_t v = px[i];
+    uint32_t bits = 0;
+    if (periodic || x + 1 < W) bits |= (v == px[(int64_t)y * W + (x + 1 == W ? 0 : x + 1)]) ? 1u : 0u;
+    if (periodic || y + 1 < H) bits |= (v == px[(int64_t)(y + 1 == H ? 0 : y + 1) * W + x]) ? 2u : 0u;
+    out |= bits << (2 * k);
   }
+  return out;
+}
+
+// Sixteen consecutive sites (in row-major order, whatever the row) per thread:
+// their pixels are one 16-byte word, the pixels after them and the pixels a row
+// further are compared four per word (unaligned words shifted together), and
+// the bond east of a row's last site is put right afterwards (closed, or to the
+// row's first pixel).  Threads that touch the last row or the array's end, and
+// images or masks that are not aligned, go site by site.  Bound by instruction
+// issue (about 9 instructions a site; 5003 x 7001: about 25 us, 130 with one
+// site at a time and its division).
+constexpr int PIXEL_THREADS = 256;
+
+__global__ void __launch_bounds__(PIXEL_THREADS)
+k_pixel_bonds(const uint8_t* __restrict__ px, uint8_t* __restrict__ mask, int H, int W, int periodic, int aligned) {
+  wait_for_previous();
+  const uint32_t n = (uint32_t)H * (uint32_t)W;   // < 2^31
+  const uint32_t t = blockIdx.x * (uint32_t)PIXEL_THREADS + threadIdx.x, i0 = 16u * t;
+  if (i0 >= n) return;
+  // the words read end at most 3 bytes past the last pixel compared
+  if (!aligned || (uint64_t)i0 + 16u + (uint32_t)W + 4u > n) {
+    for (uint32_t b = 4u * t; b < 4u * t + 4u && 4u * b < n; ++b)
+      mask[b] = (uint8_t)pixel_bond_byte(px, b, H, W, periodic);
+    return;
+  }
+  const uint4 o4 = *reinterpret_cast<const uint4*>(px + i0);
+  const uint32_t own[5] = {o4.x, o4.y, o4.z, o4.w, px[i0 + 16u]};
+  const uint32_t north0 = i0 + (uint32_t)W, sh = 8u * (north0 & 3u);
+  const uint32_t* np = reinterpret_cast<const uint32_t*>(px + (north0 & ~3u));
+  uint32_t nw[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) nw[k] = np[k];
+  uint32_t e = 0u, nb = 0u;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    e |= eq4(own[k], __funnelshift_r(own[k], own[k + 1], 8)) << (4 * k);
+    nb |= eq4(own[k], __funnelshift_r(nw[k], nw[k + 1], sh)) << (4 * k);
+  }
+  for (uint32_t j = (uint32_t)W - 1u - i0 % (uint32_t)W; j < 16u; j += (uint32_t)W) {   // row ends among the sites
+    const uint32_t i = i0 + j;
+    e &= ~(1u << j);
+    if (periodic && px[i] == px[i + 1u - (uint32_t)W]) e |= 1u << j;
+  }
+  *reinterpret_cast<uint32_t*>(mask + 4u * t) = spread_bits(e) | spread_bits(nb) << 1;
 }
 
 cudaError_t launch_pixel_bonds(const uint8_t* px, uint8_t* mask, int H, int W, int periodic,
                                cudaStream_t st) {
-  const int64_t nbytes = ((int64_t)H * W + 3) / 4;
-  const int threads = 256;
-  const int64_t blocks = std::min<int64_t>((nbytes + threads - 1) / threads, 152 * 64);
-  k_pixel_bonds<<<(unsigned)blocks, threads, 0, st>>>(px, mask, H, W, periodic);
-  return cudaGetLastError();
+  const int64_t threads = ((int64_t)H * W + 15) / 16;
+  const int aligned = (reinterpret_cast<uintptr_t>(px) & 15) == 0 && (reinterpret_cast<uintptr_t>(mask) & 3) == 0;
+  return launch_after(k_pixel_bonds, (unsigned)((threads + PIXEL_THREADS - 1) / PIXEL_THREADS), PIXEL_THREADS, st, px,
+                      mask, H, W, periodic, aligned);
 }
 
 // ---------------------------------------------------------------------------

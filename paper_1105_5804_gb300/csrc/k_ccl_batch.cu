@@ -43,12 +43,12 @@ __global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_cons
               v.limit);
 }
 
-__global__ void __launch_bounds__(256) k_cclb_final(const __grid_constant__ CclBatchView v) {
-  __shared__ int32_t table[TILE_SITES];
+__global__ void __launch_bounds__(FINAL_THREADS) k_cclb_final(const __grid_constant__ CclBatchView v) {
+  __shared__ FinalSmem fs;
   wait_for_previous();
   const int gt = blockIdx.x;
   const CclJob& J = v.jobs[job_of_tile(v, gt)];
-  final_labels_tile(J.labels, J.g, J.s, gt - J.tile0, table, v.limit);
+  final_labels_tile(J.labels, J.g, J.s, gt - J.tile0, fs, v.limit);
 }
 
 cudaError_t launch_ccl_batch(const CclBatchView& v, cudaStream_t st) {
@@ -58,7 +58,7 @@ cudaError_t launch_ccl_batch(const CclBatchView& v, cudaStream_t st) {
   const int per = merge_tiles_per_cta(v.n_tiles);
   e = launch_after(k_cclb_merge, (unsigned)((v.n_tiles + per - 1) / per), MERGE_PER_TILE, st, v, per);
   if (e != cudaSuccess) return e;
-  return launch_after(k_cclb_final, v.n_tiles, 256, st, v);
+  return launch_after(k_cclb_final, v.n_tiles, FINAL_THREADS, st, v);
 }
 
 }  // namespace swccl

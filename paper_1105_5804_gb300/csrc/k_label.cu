@@ -31,8 +31,8 @@
 // The stand-alone labeling (launch_ccl) uses k_ccl_tile, a k_tile_label that
 // keeps every site's tile root as a 16-bit local index in the tile's scratch
 // and writes label entries only for the tile roots on the tile edge (their
-// parent entries), then k_merge, then k_ccl_final: per tile, each tile root
-// finds its cluster root once and every site takes its tile root's from a
+// parent entries), then k_merge, then k_ccl_final: per tile, each edge root
+// finds its cluster root once and every site takes its tile root's label from a
 // shared-memory table -- every label written once, no gathers.
 #include "label_tile.cuh"
 
@@ -61,13 +61,11 @@ k_ccl_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid 
   ccl_label_tile<true>(mask, labels, g, s, blockIdx.x, sm);
 }
 
-constexpr int FINAL_THREADS = 256;
-
 __global__ void __launch_bounds__(FINAL_THREADS)
 k_ccl_final(int32_t* labels, Grid g, LabelScratch s, int limit) {
-  __shared__ int32_t table[TILE_SITES];
+  __shared__ FinalSmem fs;
   wait_for_previous();
-  final_labels_tile(labels, g, s, blockIdx.x, table, limit);
+  final_labels_tile(labels, g, s, blockIdx.x, fs, limit);
 }
 
 cudaError_t launch_ccl(const uint8_t* mask, int32_t* labels, const Grid& g, const LabelScratch& s, cudaStream_t st) {
@@ -163,6 +161,30 @@ LabelScratch carve_label_scratch(const Grid& g, void* base, int* err) {
   s.seams = reinterpret_cast<int32_t*>(p);
   p += al(nt * SeamLayout::INTS * 4);
   s.err = err ? err : reinterpret_cast<int*>(p);
+  return s;
+}
+
+// The stand-alone labeling keeps 16-bit tile roots, edge-root bits and seam
+// records only (2.4 bytes per site of the about 8.3 that label_scratch_bytes
+// asks a caller for).
+int64_t ccl_scratch_bytes(const Grid& g) {
+  auto al = [](int64_t b) { return (b + 255) & ~(int64_t)255; };
+  const int64_t nt = g.n_tiles();
+  return al(nt * TILE_SITES * 2) + al(nt * (TILE_SITES / 32) * 4) + al(nt * SeamLayout::INTS * 4);
+}
+
+LabelScratch carve_ccl_scratch(const Grid& g, void* base, int* err) {
+  auto al = [](int64_t b) { return (b + 255) & ~(int64_t)255; };
+  const int64_t nt = g.n_tiles();
+  char* p = static_cast<char*>(base);
+  LabelScratch s;
+  s.work = reinterpret_cast<int32_t*>(p);
+  p += al(nt * TILE_SITES * 2);
+  s.roots = reinterpret_cast<int32_t*>(p);
+  p += al(nt * (TILE_SITES / 32) * 4);
+  s.seams = reinterpret_cast<int32_t*>(p);
+  s.root_counts = nullptr;
+  s.err = err;
   return s;
 }
 

@@ -45,21 +45,29 @@ __device__ __forceinline__ unsigned long long mask_word(const uint8_t* __restric
   return nvalid < 32 ? wd & ((1ull << (2 * nvalid)) - 1ull) : wd;
 }
 
-// Local labeling of one tile for the stand-alone labeling path: every thread
-// takes the bond bits of its row of its strip from the packed mask (bits of
-// sites outside the grid and the east bond of the tile's last column
-// cleared), the engine of tile_engine.cuh labels the tile, and the warps
-// write their strips' labels (global index of the tile root, the minimum
-// site index of its tile component), the tile's root list, and the seam
-// record (labels and outgoing bond bits of the four tile edges).
-// LOCAL (the stand-alone labeling path, finished by final_labels_tile): the
-// label array receives only the parent entries of the tile roots whose
-// component reaches the tile edge (label = own global index), which the
-// seam merge and the final root walks use; every site's tile root goes, as
-// a 16-bit local index, to the tile's slot of `work`, in tile row-major order;
-// the root list holds local indices, with CCL_EDGE_ROOT set on the edge
-// roots.  final_labels_tile writes every site's label.
-constexpr int CCL_EDGE_ROOT = 1 << 30;
+// Local labeling of one tile from a bond mask: every thread takes the bond bits
+// of its row of its strip (bits of sites outside the grid and the east bond of
+// the tile's last column cleared), the engine of tile_engine.cuh labels the
+// tile, and the warps write their strips' sites and seam records (labels and
+// outgoing bond bits of the four tile edges).
+// LOCAL (the stand-alone labeling, finished by final_labels_tile): the label
+// array receives only the parent entries of the tile roots whose component
+// reaches the tile edge (label = own global index), which the seam merge and
+// the final walks use; every site's tile root goes, as a 16-bit local index, to
+// the tile's slot of `work`, in tile row-major order, and the edge-root bits to
+// its slot of `roots`.
+// Otherwise (the staged sweep) every site's label is written (global index of
+// the tile root, the minimum site index of its tile component), and the tile's
+// root list.
+// Tile t's tile roots and edge-root bits in the scratch of the stand-alone
+// labeling (carve_ccl_scratch).
+__device__ __forceinline__ uint16_t* ccl_roots(const LabelScratch& s, int t) {
+  return reinterpret_cast<uint16_t*>(s.work) + (int64_t)t * TILE_SITES;
+}
+__device__ __forceinline__ int32_t* ccl_edges(const LabelScratch& s, int t) {
+  return s.roots + (int64_t)t * (TILE_SITES / 32);
+}
+
 struct CclTileSmem {
   TileSmem tile;
   uint32_t edge_bits[TILE_SITES / 32];   // local roots on the tile edge
@@ -78,7 +86,6 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
   const int h = min(TILE_H, g.H - y0), w = min(TILE_W, g.W - x0);
   const int W = g.W;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int32_t* slot = s.roots + (int64_t)t * TILE_SITES;     // the root list
   cs.edge_bits[threadIdx.x] = 0u;                        // the engine's barriers order it before the marks
 
   // 1. bond bits of row `lane` of strip `warp`
@@ -101,12 +108,10 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
 
   // 4b. the roots of my strip's sites, eight consecutive sites per thread and
   //     step, four threads a row.  LOCAL: as 16-bit local indices into the
-  //     tile's slot of `work`.  Otherwise as global labels.  Bit 4j + k of mine
+  //     tile's slot of `work`.  Otherwise as global labels; bit 4j + k of mine
   //     flags site 2k of step j as a root, bit 16 + 4j + k site 2k + 1.
   const int lx0 = 32 * warp + 8 * (lane & 3);
   const int in = min(max(w - lx0, 0), 8);   // columns past the grid are no roots of the tile
-  const uint32_t in_mask = ((1u << ((in + 1) >> 1)) - 1u) | ((1u << (in >> 1)) - 1u) << 16;
-  uint16_t* lr = reinterpret_cast<uint16_t*>(s.work + (int64_t)t * TILE_SITES);
   uint32_t mine = 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -114,14 +119,16 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
     if (ly >= h || in == 0) continue;   // the engine wrote no entries there
     const int sidx = local_of(ly, lx0);
     const uint4 r = roots_of(par, sidx);
-    if (LOCAL) *reinterpret_cast<uint4*>(lr + ly * TILE_W + lx0) = r;
-    const uint32_t own = (uint32_t)sidx * 0x00010001u + 0x00010000u;   // (sidx, sidx + 1)
-    const uint32_t wv[4] = {r.x, r.y, r.z, r.w};
-    uint32_t m = 0;
+    if (LOCAL) {
+      *reinterpret_cast<uint4*>(ccl_roots(s, t) + ly * TILE_W + lx0) = r;
+    } else {
+      const uint32_t in_mask = ((1u << ((in + 1) >> 1)) - 1u) | ((1u << (in >> 1)) - 1u) << 16;
+      const uint32_t own = (uint32_t)sidx * 0x00010001u + 0x00010000u;   // (sidx, sidx + 1)
+      const uint32_t wv[4] = {r.x, r.y, r.z, r.w};
+      uint32_t m = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) m |= zero_halves(wv[k] ^ (own + (uint32_t)k * 0x00020002u)) >> (15 - k);
-    mine |= (m & in_mask) << (4 * j);
-    if (!LOCAL) {
+      for (int k = 0; k < 4; ++k) m |= zero_halves(wv[k] ^ (own + (uint32_t)k * 0x00020002u)) >> (15 - k);
+      mine |= (m & in_mask) << (4 * j);
       int32_t* dst = labels + (int64_t)(y0 + ly) * W + x0 + lx0;
 #pragma unroll
       for (int k = 0; k < 8; ++k)
@@ -133,7 +140,13 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
   //    roots marked
   seam_strip(sm, s.seams + (int64_t)t * SeamLayout::INTS, labels, cs.edge_bits, wn, e_last, h, w, y0, x0, W);
 
-  // 6. root list
+  // 6. LOCAL: edge-root bits; otherwise the root list
+  if (LOCAL) {
+    __syncthreads();
+    ccl_edges(s, t)[threadIdx.x] = (int32_t)cs.edge_bits[threadIdx.x];
+    return;
+  }
+  int32_t* slot = s.roots + (int64_t)t * TILE_SITES;
   int cnt = __popc(mine), incl = cnt;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -154,9 +167,7 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
     const int b = __ffs(mine) - 1;
     mine &= mine - 1;
     const int jk = b & 15;
-    const int sidx = local_of((lane >> 2) + 8 * (jk >> 2), lx0) + 2 * (jk & 3) + (b >> 4);
-    if (LOCAL) slot[base++] = sidx | (((cs.edge_bits[sidx >> 5] >> (sidx & 31)) & 1u) ? CCL_EDGE_ROOT : 0);
-    else slot[base++] = tile_global(sidx, y0, x0, W);
+    slot[base++] = tile_global(local_of((lane >> 2) + 8 * (jk >> 2), lx0) + 2 * (jk & 3) + (b >> 4), y0, x0, W);
   }
   if (threadIdx.x == 0) s.root_counts[t] = total;
   __syncthreads();
@@ -196,67 +207,89 @@ __device__ __forceinline__ void site_compress_tile(int32_t* __restrict__ labels,
 }
 
 // Final labels of tile t for the stand-alone path (after the seam merge, on
-// what ccl_label_tile<true> wrote): each tile root (local root list) finds
-// its cluster root R on the label array and stores it in `table` at its
-// local index; then every site of the tile takes table[its tile root].
-// A tile root's entry receives R (smaller than any value other walks may
-// store there), so walks of other tiles through it stay valid.  All threads
-// of the CTA call it; it synchronises the CTA.
+// what ccl_label_tile<true> wrote): `table` holds every local index's label --
+// first its own global index, the label of a component that stays in the tile;
+// then each edge root finds its cluster root R on the label array -- and every
+// site takes table[its tile root].  A walk compresses the entries it passes to
+// smaller ones of the same tree, so walks of other tiles stay valid.  The tile
+// roots come by cp.async while the table is filled and the edge roots walk; an
+// edge root is on the tile's perimeter, so a thread has at most three walks.
+// Labels go out as 16-byte words wherever the rows start (a row of any width,
+// shifted against the words of shared memory by up to three sites).  Bound by
+// the latency of the walks (long scoreboard).  With every tile root listed by
+// the labeling kernel and looked up here, and rows of odd width written site
+// by site, a labeling of 5003 x 7001 took 248 us instead of 181, of 4096^2 100
+// instead of 89.  All threads of the CTA call it.
+constexpr int FINAL_THREADS = 256;
+constexpr int EDGE_ROOTS_MAX = 2 * (TILE_H + TILE_W);
+constexpr bool FINAL_STAGED = TILE_W <= 128;   // tile roots in shared memory too (with 256 columns both exceed 48 KB)
+struct FinalSmem {
+  alignas(16) int32_t table[TILE_SITES];
+  alignas(16) uint16_t roots[FINAL_STAGED ? TILE_SITES : 8];   // tile roots, tile row-major
+  uint16_t list[EDGE_ROOTS_MAX];
+  int n_edge;
+};
 __device__ __forceinline__ void final_labels_tile(int32_t* labels, const Grid& g, const LabelScratch& s, int t,
-                                                  int32_t* table /* shared, TILE_SITES */, int limit) {
+                                                  FinalSmem& fs, int limit) {
   const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
   const int y0 = ty * TILE_H, x0 = tx * TILE_W;
   const int h = min(TILE_H, g.H - y0), w = min(TILE_W, g.W - x0);
-  const int n = __ldcg(s.root_counts + t);
-  const int32_t* list = s.roots + (int64_t)t * TILE_SITES;
-  // 1. cluster roots of the tile roots: a root whose component stays inside
-  //    the tile is its cluster's root; the others walk the label array, four
-  //    walks of a thread in flight together
-  constexpr int U = 4;
-  for (int k0 = threadIdx.x; k0 < n; k0 += U * (int)blockDim.x) {
-    int r[U], x[U];
-    bool act[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int k = k0 + u * (int)blockDim.x;
-      const int raw = k < n ? __ldcg(list + k) : 0;
-      r[u] = raw & ~CCL_EDGE_ROOT;   // local index
-      act[u] = k < n && (raw & CCL_EDGE_ROOT);
-      x[u] = tile_global(r[u], y0, x0, g.W);
-    }
-    g_find_multi<U>(labels, x, act, limit, s.err);
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (k0 + u * (int)blockDim.x < n) table[r[u]] = x[u];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint16_t* lr = ccl_roots(s, t);
+  if (FINAL_STAGED)
+    for (int k = threadIdx.x; k < h * (TILE_W / 8); k += FINAL_THREADS) copy16_async(fs.roots + 8 * k, lr + 8 * k);
+  uint32_t edge = 0u;
+  if (threadIdx.x < TILE_SITES / 32) edge = (uint32_t)__ldcg(ccl_edges(s, t) + threadIdx.x);
+  if (threadIdx.x == 0) fs.n_edge = 0;
+  // 1. the table: own global indices
+  for (int k = threadIdx.x; k < h * (TILE_W / 4); k += FINAL_THREADS) {
+    const int G = tile_global(4 * k, y0, x0, g.W);   // four local indices of a strip are four sites in a row
+    *reinterpret_cast<int4*>(fs.table + 4 * k) = make_int4(G, G + 1, G + 2, G + 3);
   }
   __syncthreads();
-  // 2. every site takes its tile root's cluster root; the tile roots are the
-  //    16-bit local indices ccl_label_tile<true> left in the tile's slot
-  //    of `work`, eight sites per 16-byte word, in tile row-major order; labels go
-  //    out four sites per 16-byte store when rows start 16-byte aligned (a
-  //    16-byte aligned array and W % 4 == 0; x0 is a multiple of TILE_W, so w
-  //    is a multiple of 4 too)
-  const uint16_t* lr = reinterpret_cast<const uint16_t*>(s.work + (int64_t)t * TILE_SITES);
-  if ((g.W & 3) == 0 && (reinterpret_cast<uintptr_t>(labels) & 15) == 0) {
-    for (int k = threadIdx.x; k < TILE_SITES / 8; k += blockDim.x) {
-      const int sidx = 8 * k;
-      const int ly = sidx >> TILE_W_LOG2, lx = sidx & (TILE_W - 1);
-      if (ly >= h || lx >= w) continue;
-      const uint4 v = __ldcg(reinterpret_cast<const uint4*>(lr + sidx));
-      int32_t* p = labels + (int64_t)(y0 + ly) * g.W + x0 + lx;
-      *reinterpret_cast<int4*>(p) =
-          make_int4(table[v.x & 0xFFFFu], table[v.x >> 16], table[v.y & 0xFFFFu], table[v.y >> 16]);
-      if (lx + 8 <= w)
-        *reinterpret_cast<int4*>(p + 4) =
-            make_int4(table[v.z & 0xFFFFu], table[v.z >> 16], table[v.w & 0xFFFFu], table[v.w >> 16]);
+  // 2. edge roots listed, then their cluster roots
+  {
+    const int cnt = __popc(edge);
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(FULL, incl, d);
+      if (lane >= d) incl += v;
     }
-  } else {
-    for (int k = threadIdx.x; k < TILE_SITES; k += blockDim.x) {
-      const int ly = k >> TILE_W_LOG2, lx = k & (TILE_W - 1);
-      if (ly < h && lx < w) labels[(int64_t)(y0 + ly) * g.W + x0 + lx] = table[__ldcg(lr + k)];
-    }
+    int base = 0;
+    if (lane == 31 && incl) base = atomicAdd(&fs.n_edge, incl);
+    int at = __shfl_sync(FULL, base, 31) + incl - cnt;
+    for (; edge; edge &= edge - 1, ++at) fs.list[at] = (uint16_t)(32 * threadIdx.x + high_bit(edge & -edge));
   }
   __syncthreads();
+  for (int k = threadIdx.x; k < fs.n_edge; k += FINAL_THREADS) {
+    const int r = fs.list[k];
+    fs.table[r] = g_find(labels, fs.table[r], limit, s.err);
+  }
+  copies_wait();
+  __syncthreads();
+  // 3. every site takes its tile root's label: a warp per row, a lane per
+  //    aligned word of four labels
+  for (int ly = warp; ly < h; ly += FINAL_THREADS / 32) {
+    int32_t* row = labels + (int64_t)(y0 + ly) * g.W + x0;
+    const int shift = (int)(reinterpret_cast<uintptr_t>(row) >> 2) & 3;   // sites of the first word before the row
+    const uint16_t* rr = (FINAL_STAGED ? fs.roots : lr) + ly * TILE_W;
+    for (int q = lane; 4 * q < w + shift; q += 32) {
+      const int lx = 4 * q - shift;
+      if (lx >= 0 && lx + 4 <= w) {
+        int4 v;
+        if (shift == 0) {
+          const uint2 r = *reinterpret_cast<const uint2*>(rr + lx);
+          v = make_int4(fs.table[r.x & 0xFFFFu], fs.table[r.x >> 16], fs.table[r.y & 0xFFFFu], fs.table[r.y >> 16]);
+        } else {
+          v = make_int4(fs.table[rr[lx]], fs.table[rr[lx + 1]], fs.table[rr[lx + 2]], fs.table[rr[lx + 3]]);
+        }
+        *reinterpret_cast<int4*>(row + lx) = v;
+      } else {
+        for (int i = max(lx, 0); i < min(lx + 4, w); ++i) row[i] = fs.table[rr[i]];
+      }
+    }
+  }
 }
 
 }  // namespace swccl

@@ -148,6 +148,32 @@ __device__ __forceinline__ uint32_t site_bits(const uint8_t* mask, int64_t i) {
   return (uint32_t)(mask[i >> 2] >> (2 * (i & 3))) & 3u;
 }
 
+// Four byte lanes of a and b compared: bit k of the result is set iff byte k
+// of a equals byte k of b.  Exact zero-byte test of a ^ b (no carry crosses a
+// byte: each byte of (x & 0x7F..) + 0x7F.. is at most 0xFE), then the four
+// flag bits are gathered by one multiply.
+__device__ __forceinline__ uint32_t eq4(uint32_t a, uint32_t b) {
+  const uint32_t x = a ^ b;
+  const uint32_t y = ((x & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x;   // bit 7 of a byte set iff the byte is non-zero
+  const uint32_t z = (~y & 0x80808080u) >> 7;                  // bit 0 of a byte set iff equal
+  return (z * 0x00204081u) >> 21 & 0xFu;
+}
+
+// Bit i of x (i < 16) to bit 2i.
+__device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
+  x = (x | (x << 8)) & 0x00FF00FFu;
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  return (x | (x << 1)) & 0x55555555u;
+}
+
+// 16 bytes from global memory (through L2) to shared memory, asynchronously.
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Record a device-side failure without trapping: the first code wins.
 __device__ __forceinline__ void set_error(int* err, int code) {
   if (err) atomicCAS(err, 0, code);

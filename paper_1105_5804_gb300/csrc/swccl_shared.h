@@ -76,8 +76,8 @@ inline Grid make_grid(int H, int W, int periodic) {
 
 // Scratch of one labeling problem.
 struct LabelScratch {
-  int32_t* roots;        // n_tiles * TILE_H * TILE_W: tile-root lists (sweeps: a tile's edge-root bits)
-  int32_t* work;         // n_tiles * TILE_H * TILE_W: stand-alone labeling: 16-bit tile roots
+  int32_t* roots;        // n_tiles * TILE_H * TILE_W: tile-root lists (fused sweeps: a tile's edge-root bits)
+  int32_t* work;         // n_tiles * TILE_H * TILE_W: unused by sweeps (stand-alone labeling: 16-bit tile roots)
   int32_t* root_counts;  // n_tiles
   int32_t* seams;        // n_tiles * SeamLayout::INTS
   int* err;              // device status word
@@ -151,6 +151,10 @@ struct CclBatchView {
 // Bytes of LabelScratch for a grid (each part 256-byte aligned).
 int64_t label_scratch_bytes(const Grid& g);
 LabelScratch carve_label_scratch(const Grid& g, void* base, int* err);
+// The same for the stand-alone labeling (launch_ccl, launch_ccl_batch), which
+// needs less: ccl_scratch_bytes(g) <= label_scratch_bytes(g).
+int64_t ccl_scratch_bytes(const Grid& g);
+LabelScratch carve_ccl_scratch(const Grid& g, void* base, int* err);
 
 // ---------------------------------------------------------------------------
 // Launchers (each enqueues on `st`, returns the launch error).

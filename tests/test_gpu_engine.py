@@ -82,3 +82,23 @@ def test_merge_with_several_tiles_per_block(tile_w, W, rows):
         sw.ccl_status()
         ref, _ = oracle.label(mask, H, W, bool(periodic))
         assert np.array_equal(lab.cpu().numpy(), ref), periodic
+
+
+@pytest.mark.parametrize("H,W", [(1, 1), (1, 16), (3, 16), (16, 1), (40, 1), (2, 3), (9, 7), (5, 17), (7, 15), (40, 33),
+                                 (64, 128), (33, 1000), (129, 515), (2, 300), (300, 2), (61, 36)])
+@pytest.mark.parametrize("px_off,mask_off", [(0, 0), (1, 0), (16, 1), (32, 4)])
+def test_pixel_bonds(H, W, px_off, mask_off):
+    """Masks of images of any width (row ends anywhere in a thread's sites, the
+    last row and the last sites), aligned or not, and nothing written past the
+    mask's end."""
+    rng = np.random.default_rng(H * 1000 + W)
+    px = rng.integers(0, 2, (H, W)).astype(np.uint8)
+    buf = torch.zeros(H * W + px_off, dtype=torch.uint8, device="cuda")
+    buf[px_off:] = torch.from_numpy(px.reshape(-1)).cuda()
+    nb = sw.mask_bytes(H * W)
+    for periodic in (False, True):
+        out = torch.full((nb + mask_off + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+        sw.ccl_bonds_from_pixels(buf[px_off:], out[mask_off:], H, W, periodic)
+        got = out.cpu().numpy()
+        assert np.array_equal(got[mask_off:mask_off + nb], oracle.bonds_from_pixels(px, periodic))
+        assert (got[:mask_off] == 0xA5).all() and (got[mask_off + nb:] == 0xA5).all()
