@@ -195,11 +195,12 @@ constexpr int QREG = QREG_MAX;   // state counts kept in registers for q <= QREG
 }  // namespace fused
 using namespace fused;
 
-// After the labeling kernel, the first TILE_SITES / 32 words of a tile's
-// root-list slot hold its edge-root bits: bit r set iff local root r's component touches the tile
-// edge, so that its cluster may continue in other tiles.  The flip and the
-// few-cluster seed selection read them.
+// The labeling kernel leaves a tile's edge-root bits in TILE_SITES / 32 words
+// of the scratch (sweep_edges): bit r set iff local root r's component touches
+// the tile edge, so that its cluster may continue in other tiles.  The flip and
+// the few-cluster seed selection read them.
 constexpr int EDGE_WORDS = TILE_SITES / 32;
+__device__ __forceinline__ int32_t* sweep_edges(const LabelScratch& s, int t) { return s.roots + (int64_t)t * EDGE_WORDS; }
 static_assert(EDGE_WORDS == LABEL_THREADS, "one edge word per thread");
 // Flag on a root-list entry (local indices are below TILE_SITES).
 constexpr uint16_t EDGE_ROOT = 0x8000u;
@@ -213,14 +214,17 @@ struct LabelTileSmem {
   int hist[128];
 };
 
-constexpr int FLIP_LIST = TILE_SITES / 4;           // roots listed per pass (at criticality a tile has 0.14 per site)
-
-struct FlipTileSmem {
-  uint4 roots[TILE_SITES / 8];  // the tile roots of every thread's sites (pass-major, thread by thread)
-  uint8_t ns[TILE_SITES];       // new state, indexed by local root
-  uint16_t rlist[FLIP_LIST];    // the tile's roots, edge roots first
+// The flip's shared memory, for tiles of TH rows.
+template <int TH>
+struct FlipTileSmemT {
+  static constexpr int SITES = TH * TILE_W;
+  static constexpr int LIST = SITES / 4;        // roots listed per pass (at criticality a tile has 0.14 per site)
+  uint4 roots[SITES / 8];       // the tile roots of every thread's sites (pass-major, thread by thread)
+  uint8_t ns[SITES];            // new state, indexed by local root
+  uint16_t rlist[LIST];         // the tile's roots, edge roots first
   int warp_cnt[LABEL_THREADS / 32];
 };
+using FlipTileSmem = FlipTileSmemT<TILE_H>;
 
 // One tile of the fused draw-and-label step (see k_fused.cu).  All threads
 // of the CTA call it; it synchronises the CTA internally and on return.
@@ -242,7 +246,6 @@ __device__ __forceinline__ void sw_label_tile(const SwRep& R, int t, uint64_t sw
   const int y0 = ty * TILE_H, x0 = tx * TILE_W;
   const int h = min(TILE_H, L - y0), w = min(TILE_W, L - x0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int32_t* slot = s.roots + (int64_t)t * TILE_SITES;
   uint32_t* edge_bits = ls.edge_bits;
   edge_bits[threadIdx.x] = 0u;        // the engine's barriers order it before the marks
   if (q > QREG) {
@@ -317,23 +320,21 @@ __device__ __forceinline__ void sw_label_tile(const SwRep& R, int t, uint64_t sw
 
   // 4. my strip's part of the seam record; parent entries of edge roots; edge
   //    roots marked
-  seam_strip(sm, s.seams + (int64_t)t * SeamLayout::INTS, gpar, edge_bits, wn, e_last, h, w, y0, x0, L);
+  seam_strip(sm.par, s.seams + (int64_t)t * SeamLayout::INTS, gpar, edge_bits, wn, e_last, h, w, y0, x0, L);
 
   __syncthreads();
-  // 5. edge-root bits into the tile's root-list slot; each thread reads
-  //    and next clears only its own word
-  slot[threadIdx.x] = (int32_t)edge_bits[threadIdx.x];
+  // 5. edge-root bits; each thread reads and next clears only its own word
+  sweep_edges(s, t)[threadIdx.x] = (int32_t)edge_bits[threadIdx.x];
 }
 
 // One tile of the fused flip step (see k_fused.cu).  All threads of the CTA
 // call it; it synchronises the CTA internally and on return.
-// Site ownership of the flip: with G = TILE_W / 8 column groups, thread k
-// owns, in each of four passes j, the eight sites (row 8j + k / G, columns
-// 8 (k % G) .. 8 (k % G) + 7) of the tile; their tile roots are one 16-byte
-// word per pass.
+// Site ownership of the flip: with G = TILE_W / 8 column groups, thread k owns,
+// in each pass j (four for a 32-row tile), the eight sites (row 8j + k / G,
+// columns 8 (k % G) .. 8 (k % G) + 7) of the tile; their tile roots are one
+// 16-byte word per pass.
 constexpr int FLIP_GROUPS = TILE_W / 8;
-constexpr int FLIP_PASSES = TILE_SITES / (8 * LABEL_THREADS);
-static_assert(FLIP_PASSES * 8 * LABEL_THREADS == TILE_SITES && LABEL_THREADS / FLIP_GROUPS == 8, "site ownership");
+static_assert(LABEL_THREADS / FLIP_GROUPS == 8, "site ownership");
 
 // Local root (16 bits) of site i (0..7) of a pass word.
 __device__ __forceinline__ int root_in(const uint4& v, int i) {
@@ -356,11 +357,12 @@ __device__ __forceinline__ int root_in(const uint4& v, int i) {
 // site, a third of them the draws); critical Ising, L = 16384: 0.298 ms against
 // 0.389 ms with the roots read twice, flags looked up root by root and four
 // walks per thread in step.
-template <bool FEW = false, class Keys = SeedKey>
-__device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t sweep, int limit, FlipTileSmem& fs,
+// TH: rows of the lattice's tiles.
+template <bool FEW = false, int TH = TILE_H, class Keys = SeedKey>
+__device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t sweep, int limit, FlipTileSmemT<TH>& fs,
                                              const Keys& keys, const uint32_t* __restrict__ sel = nullptr,
                                              uint64_t P = 0) {
-  constexpr int PASSES = FLIP_PASSES;
+  constexpr int PASSES = TH / 8, FLIP_LIST = FlipTileSmemT<TH>::LIST;
   uint8_t* ns = fs.ns;
   int8_t* __restrict__ spins = R.spins;
   int32_t* __restrict__ gpar = R.gpar;
@@ -368,8 +370,8 @@ __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t swe
   int* err = R.s.err;
   const int L = R.g.W;
   const int ty = t / R.g.tiles_x, tx = t - ty * R.g.tiles_x;
-  const int y0 = ty * TILE_H, x0 = tx * TILE_W;
-  const int h = min(TILE_H, L - y0), w = min(TILE_W, L - x0);
+  const int y0 = ty * TH, x0 = tx * TILE_W;
+  const int h = min(TH, L - y0), w = min(TILE_W, L - x0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int orow = threadIdx.x / FLIP_GROUPS, lx0 = 8 * (threadIdx.x % FLIP_GROUPS);   // my sites
 
@@ -381,12 +383,12 @@ __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t swe
   const int id0 = local_of(orow, lx0);              // local index of my first site; pass j: id0 + 8 j TILE_W
   uint32_t edges = 0u;   // bit 8j + i: edge-root bit of site i of pass j
   {
-    const uint8_t* eb = reinterpret_cast<const uint8_t*>(R.s.roots + (int64_t)t * TILE_SITES) + (id0 >> 3);
+    const uint8_t* eb = reinterpret_cast<const uint8_t*>(sweep_edges(R.s, t)) + (id0 >> 3);
     const uint16_t* src = R.lroot + (int64_t)(y0 + orow) * L + x0 + lx0;
     const int64_t step = (int64_t)8 * L;
 #pragma unroll
     for (int j = 0; j < PASSES; ++j) edges |= (uint32_t)__ldcg(eb + j * TILE_W) << (8 * j);
-    if ((L & 7) == 0 && h == TILE_H && lx0 < w) {   // w is a multiple of 8
+    if ((L & 7) == 0 && h == TH && lx0 < w) {   // w is a multiple of 8
 #pragma unroll
       for (int j = 0; j < PASSES; ++j) copy16_async(my_roots + j * LABEL_THREADS, src + j * step);
       copies_wait();   // a thread reads back only what it copied itself
@@ -535,8 +537,8 @@ __device__ __forceinline__ void observe_tile(const SwRep& R, int t, uint64_t don
   const Grid& g = R.g;
   const int L = g.W, q = R.q;
   const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-  const int y0 = ty * TILE_H, x0 = tx * TILE_W;
-  const int h = min(TILE_H, L - y0), w = min(TILE_W, L - x0);
+  const int y0 = ty * g.th, x0 = tx * TILE_W;
+  const int h = min(g.th, L - y0), w = min(TILE_W, L - x0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int k = threadIdx.x; k < 128; k += LABEL_THREADS) ls.hist[k] = 0;
   __syncthreads();
@@ -591,10 +593,10 @@ __device__ __forceinline__ void few_select_seed(const SwRep& R, int ell, int64_t
   const uint4 w = philox(make_uint4((uint32_t)b, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_SEED),
                          (uint32_t)R.seed, (uint32_t)(R.seed >> 32));
   const int x = bx * B + state_of(w.x, B), y = by * B + state_of(w.y, B);
-  const int ty = y / TILE_H, tx = x / TILE_W;
+  const int ty = y / g.th, tx = x / TILE_W;
   const int r = R.lroot[(int64_t)y * L + x];
-  const int G = tile_global(r, ty * TILE_H, tx * TILE_W, L);
-  const int32_t* edge_bits = R.s.roots + (int64_t)(ty * g.tiles_x + tx) * TILE_SITES;
+  const int G = tile_global(r, ty * g.th, tx * TILE_W, L);
+  const int32_t* edge_bits = sweep_edges(R.s, ty * g.tiles_x + tx);
   const bool edge = (__ldcg(edge_bits + (r >> 5)) >> (r & 31)) & 1;
   const int root = edge ? g_find(R.gpar, G, limit, R.s.err) : G;
   atomicOr(sel + (root >> 5), 1u << (root & 31));

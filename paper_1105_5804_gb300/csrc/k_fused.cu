@@ -30,7 +30,7 @@
 // k_merge; between the merge and the flip, k_few_select marks the global
 // roots of the clusters holding the ell^2 seeds in a bit array, and
 // k_sw_flip_few moves only those clusters (each with probability p_flip).
-#include "fused_tile.cuh"
+#include "low_tile.cuh"
 
 namespace swccl {
 
@@ -44,19 +44,33 @@ k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_con
   sw_label_tile(R, blockIdx.x, sweep, do_obs, obs_cap, ls, keys);
 }
 
-__global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
-k_sw_flip(SwRep R, const SwCtl* __restrict__ ctl, int limit, const __grid_constant__ PhiloxKeys keys) {
-  __shared__ FlipTileSmem fs;
+// The same for a lattice cut into low tiles.
+template <int TH>
+__global__ void __launch_bounds__(LABEL_THREADS)
+k_sw_label_low(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys) {
+  __shared__ LowTileSmem<TH> ls;
   wait_for_previous();
-  sw_flip_tile(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys);   // the merge has advanced the counter
+  const uint64_t sweep = ctl->sweep;
+  const bool do_obs = sweep > 0 && ctl->obs_done != (long long)(sweep - 1);
+  sw_label_low_tile(R, blockIdx.x, sweep, do_obs, obs_cap, ls, keys);
 }
 
+// The merge has advanced the counter.
+template <int TH>
+__global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
+k_sw_flip(SwRep R, const SwCtl* __restrict__ ctl, int limit, const __grid_constant__ PhiloxKeys keys) {
+  __shared__ FlipTileSmemT<TH> fs;
+  wait_for_previous();
+  sw_flip_tile<false, TH>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys);
+}
+
+template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
 k_sw_flip_few(SwRep R, const SwCtl* __restrict__ ctl, int limit, const uint32_t* __restrict__ sel, uint64_t P,
               const __grid_constant__ PhiloxKeys keys) {
-  __shared__ FlipTileSmem fs;
+  __shared__ FlipTileSmemT<TH> fs;
   wait_for_previous();
-  sw_flip_tile<true>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys, sel, P);
+  sw_flip_tile<true, TH>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys, sel, P);
 }
 
 constexpr int SELECT_THREADS = 256;
@@ -134,14 +148,16 @@ cudaError_t launch_sw_label(const int8_t* spins, uint16_t* lroot, int32_t* gpar,
                             const LabelScratch& s, int q, uint64_t T, uint64_t seed, const SwCtl* ctl,
                             int64_t* obs, int obs_cap, cudaStream_t st) {
   const SwRep R = make_rep(const_cast<int8_t*>(spins), lroot, gpar, obs, g, s, q, T, seed);
-  return launch_after(k_sw_label, g.n_tiles(), LABEL_THREADS, st, R, ctl, obs_cap, philox_keys(seed));
+  auto* kernel = g.th == 8 ? k_sw_label_low<8> : g.th == 16 ? k_sw_label_low<16> : k_sw_label;
+  return launch_after(kernel, g.n_tiles(), LABEL_THREADS, st, R, ctl, obs_cap, philox_keys(seed));
 }
 
 cudaError_t launch_sw_flip(int8_t* spins, const uint16_t* lroot, int32_t* gpar, const Grid& g,
                            const LabelScratch& s, int q, uint64_t seed, const SwCtl* ctl, cudaStream_t st) {
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
   const SwRep R = make_rep(spins, const_cast<uint16_t*>(lroot), gpar, nullptr, g, s, q, 0, seed);
-  return launch_after(k_sw_flip, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, philox_keys(seed));
+  auto* kernel = g.th == 8 ? k_sw_flip<8> : g.th == 16 ? k_sw_flip<16> : k_sw_flip<TILE_H>;
+  return launch_after(kernel, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, philox_keys(seed));
 }
 
 // The same for L % 16 == 0 at HBM speed: a thread owns 16 columns (one
@@ -234,7 +250,29 @@ cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gp
                                const SwCtl* ctl, cudaStream_t st) {
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
   const SwRep R = make_rep(spins, const_cast<uint16_t*>(lroot), gpar, nullptr, g, s, q, 0, seed);
-  return launch_after(k_sw_flip_few, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, sel, P, philox_keys(seed));
+  auto* kernel = g.th == 8 ? k_sw_flip_few<8> : g.th == 16 ? k_sw_flip_few<16> : k_sw_flip_few<TILE_H>;
+  return launch_after(kernel, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, sel, P, philox_keys(seed));
 }
+
+// The lowest tiles that still leave few warps per SM: below about 16 (24 for
+// tiles of 16 rows) a tile's time is the latency of its chains, above it the
+// tiles share an SM's issue slots and the engine's work per tile counts.
+// Critical Ising, us per sweep with tiles of 32 / 16 / 8 rows: L = 256
+// 25.5 / 21.8 / 20.2, L = 768 (288 tiles of 8 rows) 27.7 / 24.1 / 23.5, L = 1000
+// (252 of 16, 500 of 8) 28.9 / 26.7 / 27.3, L = 1280 (400 of 16) 31.8 / 29.3 / 33.2,
+// L = 1440 (540 of 16) 31.6 / 31.9 / 37.3, L = 2048 42.4 / 45.5 / 53.8.
+int sweep_tile_rows(int L) {
+  constexpr int SMS = 152;
+  auto warps = [&](int th) { return make_grid(L, L, 1, th).n_tiles() * STRIPS; };
+  return warps(8) <= 16 * SMS ? 8 : warps(16) <= 24 * SMS ? 16 : TILE_H;
+}
+
+LabelScratch sweep_scratch(const Grid& g, const LabelScratch& s) {
+  LabelScratch low = s;
+  if (g.th < TILE_H) low.seams = s.work;   // up to TILE_H / th as many records in the sweep's unused part
+  return low;
+}
+static_assert((TILE_H / 8) * SeamLayout::INTS <= TILE_SITES, "the records of a 32-row tile's low tiles fit its slot");
+static_assert((TILE_H / 8) * EDGE_WORDS <= TILE_SITES, "and their edge-root words");
 
 }  // namespace swccl

@@ -138,7 +138,7 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
 
   // 5. my strip's part of the seam record; parent entries of edge roots; edge
   //    roots marked
-  seam_strip(sm, s.seams + (int64_t)t * SeamLayout::INTS, labels, cs.edge_bits, wn, e_last, h, w, y0, x0, W);
+  seam_strip(par, s.seams + (int64_t)t * SeamLayout::INTS, labels, cs.edge_bits, wn, e_last, h, w, y0, x0, W);
 
   // 6. LOCAL: edge-root bits; otherwise the root list
   if (LOCAL) {

@@ -75,7 +75,9 @@ struct sw_handle {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int device = 0;
-  Grid grid{};
+  Grid grid{};          // 32-row tiles: staged sweeps, and the size of every buffer
+  Grid grid_f{};        // tiles of the fused sweeps
+  LabelScratch ls_f{};  // their scratch
   int8_t* spins = nullptr;
   uint8_t* mask = nullptr;
   int32_t* labels = nullptr;
@@ -155,21 +157,21 @@ cudaError_t enqueue_sweep_fused(sw_handle* h, cudaEvent_t* ev) {
   const cudaStream_t st = h->stream;
   if (ev && ((e = cudaEventRecord(ev[0], st)) != cudaSuccess || (e = cudaEventRecord(ev[1], st)) != cudaSuccess))
     return e;
-  if ((e = launch_sw_label(h->spins, h->lroot, h->labels, h->grid, h->ls, h->q, h->T, h->seed, h->ctl, h->obs,
+  if ((e = launch_sw_label(h->spins, h->lroot, h->labels, h->grid_f, h->ls_f, h->q, h->T, h->seed, h->ctl, h->obs,
                            OBS_CAP, st)))
     return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
-  if ((e = launch_merge(h->labels, h->grid, h->ls, h->ctl, h->obs, OBS_CAP, h->q, st))) return e;
+  if ((e = launch_merge(h->labels, h->grid_f, h->ls_f, h->ctl, h->obs, OBS_CAP, h->q, st))) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
   if (h->update == SW_UPDATE_FEW &&
-      (e = launch_few_select(h->lroot, h->labels, h->grid, h->ls, h->seed, h->ell, h->sel, h->ctl, st)))
+      (e = launch_few_select(h->lroot, h->labels, h->grid_f, h->ls_f, h->seed, h->ell, h->sel, h->ctl, st)))
     return e;
   if (ev && (e = cudaEventRecord(ev[4], st)) != cudaSuccess) return e;
   if (h->update == SW_UPDATE_FEW) {
-    if ((e = launch_sw_flip_few(h->spins, h->lroot, h->labels, h->grid, h->ls, h->q, h->seed, h->sel, h->P_flip,
+    if ((e = launch_sw_flip_few(h->spins, h->lroot, h->labels, h->grid_f, h->ls_f, h->q, h->seed, h->sel, h->P_flip,
                                 h->ctl, st)))
       return e;
-  } else if ((e = launch_sw_flip(h->spins, h->lroot, h->labels, h->grid, h->ls, h->q, h->seed, h->ctl, st))) {
+  } else if ((e = launch_sw_flip(h->spins, h->lroot, h->labels, h->grid_f, h->ls_f, h->q, h->seed, h->ctl, st))) {
     return e;
   }
   return ev ? cudaEventRecord(ev[5], st) : cudaSuccess;
@@ -303,6 +305,7 @@ sw_handle* sw_create_threshold(int L, int q, uint64_t T, uint64_t seed, int hot_
   h->T = T;
   h->seed = seed;
   h->grid = make_grid(L, L, 1);
+  h->grid_f = make_grid(L, L, 1, sweep_tile_rows(L));
   const int64_t N = (int64_t)L * L;
   auto bad = [&](cudaError_t e, const char* what) -> sw_handle* {
     cuda_fail(e, what);
@@ -331,6 +334,7 @@ sw_handle* sw_create_threshold(int L, int q, uint64_t T, uint64_t seed, int hot_
   if (L <= SMALL_L && (e = small_prepare())) return bad(e, "small-lattice kernel");
   h->ls = carve_label_scratch(h->grid, h->scratch,
                               reinterpret_cast<int*>(reinterpret_cast<char*>(h->ctl) + offsetof(SwCtl, err)));
+  h->ls_f = sweep_scratch(h->grid_f, h->ls);
   {
     static const SwCtl init_ctl = {0ull, -1ll, 0, 0};
     if ((e = cudaMemcpyAsync(h->ctl, &init_ctl, sizeof(SwCtl), cudaMemcpyHostToDevice, h->stream)))

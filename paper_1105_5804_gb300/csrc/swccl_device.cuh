@@ -131,6 +131,17 @@ __device__ __forceinline__ void philox_draws(uint4 (&ctr)[N], const PhiloxKeys& 
   }
 }
 
+template <int N>
+__device__ __forceinline__ void philox_draws(uint4 (&ctr)[N], const SeedKey& k) {
+  PhiloxKeys all;
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    all.lo[r] = k.lo + (uint32_t)r * 0x9E3779B9u;
+    all.hi[r] = k.hi + (uint32_t)r * 0xBB67AE85u;
+  }
+  philox_draws(ctr, all);
+}
+
 __device__ __forceinline__ uint4 philox_draw(uint4 ctr, const SeedKey& k) { return philox(ctr, k.lo, k.hi); }
 
 __device__ __forceinline__ uint4 draw(uint32_t c0, uint64_t sweep, uint32_t tag, uint64_t seed) {

@@ -52,6 +52,7 @@ struct Grid {
   int H, W;
   int tiles_x, tiles_y;
   int periodic;
+  int th;               // rows of a tile: TILE_H, or fewer for a sweep of a small lattice (low_tile.cuh)
   __host__ __device__ int64_t n_sites() const { return (int64_t)H * W; }
   __host__ __device__ int n_tiles() const { return tiles_x * tiles_y; }
 };
@@ -64,19 +65,20 @@ struct Box3 {
   __host__ __device__ int64_t n_bricks() const { return (int64_t)bx * by * bz; }
 };
 
-inline Grid make_grid(int H, int W, int periodic) {
+inline Grid make_grid(int H, int W, int periodic, int th = TILE_H) {
   Grid g;
+  g.th = th;
   g.H = H;
   g.W = W;
   g.tiles_x = (W + TILE_W - 1) / TILE_W;
-  g.tiles_y = (H + TILE_H - 1) / TILE_H;
+  g.tiles_y = (H + th - 1) / th;
   g.periodic = periodic ? 1 : 0;
   return g;
 }
 
 // Scratch of one labeling problem.
 struct LabelScratch {
-  int32_t* roots;        // n_tiles * TILE_H * TILE_W: tile-root lists (fused sweeps: a tile's edge-root bits)
+  int32_t* roots;        // n_tiles * TILE_H * TILE_W: tile-root lists (fused sweeps: TILE_SITES / 32 edge-root words per tile)
   int32_t* work;         // n_tiles * TILE_H * TILE_W: unused by sweeps (stand-alone labeling: 16-bit tile roots)
   int32_t* root_counts;  // n_tiles
   int32_t* seams;        // n_tiles * SeamLayout::INTS
@@ -151,6 +153,10 @@ struct CclBatchView {
 // Bytes of LabelScratch for a grid (each part 256-byte aligned).
 int64_t label_scratch_bytes(const Grid& g);
 LabelScratch carve_label_scratch(const Grid& g, void* base, int* err);
+// Rows of the tiles a fused sweep of an L x L lattice is cut into, and its
+// scratch: that of the 32-row grid, whose parts the lower tiles share.
+int sweep_tile_rows(int L);
+LabelScratch sweep_scratch(const Grid& g, const LabelScratch& s);
 // The same for the stand-alone labeling (launch_ccl, launch_ccl_batch), which
 // needs less: ccl_scratch_bytes(g) <= label_scratch_bytes(g).
 int64_t ccl_scratch_bytes(const Grid& g);

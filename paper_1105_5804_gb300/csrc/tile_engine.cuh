@@ -290,13 +290,13 @@ __device__ __forceinline__ void tile_engine(TileSmemT<ROWS>& sm, uint32_t we, ui
 // gpar[g] = g of those roots and their marks in edge_bits (TILE_SITES / 32
 // words, zeroed before the engine).  wn: my row's north bonds; e_last: raw
 // east bits of column w - 1 (bit = row) in the warp that holds that column.
-__device__ __forceinline__ void seam_strip(const TileSmem& sm, int32_t* rec, int32_t* gpar, uint32_t* edge_bits,
+__device__ __forceinline__ void seam_strip(const uint16_t* par, int32_t* rec, int32_t* gpar, uint32_t* edge_bits,
                                            uint32_t wn, uint32_t e_last, int h, int w, int y0, int x0, int W) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   auto edge_root = [&](bool ok, int i) -> int32_t {
     // global index of the tile root of local site i; the first of a run of
     // equal roots among consecutive lanes writes its parent entry and its mark
-    const int r = ok ? root_of(sm.par, i) : -1;
+    const int r = ok ? root_of(par, i) : -1;
     const int left = __shfl_up_sync(FULL, r, 1);
     if (!ok) return -1;
     const int32_t gr = tile_global(r, y0, x0, W);
