@@ -39,20 +39,20 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "b79bdb9c1397e87a"
+SWEEP_COUNTER_HASH = "5170107d943b40a9"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
-    "k_sw_label": ((88.861440 + 130.782976) * 1e6 / 67108864, 184026506 / 67108864),
-    "k_merge": ((56.304640 + 0.724736) * 1e6 / 67108864, 15167883 / 67108864),
-    "k_sw_flip": ((203.574784 + 48.139008) * 1e6 / 67108864, 71162469 / 67108864),
+    "k_sw_label": ((88.993536 + 130.604544) * 1e6 / 67108864, 184026607 / 67108864),
+    "k_merge": ((56.304896 + 0.751872) * 1e6 / 67108864, 15152868 / 67108864),
+    "k_sw_flip": ((203.557632 + 47.628288) * 1e6 / 67108864, 71157729 / 67108864),
 }
 # The stand-alone labeling call (k_ccl_tile, k_merge, k_ccl_final), one ncu
 # capture per kernel of a 4096^2 critical percolation mask: DRAM bytes per site,
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "ad769f64540b9ac8"
+CCL_COUNTER_HASH = "28b8517f05bf3fa4"
 CCL_COUNTER_TILE_W = 128
-CCL_TRAFFIC_BYTES_PER_SITE = ((6.654208 + 2.559232) + (16.646144 + 0.000000) + (53.508096 + 10.329600)) * 1e6 / 16777216
+CCL_TRAFFIC_BYTES_PER_SITE = ((6.648832 + 2.544384) + (16.644864 + 0.000000) + (53.508096 + 10.391296)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8
 # spins once (2 B, the minimum of any sweep); the kernel split adds the
 # 16-bit tile roots written by k_sw_label and read by k_sw_flip (6 B).
