@@ -79,6 +79,24 @@ __device__ __forceinline__ bool grid_barrier(BatchCtl* ctl, unsigned nblocks, lo
 
 }  // namespace
 
+// Initial state of every chain: its tiles' blocks share its sites, four per
+// thread and step (L % 4 == 0), and the clearing of its observable ring.
+__global__ void __launch_bounds__(LABEL_THREADS) k_batch_init(BatchView b, int hot) {
+  const SwRep& R = b.reps[b.tile_rep[blockIdx.x]];
+  const int64_t i0 = (int64_t)(blockIdx.x - R.tile0) * LABEL_THREADS + threadIdx.x;
+  const int64_t stride = (int64_t)R.g.n_tiles() * LABEL_THREADS;
+  for (int64_t i = i0; i < R.g.n_sites() / 4; i += stride) {
+    uint32_t w = 0u;
+    if (hot) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        w |= (uint32_t)state_of(draw((uint32_t)(4 * i + k), 0, TAG_INIT, R.seed).x, R.q) << (8 * k);
+    }
+    reinterpret_cast<uint32_t*>(R.spins)[i] = w;
+  }
+  for (int64_t i = i0; i < (int64_t)b.obs_cap * (R.q + 1); i += stride) R.obs[i] = 0;
+}
+
 // ---------------------------------------------------------------------------
 // Phase kernels: one CTA per global tile (merge: per few tiles).
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_batch_label(BatchView b, const BatchCtl* __restrict__ ctl) {
@@ -162,6 +180,11 @@ __global__ void __launch_bounds__(LABEL_THREADS, 4 * 256 / TILE_W) k_batch_persi
 }
 
 // ---------------------------------------------------------------------------
+cudaError_t launch_batch_init(const BatchView& b, int hot, cudaStream_t st) {
+  k_batch_init<<<b.n_tiles, LABEL_THREADS, 0, st>>>(b, hot);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_batch_label(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
   return launch_after(k_batch_label, b.n_tiles, LABEL_THREADS, st, b, ctl);
 }

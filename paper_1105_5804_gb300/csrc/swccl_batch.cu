@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cstdint>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -88,11 +89,10 @@ cudaError_t finish_batch_observables(sw_batch* b) {
   return launch_batch_observe(b->view, b->ctl, b->stream);
 }
 
+// Wait for the batch's work; report failures the device recorded.
 int batch_status(sw_batch* b) {
-  cudaError_t e = cudaStreamSynchronize(b->stream);
-  if (e != cudaSuccess) return set_last_error(SW_ERR_CUDA, std::string("batch: ") + cudaGetErrorString(e));
   BatchCtl c;
-  e = cudaMemcpyAsync(&c, b->ctl, sizeof(c), cudaMemcpyDeviceToHost, b->stream);
+  cudaError_t e = cudaMemcpyAsync(&c, b->ctl, sizeof(c), cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return set_last_error(SW_ERR_CUDA, std::string("batch: ") + cudaGetErrorString(e));
   if (c.err) b->failed = c.err;
@@ -210,7 +210,13 @@ sw_batch* create_batch(int n, const int* L, const int* q, const double* beta, co
   b->d_tile_rep = reinterpret_cast<int*>(base + lay.tile_rep);
   b->total_sites = lay.total_sites;
   int* err = reinterpret_cast<int*>(reinterpret_cast<char*>(b->ctl) + offsetof(BatchCtl, err));
-  std::vector<int> tile_rep(lay.n_tiles);
+  // the tables (control block, chains, tile map) lie together at the start of the
+  // arena: one copy brings them, one kernel sets up every chain from them (eight
+  // chains of a served group: two calls where there were nineteen)
+  std::vector<char> tables(lay.chain[0], 0);
+  static const BatchCtl init_ctl = {0ull, -1ll, 0, 0u, 0u, 0};
+  memcpy(tables.data() + lay.ctl, &init_ctl, sizeof(BatchCtl));
+  int* tile_rep = reinterpret_cast<int*>(tables.data() + lay.tile_rep);
   int t0 = 0;
   for (int r = 0; r < n; ++r) {
     const int64_t N = (int64_t)L[r] * L[r];
@@ -233,28 +239,22 @@ sw_batch* create_batch(int n, const int* L, const int* q, const double* beta, co
     for (int k = 0; k < lay.grids[r].n_tiles(); ++k) tile_rep[t0 + k] = r;
     t0 += lay.grids[r].n_tiles();
     b->reps.push_back(R);
-    if ((e = launch_init_spins(R.spins, L[r], q[r], seed[r], hot_start, b->stream))) return bad(e, "init spins");
-    if ((e = cudaMemsetAsync(R.obs, 0, (int64_t)BATCH_OBS_CAP * (q[r] + 1) * 8, b->stream))) return bad(e, "memset");
   }
-  if ((e = cudaMemcpyAsync(b->d_reps, b->reps.data(), sizeof(SwRep) * n, cudaMemcpyHostToDevice, b->stream)))
-    return bad(e, "chain table");
-  if ((e = cudaMemcpyAsync(b->d_tile_rep, tile_rep.data(), sizeof(int) * lay.n_tiles, cudaMemcpyHostToDevice,
-                           b->stream)))
-    return bad(e, "tile map");
-  static const BatchCtl init_ctl = {0ull, -1ll, 0, 0u, 0u, 0};
-  if ((e = cudaMemcpyAsync(b->ctl, &init_ctl, sizeof(BatchCtl), cudaMemcpyHostToDevice, b->stream)))
-    return bad(e, "control block");
+  memcpy(tables.data() + lay.reps, b->reps.data(), sizeof(SwRep) * n);
+  if ((e = cudaMemcpyAsync(base, tables.data(), tables.size(), cudaMemcpyHostToDevice, b->stream)))
+    return bad(e, "chain tables");
   b->view.reps = b->d_reps;
   b->view.tile_rep = b->d_tile_rep;
   b->view.n_reps = n;
   b->view.n_tiles = lay.n_tiles;
   b->view.obs_cap = BATCH_OBS_CAP;
   b->view.limit = (int)std::min<int64_t>(lay.max_sites + 64, (int64_t)1 << 30);
+  if ((e = launch_batch_init(b->view, hot_start, b->stream))) return bad(e, "init spins");
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->blocks = std::max(1, batch_persistent_blocks_per_sm()) * std::max(1, sms);
-  // the host tables above are copied from pageable memory: the copies are
+  // the host tables above are copied from pageable memory: the copy is
   // staged before cudaMemcpyAsync returns, so no wait is needed here
   return b;
 }
@@ -424,11 +424,17 @@ int sw_batch_observables_async(sw_batch* b, int replica, int64_t* dst, int max_s
 
 int sw_batch_get_spins(sw_batch* b, int replica, int8_t* dst, int is_device) {
   if (!b || replica < 0 || replica >= b->n || !dst) return set_last_error(SW_ERR_ARG, "sw_batch_get_spins: bad arguments");
-  int rc = batch_status(b);
-  if (rc) return rc;
   const int64_t n = (int64_t)b->L[replica] * b->L[replica];
-  cudaError_t e = is_device ? launch_copy_if(dst, b->reps[replica].spins, n, nullptr, b->stream)
-                            : cudaMemcpyAsync(dst, b->reps[replica].spins, n, cudaMemcpyDeviceToHost, b->stream);
+  const int8_t* src = b->reps[replica].spins;
+  cudaError_t e = cudaSuccess;
+  if (is_device) {
+    // the copy looks at the device's status itself, so that the host waits once
+    e = launch_copy_if(dst, src, n, &b->ctl->err, b->stream);
+    if (e == cudaSuccess) return batch_status(b);
+  } else {
+    if (const int rc = batch_status(b)) return rc;
+    e = cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToHost, b->stream);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return set_last_error(SW_ERR_CUDA, std::string("sw_batch_get_spins: ") + cudaGetErrorString(e));
   return SW_OK;

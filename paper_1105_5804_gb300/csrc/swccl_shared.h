@@ -238,7 +238,8 @@ cudaError_t small_prepare();
 cudaError_t launch_sw_small(int8_t* spins, int L, int q, uint64_t T, uint64_t seed, SwCtl* ctl, int64_t* obs,
                             int obs_cap, int n, cudaStream_t st);
 
-// Batched chains (k_batch.cu).
+// Batched chains (k_batch.cu).  init: spins of every chain, observable rings cleared.
+cudaError_t launch_batch_init(const BatchView& b, int hot, cudaStream_t st);
 cudaError_t launch_batch_label(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
 cudaError_t launch_batch_merge(const BatchView& b, BatchCtl* ctl, cudaStream_t st);   // and advance (see launch_merge)
 cudaError_t launch_batch_flip(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
