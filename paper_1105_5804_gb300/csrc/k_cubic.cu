@@ -19,8 +19,8 @@
 //              G), writes the open bonds that leave the brick as face words,
 //              and counts the observables of the spins it read (the previous
 //              sweep's);
-//  k3_merge    one thread per face bond: if its bit is set, joins the brick
-//              roots on its two ends on gpar with global atomics;
+//  k3_merge    one CTA per brick: lists the pairs of brick roots that its open
+//              face bonds join, then joins them on gpar with global atomics;
 //  k3_flip     one CTA per brick: lists the brick's roots; an edge root looks
 //              up its cluster root R on gpar, any other root is its own
 //              cluster's root; one FLIP draw per root (keyed by R, Sec. II.D)
@@ -36,7 +36,7 @@ namespace swccl {
 constexpr int B3X = 32, B3Y = 8, B3Z = 16;
 constexpr int B3_SITES = B3X * B3Y * B3Z;
 constexpr int B3_THREADS = 256;
-static_assert(B3_THREADS == B3X * B3Y, "thread (lx, ly) walks the brick along z");
+static_assert(B3_THREADS == 32 * B3Y && 32 == 2 * B3Z, "a warp per plane, two lanes per row");
 
 __device__ __forceinline__ int64_t site3(const Box3& b, int x, int y, int z) {
   return ((int64_t)z * b.Y + y) * b.X + x;
@@ -93,57 +93,50 @@ constexpr int Y_LIST = 256;
 struct Local3Smem {
   TileSmemT<B3Z> tile;
   uint32_t edge[B3_EDGE_WORDS];
-  union {
-    uint32_t plane[B3Y][4][B3X];             // every plane's spins: byte z of word z / 4 of column lx
-    uint16_t list[B3Y][Y_LIST];              // then: the +y contacts of every plane
-  };
-  alignas(16) uint8_t xface[B3Y][B3Z];       // spins of the column at x0 + w
+  uint16_t list[B3Y][Y_LIST];                // the +y contacts of every plane
   unsigned red[(1 + QREG) * (B3_THREADS / 32)];
   int hist[128];
 };
 
-// Transposes a 32 x 32 bit matrix held one row per lane.
-__device__ __forceinline__ uint32_t transpose32(uint32_t x) {
-  const int lane = threadIdx.x & 31;
-  constexpr uint32_t M[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int s = 16 >> i;
-    const bool up = lane & s;
-    const uint32_t y = __shfl_xor_sync(FULL, x, s);
-    const uint32_t keep = up ? ~M[i] : M[i];
-    x = (x & keep) | (__funnelshift_l(y, y, up ? 32 - s : s) & ~keep);
+// Sixteen consecutive spins from site i on, of which the first nv are wanted
+// (the others are arbitrary).  whole: rows start 16-byte aligned and nv is 0 or
+// 16; otherwise aligned words are shifted into place (a word is read only if it
+// holds a wanted spin, so reads stay inside the array's last word).
+__device__ __forceinline__ void load_row(const int8_t* __restrict__ spins, uint32_t i, int nv, bool whole,
+                                         uint32_t (&c)[4]) {
+  if (whole) {
+    const uint4 v = nv > 0 ? *reinterpret_cast<const uint4*>(spins + i) : make_uint4(0u, 0u, 0u, 0u);
+    c[0] = v.x;
+    c[1] = v.y;
+    c[2] = v.z;
+    c[3] = v.w;
+    return;
   }
-  return x;
+  const int off = (int)(i & 3u);
+  const uint32_t* p = reinterpret_cast<const uint32_t*>(spins + (i - off));
+  uint32_t v[5];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) v[j] = nv > 0 && 4 * j < off + nv ? p[j] : 0u;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) c[j] = __funnelshift_r(v[j], v[j + 1], 8 * off);
 }
 
-// Spins of the 16 sites along z at column (x, y) of brick k, four per word;
-// zero past the brick's depth.
-__device__ __forceinline__ void load_column(const int8_t* __restrict__ spins, const Box3& b, const Brick& k, int x,
-                                            int y, bool in, uint32_t (&c)[4]) {
-  const int64_t XY = (int64_t)b.X * b.Y;
-  const int8_t* p = spins + site3(b, in ? x : 0, in ? y : 0, k.z0);
-  uint32_t v[B3Z];
-#pragma unroll
-  for (int lz = 0; lz < B3Z; ++lz) v[lz] = (in && lz < k.d) ? (uint32_t)(uint8_t)p[lz * XY] : 0u;
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    c[j] = v[4 * j] | v[4 * j + 1] << 8 | v[4 * j + 2] << 16 | v[4 * j + 3] << 24;
-}
-
-// Bit lz set iff byte lz of the columns a and b is equal.
-__device__ __forceinline__ uint32_t eq_column(const uint32_t (&a)[4], const uint32_t (&b)[4]) {
+// Bit i set iff byte i of the rows a and b is equal.
+__device__ __forceinline__ uint32_t eq_row(const uint32_t (&a)[4], const uint32_t (&b)[4]) {
   return eq4(a[0], b[0]) | eq4(a[1], b[1]) << 4 | eq4(a[2], b[2]) << 8 | eq4(a[3], b[3]) << 12;
 }
 
-// Local step of a brick.  Bound by instruction issue: 16 draws per thread
-// (about 45 instructions each) and the engine; the comparisons work on four
-// spins of a column per word, the bond bits of a column (one thread) become
-// the engine's row words (one lane per row) by two bit-matrix transposes, and
-// the +y bonds are joined in three rounds between disjoint pairs of plane
-// groups, so that plain stores do (one warp per round and boundary, no shared
-// atomics).
-__global__ void __launch_bounds__(B3_THREADS, 6)
+// Local step of a brick.  Bound by instruction issue and by the latency of the
+// shared-memory walks: 16 draws per thread (about 45 instructions each, 18 % of
+// a warp's time), the engine (17 %), the +y joins (22 %), so eight CTAs per SM
+// (32 registers) beat six.  A lane has half a row: its spins and those at +y and
+// +z are three 16-byte loads (the neighbours' from L1), compared four per word,
+// and the bond bits are row words already.  With a thread per column (byte
+// loads, neighbours' spins through shared memory, bit-matrix transposes) and
+// the +y joins in three rounds between disjoint planes (plain stores, but one to
+// four warps of eight busy): 185 us at 256^3 and six CTAs, 172 with joins by
+// compare-and-swap all at once, 159 with rows, 153 with eight CTAs.
+__global__ void __launch_bounds__(B3_THREADS, 8)
 k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t* __restrict__ gpar,
          uint32_t* __restrict__ words, Box3 b, int q, uint64_t T, const __grid_constant__ PhiloxKeys keys,
          const SwCtl* __restrict__ ctl, int64_t* obs, int obs_cap, int* err) {
@@ -156,93 +149,76 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
   const uint64_t sweep = ctl->sweep;
   const bool do_obs = sweep > 0 && ctl->obs_done != (long long)(sweep - 1);
   const bool plane = ly < k.h;               // the warp has a plane
-  const bool col = plane && lane < k.w;      // the thread has a column
-  const uint32_t depth = (1u << k.d) - 1u;   // bit lz: the brick has row lz
   if (threadIdx.x < B3_EDGE_WORDS) ls.edge[threadIdx.x] = 0u;
   if (q > QREG)
     for (int j = threadIdx.x; j < 128; j += B3_THREADS) ls.hist[j] = 0;
 
-  // 1. spins of my column, of the columns past the brick (+x, +y) and of the
-  //    row past it (+z); which neighbours are equal (bit = lz)
-  uint32_t ex, ey, ez;
+  // 1. lane (lz, half) has sixteen sites of a row of its warp's plane: their
+  //    spins, the rows at +y and +z and the spin at +x; which neighbours are
+  //    equal (bit = site)
+  const int lz = lane >> 1, half = lane & 1;
+  const int nv = plane && lz < k.d ? min(max(k.w - 16 * half, 0), 16) : 0;
+  const uint32_t row0 = (uint32_t)site3(b, k.x0, k.y0 + ly, k.z0 + lz);   // my row's first site; past the box without sites
+  const uint32_t site0 = row0 + 16 * half;
+  uint32_t ex = 0u, ey = 0u, ez = 0u;
   {
-    uint32_t c[4];
-    load_column(spins, b, k, k.x0 + lane, k.y0 + ly, col, c);
-    const int zf = k.z0 + k.d == b.Z ? 0 : k.z0 + k.d;
-    const uint32_t top = col ? (uint32_t)(uint8_t)spins[site3(b, k.x0 + lane, k.y0 + ly, zf)] : 0u;
-    const int xf = k.x0 + k.w == b.X ? 0 : k.x0 + k.w, yf = k.y0 + k.h == b.Y ? 0 : k.y0 + k.h;
-    if (lane < B3Z)
-      ls.xface[ly][lane] = plane && lane < k.d ? (uint8_t)spins[site3(b, xf, k.y0 + ly, k.z0 + lane)] : 0;
-    uint32_t n[4];
-    if (ly == k.h - 1) load_column(spins, b, k, k.x0 + lane, yf, col, n);   // the plane past the brick
+    const bool whole = (b.X & 15) == 0;
+    const int y = k.y0 + ly, z = k.z0 + lz, x1 = k.x0 + 16 * half + nv;
+    uint32_t c[4], n[4], ny[4], nz[4];
+    load_row(spins, site0, nv, whole, c);
+    load_row(spins, site0 + (y + 1 == b.Y ? -(uint32_t)y : 1u) * (uint32_t)b.X, nv, whole, ny);
+    load_row(spins, site0 + (z + 1 == b.Z ? -(uint32_t)z : 1u) * ((uint32_t)b.X * (uint32_t)b.Y), nv, whole, nz);
+    const uint32_t next = nv > 0 ? (uint32_t)(uint8_t)spins[x1 == b.X ? row0 - k.x0 : row0 - k.x0 + x1] : 0u;
+    const uint32_t mine = (1u << nv) - 1u;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) ls.plane[ly][j][lane] = c[j];
-    __syncthreads();
-    if (ly < k.h - 1) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) n[j] = ls.plane[ly + 1][j][lane];
+    for (int j = 0; j < 4; ++j) {
+      n[j] = __funnelshift_r(c[j], j < 3 ? c[j + 1] : next, 8);
+      if (nv < 16 && (nv - 1) >> 2 == j) {
+        const int sh = 8 * ((nv - 1) & 3);
+        n[j] = (n[j] & ~(0xFFu << sh)) | next << sh;
+      }
     }
-    ey = plane ? eq_column(c, n) : 0u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) n[j] = __shfl_down_sync(FULL, c[j], 1);
-    if (lane == k.w - 1) {
-      const uint4 f = *reinterpret_cast<const uint4*>(ls.xface[ly]);
-      n[0] = f.x;
-      n[1] = f.y;
-      n[2] = f.z;
-      n[3] = f.w;
-    }
-    ex = eq_column(c, n);
-    // the column moved down by one row, the row past the brick on top
-#pragma unroll
-    for (int j = 0; j < 4; ++j) n[j] = (c[j] >> 8) | (j < 3 ? c[j + 1] << 24 : 0u);
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if ((k.d - 1) >> 2 == j) n[j] |= top << (8 * ((k.d - 1) & 3));
-    ez = eq_column(c, n);
-    const uint32_t mine = col ? depth : 0u;
-    ex &= mine;
-    ey &= mine;
-    ez &= mine;
+    ex = eq_row(c, n) & mine;
+    ey = eq_row(c, ny) & mine;
+    ez = eq_row(c, nz) & mine;
     if (do_obs) {
       int cnt[QREG];
 #pragma unroll
       for (int s = 0; s < QREG; ++s) {
         const uint32_t same = 0x01010101u * (uint32_t)s;
         const uint32_t v[4] = {same, same, same, same};
-        cnt[s] = s < q && q <= QREG ? __popc(eq_column(c, v) & mine) : 0;
+        cnt[s] = s < q && q <= QREG ? __popc(eq_row(c, v) & mine) : 0;
       }
-      if (q > QREG && col)
-        for (int lz = 0; lz < k.d; ++lz)
-          atomicAdd(&ls.hist[(uint8_t)spins[site3(b, k.x0 + lane, k.y0 + ly, k.z0 + lz)]], 1);
+      if (q > QREG) {
+        __syncthreads();   // the histogram is cleared
+        for (int i = 0; i < nv; ++i) atomicAdd(&ls.hist[(uint8_t)spins[site0 + i]], 1);
+      }
       observables_warp_sums<B3_THREADS>((unsigned)(__popc(ex) + __popc(ey) + __popc(ez)), cnt, q <= QREG ? q : 0,
                                         ls.red);
     }
   }
 
-  // 2. open bonds of my column
+  // 2. open bonds of my sites
   if (T == 0) {
     ex = ey = ez = 0u;
   } else if (T < (1ull << 32) && plane) {
-    const uint32_t thr = (uint32_t)T, XY = (uint32_t)b.X * (uint32_t)b.Y;
-    uint32_t site = (uint32_t)site3(b, k.x0 + lane, k.y0 + ly, k.z0);   // wraps past the box in lanes without a column
+    const uint32_t thr = (uint32_t)T;
     uint32_t ox = 0u, oy = 0u, oz = 0u;
     constexpr int U = 8;
 #pragma unroll 1
-    for (int z0 = 0; z0 < k.d; z0 += U) {
+    for (int i0 = 0; i0 < min(k.w, 16); i0 += U) {
       uint32_t bx = 0u, by = 0u, bz = 0u;
 #pragma unroll
       for (int i = 0; i < U; ++i) {
-        const uint4 r =
-            philox_draw(make_uint4(site, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_BOND3), keys);
+        const uint4 r = philox_draw(
+            make_uint4(site0 + (uint32_t)(i0 + i), (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_BOND3), keys);
         set_if_below(bx, r.x, thr, 1u << i);
         set_if_below(by, r.y, thr, 1u << i);
         set_if_below(bz, r.z, thr, 1u << i);
-        site += XY;
       }
-      ox |= bx << z0;
-      oy |= by << z0;
-      oz |= bz << z0;
+      ox |= bx << i0;
+      oy |= by << i0;
+      oz |= bz << i0;
     }
     ex &= ox;
     ey &= oy;
@@ -252,11 +228,15 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
   // 3. row words (lane = row lz) of the plane's bonds: inside the brick for
   //    the engine and the +y joins, leaving it for the merge, wrapping inside
   //    it where the axis is one brick long
-  const uint32_t xz = transpose32(ex | ez << 16);
-  uint32_t yb = transpose32(ey);                                   // lanes 0 .. 15
-  uint32_t we = lane < B3Z ? xz : 0u;
-  uint32_t wn = __shfl_sync(FULL, xz, (lane & 15) + 16);
-  if (lane >= B3Z) wn = 0u;
+  auto row_word = [&](uint32_t e) {
+    e <<= 16 * half;
+    e |= __shfl_xor_sync(FULL, e, 1);
+    e = __shfl_sync(FULL, e, 2 * (lane & 15));
+    return lane < B3Z ? e : 0u;
+  };
+  uint32_t we = row_word(ex);
+  uint32_t wn = row_word(ez);
+  const uint32_t yb = row_word(ey);
   const uint32_t last_x = 1u << (k.w - 1);
   const uint32_t x_out = __ballot_sync(FULL, (we & last_x) != 0u);  // bit = lz
   const uint32_t z_out = __shfl_sync(FULL, wn, k.d - 1);            // bit = lx
@@ -276,9 +256,8 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
 
   // 5. +y bonds between planes ly and ly + 1.  One contact per overlap of an
   //    x run with a run of the next plane is kept, and none whose row below
-  //    has the bond too and +z bonds up on both sides.  Rounds: boundaries
-  //    0 2 4 6, then 1 5, then 3 (each warp's pairs lie in planes that no other
-  //    warp of the round touches).
+  //    has the bond too and +z bonds up on both sides.  Every join hooks one
+  //    root, which takes the contact's place in the list.
   uint16_t* list = ls.list[ly];
   int n_list = 0;
   {
@@ -291,6 +270,7 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
       C = yb & ~((seg_or_up(yb, j2) << 1) & (j2 << 1));
       if (lane > 0) C &= ~implied;
     }
+    C = __shfl_sync(FULL, C, lz) >> (16 * half) & 0xFFFFu;   // my sixteen sites' contacts
     const int cnt = __popc(C);
     int incl = cnt;
 #pragma unroll
@@ -299,33 +279,27 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
       if (lane >= o) incl += v;
     }
     n_list = __shfl_sync(FULL, incl, 31);
-    const int row = brick_local(0, ly, lane);
-    const int my_round = !(ly & 1) ? 0 : (ly & 3) == 1 ? 1 : 2;
-#pragma unroll 1
-    for (int round = 0; round < 3; ++round) {
-      if (round == my_round) {
-        for (int first = 0; first < n_list; first += Y_LIST) {
-          int at = incl - cnt - first;
-          for (uint32_t x = C; x; x &= x - 1, ++at)
-            if ((unsigned)at < Y_LIST) list[at] = (uint16_t)(row + high_bit(x & -x));
-          __syncwarp();
-          const int n = min(n_list - first, Y_LIST);
-          for (int j = lane; j - lane < n; j += 32) {
-            int a = 2 * brick_local(0, ly, 0), c = a;
-            if (j < n) {
-              const int site = list[j];
-              const int lz = local_y(site);
-              a = par[site];
-              c = par[brick_local(0, ly + 1, lz) + (site & (B3X - 1))];
-            }
-            const int hooked = sm_union_strips(par, a, c, err);
-            if (j < n) list[j] = (uint16_t)hooked;
-          }
-          __syncwarp();
+    const int row = brick_local(16 * half, ly, lz);
+    for (int first = 0; first < n_list; first += Y_LIST) {
+      int at = incl - cnt - first;
+      for (uint32_t x = C; x; x &= x - 1, ++at)
+        if ((unsigned)at < Y_LIST) list[at] = (uint16_t)(row + high_bit(x & -x));
+      __syncwarp();
+      const int n = min(n_list - first, Y_LIST);
+      for (int j = lane; j - lane < n; j += 32) {
+        int a[1], c[1], hooked[1];
+        a[0] = c[0] = 2 * brick_local(0, ly, 0);
+        if (j < n) {
+          const int site = list[j];
+          a[0] = par[site];
+          c[0] = par[brick_local(0, ly + 1, local_y(site)) + (site & (B3X - 1))];
         }
+        sm_union_tile(par, a, c, hooked, err);
+        if (j < n) list[j] = (uint16_t)hooked[0];
       }
-      __syncthreads();
+      __syncwarp();
     }
+    __syncthreads();
   }
   // wraps of an axis one brick long
   const bool wraps = b.bx == 1 || b.by == 1 || b.bz == 1;
@@ -424,7 +398,13 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
         }
       } else {
         if (lx0 == 0) mark(wv[0] & 0xFFFFu);
-        if (lx0 + in == k.w && in > 0) mark((wv[(in - 1) >> 1] >> (16 * ((in - 1) & 1))) & 0xFFFFu);
+        if (lx0 + in == k.w) {
+          uint32_t last = wv[0];
+#pragma unroll
+          for (int i = 1; i < 4; ++i)
+            if (2 * i < in) last = wv[i];
+          mark((last >> (16 * ((in - 1) & 1))) & 0xFFFFu);
+        }
       }
     }
   }
@@ -448,16 +428,22 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
   if (threadIdx.x < B3_EDGE_WORDS) out[threadIdx.x] = ls.edge[threadIdx.x];
 }
 
-// One warp per face word of a brick (x: two words): z faces 0 .. 7 (bit lx of
-// word ly), y face 8 .. 23 (bit lx of word lz), x face 24 .. 27 (bits lz of
+// One CTA per brick, a warp per face word (x: two words): z faces 0 .. 7 (bit lx
+// of word ly), y face 8 .. 23 (bit lx of word lz), x face 24 .. 27 (bits lz of
 // words ly, ly + 1).  A lane whose root pair equals its left neighbour's skips
-// the union.  Bound by the latency of the root loads and parent walks.
+// the union; the others' pairs are listed and joined with all lanes busy (see
+// merge_tiles).  Bound by the latency of the root loads and parent walks;
+// 256^3: 37 us against 61 with a union per lane where its bond stands (blocks of
+// 128 threads 40 us, of 448 45).
 constexpr int B3_MERGE_UNITS = B3Y + B3Z + B3Y / 2;
 constexpr int MERGE3_THREADS = 256;
 
 __global__ void __launch_bounds__(MERGE3_THREADS)
 k3_merge(const uint16_t* __restrict__ lroot, int32_t* gpar, const uint32_t* __restrict__ words, Box3 b, int limit,
          SwCtl* ctl, int64_t* obs, int obs_cap, int q) {
+  constexpr int WARPS = MERGE3_THREADS / 32, UNITS = (B3_MERGE_UNITS + WARPS - 1) / WARPS;
+  __shared__ int2 pairs[B3_MERGE_UNITS * 32];
+  __shared__ int n_pairs;
   wait_for_previous();
   int* err = &ctl->err;
   if (blockIdx.x == 0) {   // the next sweep's local step fills this sweep's observable slot
@@ -466,58 +452,68 @@ k3_merge(const uint16_t* __restrict__ lroot, int32_t* gpar, const uint32_t* __re
     __syncthreads();
     if (threadIdx.x == 0) ctl->sweep = s + 1;
   }
-  const int64_t unit = blockIdx.x * (int64_t)(MERGE3_THREADS / 32) + (threadIdx.x >> 5);
-  if (unit >= b.n_bricks() * B3_MERGE_UNITS) return;
-  const int t = (int)(unit / B3_MERGE_UNITS), u = (int)(unit - (int64_t)t * B3_MERGE_UNITS);
-  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) n_pairs = 0;
+  const int t = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t* wd = words + (int64_t)t * B3_WORDS;
-  int lx = lane, ly = u, lz = 0, axis = 2;
-  uint32_t bits;
-  if (u < B3Y) {
-    bits = wd[B3_FACE_Z + u] >> lane;
-  } else if (u < B3Y + B3Z) {
-    lz = u - B3Y;
-    axis = 1;
-    bits = wd[B3_FACE_Y + lz] >> lane;
-  } else {
-    ly = 2 * (u - B3Y - B3Z) + (lane >> 4);
-    lz = lane & 15;
-    axis = 0;
-    bits = wd[B3_FACE_X + ly] >> lz;
-  }
-  bool valid = bits & 1u;
-  if (!__any_sync(FULL, valid)) return;
   const Brick k = brick_of(b, t);
-  if (axis == 2) lz = k.d - 1;
-  if (axis == 1) ly = k.h - 1;
-  if (axis == 0) lx = k.w - 1;
-  const Brick kn = brick_at(b, axis == 0 ? (k.tbx + 1 == b.bx ? 0 : k.tbx + 1) : k.tbx,
-                            axis == 1 ? (k.tby + 1 == b.by ? 0 : k.tby + 1) : k.tby,
-                            axis == 2 ? (k.tbz + 1 == b.bz ? 0 : k.tbz + 1) : k.tbz);
-  int ga = 0, gb = 0;
-  if (valid) {   // the brick roots on the two ends (both edge roots)
-    const int ra = lroot[site3(b, k.x0 + lx, k.y0 + ly, k.z0 + lz)];
-    const int rb = lroot[site3(b, kn.x0 + (axis == 0 ? 0 : lx), kn.y0 + (axis == 1 ? 0 : ly),
-                               kn.z0 + (axis == 2 ? 0 : lz))];
-    ga = (int)brick_global(b, k, ra);
-    gb = (int)brick_global(b, kn, rb);
+  uint32_t bit[UNITS];
+  int ga[UNITS], gb[UNITS];
+#pragma unroll
+  for (int i = 0; i < UNITS; ++i) {
+    const int u = warp + WARPS * i;
+    bit[i] = u >= B3_MERGE_UNITS ? 0u
+             : u < B3Y + B3Z     ? wd[B3_FACE_Z + u] >> lane
+                                 : wd[B3_FACE_X + 2 * (u - B3Y - B3Z) + (lane >> 4)] >> (lane & 15);
   }
-  valid = valid && ga != gb;
-  const unsigned long long key =
-      valid ? ((unsigned long long)(unsigned)min(ga, gb) << 32) | (unsigned)max(ga, gb) : ~0ull;
-  const unsigned long long left = __shfl_up_sync(FULL, key, 1);
-  if (valid && (lane == 0 || left != key)) g_union(gpar, ga, gb, limit, err);
+#pragma unroll
+  for (int i = 0; i < UNITS; ++i) {
+    const int u = warp + WARPS * i;
+    ga[i] = gb[i] = 0;
+    if (bit[i] & 1u) {   // the brick roots on the two ends (both edge roots)
+      const int axis = u < B3Y ? 2 : u < B3Y + B3Z ? 1 : 0;
+      const int lx = axis ? lane : k.w - 1;
+      const int ly = axis == 2 ? u : axis == 1 ? k.h - 1 : 2 * (u - B3Y - B3Z) + (lane >> 4);
+      const int lz = axis == 2 ? k.d - 1 : axis == 1 ? u - B3Y : lane & 15;
+      const Brick kn = brick_at(b, axis == 0 ? (k.tbx + 1 == b.bx ? 0 : k.tbx + 1) : k.tbx,
+                                axis == 1 ? (k.tby + 1 == b.by ? 0 : k.tby + 1) : k.tby,
+                                axis == 2 ? (k.tbz + 1 == b.bz ? 0 : k.tbz + 1) : k.tbz);
+      const int ra = lroot[site3(b, k.x0 + lx, k.y0 + ly, k.z0 + lz)];
+      const int rb = lroot[site3(b, kn.x0 + (axis == 0 ? 0 : lx), kn.y0 + (axis == 1 ? 0 : ly),
+                                 kn.z0 + (axis == 2 ? 0 : lz))];
+      ga[i] = (int)brick_global(b, k, ra);
+      gb[i] = (int)brick_global(b, kn, rb);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < UNITS; ++i) {
+    const int lo = min(ga[i], gb[i]), hi = max(ga[i], gb[i]);
+    const bool valid = lo != hi;
+    const unsigned long long key = valid ? ((unsigned long long)(unsigned)lo << 32) | (unsigned)hi : ~0ull;
+    const unsigned long long left = __shfl_up_sync(FULL, key, 1);
+    const bool join = valid && (lane == 0 || left != key);
+    const uint32_t m = __ballot_sync(FULL, join);
+    if (m == 0u) continue;
+    int at = 0;
+    if (lane == 0) at = atomicAdd(&n_pairs, __popc(m));
+    at = __shfl_sync(FULL, at, 0) + __popc(m & ((1u << lane) - 1u));
+    if (join) pairs[at] = make_int2(lo, hi);
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < n_pairs; j += MERGE3_THREADS) seam_join(gpar, pairs[j].x, pairs[j].y, limit, err);
 }
 
 // Flip of a brick: a thread owns the sites it wrote in k3_local's step 7 (two
 // steps of eight consecutive sites of a row, one 16-byte load of roots each).
+// Edge roots come first in the list, as in sw_flip_tile: the first walks' loads
+// are in flight while the interior roots are drawn.  256^3: 54 us against 71 with
+// flags looked up root by root and walks and draws in turn.
 __global__ void __launch_bounds__(B3_THREADS, 6)
 k3_flip(int8_t* __restrict__ spins, const uint16_t* __restrict__ lroot, int32_t* gpar,
         const uint32_t* __restrict__ words, Box3 b, int q, const __grid_constant__ PhiloxKeys keys,
         const SwCtl* __restrict__ ctl, int limit, int* err) {
   __shared__ uint16_t rlist[B3_SITES];
   __shared__ uint8_t ns[B3_SITES];
-  __shared__ uint32_t edge[B3_EDGE_WORDS];
   __shared__ int warp_cnt[B3_THREADS / 32];
   const Brick k = brick_of(b, blockIdx.x);
   wait_for_previous();
@@ -526,10 +522,12 @@ k3_flip(int8_t* __restrict__ spins, const uint16_t* __restrict__ lroot, int32_t*
   const int lx0 = 8 * (lane & 3);
   const int in = ly < k.h ? min(max(k.w - lx0, 0), 8) : 0;
   const bool whole = (b.X & 7) == 0;   // rows start 16-byte aligned, in is 0 or 8
-  if (threadIdx.x < B3_EDGE_WORDS) edge[threadIdx.x] = words[(int64_t)blockIdx.x * B3_WORDS + threadIdx.x];
+  const int id0 = brick_local(lx0, ly, lane >> 2);   // local index of my first site; step j is 8 rows further
+  const uint8_t* eb = reinterpret_cast<const uint8_t*>(words + (int64_t)blockIdx.x * B3_WORDS) + (id0 >> 3);
   // 1. brick roots of my sites (0xFFFF outside the brick), and which are roots
+  //    and edge roots (bit 8j + i: site i of step j)
   uint4 roots[B3Z / 8];
-  uint32_t mine = 0;
+  uint32_t m = 0, edges = 0;
 #pragma unroll
   for (int j = 0; j < B3Z / 8; ++j) {
     const int lz = (lane >> 2) + 8 * j;
@@ -548,13 +546,17 @@ k3_flip(int8_t* __restrict__ spins, const uint16_t* __restrict__ lroot, int32_t*
           if (i < in) v[i >> 1] = i & 1 ? (v[i >> 1] & 0xFFFFu) | (uint32_t)src[i] << 16 : 0xFFFF0000u | src[i];
       }
     }
-    const uint32_t own = (uint32_t)brick_local(lx0, ly, lz) * 0x00010001u + 0x00010000u;
+    edges |= (uint32_t)eb[j * TILE_W] << (8 * j);
+    const uint32_t own = (uint32_t)(id0 + 8 * j * TILE_W) * 0x00010001u + 0x00010000u;   // (site, site + 1)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) mine |= zero_halves(v[i] ^ (own + (uint32_t)i * 0x00020002u)) >> (15 - (4 * j + i));
+    for (int i = 0; i < 4; ++i) m |= zero_halves(v[i] ^ (own + (uint32_t)i * 0x00020002u)) >> (15 - (4 * j + i));
     roots[j] = make_uint4(v[0], v[1], v[2], v[3]);
   }
-  // 2. the brick's root list, edge roots flagged
-  const int cnt = __popc(mine);
+  // 2. the brick's root list: edge roots, then the others (counts of both in
+  //    one scan)
+  const uint32_t mine = spread_bits(m & 0xFFFFu) | spread_bits(m >> 16) << 1;
+  const uint32_t on_edge = mine & edges, inner = mine & ~edges;
+  const int cnt = __popc(on_edge) << 16 | __popc(inner);
   int incl = cnt;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -563,42 +565,50 @@ k3_flip(int8_t* __restrict__ spins, const uint16_t* __restrict__ lroot, int32_t*
   }
   if (lane == 31) warp_cnt[warp] = incl;
   __syncthreads();
-  int base = 0, n_roots = 0;
+  int before = incl - cnt, total = 0;
 #pragma unroll
   for (int j = 0; j < B3_THREADS / 32; ++j) {
-    base += (j < warp) ? warp_cnt[j] : 0;
-    n_roots += warp_cnt[j];
+    before += (j < warp) ? warp_cnt[j] : 0;
+    total += warp_cnt[j];
   }
-  base += incl - cnt;
-  while (mine) {
-    const int bit = __ffs(mine) - 1;
-    mine &= mine - 1;
-    const int jk = bit & 15;
-    const int l = brick_local(lx0, ly, (lane >> 2) + 8 * (jk >> 2)) + 2 * (jk & 3) + (bit >> 4);
-    rlist[base++] = (uint16_t)l | (((edge[l >> 5] >> (l & 31)) & 1u) ? EDGE_ROOT : (uint16_t)0);
-  }
+  const int n_edge = total >> 16, n_roots = n_edge + (total & 0xFFFF);
+  auto list = [&](uint32_t bits, int at) {
+    while (bits) {
+      const int n = high_bit(bits);
+      bits ^= 1u << n;
+      rlist[at++] = (uint16_t)(id0 + n + (n & 24) * (TILE_W - 1));
+    }
+  };
+  list(on_edge, before >> 16);
+  list(inner, n_edge + (before & 0xFFFF));
   __syncthreads();
-  // 3. one draw per brick root, keyed by its cluster's root; a thread takes
-  //    its roots two at a time, their parent walks in lock step
-  constexpr int U = 2;
-  for (int j0 = threadIdx.x; j0 < n_roots; j0 += U * B3_THREADS) {
-    int r[U], R[U];
-    bool act[U];
+  // 3. one draw per brick root, keyed by its cluster's root.  A thread's first
+  //    edge roots have their parents loaded before it draws its interior roots.
+  auto set_state = [&](int r, int G) {
+    const uint4 w = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
+    ns[r] = (uint8_t)state_of(w.x, q);
+  };
+  constexpr int U = 3;   // of about 500 edge roots per brick at criticality (two: 56 us, four: as three)
+  int x[U], p[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int j = j0 + u * B3_THREADS;
-      const int raw = j < n_roots ? (int)rlist[j] : 0;
-      r[u] = raw & ROOT_MASK;
-      R[u] = (int)brick_global(b, k, r[u]);
-      act[u] = j < n_roots && (raw & EDGE_ROOT);
-    }
-    g_find_multi<U>(gpar, R, act, limit, err);
+  for (int u = 0; u < U; ++u) {
+    const int j = threadIdx.x + u * B3_THREADS;
+    x[u] = j < n_edge ? (int)brick_global(b, k, rlist[j]) : 0;
+    p[u] = j < n_edge ? g_load(gpar + x[u]) : 0;
+  }
+  for (int j = n_edge + threadIdx.x; j < n_roots; j += B3_THREADS) {
+    const int r = rlist[j];
+    set_state(r, (int)brick_global(b, k, r));
+  }
+  g_find_multi<U>(gpar, x, p, limit, err);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (j0 + u * B3_THREADS >= n_roots) break;
-      const uint4 w = philox_draw(make_uint4((uint32_t)R[u], (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
-      ns[r[u]] = (uint8_t)state_of(w.x, q);
-    }
+  for (int u = 0; u < U; ++u) {
+    const int j = threadIdx.x + u * B3_THREADS;
+    if (j < n_edge) set_state(rlist[j], x[u]);
+  }
+  for (int j = threadIdx.x + U * B3_THREADS; j < n_edge; j += B3_THREADS) {
+    const int r = rlist[j];
+    set_state(r, g_find(gpar, (int)brick_global(b, k, r), limit, err));
   }
   __syncthreads();
   // 4. every site takes its brick root's state
@@ -728,9 +738,8 @@ cudaError_t launch_sweep3(int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
   // a box of one brick has no face bonds: one block only advances the counter
-  constexpr int WARPS = MERGE3_THREADS / 32;
   const bool faces = b.bx > 1 || b.by > 1 || b.bz > 1;
-  const int64_t blocks = faces ? (b.n_bricks() * B3_MERGE_UNITS + WARPS - 1) / WARPS : 1;
+  const int64_t blocks = faces ? b.n_bricks() : 1;
   e = launch_after(k3_merge, (unsigned)blocks, MERGE3_THREADS, st, lroot, gpar, words, b, limit3(b), ctl, obs, obs_cap, q);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;

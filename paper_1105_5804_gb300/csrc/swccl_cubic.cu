@@ -123,7 +123,7 @@ sw3_handle* sw3_create(int X, int Y, int Z, int q, uint64_t T, uint64_t seed, in
       return bail(SW_ERR_CUDA, "sw3_create: cudaStreamCreate failed");
     h->own_stream = true;
   }
-  if (cudaMalloc(&h->spins, (size_t)n) != cudaSuccess || cudaMalloc(&h->gpar, (size_t)n * 4) != cudaSuccess ||
+  if (cudaMalloc(&h->spins, ((size_t)n + 3) & ~(size_t)3) != cudaSuccess || cudaMalloc(&h->gpar, (size_t)n * 4) != cudaSuccess ||
       cudaMalloc(&h->lroot, (size_t)n * 2) != cudaSuccess ||
       cudaMalloc(&h->words, (size_t)brick_words3(h->box) * 4) != cudaSuccess ||
       cudaMalloc(&h->ctl, sizeof(SwCtl)) != cudaSuccess || cudaMalloc(&h->chk, sizeof(int)) != cudaSuccess ||

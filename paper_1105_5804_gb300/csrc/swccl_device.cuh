@@ -275,9 +275,12 @@ __device__ __forceinline__ void sm_find_tile(const uint16_t* par, int (&x)[N], i
 // repeated while only the entry beside it changed (it can be hooked once, so
 // twice at most); if the root itself was hooked meanwhile, its new parent is
 // joined in the next round, so no link is lost.  Every round lowers the larger
-// operand, so at most WALK_LIMIT rounds run.
+// operand, so at most WALK_LIMIT rounds run.  hooked[u]: the root that the pair
+// hooked, or -1.
 template <class Order = TileOrder, int N>
-__device__ __forceinline__ void sm_union_tile(uint16_t* par, int (&a)[N], int (&b)[N], int* err) {
+__device__ __forceinline__ void sm_union_tile(uint16_t* par, int (&a)[N], int (&b)[N], int (&hooked)[N], int* err) {
+#pragma unroll
+  for (int u = 0; u < N; ++u) hooked[u] = -1;
   for (int rounds = 0; rounds <= WALK_LIMIT; ++rounds) {
     int x[2 * N];
 #pragma unroll
@@ -305,7 +308,10 @@ __device__ __forceinline__ void sm_union_tile(uint16_t* par, int (&a)[N], int (&
             break;
           }
           const unsigned seen = atomicCAS(word, old, old ^ ((unsigned)(lo ^ hi) << sh));
-          if (seen == old) break;
+          if (seen == old) {
+            hooked[u] = hi;
+            break;
+          }
           old = seen;
         }
         more |= a[u] != b[u];
@@ -314,6 +320,11 @@ __device__ __forceinline__ void sm_union_tile(uint16_t* par, int (&a)[N], int (&
     if (!__any_sync(0xFFFFFFFFu, more)) return;
   }
   set_error(err, SW_ERR_STATE);
+}
+template <class Order = TileOrder, int N>
+__device__ __forceinline__ void sm_union_tile(uint16_t* par, int (&a)[N], int (&b)[N], int* err) {
+  int hooked[N];
+  sm_union_tile<Order>(par, a, b, hooked, err);
 }
 template <class Order = TileOrder>
 __device__ __forceinline__ void sm_union_tile(uint16_t* par, int a, int b, int* err) {
@@ -348,30 +359,6 @@ __device__ __forceinline__ int sm_union_strip(uint16_t* par, int a, int b) {
   return hooked;
 }
 
-// sm_union_strip for pairs whose trees lie in several strips that no other
-// warp touches meanwhile.
-__device__ __forceinline__ int sm_union_strips(uint16_t* par, int a, int b, int* err) {
-  int hooked = -1;
-  for (int rounds = 0; rounds <= WALK_LIMIT; ++rounds) {
-    int x[2] = {a, b};
-    sm_find_tile(par, x, err);
-    const bool first = node_key(x[0]) < node_key(x[1]);
-    a = first ? x[0] : x[1];
-    b = first ? x[1] : x[0];
-    __syncwarp();
-    if (a != b) sm_set(par, b, a);
-    __syncwarp();
-    if (a != b) {
-      const int won = sm_at(par, b);
-      if (won == a) hooked = b;
-      b = won;
-    }
-    if (!__any_sync(0xFFFFFFFFu, a != b)) return hooked;
-  }
-  set_error(err, SW_ERR_STATE);
-  return hooked;
-}
-
 // ---------------------------------------------------------------------------
 // Union-find on a global int32 array (the label array itself: the entry of a
 // tile root is its parent pointer).  Loads bypass L1 (ld.cg) because other
@@ -396,14 +383,12 @@ __device__ __forceinline__ int g_find(int* lab, int x, int limit, int* err) {
   return g_find_from(lab, x, g_load(lab + x), limit, err);
 }
 
-// g_find of up to U nodes at once (those with act[u] set): the walks run in
-// lock step so that their loads are in flight together.  x[u] is replaced by
-// its root; same path halving and step limit as g_find.
+// g_find of U nodes at once, p[u] being the loaded parent of x[u] (x[u] itself:
+// no walk): the walks run in lock step so that their loads are in flight
+// together.  x[u] is replaced by its root; same path halving and step limit as
+// g_find.
 template <int U>
-__device__ __forceinline__ void g_find_multi(int* lab, int (&x)[U], const bool (&act)[U], int limit, int* err) {
-  int p[U];
-#pragma unroll
-  for (int u = 0; u < U; ++u) p[u] = act[u] ? g_load(lab + x[u]) : x[u];
+__device__ __forceinline__ void g_find_multi(int* lab, int (&x)[U], int (&p)[U], int limit, int* err) {
   for (int steps = 0;; ++steps) {
     int gp[U];
     bool more = false;
@@ -433,8 +418,8 @@ __device__ __forceinline__ void g_find_multi(int* lab, int (&x)[U], const bool (
 __device__ __forceinline__ void g_union(int* lab, int a, int b, int limit, int* err) {
   for (int rounds = 0; rounds <= limit; ++rounds) {
     int x[2] = {a, b};
-    const bool act[2] = {true, true};
-    g_find_multi<2>(lab, x, act, limit, err);
+    int p[2] = {g_load(lab + a), g_load(lab + b)};
+    g_find_multi<2>(lab, x, p, limit, err);
     a = x[0];
     b = x[1];
     if (a == b) return;
