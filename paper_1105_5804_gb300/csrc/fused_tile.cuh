@@ -344,10 +344,6 @@ __device__ __forceinline__ int root_in(const uint4& v, int i) {
 
 // The flip of tile t (see k_fused.cu).  All threads of the CTA call it; it
 // ends with a barrier.
-// FEW: the few-cluster update (Sec. III, variant (c)).  Only clusters whose
-// global root has its bit set in `sel` (seeded clusters) move: with FLIP draw
-// w of the root, iff (uint64)w.y < P, to state (s + 1 + F_{q-1}(w.x)) mod q,
-// s being the cluster's current state (read at the tile root).
 // The tile roots wait in shared memory for the site pass (held in registers
 // across the draws they spill at six CTAs per SM, read again through L2 they
 // cost its traffic twice).  Edge roots, whose cluster root has to be found on
@@ -358,10 +354,9 @@ __device__ __forceinline__ int root_in(const uint4& v, int i) {
 // 0.389 ms with the roots read twice, flags looked up root by root and four
 // walks per thread in step.
 // TH: rows of the lattice's tiles.
-template <bool FEW = false, int TH = TILE_H, class Keys = SeedKey>
+template <int TH = TILE_H, class Keys = SeedKey>
 __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t sweep, int limit, FlipTileSmemT<TH>& fs,
-                                             const Keys& keys, const uint32_t* __restrict__ sel = nullptr,
-                                             uint64_t P = 0) {
+                                             const Keys& keys) {
   constexpr int PASSES = TH / 8, FLIP_LIST = FlipTileSmemT<TH>::LIST;
   uint8_t* ns = fs.ns;
   int8_t* __restrict__ spins = R.spins;
@@ -452,19 +447,8 @@ __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t swe
   const int at_edge = before >> 16, at_inner = n_edge + (before & 0xFFFF);
 
   auto set_state = [&](int r, int G) {   // new state of the component with local root r and cluster root G
-    if (FEW) {
-      // the cluster's current state, read at the tile root (this tile's own
-      // site: the site pass rewrites it only after a barrier)
-      int v = spins[(uint32_t)tile_global(r, y0, x0, L)];
-      if ((__ldcg(sel + (G >> 5)) >> (G & 31)) & 1u) {
-        const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
-        if ((uint64_t)d.y < P) v = (v + 1 + state_of(d.x, q - 1)) % q;
-      }
-      ns[r] = (uint8_t)v;
-    } else {
-      const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
-      ns[r] = (uint8_t)state_of(d.x, q);
-    }
+    const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
+    ns[r] = (uint8_t)state_of(d.x, q);
   };
 
   for (int first = 0; first < n_roots; first += FLIP_LIST) {
@@ -528,6 +512,141 @@ __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t swe
     }
   }
   __syncthreads();
+}
+
+// The flip of the few-cluster update (Sec. III, variant (c)).  Only clusters
+// whose global root has its bit set in `sel` (seeded clusters) move: with FLIP
+// draw w of the root, iff (uint64)w.y < P, to state (s + 1 + F_{q-1}(w.x)) mod q,
+// s being the cluster's current state, that is by the same step on every site.
+// Few clusters are seeded, and which of a tile's components belong to one can be
+// seen without the sites' roots: the interior ones have their own bit set in
+// sel, the others are edge roots (at most 576 of a tile's 8192 sites).  So a
+// tile reads a bit per site of each kind, walks from its edge roots, and reads
+// roots and spins only if some component of it moves.  Bound by instruction
+// issue and the walks' latency; critical Ising, L = 4096, 16 x 16 seeds: 17 us
+// against 53 with the state of every tile root looked up.
+template <int TH>
+struct FewFlipSmem {
+  static constexpr int LIST = 1024;
+  alignas(16) uint8_t step[TH * TILE_W];   // by local root; 0: stays
+  uint16_t rlist[LIST];                    // the tile's edge roots, then its selected interior roots
+  int warp_cnt[LABEL_THREADS / 32];
+};
+
+template <int TH, class Keys>
+__device__ __forceinline__ void sw_flip_few_tile(const SwRep& R, int t, uint64_t sweep, int limit, FewFlipSmem<TH>& fs,
+                                                 const Keys& keys, const uint32_t* __restrict__ sel, uint64_t P) {
+  constexpr int LIST = FewFlipSmem<TH>::LIST, WORDS = TH * TILE_W / 32;
+  int8_t* __restrict__ spins = R.spins;
+  int32_t* __restrict__ gpar = R.gpar;
+  const int q = R.q, L = R.g.W;
+  int* err = R.s.err;
+  const int ty = t / R.g.tiles_x, tx = t - ty * R.g.tiles_x;
+  const int y0 = ty * TH, x0 = tx * TILE_W;
+  const int h = min(TH, L - y0), w = min(TILE_W, L - x0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+
+  // 1. roots that may move, 32 sites (a word of local indices) per thread
+  uint32_t on_edge = 0u, inner = 0u;
+  if (threadIdx.x < WORDS) {
+    const int ly = local_y(32 * threadIdx.x), lx = local_x(32 * threadIdx.x);
+    const int nv = ly < h ? min(max(w - lx, 0), 32) : 0;
+    if (nv > 0) {
+      const uint32_t G = (uint32_t)(y0 + ly) * (uint32_t)L + (uint32_t)(x0 + lx), at = G >> 5, off = G & 31u;
+      on_edge = (uint32_t)sweep_edges(R.s, t)[threadIdx.x];
+      const uint32_t lo = sel[at], hi = off + nv > 32 ? sel[at + 1] : 0u;
+      inner = __funnelshift_r(lo, hi, off) & (FULL >> (32 - nv)) & ~on_edge;
+    }
+  }
+  for (int k = threadIdx.x; k < TH * TILE_W / 16; k += LABEL_THREADS)
+    reinterpret_cast<uint4*>(fs.step)[k] = make_uint4(0u, 0u, 0u, 0u);
+  // 2. their list (counts of both kinds in one scan; several passes if it is full)
+  const int cnt = __popc(on_edge) << 16 | __popc(inner);
+  int incl = cnt;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(FULL, incl, d);
+    if (lane >= d) incl += v;
+  }
+  if (lane == 31) fs.warp_cnt[warp] = incl;
+  __syncthreads();
+  int before = incl - cnt, total = 0;
+#pragma unroll
+  for (int k = 0; k < LABEL_THREADS / 32; ++k) {
+    before += (k < warp) ? fs.warp_cnt[k] : 0;
+    total += fs.warp_cnt[k];
+  }
+  const int n_edge = total >> 16, n_roots = n_edge + (total & 0xFFFF);
+  bool moved = false;
+  for (int first = 0; first < n_roots; first += LIST) {
+    auto list = [&](uint32_t bits, int at) {
+      while (bits) {
+        const int n = high_bit(bits);
+        bits ^= 1u << n;
+        if ((unsigned)at < LIST) fs.rlist[at] = (uint16_t)(32 * threadIdx.x + n);
+        ++at;
+      }
+    };
+    list(on_edge, (before >> 16) - first);
+    list(inner, n_edge + (before & 0xFFFF) - first);
+    __syncthreads();
+    // 3. the steps of the selected ones, keyed by their clusters' final roots
+    const int n = min(n_roots - first, LIST), ne = min(max(n_edge - first, 0), n);
+    for (int k = threadIdx.x; k < n; k += LABEL_THREADS) {
+      const int r = fs.rlist[k];
+      int G = tile_global(r, y0, x0, L);
+      if (k < ne) {
+        G = g_find(gpar, G, limit, err);
+        if (!((__ldg(sel + (G >> 5)) >> (G & 31)) & 1u)) continue;
+      }
+      const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
+      if ((uint64_t)d.y < P) {
+        fs.step[r] = (uint8_t)(1 + state_of(d.x, q - 1));
+        moved = true;
+      }
+    }
+    __syncthreads();
+  }
+  if (!__syncthreads_or(moved)) return;
+
+  // 4. every site takes its tile root's step (s + step <= 252: four spins are
+  //    added and reduced per word)
+  const int orow = threadIdx.x / FLIP_GROUPS, lx0 = 8 * (threadIdx.x % FLIP_GROUPS);   // my sites, as in sw_flip_tile
+  const uint32_t qq = 0x01010101u * (uint32_t)q;
+  auto shift = [&](uint32_t s, uint32_t step) {
+    const uint32_t v = __vadd4(s, step);
+    return __vsub4(v, __vcmpgeu4(v, qq) & qq);
+  };
+  if (lx0 >= w) return;
+#pragma unroll
+  for (int j = 0; j < TH / 8; ++j) {
+    const int ly = 8 * j + orow;
+    if (ly >= h) break;
+    const int64_t at = (int64_t)(y0 + ly) * L + x0 + lx0;
+    const bool two = lx0 + 8 <= w;         // w is a multiple of 4
+    uint4 rv = make_uint4(0u, 0u, 0u, 0u);
+    if ((L & 7) == 0) {
+      rv = __ldcs(reinterpret_cast<const uint4*>(R.lroot + at));
+    } else {
+      const uint2 a = *reinterpret_cast<const uint2*>(R.lroot + at);
+      rv.x = a.x;
+      rv.y = a.y;
+      if (two) {
+        const uint2 c = *reinterpret_cast<const uint2*>(R.lroot + at + 4);
+        rv.z = c.x;
+        rv.w = c.y;
+      }
+    }
+    uint32_t lo = 0, hi = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      lo |= (uint32_t)fs.step[root_in(rv, i)] << (8 * i);
+      hi |= (uint32_t)fs.step[root_in(rv, 4 + i)] << (8 * i);
+    }
+    uint32_t* dst = reinterpret_cast<uint32_t*>(spins + at);
+    if (lo) dst[0] = shift(dst[0], lo);
+    if (two && hi) dst[1] = shift(dst[1], hi);
+  }
 }
 
 // Observables of the current spins of tile t (bonds joining equal spins, the
@@ -599,7 +718,10 @@ __device__ __forceinline__ void few_select_seed(const SwRep& R, int ell, int64_t
   const int32_t* edge_bits = sweep_edges(R.s, ty * g.tiles_x + tx);
   const bool edge = (__ldcg(edge_bits + (r >> 5)) >> (r & 31)) & 1;
   const int root = edge ? g_find(R.gpar, G, limit, R.s.err) : G;
-  atomicOr(sel + (root >> 5), 1u << (root & 31));
+  // most seeds of a critical lattice are in one cluster: only the first few set
+  // its bit (a seed per site, L = 1024: 27 us, 290 with an atomic each)
+  const uint32_t bit = 1u << (root & 31);
+  if (!(__ldcg(sel + (root >> 5)) & bit)) atomicOr(sel + (root >> 5), bit);
 }
 
 }  // namespace swccl

@@ -34,11 +34,24 @@
 
 namespace swccl {
 
+// The few-cluster update's selection bits, cleared by the labeling kernel (null:
+// none), the last one in a sweep before they are set.
+struct ClearBits {
+  uint32_t* words;
+  int64_t n;
+};
+__device__ __forceinline__ void clear_bits(const ClearBits& c) {
+  if (!c.words) return;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < c.n; k += (int64_t)gridDim.x * blockDim.x)
+    c.words[k] = 0u;
+}
+
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
-k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys) {
+k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys, ClearBits clear) {
   __shared__ LabelTileSmem ls;
   wait_for_previous();
+  clear_bits(clear);
   const uint64_t sweep = ctl->sweep;
   const bool do_obs = sweep > 0 && ctl->obs_done != (long long)(sweep - 1);
   sw_label_tile(R, blockIdx.x, sweep, do_obs, obs_cap, ls, keys);
@@ -47,9 +60,11 @@ k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_con
 // The same for a lattice cut into low tiles.
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS)
-k_sw_label_low(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys) {
+k_sw_label_low(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys,
+               ClearBits clear) {
   __shared__ LowTileSmem<TH> ls;
   wait_for_previous();
+  clear_bits(clear);
   const uint64_t sweep = ctl->sweep;
   const bool do_obs = sweep > 0 && ctl->obs_done != (long long)(sweep - 1);
   sw_label_low_tile(R, blockIdx.x, sweep, do_obs, obs_cap, ls, keys);
@@ -61,16 +76,16 @@ __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
 k_sw_flip(SwRep R, const SwCtl* __restrict__ ctl, int limit, const __grid_constant__ PhiloxKeys keys) {
   __shared__ FlipTileSmemT<TH> fs;
   wait_for_previous();
-  sw_flip_tile<false, TH>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys);
+  sw_flip_tile<TH>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys);
 }
 
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
 k_sw_flip_few(SwRep R, const SwCtl* __restrict__ ctl, int limit, const uint32_t* __restrict__ sel, uint64_t P,
               const __grid_constant__ PhiloxKeys keys) {
-  __shared__ FlipTileSmemT<TH> fs;
+  __shared__ FewFlipSmem<TH> fs;
   wait_for_previous();
-  sw_flip_tile<true, TH>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys, sel, P);
+  sw_flip_few_tile(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys, sel, P);
 }
 
 constexpr int SELECT_THREADS = 256;
@@ -78,6 +93,7 @@ constexpr int SELECT_THREADS = 256;
 __global__ void __launch_bounds__(SELECT_THREADS)
 k_few_select(SwRep R, const SwCtl* __restrict__ ctl, int ell, uint32_t* sel, int limit) {
   const int64_t b = blockIdx.x * (int64_t)SELECT_THREADS + threadIdx.x;   // one thread per seed
+  wait_for_previous();
   if (b < (int64_t)ell * ell) few_select_seed(R, ell, b, ctl->sweep - 1, sel, limit);
 }
 
@@ -146,10 +162,11 @@ SwRep make_rep(int8_t* spins, uint16_t* lroot, int32_t* gpar, int64_t* obs, cons
 
 cudaError_t launch_sw_label(const int8_t* spins, uint16_t* lroot, int32_t* gpar, const Grid& g,
                             const LabelScratch& s, int q, uint64_t T, uint64_t seed, const SwCtl* ctl,
-                            int64_t* obs, int obs_cap, cudaStream_t st) {
+                            int64_t* obs, int obs_cap, uint32_t* sel, cudaStream_t st) {
   const SwRep R = make_rep(const_cast<int8_t*>(spins), lroot, gpar, obs, g, s, q, T, seed);
   auto* kernel = g.th == 8 ? k_sw_label_low<8> : g.th == 16 ? k_sw_label_low<16> : k_sw_label;
-  return launch_after(kernel, g.n_tiles(), LABEL_THREADS, st, R, ctl, obs_cap, philox_keys(seed));
+  return launch_after(kernel, g.n_tiles(), LABEL_THREADS, st, R, ctl, obs_cap, philox_keys(seed),
+                      ClearBits{sel, sel ? few_sel_bytes(g.n_sites()) / 4 : 0});
 }
 
 cudaError_t launch_sw_flip(int8_t* spins, const uint16_t* lroot, int32_t* gpar, const Grid& g,
@@ -235,14 +252,11 @@ cudaError_t launch_observe(const int8_t* spins, int L, int q, SwCtl* ctl, int64_
 
 cudaError_t launch_few_select(const uint16_t* lroot, int32_t* gpar, const Grid& g, const LabelScratch& s,
                               uint64_t seed, int ell, uint32_t* sel, const SwCtl* ctl, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(sel, 0, few_sel_bytes(g.n_sites()), st);
-  if (e != cudaSuccess) return e;
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
   const SwRep R = make_rep(nullptr, const_cast<uint16_t*>(lroot), gpar, nullptr, g, s, 2, 0, seed);
   const int64_t seeds = (int64_t)ell * ell;
   const int64_t blocks = (seeds + SELECT_THREADS - 1) / SELECT_THREADS;
-  k_few_select<<<(unsigned)blocks, SELECT_THREADS, 0, st>>>(R, ctl, ell, sel, limit);
-  return cudaGetLastError();
+  return launch_after(k_few_select, (unsigned)blocks, SELECT_THREADS, st, R, ctl, ell, sel, limit);
 }
 
 cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gpar, const Grid& g,

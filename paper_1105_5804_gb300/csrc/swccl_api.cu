@@ -158,7 +158,7 @@ cudaError_t enqueue_sweep_fused(sw_handle* h, cudaEvent_t* ev) {
   if (ev && ((e = cudaEventRecord(ev[0], st)) != cudaSuccess || (e = cudaEventRecord(ev[1], st)) != cudaSuccess))
     return e;
   if ((e = launch_sw_label(h->spins, h->lroot, h->labels, h->grid_f, h->ls_f, h->q, h->T, h->seed, h->ctl, h->obs,
-                           OBS_CAP, st)))
+                           OBS_CAP, h->update == SW_UPDATE_FEW ? h->sel : nullptr, st)))
     return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if ((e = launch_merge(h->labels, h->grid_f, h->ls_f, h->ctl, h->obs, OBS_CAP, h->q, st))) return e;

@@ -214,14 +214,14 @@ cudaError_t launch_advance(SwCtl* ctl, cudaStream_t st);
 // Fused sweep (activation inside labeling; no mask or int32 labels in HBM).
 cudaError_t launch_sw_label(const int8_t* spins, uint16_t* lroot, int32_t* gpar, const Grid& g,
                             const LabelScratch& s, int q, uint64_t T, uint64_t seed, const SwCtl* ctl,
-                            int64_t* obs, int obs_cap, cudaStream_t st);
+                            int64_t* obs, int obs_cap, uint32_t* sel, cudaStream_t st);
 cudaError_t launch_sw_flip(int8_t* spins, const uint16_t* lroot, int32_t* gpar, const Grid& g,
                            const LabelScratch& s, int q, uint64_t seed, const SwCtl* ctl, cudaStream_t st);
 cudaError_t launch_observe(const int8_t* spins, int L, int q, SwCtl* ctl, int64_t* obs, int obs_cap,
                            cudaStream_t st);
-// Few-cluster update: bytes of the seed-selection bit array of n sites, the
-// selection (clears the array, then marks the seeded clusters' roots), and
-// the flip of the selected clusters.
+// Few-cluster update: bytes of the seed-selection bit array of n sites (cleared
+// by launch_sw_label, `sel`), the selection (marks the seeded clusters' roots),
+// and the flip of the selected clusters.
 inline int64_t few_sel_bytes(int64_t n_sites) { return (n_sites + 31) / 32 * 4; }
 cudaError_t launch_few_select(const uint16_t* lroot, int32_t* gpar, const Grid& g, const LabelScratch& s,
                               uint64_t seed, int ell, uint32_t* sel, const SwCtl* ctl, cudaStream_t st);
