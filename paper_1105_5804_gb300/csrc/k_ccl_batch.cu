@@ -21,13 +21,14 @@ __device__ __forceinline__ int job_of_tile(const CclBatchView& v, int gt) {
   return lo;
 }
 
+template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_cclb_tile(const __grid_constant__ CclBatchView v) {
-  __shared__ CclTileSmem sm;
+  __shared__ CclTileSmemT<TH> sm;
   wait_for_previous();
   let_next_start();
   const int gt = blockIdx.x;
   const CclJob& J = v.jobs[job_of_tile(v, gt)];
-  ccl_label_tile<true>(J.mask, J.labels, J.g, J.s, gt - J.tile0, sm);
+  ccl_label_tile<true, TH>(J.mask, J.labels, J.g, J.s, gt - J.tile0, sm);
 }
 
 __global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_constant__ CclBatchView v, int per) {
@@ -43,22 +44,26 @@ __global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_cons
               v.limit);
 }
 
+template <int TH>
 __global__ void __launch_bounds__(FINAL_THREADS) k_cclb_final(const __grid_constant__ CclBatchView v) {
-  __shared__ FinalSmem fs;
+  __shared__ FinalSmem<TH> fs;
   wait_for_previous();
   const int gt = blockIdx.x;
   const CclJob& J = v.jobs[job_of_tile(v, gt)];
-  final_labels_tile(J.labels, J.g, J.s, gt - J.tile0, fs, v.limit);
+  final_labels_tile<TH>(J.labels, J.g, J.s, gt - J.tile0, fs, v.limit);
 }
 
 cudaError_t launch_ccl_batch(const CclBatchView& v, cudaStream_t st) {
   if (v.n_tiles == 0) return cudaSuccess;
-  cudaError_t e = launch_after(k_cclb_tile, v.n_tiles, LABEL_THREADS, st, v);
+  const int th = v.jobs[0].g.th;   // of all grids
+  auto* tile = th == 8 ? k_cclb_tile<8> : th == 16 ? k_cclb_tile<16> : k_cclb_tile<TILE_H>;
+  auto* final_labels = th == 8 ? k_cclb_final<8> : th == 16 ? k_cclb_final<16> : k_cclb_final<TILE_H>;
+  cudaError_t e = launch_after(tile, v.n_tiles, LABEL_THREADS, st, v);
   if (e != cudaSuccess) return e;
   const int per = merge_tiles_per_cta(v.n_tiles);
   e = launch_after(k_cclb_merge, (unsigned)((v.n_tiles + per - 1) / per), MERGE_PER_TILE, st, v, per);
   if (e != cudaSuccess) return e;
-  return launch_after(k_cclb_final, v.n_tiles, FINAL_THREADS, st, v);
+  return launch_after(final_labels, v.n_tiles, FINAL_THREADS, st, v);
 }
 
 }  // namespace swccl

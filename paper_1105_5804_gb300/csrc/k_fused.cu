@@ -268,18 +268,11 @@ cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gp
   return launch_after(kernel, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, sel, P, philox_keys(seed));
 }
 
-// The lowest tiles that still leave few warps per SM: below about 16 (24 for
-// tiles of 16 rows) a tile's time is the latency of its chains, above it the
-// tiles share an SM's issue slots and the engine's work per tile counts.
 // Critical Ising, us per sweep with tiles of 32 / 16 / 8 rows: L = 256
 // 25.5 / 21.8 / 20.2, L = 768 (288 tiles of 8 rows) 27.7 / 24.1 / 23.5, L = 1000
 // (252 of 16, 500 of 8) 28.9 / 26.7 / 27.3, L = 1280 (400 of 16) 31.8 / 29.3 / 33.2,
 // L = 1440 (540 of 16) 31.6 / 31.9 / 37.3, L = 2048 42.4 / 45.5 / 53.8.
-int sweep_tile_rows(int L) {
-  constexpr int SMS = 152;
-  auto warps = [&](int th) { return make_grid(L, L, 1, th).n_tiles() * STRIPS; };
-  return warps(8) <= 16 * SMS ? 8 : warps(16) <= 24 * SMS ? 16 : TILE_H;
-}
+int sweep_tile_rows(int L) { return low_tile_rows(make_grid(L, L, 1, 8).n_tiles(), make_grid(L, L, 1, 16).n_tiles()); }
 
 LabelScratch sweep_scratch(const Grid& g, const LabelScratch& s) {
   LabelScratch low = s;

@@ -53,28 +53,39 @@ cudaError_t launch_tile_label(const uint8_t* mask, int32_t* labels, const Grid& 
 
 // Stand-alone labeling: local labeling with local-root labels, then (after
 // the seam merge) the final labels of every tile in one pass.
+template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
 k_ccl_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid g, LabelScratch s) {
-  __shared__ CclTileSmem sm;
+  __shared__ CclTileSmemT<TH> sm;
   wait_for_previous();
   let_next_start();
-  ccl_label_tile<true>(mask, labels, g, s, blockIdx.x, sm);
+  ccl_label_tile<true, TH>(mask, labels, g, s, blockIdx.x, sm);
 }
 
+template <int TH>
 __global__ void __launch_bounds__(FINAL_THREADS)
 k_ccl_final(int32_t* labels, Grid g, LabelScratch s, int limit) {
-  __shared__ FinalSmem fs;
+  __shared__ FinalSmem<TH> fs;
   wait_for_previous();
-  final_labels_tile(labels, g, s, blockIdx.x, fs, limit);
+  final_labels_tile<TH>(labels, g, s, blockIdx.x, fs, limit);
 }
 
 cudaError_t launch_ccl(const uint8_t* mask, int32_t* labels, const Grid& g, const LabelScratch& s, cudaStream_t st) {
-  cudaError_t e = launch_after(k_ccl_tile, g.n_tiles(), LABEL_THREADS, st, mask, labels, g, s);
+  auto* tile = g.th == 8 ? k_ccl_tile<8> : g.th == 16 ? k_ccl_tile<16> : k_ccl_tile<TILE_H>;
+  auto* final_labels = g.th == 8 ? k_ccl_final<8> : g.th == 16 ? k_ccl_final<16> : k_ccl_final<TILE_H>;
+  cudaError_t e = launch_after(tile, g.n_tiles(), LABEL_THREADS, st, mask, labels, g, s);
   if (e != cudaSuccess) return e;
   if ((e = launch_merge(labels, g, s, nullptr, nullptr, 0, 0, st)) != cudaSuccess) return e;
   const int limit = (int)std::min<int64_t>(g.n_sites() + 64, (int64_t)1 << 30);
-  return launch_after(k_ccl_final, g.n_tiles(), FINAL_THREADS, st, labels, g, s, limit);
+  return launch_after(final_labels, g.n_tiles(), FINAL_THREADS, st, labels, g, s, limit);
 }
+
+// Critical percolation, 128-wide tiles, us per labeling with tiles of
+// 32 / 16 / 8 rows: 28 x 64 14.5 / 14.4 / 14.2, 200 x 300 20.1 / 18.1 / 17.1,
+// 512^2 21.5 / 19.2 / 18.7, 768^2 (576 tiles of 8 rows) 24.9 / 20.7 / 20.5, 900^2
+// (456 of 16, 912 of 8) 26.5 / 22.5 / 23.2, 1280^2 (800 of 16) 27.7 / 24.8 / 31.1,
+// 1440^2 (1080 of 16) 27.3 / 26.6 / 36.4, 2048^2 32.7 / 39.6 / 55.6.
+int ccl_tile_rows(int64_t tiles8, int64_t tiles16) { return low_tile_rows(tiles8, tiles16); }
 
 // ---------------------------------------------------------------------------
 // Seam merge: one CTA per `per` consecutive tiles (merge_tiles).
@@ -169,19 +180,19 @@ LabelScratch carve_label_scratch(const Grid& g, void* base, int* err) {
 // asks a caller for).
 int64_t ccl_scratch_bytes(const Grid& g) {
   auto al = [](int64_t b) { return (b + 255) & ~(int64_t)255; };
-  const int64_t nt = g.n_tiles();
-  return al(nt * TILE_SITES * 2) + al(nt * (TILE_SITES / 32) * 4) + al(nt * SeamLayout::INTS * 4);
+  const int64_t nt = g.n_tiles(), sites = nt * g.th * TILE_W;
+  return al(sites * 2) + al(sites / 8) + al(nt * SeamLayout::INTS * 4);
 }
 
 LabelScratch carve_ccl_scratch(const Grid& g, void* base, int* err) {
   auto al = [](int64_t b) { return (b + 255) & ~(int64_t)255; };
-  const int64_t nt = g.n_tiles();
+  const int64_t sites = (int64_t)g.n_tiles() * g.th * TILE_W;
   char* p = static_cast<char*>(base);
   LabelScratch s;
   s.work = reinterpret_cast<int32_t*>(p);
-  p += al(nt * TILE_SITES * 2);
+  p += al(sites * 2);
   s.roots = reinterpret_cast<int32_t*>(p);
-  p += al(nt * (TILE_SITES / 32) * 4);
+  p += al(sites / 8);
   s.seams = reinterpret_cast<int32_t*>(p);
   s.root_counts = nullptr;
   s.err = err;

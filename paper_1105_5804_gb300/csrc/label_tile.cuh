@@ -60,33 +60,37 @@ __device__ __forceinline__ unsigned long long mask_word(const uint8_t* __restric
 // the tile root, the minimum site index of its tile component), and the tile's
 // root list.
 // Tile t's tile roots and edge-root bits in the scratch of the stand-alone
-// labeling (carve_ccl_scratch).
+// labeling (carve_ccl_scratch); TH: rows of a tile.
+template <int TH>
 __device__ __forceinline__ uint16_t* ccl_roots(const LabelScratch& s, int t) {
-  return reinterpret_cast<uint16_t*>(s.work) + (int64_t)t * TILE_SITES;
+  return reinterpret_cast<uint16_t*>(s.work) + (int64_t)t * (TH * TILE_W);
 }
+template <int TH>
 __device__ __forceinline__ int32_t* ccl_edges(const LabelScratch& s, int t) {
-  return s.roots + (int64_t)t * (TILE_SITES / 32);
+  return s.roots + (int64_t)t * (TH * TILE_W / 32);
 }
 
-struct CclTileSmem {
-  TileSmem tile;
-  uint32_t edge_bits[TILE_SITES / 32];   // local roots on the tile edge
+template <int TH>
+struct CclTileSmemT {
+  TileSmemT<TH> tile;
+  uint32_t edge_bits[TH * TILE_W / 32];   // local roots on the tile edge
 };
-static_assert(TILE_SITES / 32 == LABEL_THREADS, "one edge word per thread");
+using CclTileSmem = CclTileSmemT<TILE_H>;
+static_assert(TILE_SITES / 32 == LABEL_THREADS, "at most one edge word per thread");
 
-template <bool LOCAL = false>
+template <bool LOCAL = false, int TH = TILE_H>
 __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels,
-                                               const Grid& g, const LabelScratch& s, int t, CclTileSmem& cs) {
-  TileSmem& sm = cs.tile;
+                                               const Grid& g, const LabelScratch& s, int t, CclTileSmemT<TH>& cs) {
+  TileSmemT<TH>& sm = cs.tile;
   const uint16_t* par = sm.par;
   int* warp_roots = sm.warp_roots;
 
   const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-  const int y0 = ty * TILE_H, x0 = tx * TILE_W;
-  const int h = min(TILE_H, g.H - y0), w = min(TILE_W, g.W - x0);
+  const int y0 = ty * TH, x0 = tx * TILE_W;
+  const int h = min(TH, g.H - y0), w = min(TILE_W, g.W - x0);
   const int W = g.W;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  cs.edge_bits[threadIdx.x] = 0u;                        // the engine's barriers order it before the marks
+  if (threadIdx.x < TH * TILE_W / 32) cs.edge_bits[threadIdx.x] = 0u;                        // the engine's barriers order it before the marks
 
   // 1. bond bits of row `lane` of strip `warp`
   const int nvalid = min(max(w - 32 * warp, 0), 32);
@@ -114,13 +118,13 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
   const int in = min(max(w - lx0, 0), 8);   // columns past the grid are no roots of the tile
   uint32_t mine = 0;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < TH / 8; ++j) {
     const int ly = (lane >> 2) + 8 * j;
     if (ly >= h || in == 0) continue;   // the engine wrote no entries there
     const int sidx = local_of(ly, lx0);
     const uint4 r = roots_of(par, sidx);
     if (LOCAL) {
-      *reinterpret_cast<uint4*>(ccl_roots(s, t) + ly * TILE_W + lx0) = r;
+      *reinterpret_cast<uint4*>(ccl_roots<TH>(s, t) + ly * TILE_W + lx0) = r;
     } else {
       const uint32_t in_mask = ((1u << ((in + 1) >> 1)) - 1u) | ((1u << (in >> 1)) - 1u) << 16;
       const uint32_t own = (uint32_t)sidx * 0x00010001u + 0x00010000u;   // (sidx, sidx + 1)
@@ -143,7 +147,7 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
   // 6. LOCAL: edge-root bits; otherwise the root list
   if (LOCAL) {
     __syncthreads();
-    ccl_edges(s, t)[threadIdx.x] = (int32_t)cs.edge_bits[threadIdx.x];
+    if (threadIdx.x < TH * TILE_W / 32) ccl_edges<TH>(s, t)[threadIdx.x] = (int32_t)cs.edge_bits[threadIdx.x];
     return;
   }
   int32_t* slot = s.roots + (int64_t)t * TILE_SITES;
@@ -221,25 +225,26 @@ __device__ __forceinline__ void site_compress_tile(int32_t* __restrict__ labels,
 // by site, a labeling of 5003 x 7001 took 248 us instead of 181, of 4096^2 100
 // instead of 89.  All threads of the CTA call it.
 constexpr int FINAL_THREADS = 256;
-constexpr int EDGE_ROOTS_MAX = 2 * (TILE_H + TILE_W);
 constexpr bool FINAL_STAGED = TILE_W <= 128;   // tile roots in shared memory too (with 256 columns both exceed 48 KB)
+template <int TH>
 struct FinalSmem {
-  alignas(16) int32_t table[TILE_SITES];
-  alignas(16) uint16_t roots[FINAL_STAGED ? TILE_SITES : 8];   // tile roots, tile row-major
-  uint16_t list[EDGE_ROOTS_MAX];
+  alignas(16) int32_t table[TH * TILE_W];
+  alignas(16) uint16_t roots[FINAL_STAGED ? TH * TILE_W : 8];   // tile roots, tile row-major
+  uint16_t list[2 * (TH + TILE_W)];
   int n_edge;
 };
+template <int TH>
 __device__ __forceinline__ void final_labels_tile(int32_t* labels, const Grid& g, const LabelScratch& s, int t,
-                                                  FinalSmem& fs, int limit) {
+                                                  FinalSmem<TH>& fs, int limit) {
   const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-  const int y0 = ty * TILE_H, x0 = tx * TILE_W;
-  const int h = min(TILE_H, g.H - y0), w = min(TILE_W, g.W - x0);
+  const int y0 = ty * TH, x0 = tx * TILE_W;
+  const int h = min(TH, g.H - y0), w = min(TILE_W, g.W - x0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint16_t* lr = ccl_roots(s, t);
+  const uint16_t* lr = ccl_roots<TH>(s, t);
   if (FINAL_STAGED)
     for (int k = threadIdx.x; k < h * (TILE_W / 8); k += FINAL_THREADS) copy16_async(fs.roots + 8 * k, lr + 8 * k);
   uint32_t edge = 0u;
-  if (threadIdx.x < TILE_SITES / 32) edge = (uint32_t)__ldcg(ccl_edges(s, t) + threadIdx.x);
+  if (threadIdx.x < TH * TILE_W / 32) edge = (uint32_t)__ldcg(ccl_edges<TH>(s, t) + threadIdx.x);
   if (threadIdx.x == 0) fs.n_edge = 0;
   // 1. the table: own global indices
   for (int k = threadIdx.x; k < h * (TILE_W / 4); k += FINAL_THREADS) {

@@ -624,16 +624,16 @@ int ccl_label_ws(const uint8_t* bond_mask, int32_t* labels, int H, int W, int pe
     return fail(SW_ERR_ARG, "ccl_label_ws: workspace missing, too small or not 256-byte aligned");
   int* status = ccl_status_ptr();
   if (!status) return fail(SW_ERR_CUDA, "ccl: cannot resolve the device status word");
-  const LabelScratch s = carve_ccl_scratch(g, workspace, status);
+  const Grid gl = make_ccl_grid(H, W, periodic);
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  CK(launch_ccl(bond_mask, labels, g, s, st));
+  CK(launch_ccl(bond_mask, labels, gl, carve_ccl_scratch(gl, workspace, status), st));
   return SW_OK;
 }
 
 int ccl_label(const uint8_t* bond_mask, int32_t* labels, int H, int W, int periodic, void* stream) {
   int rc = ccl_validate(bond_mask, labels, H, W);
   if (rc) return rc;
-  const Grid g = make_grid(H, W, periodic);
+  const Grid g = make_ccl_grid(H, W, periodic);
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   int* status = ccl_status_ptr();
   if (!status) return fail(SW_ERR_CUDA, "ccl: cannot resolve the device status word");
@@ -722,11 +722,17 @@ int ccl_label_batch(int n, const uint8_t* const* masks, int32_t* const* labels, 
   for (int j0 = 0; j0 < n; j0 += CCL_PARAM_JOBS) {
     CclBatchView v;
     v.n_jobs = std::min(CCL_PARAM_JOBS, n - j0);
+    int64_t tiles8 = 0, tiles16 = 0;
+    for (int u = j0; u < j0 + v.n_jobs; ++u) {
+      tiles8 += make_grid(H[u], W[u], periodic[u], 8).n_tiles();
+      tiles16 += make_grid(H[u], W[u], periodic[u], 16).n_tiles();
+    }
+    const int th = ccl_tile_rows(tiles8, tiles16);
     int t0 = 0;
     int64_t max_sites = 0;
     for (int u = 0; u < v.n_jobs; ++u) {
       const int j = j0 + u;
-      const Grid g = make_grid(H[j], W[j], periodic[j]);
+      const Grid g = make_grid(H[j], W[j], periodic[j], th);
       CclJob& J = v.jobs[u];
       J.mask = masks[j];
       J.labels = labels[j];
@@ -734,7 +740,7 @@ int ccl_label_batch(int n, const uint8_t* const* masks, int32_t* const* labels, 
       J.g = g;
       J.tile0 = t0;
       J.pad = 0;
-      p += al256b(label_scratch_bytes(g));
+      p += al256b(label_scratch_bytes(make_grid(H[j], W[j], periodic[j])));
       t0 += g.n_tiles();
       v.tile_end[u] = t0;
       max_sites = std::max<int64_t>(max_sites, g.n_sites());

@@ -82,10 +82,11 @@ extern "C" int ccl_label_noalloc(const uint8_t* bond_mask, int32_t* labels, int 
   if (!ws) return set_last_error(SW_ERR_CUDA, "ccl_label_noalloc: " + msg);
   int* status = ccl_status_word();
   if (!status) return set_last_error(SW_ERR_CUDA, "ccl_label_noalloc: cannot resolve the device status word");
-  const LabelScratch s = carve_ccl_scratch(g, ws, status);
+  const Grid gl = make_ccl_grid(H, W, periodic);
+  const LabelScratch s = carve_ccl_scratch(gl, ws, status);
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  if ((e = launch_ccl(bond_mask, labels, g, s, st)) != cudaSuccess)
+  if ((e = launch_ccl(bond_mask, labels, gl, s, st)) != cudaSuccess)
     return set_last_error(SW_ERR_CUDA, std::string("ccl_label_noalloc: launch: ") + cudaGetErrorString(e));
   return SW_OK;
 }

@@ -52,7 +52,7 @@ struct Grid {
   int H, W;
   int tiles_x, tiles_y;
   int periodic;
-  int th;               // rows of a tile: TILE_H, or fewer for a sweep of a small lattice (low_tile.cuh)
+  int th;               // rows of a tile: TILE_H, or 8 or 16 where tiles are few (low_tile_rows)
   __host__ __device__ int64_t n_sites() const { return (int64_t)H * W; }
   __host__ __device__ int n_tiles() const { return tiles_x * tiles_y; }
 };
@@ -153,6 +153,20 @@ struct CclBatchView {
 // Bytes of LabelScratch for a grid (each part 256-byte aligned).
 int64_t label_scratch_bytes(const Grid& g);
 LabelScratch carve_label_scratch(const Grid& g, void* base, int* err);
+// Rows of the tiles for work that tiles of 8 or 16 rows cut into so many: the
+// lowest tiles that still leave few warps per SM.  Below about 16 (24 for
+// tiles of 16 rows) a tile's time is the latency of its chains, above it the
+// tiles share an SM's issue slots and the engine's work per tile counts.
+inline int low_tile_rows(int64_t tiles8, int64_t tiles16) {
+  constexpr int SMS = 152, WARPS = TILE_W / 32;
+  return tiles8 * WARPS <= 16 * SMS ? 8 : tiles16 * WARPS <= 24 * SMS ? 16 : TILE_H;
+}
+// Rows of the tiles of a stand-alone labeling.
+int ccl_tile_rows(int64_t tiles8, int64_t tiles16);
+inline Grid make_ccl_grid(int H, int W, int periodic) {
+  return make_grid(H, W, periodic,
+                   ccl_tile_rows(make_grid(H, W, periodic, 8).n_tiles(), make_grid(H, W, periodic, 16).n_tiles()));
+}
 // Rows of the tiles a fused sweep of an L x L lattice is cut into, and its
 // scratch: that of the 32-row grid, whose parts the lower tiles share.
 int sweep_tile_rows(int L);
