@@ -16,7 +16,7 @@
 // Small lattices alone leave most SMs idle (L = 64 is two tiles); in one
 // batch their tiles fill the machine.  Every chain draws from its own seed,
 // so a chain's result is the same alone or in any batch.
-#include "fused_tile.cuh"
+#include "low_tile.cuh"
 
 namespace swccl {
 
@@ -130,6 +130,60 @@ __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM) k_batch_flip(
   sw_flip_tile(R, gt - R.tile0, ctl->sweep - 1, b.limit, fs, SeedKey{(uint32_t)R.seed, (uint32_t)(R.seed >> 32)});
 }
 
+// The same over the low tiles of a batch that has few tiles (low_tile.cuh).
+// Tile gt of the batch: its chain with the grid and records of its low tiles,
+// and the tile's number in the chain.
+struct LowChain {
+  SwRep R;
+  int t;
+};
+template <int TH>
+__device__ __forceinline__ LowChain low_chain(const BatchView& b, const LowBatch& low, int gt) {
+  int lo = 0, hi = b.n_reps - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (gt < low.end[mid]) hi = mid;
+    else lo = mid + 1;
+  }
+  LowChain c;
+  c.R = b.reps[lo];
+  c.R.g.th = TH;
+  c.R.g.tiles_y = (c.R.g.H + TH - 1) / TH;
+  c.R.s.seams = c.R.s.work;   // see sweep_scratch
+  c.t = gt - (lo > 0 ? low.end[lo - 1] : 0);
+  return c;
+}
+
+template <int TH>
+__global__ void __launch_bounds__(LABEL_THREADS)
+k_batch_label_low(BatchView b, const __grid_constant__ LowBatch low, const BatchCtl* __restrict__ ctl) {
+  __shared__ LowTileSmem<TH> ls;
+  const LowChain c = low_chain<TH>(b, low, blockIdx.x);   // tables: not written by the kernels ahead
+  wait_for_previous();
+  const uint64_t sweep = ctl->sweep;
+  sw_label_low_tile(c.R, c.t, sweep, batch_do_obs(ctl, sweep), b.obs_cap, ls,
+                    SeedKey{(uint32_t)c.R.seed, (uint32_t)(c.R.seed >> 32)});
+}
+
+template <int TH>
+__global__ void __launch_bounds__(MERGE_PER_TILE)
+k_batch_merge_low(BatchView b, const __grid_constant__ LowBatch low, BatchCtl* ctl) {
+  __shared__ MergeSmem ms;
+  const LowChain c = low_chain<TH>(b, low, blockIdx.x);
+  wait_for_previous();
+  if (blockIdx.x == 0) batch_advance_block(b, ctl, ctl->sweep);
+  merge_tiles(ms, 1, [&](int) { return MergeTile{&c.R.g, c.R.gpar, c.R.s.seams, c.R.s.err, c.t}; }, b.limit);
+}
+
+template <int TH>
+__global__ void __launch_bounds__(LABEL_THREADS)
+k_batch_flip_low(BatchView b, const __grid_constant__ LowBatch low, const BatchCtl* __restrict__ ctl) {
+  __shared__ FlipTileSmemT<TH> fs;
+  const LowChain c = low_chain<TH>(b, low, blockIdx.x);
+  wait_for_previous();
+  sw_flip_tile<TH>(c.R, c.t, ctl->sweep - 1, b.limit, fs, SeedKey{(uint32_t)c.R.seed, (uint32_t)(c.R.seed >> 32)});
+}
+
 __global__ void __launch_bounds__(LABEL_THREADS) k_batch_observe(BatchView b, BatchCtl* ctl) {
   __shared__ LabelTileSmem ls;
   const uint64_t done = ctl->sweep - 1;
@@ -185,16 +239,25 @@ cudaError_t launch_batch_init(const BatchView& b, int hot, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_label(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
+cudaError_t launch_batch_label(const BatchView& b, const LowBatch& low, BatchCtl* ctl, cudaStream_t st) {
+  if (low.th)
+    return launch_after(low.th == 8 ? k_batch_label_low<8> : k_batch_label_low<16>, low.n_tiles, LABEL_THREADS, st, b, low,
+                        ctl);
   return launch_after(k_batch_label, b.n_tiles, LABEL_THREADS, st, b, ctl);
 }
 
-cudaError_t launch_batch_merge(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
+cudaError_t launch_batch_merge(const BatchView& b, const LowBatch& low, BatchCtl* ctl, cudaStream_t st) {
+  if (low.th)
+    return launch_after(low.th == 8 ? k_batch_merge_low<8> : k_batch_merge_low<16>, low.n_tiles, MERGE_PER_TILE, st, b, low,
+                        ctl);
   const int per = merge_tiles_per_cta(b.n_tiles);
   return launch_after(k_batch_merge, (unsigned)((b.n_tiles + per - 1) / per), MERGE_PER_TILE, st, b, ctl, per);
 }
 
-cudaError_t launch_batch_flip(const BatchView& b, BatchCtl* ctl, cudaStream_t st) {
+cudaError_t launch_batch_flip(const BatchView& b, const LowBatch& low, BatchCtl* ctl, cudaStream_t st) {
+  if (low.th)
+    return launch_after(low.th == 8 ? k_batch_flip_low<8> : k_batch_flip_low<16>, low.n_tiles, LABEL_THREADS, st, b, low,
+                        ctl);
   return launch_after(k_batch_flip, b.n_tiles, LABEL_THREADS, st, b, ctl);
 }
 

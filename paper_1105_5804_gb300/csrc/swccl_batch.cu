@@ -38,6 +38,7 @@ struct sw_batch {
   BatchCtl* ctl = nullptr;
   std::vector<SwRep> reps;
   BatchView view{};
+  LowBatch low{};                 // lower tiles for the phase schedule, if the batch has few
   int schedule = SW_BATCH_PHASES;
   int blocks = 0;                 // persistent CTAs
   long long barrier_limit = SW_BATCH_BARRIER_LIMIT_DEFAULT;   // clock64() cycles per barrier wait
@@ -52,6 +53,25 @@ struct sw_batch {
 };
 
 namespace {
+
+// The low tiles of a batch with few tiles (th = 0: it keeps the 32-row ones).
+LowBatch low_batch(int n, const int* L) {
+  LowBatch low{};
+  if (n > LOW_BATCH_CHAINS) return low;
+  int64_t tiles8 = 0, tiles16 = 0;
+  for (int r = 0; r < n; ++r) {
+    tiles8 += make_grid(L[r], L[r], 1, 8).n_tiles();
+    tiles16 += make_grid(L[r], L[r], 1, 16).n_tiles();
+  }
+  const int th = low_tile_rows(tiles8, tiles16);
+  if (th == TILE_H) return low;
+  low.th = th;
+  for (int r = 0; r < n; ++r) {
+    low.n_tiles += make_grid(L[r], L[r], 1, th).n_tiles();
+    low.end[r] = (uint16_t)low.n_tiles;
+  }
+  return low;
+}
 
 void free_batch(sw_batch* b) {
   if (!b) return;
@@ -69,9 +89,9 @@ cudaError_t enqueue_batch_sweep(sw_batch* b) {
   cudaError_t e;
   if (b->schedule == SW_BATCH_PERSISTENT)
     return launch_batch_persistent(b->view, b->ctl, b->blocks, b->barrier_limit, b->stream);
-  if ((e = launch_batch_label(b->view, b->ctl, b->stream))) return e;
-  if ((e = launch_batch_merge(b->view, b->ctl, b->stream))) return e;
-  return launch_batch_flip(b->view, b->ctl, b->stream);
+  if ((e = launch_batch_label(b->view, b->low, b->ctl, b->stream))) return e;
+  if ((e = launch_batch_merge(b->view, b->low, b->ctl, b->stream))) return e;
+  return launch_batch_flip(b->view, b->low, b->ctl, b->stream);
 }
 
 // Forget the captured sweep of schedule k (its launch arguments changed).
@@ -243,6 +263,7 @@ sw_batch* create_batch(int n, const int* L, const int* q, const double* beta, co
   memcpy(tables.data() + lay.reps, b->reps.data(), sizeof(SwRep) * n);
   if ((e = cudaMemcpyAsync(base, tables.data(), tables.size(), cudaMemcpyHostToDevice, b->stream)))
     return bad(e, "chain tables");
+  b->low = low_batch(n, L);
   b->view.reps = b->d_reps;
   b->view.tile_rep = b->d_tile_rep;
   b->view.n_reps = n;

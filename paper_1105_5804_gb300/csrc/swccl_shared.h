@@ -127,6 +127,15 @@ struct BatchView {
   int limit;          // union-find step bound: largest replica's sites + 64
 };
 
+// The tiles of 8 or 16 rows of a batch that has few tiles (low_tile_rows), passed
+// to the kernels of the phase schedule by value: chain r's end at end[r].
+constexpr int LOW_BATCH_CHAINS = 256;
+struct LowBatch {
+  int th;             // rows of a tile; 0: the batch runs on the 32-row tiles
+  int n_tiles;
+  uint16_t end[LOW_BATCH_CHAINS];
+};
+
 // One grid of a batched labeling call.
 struct CclJob {
   const uint8_t* mask;
@@ -254,9 +263,9 @@ cudaError_t launch_sw_small(int8_t* spins, int L, int q, uint64_t T, uint64_t se
 
 // Batched chains (k_batch.cu).  init: spins of every chain, observable rings cleared.
 cudaError_t launch_batch_init(const BatchView& b, int hot, cudaStream_t st);
-cudaError_t launch_batch_label(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
-cudaError_t launch_batch_merge(const BatchView& b, BatchCtl* ctl, cudaStream_t st);   // and advance (see launch_merge)
-cudaError_t launch_batch_flip(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
+cudaError_t launch_batch_label(const BatchView& b, const LowBatch& low, BatchCtl* ctl, cudaStream_t st);
+cudaError_t launch_batch_merge(const BatchView& b, const LowBatch& low, BatchCtl* ctl, cudaStream_t st);   // and advance (see launch_merge)
+cudaError_t launch_batch_flip(const BatchView& b, const LowBatch& low, BatchCtl* ctl, cudaStream_t st);
 cudaError_t launch_batch_observe(const BatchView& b, BatchCtl* ctl, cudaStream_t st);
 // One persistent cooperative launch for the whole sweep; `blocks` CTAs; a
 // grid-barrier wait gives up after limit_cycles of clock64().
