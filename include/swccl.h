@@ -191,9 +191,11 @@ int sw_set_mode(sw_handle* h, int mode);
 /* The CUDA stream (cudaStream_t) all work of the handle is ordered on. */
 void* sw_stream(sw_handle* h);
 
-/* Per-phase timing.  With timing on, sw_sweep launches each phase directly
- * with CUDA events between phases (no graph); with it off (default) one
- * sweep is a captured CUDA graph.  Both compute the same chain. */
+/* Per-phase timing.  With timing on, sw_sweep launches each phase with CUDA
+ * events between phases; with it off (default) phases and sweeps follow each
+ * other by programmatic launches, or many sweeps of a small lattice run in one
+ * launch (staged mode: one sweep is a captured CUDA graph).  Both compute the
+ * same chain. */
 int sw_set_timing(sw_handle* h, int enable);
 
 /* Milliseconds spent in each phase (ms[SW_N_PHASES]) summed over the sweeps
@@ -253,8 +255,8 @@ uint64_t sw_prob_threshold(double p);
  * library owns the device memory: about 7.2 bytes per site (spins, brick
  * roots, parent array, edge and face bits) plus the observable ring.  NULL on failure (see sw_last_error).  Each sweep is
  * three kernels (brick-local union-find with the previous sweep's
- * observables, face merge, flip) and a counter advance, replayed as a
- * captured CUDA graph unless timing is on. */
+ * observables, face merge and counter advance, flip), launched so that each
+ * launch overlaps the kernel before it. */
 typedef struct sw3_handle sw3_handle;
 #define SW3_N_PHASES 4   /* local (+ observables), merge, flip, advance */
 

@@ -1,7 +1,7 @@
 // k_small.cu -- many Swendsen-Wang sweeps of a small lattice in one launch.
 //
-// A lattice up to SMALL_L = 128 on a side leaves the GPU all but empty, and its
-// sweep is bound by latency: of the 21 us that a sweep at L = 64 takes as three
+// A lattice up to SMALL_L = 112 on a side leaves the GPU all but empty, and its
+// sweep is bound by latency: of the 14.3 us that a sweep at L = 64 takes as three
 // kernels (k_fused.cu), most goes into launches and into loads and atomics that
 // go through L2.  Here one block keeps the whole lattice in shared memory --
 // int8 spins, and 16-bit union-find entries laid out like the sites, so that no
@@ -23,10 +23,11 @@
 //     the root) into their own spins;
 //  5. after a barrier, every site takes its root's spin.
 // Bound by the latency of its chains up to about L = 80 (an instruction every
-// five cycles in a warp, 4 warps per scheduler) and by issue at L = 128.  A
-// sweep takes 4.6 us at L = 16, 7.8 at 64, 12.0 at 96 and 17.1 at 128 against
-// 21.0 (L = 64) and 22.9 (128) as three kernels; beyond that one SM no longer
-// keeps up with tiles spread over the GPU (24.8 us at L = 132).
+// five cycles in a warp, 4 warps per scheduler) and by issue above.  Critical
+// Ising, us per sweep here / as three kernels on low tiles: L = 16 4.8 / 11.4, 64
+// 7.8 / 14.3, 96 12.1 / 15.2, 100 15.1 / 15.5, 112 15.3 / 16.6, 116 16.8 / 17.0,
+// 124 19.8 / 16.9 (q = 3: 112 16.2 / 16.6, 116 17.7 / 16.8); the line lies where
+// one SM no longer keeps up with tiles spread over the GPU.
 #include "fused_tile.cuh"
 
 namespace swccl {
@@ -58,7 +59,7 @@ static size_t small_smem_bytes(int L) { return sizeof(SmallSmem) + (size_t)3 * L
 // chains, more warps: L = 64 8.1 against 9.9 us a sweep with 16), else 16.
 static int small_units(int L, int H) { return ((L + 31) / 32) * ((L + H - 1) / H); }
 static int small_rows(int L) { return small_units(L, 8) <= SMALL_UNITS ? 8 : 16; }
-static_assert((SMALL_L / 32) * (SMALL_L / 16) <= SMALL_UNITS, "one warp per unit");
+static_assert(((SMALL_L + 31) / 32) * ((SMALL_L + 15) / 16) <= SMALL_UNITS, "one warp per unit");
 
 // Shared memory is read before it is written within each step (loads of all
 // rows first, then the chain, then the stores): the compiler cannot tell the

@@ -1,10 +1,11 @@
 // swccl_api.cu -- host driver and C ABI of libswccl (declared in include/swccl.h).
 //
-// A Swendsen-Wang sweep (Sec. II, three steps) is five kernels on the
-// handle's stream: activation, tile labeling, seam merge, root compression
-// with root draws, flip with observables; a one-thread kernel then advances
-// the sweep counter held in device memory, so one captured CUDA graph serves
-// every sweep.  Nothing crosses to the host inside a sweep (the paper's
+// A Swendsen-Wang sweep (Sec. II, three steps) is three kernels on the
+// handle's stream (k_fused.cu), many sweeps of a small lattice one (k_small.cu).
+// In staged mode it is five: activation, tile labeling, seam merge, root
+// compression with root draws, flip with observables; a one-thread kernel then
+// advances the sweep counter held in device memory, so one captured CUDA graph
+// serves every such sweep.  Nothing crosses to the host inside a sweep (the paper's
 // relaxation checked its stopping rule on the CPU between launches,
 // Sec. II.C.1; the atomic merge needs no such loop).
 #include <cmath>
@@ -93,8 +94,6 @@ struct sw_handle {
   uint64_t obs_read = 0;   // next sweep whose observables are unread
   cudaGraph_t graph = nullptr;        // one staged sweep
   cudaGraphExec_t exec = nullptr;
-  cudaGraph_t graph_fused = nullptr;  // one fused sweep
-  cudaGraphExec_t exec_fused = nullptr;
   int update = SW_UPDATE_SW;         // SW_UPDATE_SW or SW_UPDATE_FEW (fused mode only)
   int ell = 0;                       // few-cluster: ell x ell seed blocks
   uint64_t P_flip = 0;               // few-cluster: flip threshold
@@ -113,8 +112,6 @@ void free_handle(sw_handle* h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   if (h->exec) cudaGraphExecDestroy(h->exec);
   if (h->graph) cudaGraphDestroy(h->graph);
-  if (h->exec_fused) cudaGraphExecDestroy(h->exec_fused);
-  if (h->graph_fused) cudaGraphDestroy(h->graph_fused);
   for (auto e : h->ev_pending) cudaEventDestroy(e);
   for (auto e : h->ev_free) cudaEventDestroy(e);
   cudaFree(h->spins);
@@ -275,11 +272,6 @@ int sw_set_update(sw_handle* h, int update, int ell, uint64_t P) {
       return fail(SW_ERR_OOM, "sw_set_update: cudaMalloc of the selection bits failed");
     }
   }
-  // ell and P are launch arguments of the captured sweep: capture it again
-  if (h->exec_fused) cudaGraphExecDestroy(h->exec_fused);
-  if (h->graph_fused) cudaGraphDestroy(h->graph_fused);
-  h->exec_fused = nullptr;
-  h->graph_fused = nullptr;
   h->update = update;
   h->ell = ell;
   h->P_flip = P;
@@ -371,6 +363,11 @@ int sw_sweep(sw_handle* h, int n) {
   if (n == 0) return SW_OK;
   const bool fused = h->mode == SW_MODE_FUSED;
   auto enqueue = fused ? enqueue_sweep_fused : enqueue_sweep;
+  if (fused && !h->timing) {   // a captured sweep would not be counted: refused
+    cudaStreamCaptureStatus capture;
+    CK(cudaStreamIsCapturing(h->stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) return fail(SW_ERR_CUDA, "sw_sweep: the stream is being captured");
+  }
   if (fused && !h->timing && h->update == SW_UPDATE_SW && h->L <= SMALL_L) {
     // all sweeps of the call by one block, which writes their observables too
     for (int done = 0; done < n; done += SMALL_SWEEPS) {
@@ -397,21 +394,28 @@ int sw_sweep(sw_handle* h, int n) {
       CK(enqueue(h, ev));
       h->sweeps++;
     }
+  } else if (fused) {
+    // three programmatic launches per sweep, 4 us of host time: a sweep's first
+    // kernel is then launched while the sweep before ends, which graphs of one
+    // sweep each do not do (L = 256: 17.5 us per sweep against 20.2, L = 1000
+    // 24.1 against 26.7, L = 2048 40.6 against 42.6)
+    for (int k = 0; k < n; ++k) {
+      CK(enqueue(h, nullptr));
+      h->sweeps++;
+    }
   } else {
-    cudaGraph_t& graph = fused ? h->graph_fused : h->graph;
-    cudaGraphExec_t& exec = fused ? h->exec_fused : h->exec;
-    if (!exec) {
+    if (!h->exec) {
       CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
       cudaError_t e = enqueue(h, nullptr);
       cudaGraph_t gr = nullptr;
       cudaError_t e2 = cudaStreamEndCapture(h->stream, &gr);
       if (e != cudaSuccess) { if (gr) cudaGraphDestroy(gr); return cuda_fail(e, "capture of one sweep"); }
       if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamEndCapture");
-      graph = gr;
-      CK(cudaGraphInstantiate(&exec, graph, 0));
+      h->graph = gr;
+      CK(cudaGraphInstantiate(&h->exec, h->graph, 0));
     }
     for (int k = 0; k < n; ++k) {
-      CK(cudaGraphLaunch(exec, h->stream));
+      CK(cudaGraphLaunch(h->exec, h->stream));
       h->sweeps++;
     }
   }

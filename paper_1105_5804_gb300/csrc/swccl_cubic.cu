@@ -41,8 +41,6 @@ struct sw3_handle {
   int* chk = nullptr;             // spin-check flag of sw3_set_spins
   int64_t* obs = nullptr;
   uint64_t sweeps = 0, obs_read = 0;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
   bool timing = false;
   bool labels_valid = false;
   bool final_obs_pending = false;   // the last sweep's observables are counted when read
@@ -55,8 +53,6 @@ namespace {
 void free3(sw3_handle* h) {
   if (!h) return;
   if (h->stream) cudaStreamSynchronize(h->stream);
-  if (h->exec) cudaGraphExecDestroy(h->exec);
-  if (h->graph) cudaGraphDestroy(h->graph);
   for (auto e : h->ev_pending) cudaEventDestroy(e);
   for (auto e : h->ev_free) cudaEventDestroy(e);
   cudaFree(h->spins);
@@ -175,22 +171,12 @@ int sw3_sweep(sw3_handle* h, int n) {
       h->sweeps++;
     }
   } else {
-    if (!h->exec) {
-      CK3(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-      cudaError_t e = launch_sweep3(h->spins, h->lroot, h->gpar, h->words, h->box, h->q, h->T,
-                                    h->seed, h->ctl, h->obs, OBS3_CAP, h->stream, nullptr);
-      cudaGraph_t gr = nullptr;
-      cudaError_t e2 = cudaStreamEndCapture(h->stream, &gr);
-      if (e != cudaSuccess) {
-        if (gr) cudaGraphDestroy(gr);
-        return cuda_fail3(e, "capture of one 3D sweep");
-      }
-      if (e2 != cudaSuccess) return cuda_fail3(e2, "cudaStreamEndCapture");
-      h->graph = gr;
-      CK3(cudaGraphInstantiate(&h->exec, h->graph, 0));
-    }
+    cudaStreamCaptureStatus capture;   // a captured sweep would not be counted: refused
+    CK3(cudaStreamIsCapturing(h->stream, &capture));
+    if (capture != cudaStreamCaptureStatusNone) return fail3(SW_ERR_CUDA, "sw3_sweep: the stream is being captured");
     for (int k = 0; k < n; ++k) {
-      CK3(cudaGraphLaunch(h->exec, h->stream));
+      CK3(launch_sweep3(h->spins, h->lroot, h->gpar, h->words, h->box, h->q, h->T, h->seed, h->ctl, h->obs, OBS3_CAP,
+                        h->stream, nullptr));
       h->sweeps++;
     }
   }

@@ -256,7 +256,7 @@ cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gp
 // in one launch, their observables (and the pending ones of the sweep before)
 // written to the ring, ctl advanced.  small_prepare: once per device before the
 // first launch.
-constexpr int SMALL_L = 128;
+constexpr int SMALL_L = 112;
 cudaError_t small_prepare();
 cudaError_t launch_sw_small(int8_t* spins, int L, int q, uint64_t T, uint64_t seed, SwCtl* ctl, int64_t* obs,
                             int obs_cap, int n, cudaStream_t st);

@@ -21,6 +21,7 @@ def test_initial_state(hot):
         for r in range(6):
             s = oracle.init_spins(L[r], q[r], seed[r], hot).reshape(-1)
             out = torch.full((L[r] * L[r] + 1,), -1, dtype=torch.int8, device="cuda")
+            torch.cuda.synchronize()   # the batch copies on its own stream
             sw.sw_batch_get_spins(b, r, L[r], out[1:])   # a destination that is not 16-byte aligned
             assert np.array_equal(out[1:].cpu().numpy(), s) and int(out[0]) == -1, r
             assert np.array_equal(sw.sw_batch_get_spins(b, r, L[r]), s), r
@@ -33,6 +34,7 @@ def test_failed_batch_leaves_the_destination():
     b = sw.sw_batch_create([64, 256], [2, 2], [0.4, 0.4], [1, 2], sw.SW_CONV_AUTO, True)
     try:
         out = torch.full((64 * 64,), 77, dtype=torch.int8, device="cuda")
+        torch.cuda.synchronize()
         sw.sw_batch_set_schedule(b, sw.SW_BATCH_PERSISTENT)
         sw.sw_batch_set_barrier_limit(b, 0)
         sw.sw_batch_sweep(b, 1)
