@@ -25,7 +25,6 @@ template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_cclb_tile(const __grid_constant__ CclBatchView v) {
   __shared__ CclTileSmemT<TH> sm;
   wait_for_previous();
-  let_next_start();
   const int gt = blockIdx.x;
   const CclJob& J = v.jobs[job_of_tile(v, gt)];
   ccl_label_tile<true, TH>(J.mask, J.labels, J.g, J.s, gt - J.tile0, sm);
@@ -34,7 +33,6 @@ __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_cclb_tile(
 __global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_constant__ CclBatchView v, int per) {
   __shared__ MergeSmem ms;
   wait_for_previous();
-  let_next_start();
   const int gt0 = blockIdx.x * per;
   merge_tiles(ms, min(per, v.n_tiles - gt0),
               [&](int u) {

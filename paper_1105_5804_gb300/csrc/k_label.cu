@@ -58,7 +58,6 @@ __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
 k_ccl_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid g, LabelScratch s) {
   __shared__ CclTileSmemT<TH> sm;
   wait_for_previous();
-  let_next_start();
   ccl_label_tile<true, TH>(mask, labels, g, s, blockIdx.x, sm);
 }
 
@@ -95,7 +94,6 @@ k_merge(int32_t* __restrict__ labels, const __grid_constant__ Grid g, LabelScrat
         int64_t* obs, int obs_cap, int q) {
   __shared__ MergeSmem ms;
   wait_for_previous();
-  if (!adv) let_next_start();
   if (adv && blockIdx.x == 0) {   // end of the drawing step: the next sweep's fills this sweep's observable slot
     const uint64_t sweep = adv->sweep;
     for (int k = threadIdx.x; k <= q; k += MERGE_PER_TILE) obs[(int64_t)(sweep % (uint64_t)obs_cap) * (q + 1) + k] = 0;

@@ -18,15 +18,15 @@ namespace swccl {
 // launched before the kernels ahead of it in the stream have ended, so that its
 // launch overlaps them.  Every thread of such a kernel calls wait_for_previous
 // first: it returns when the kernels ahead have completed and their writes are
-// visible (at once in a kernel launched plainly).  A sweep at L = 256 takes 25.0
-// us instead of 27.4.  let_next_start lets the next kernel's blocks become
-// resident as soon as all of this one's run: 1 us more for a chain of kernels
-// that leave the GPU mostly empty (labeling 200 x 300), but the heavy blocks of
-// the next step then land unevenly (a sweep at L = 2048 46 instead of 42 us), so
-// only the stand-alone labeling uses it.
+// visible (at once in a kernel launched plainly).  A sweep at L = 256 took 25.0
+// us instead of 27.4 with it, 17.5 instead of 20.2 on low tiles where it also
+// joins the sweeps.  The other half, a trigger that lets the next kernel's blocks
+// become resident while this one's run, made everything slower (they take issue
+// slots and place its blocks unevenly): L = 256 19.0 instead of 17.5 us, L = 2048
+// 46 instead of 42, a labeling of 200 x 300 17.8 instead of 17.1, of 2048^2 34.1
+// instead of 31.8.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class... P, class... A>
 inline cudaError_t launch_after_smem(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem,
