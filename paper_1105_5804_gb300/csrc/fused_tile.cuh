@@ -352,7 +352,10 @@ __device__ __forceinline__ int root_in(const uint4& v, int i) {
 // Bound by instruction issue (74 % of the slots, 1.03 warp instructions per
 // site, a third of them the draws); critical Ising, L = 16384: 0.298 ms against
 // 0.389 ms with the roots read twice, flags looked up root by root and four
-// walks per thread in step.
+// walks per thread in step.  Above the critical temperature the draws are most
+// of it (0.4 roots per site at 0.6 beta_c): L = 8192 there 146 us against 180 with
+// every root listed and threads looking through their roots once per pass of
+// the list (T = infinity 210 against 345).
 // TH: rows of the lattice's tiles.
 template <int TH = TILE_H, class Keys = SeedKey>
 __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t sweep, int limit, FlipTileSmemT<TH>& fs,
@@ -423,7 +426,21 @@ __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t swe
     mine = spread_bits(m & 0xFFFFu) | spread_bits(m >> 16) << 1;
   }
   const uint32_t on_edge = mine & edges;
-  const uint32_t inner = mine & ~edges;
+  uint32_t inner = mine & ~edges;
+  auto set_state = [&](int r, int G) {   // new state of the component with local root r and cluster root G
+    const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
+    ns[r] = (uint8_t)state_of(d.x, q);
+  };
+  auto root_at = [&](int n) { return id0 + n + (n & 24) * (TILE_W - 1); };   // local index of bit n's site
+  // as many interior roots as every lane of the warp has are drawn where they
+  // stand (hardly any at criticality, two in three at 0.6 beta_c); the list
+  // spreads the others over the lanes
+  for (int k = __reduce_min_sync(FULL, __popc(inner)); k > 0; --k) {
+    const int n = high_bit(inner);
+    inner ^= 1u << n;
+    const int r = root_at(n);
+    set_state(r, tile_global(r, y0, x0, L));
+  }
 
   // 3. the tile's root list: edge roots, then the others (counts of both in
   //    one scan; a tile with more roots than the list holds takes several
@@ -446,18 +463,15 @@ __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t swe
   const int n_edge = total >> 16, n_roots = n_edge + (total & 0xFFFF);
   const int at_edge = before >> 16, at_inner = n_edge + (before & 0xFFFF);
 
-  auto set_state = [&](int r, int G) {   // new state of the component with local root r and cluster root G
-    const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
-    ns[r] = (uint8_t)state_of(d.x, q);
-  };
-
   for (int first = 0; first < n_roots; first += FLIP_LIST) {
-    // my roots as local indices id0 + (site of a pass) + 8 (pass) TILE_W
+    // my roots as local indices id0 + (site of a pass) + 8 (pass) TILE_W; a
+    // thread whose roots all belong to another pass lists none
     auto list = [&](uint32_t bits, int at, bool fits) {
+      if (!fits && (at >= FLIP_LIST || at + __popc(bits) <= 0)) return;
       while (bits) {
         const int n = high_bit(bits);
         bits ^= 1u << n;
-        if (fits || (unsigned)at < FLIP_LIST) fs.rlist[at] = (uint16_t)(id0 + n + (n & 24) * (TILE_W - 1));
+        if (fits || (unsigned)at < FLIP_LIST) fs.rlist[at] = (uint16_t)root_at(n);
         ++at;
       }
     };
