@@ -29,10 +29,10 @@ L_BENCH, Q_BENCH, SEED_BENCH = 16384, 2, 7
 # self-labeling + sewing on a Tesla M2070, 3.573 ns per site and sweep (Table I)
 PAPER_SITE_UPDATES_PER_NS = 1.0 / 3.573
 WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
-# Counters of the fused sweep's kernels from one ncu capture each (--set
-# full, one launch, L = 8192, the third sweep from the hot start; the
-# full-size launch is too large to capture under ncu's replay, and DRAM
-# bytes and instructions grow with the sites processed), per site:
+# Counters of the fused sweep's kernels from one ncu capture each (one
+# launch, L = 8192, the eleventh sweep from the hot start; the full-size
+# launch is too large to capture under ncu's replay, and DRAM bytes and
+# instructions grow with the sites processed), per site:
 # DRAM bytes = dram__bytes_read.sum + dram__bytes_write.sum, warp
 # instructions = smsp__inst_executed.sum.  Valid only for the code they were
 # taken with (a hash of the sources without comments); otherwise the line
@@ -629,13 +629,13 @@ def run_ours(args):
         if world > 1:
             torch.distributed.barrier()
 
-    # warm-up (graph capture happens in the first call of graph mode)
+    # warm-up
     sw.sw_sweep(h, max(args.warmup, 3))
     sw.sw_sync(h)
     sw.sw_observables(h, 4096)
 
-    # timed region: the sweeps as a user runs them (one captured CUDA graph per
-    # sweep, replayed), events on the handle's stream
+    # timed region: the sweeps as a user runs them (three programmatic launches
+    # per sweep), events on the handle's stream
     uuid = None
     try:
         uuid = "GPU-" + str(torch.cuda.get_device_properties(local).uuid)
@@ -822,7 +822,7 @@ def run_ours(args):
                    "start": "hot", "seed": SEED_BENCH, "replicas": world, "parallelism": "replicas",
                    "l2": "inputs larger than L2 (spins %d MiB, 16-bit tile roots %d MiB per replica)"
                          % (N >> 20, (2 * N) >> 20),
-                   "timed_path": "sw_sweep replaying one captured CUDA graph per sweep; the per-kernel split comes "
+                   "timed_path": "sw_sweep, three programmatic launches per sweep; the per-kernel split comes "
                                  "from a separate pass of %d eagerly launched sweeps with events" % PHASE_SWEEPS},
         "clocks": clk,
         "gpu_launches": 3 * args.steps,

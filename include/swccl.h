@@ -407,7 +407,7 @@ void* sw_batch_stream(sw_batch* b);
  * periodic == 0: those bonds are ignored (image segmentation).
  * Requires H, W >= 1 and H*W < 2^31.  Enqueued on `stream` (a
  * cudaStream_t, NULL = legacy default stream); returns without waiting.
- * Scratch memory (about 8.3 bytes per site) is taken with cudaMallocAsync
+ * Scratch memory (2.4 to 3.4 bytes per site) is taken with cudaMallocAsync
  * on the same stream and released in stream order. */
 int ccl_label(const uint8_t* bond_mask, int32_t* labels, int H, int W, int periodic, void* stream);
 

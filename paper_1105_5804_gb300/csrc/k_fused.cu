@@ -9,15 +9,15 @@
 //              and east column beyond it), draws the tile's bonds (rule of
 //              Eq. 7, Sec. II.A) into shared memory, labels the tile with
 //              the engine of tile_engine.cuh, and writes each site's tile
-//              root as a 16-bit local index (the root's own entry flagged
-//              if its component touches the tile edge), the seam record of
-//              the tile, and a parent entry gpar[r] = r for every tile root
-//              r on the tile's edge.  It also counts, for the spins it read
+//              root as a 16-bit local index, a bit per local index that is
+//              set for the roots whose component touches the tile edge, the
+//              seam record of the tile, and a parent entry gpar[r] = r for
+//              every such root r.  It also counts, for the spins it read
 //              (the result of the previous sweep), the bonds joining equal
 //              spins and the sites per state, the observables of that sweep.
-//  k_merge     (k_label.cu) joins tile roots across seams on gpar.
-//  k_sw_flip   one CTA per tile: lists the tile's roots; a flagged root
-//              (on the tile edge) looks up its final root R in gpar, any
+//  k_merge     (k_label.cu) joins tile roots across seams on gpar, clears the
+//              sweep's observable slot and advances the sweep counter.
+//  k_sw_flip   one CTA per tile: lists the tile's roots; an edge root looks up its final root R in gpar, any
 //              other root is its own final root; each root draws its
 //              cluster's new state once
 //              (FLIP draw keyed by R, Sec. II.D) and every site copies the
@@ -268,7 +268,8 @@ cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gp
   return launch_after(kernel, g.n_tiles(), LABEL_THREADS, st, R, ctl, limit, sel, P, philox_keys(seed));
 }
 
-// Critical Ising, us per sweep with tiles of 32 / 16 / 8 rows: L = 256
+// Critical Ising, us per sweep with tiles of 32 / 16 / 8 rows (measured with a
+// graph per sweep; 2 to 3 us less each without): L = 256
 // 25.5 / 21.8 / 20.2, L = 768 (288 tiles of 8 rows) 27.7 / 24.1 / 23.5, L = 1000
 // (252 of 16, 500 of 8) 28.9 / 26.7 / 27.3, L = 1280 (400 of 16) 31.8 / 29.3 / 33.2,
 // L = 1440 (540 of 16) 31.6 / 31.9 / 37.3, L = 2048 42.4 / 45.5 / 53.8.

@@ -5,17 +5,11 @@
 // (self-labeling, BFS, serial union-find) and its consolidation schemes
 // (relaxation, hierarchical sewing) are replaced:
 //
-//  k_tile_label   one CTA per TILE_H x TILE_W tile.  Bond bits go to shared
-//                 memory; each row is cut into runs of east-connected sites
-//                 with one warp ballot per 32 sites (the run's leftmost site
-//                 is its root); north bonds are joined with a lock-free
-//                 shared-memory union-find that hooks larger roots under
-//                 smaller ones, skipping a north bond whose left neighbour
-//                 already joined the same two runs.  Each site's label is the
-//                 global index of its tile-local root (the tile component's
-//                 minimum site index); roots are appended to a per-tile list,
-//                 and the labels and bond bits of the four tile edges go to a
-//                 compact seam record.
+//  k_tile_label   one CTA per TILE_H x TILE_W tile, labeled by the tile engine
+//                 (tile_engine.cuh).  Each site's label is the global index of
+//                 its tile-local root (the tile component's minimum site index);
+//                 roots are appended to a per-tile list, and the labels and
+//                 bond bits of the four tile edges go to a compact seam record.
 //  k_merge        the bonds leaving a tile (the periodic wrap included,
 //                 Sec. II.C): union of the two tile roots on the
 //                 global label array with atomicMin hooking.  A lane whose

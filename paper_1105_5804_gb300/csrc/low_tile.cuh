@@ -8,7 +8,7 @@
 // the bonds of 8 or 16 sites, all its Philox calls in step, and a strip sweeps
 // 8 or 16 rows.  The seams they add cost the merge little, which is bound by
 // the latency of its walks.  A whole sweep at L = 256: 25.5 us with 32 rows, 20.2
-// with 8.  Everything but the bonds' division among the lanes is as in
+// with 8 (17.5 since the sweeps' launches overlap).  Everything but the bonds' division among the lanes is as in
 // sw_label_tile.
 #pragma once
 #include "fused_tile.cuh"
