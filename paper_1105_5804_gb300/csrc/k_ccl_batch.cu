@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(MERGE_PER_TILE) k_cclb_merge(const __grid_cons
 }
 
 template <int TH>
-__global__ void __launch_bounds__(FINAL_THREADS) k_cclb_final(const __grid_constant__ CclBatchView v) {
+__global__ void __launch_bounds__(FINAL_THREADS, FINAL_CTAS) k_cclb_final(const __grid_constant__ CclBatchView v) {
   __shared__ FinalSmem<TH> fs;
   wait_for_previous();
   const int gt = blockIdx.x;

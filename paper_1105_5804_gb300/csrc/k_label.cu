@@ -56,7 +56,7 @@ k_ccl_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid 
 }
 
 template <int TH>
-__global__ void __launch_bounds__(FINAL_THREADS)
+__global__ void __launch_bounds__(FINAL_THREADS, FINAL_CTAS)
 k_ccl_final(int32_t* labels, Grid g, LabelScratch s, int limit) {
   __shared__ FinalSmem<TH> fs;
   wait_for_previous();

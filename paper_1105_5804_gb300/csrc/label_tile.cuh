@@ -216,43 +216,69 @@ __device__ __forceinline__ void site_compress_tile(int32_t* __restrict__ labels,
 // then each edge root finds its cluster root R on the label array -- and every
 // site takes table[its tile root].  A walk compresses the entries it passes to
 // smaller ones of the same tree, so walks of other tiles stay valid.  The tile
-// roots come by cp.async while the table is filled and the edge roots walk; an
-// edge root is on the tile's perimeter, so a thread has at most three walks.
-// Labels go out as 16-byte words wherever the rows start (a row of any width,
-// shifted against the words of shared memory by up to three sites).  Bound by
-// the latency of the walks (long scoreboard).  With every tile root listed by
-// the labeling kernel and looked up here, and rows of odd width written site
-// by site, a labeling of 5003 x 7001 took 248 us instead of 181, of 4096^2 100
-// instead of 89.  All threads of the CTA call it.
-constexpr int FINAL_THREADS = 256;
-constexpr bool FINAL_STAGED = TILE_W <= 128;   // tile roots in shared memory too (with 256 columns both exceed 48 KB)
+// roots of a thread's sites wait in registers while the table is filled and the
+// edge roots walk; an edge root is on the tile's perimeter, so a thread has at
+// most five walks.  Labels go out as 16-byte words wherever the rows start (a row
+// of any width, its roots shifted by up to three sites against the words they
+// come in).  Bound by the latency of the walks, so what counts is tiles in
+// flight: ten per SM, with a thread per column and no roots in shared memory,
+// against eight of 256 threads with them: 4096^2 83.5 against 87.2 us per
+// labeling, 8192^2 290 against 303, 5003 x 7001 176 against 181 (248 with every
+// tile root listed and looked up and rows of odd width written site by site).
+// All threads of the CTA call it.
+constexpr int FINAL_THREADS = TILE_W;
+constexpr int FINAL_CTAS = 1280 / FINAL_THREADS;   // 48 registers (1536: 84.2 us at 4096^2, 1024: 86.5)
 template <int TH>
 struct FinalSmem {
   alignas(16) int32_t table[TH * TILE_W];
-  alignas(16) uint16_t roots[FINAL_STAGED ? TH * TILE_W : 8];   // tile roots, tile row-major
+  unsigned long long last[TH];             // tile roots of the rows' last four sites
   uint16_t list[2 * (TH + TILE_W)];
   int n_edge;
 };
 template <int TH>
 __device__ __forceinline__ void final_labels_tile(int32_t* labels, const Grid& g, const LabelScratch& s, int t,
                                                   FinalSmem<TH>& fs, int limit) {
+  constexpr int WORDS = TILE_W / 4, STEP = FINAL_THREADS / WORDS, PER = TH / STEP;
   const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
   const int y0 = ty * TH, x0 = tx * TILE_W;
   const int h = min(TH, g.H - y0), w = min(TILE_W, g.W - x0);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  // 1. tile roots of my sites: of the rows row0 + STEP j, the aligned word q of
+  //    four labels, whose first site is 4q less the sites that the row starts
+  //    after a word
+  const int q = threadIdx.x % WORDS, row0 = threadIdx.x / WORDS;
   const uint16_t* lr = ccl_roots<TH>(s, t);
-  if (FINAL_STAGED)
-    for (int k = threadIdx.x; k < h * (TILE_W / 8); k += FINAL_THREADS) copy16_async(fs.roots + 8 * k, lr + 8 * k);
+  auto row_at = [&](int ly) { return labels + (int64_t)(y0 + ly) * g.W + x0; };
+  auto shift_of = [&](const int32_t* row) { return (int)(reinterpret_cast<uintptr_t>(row) >> 2) & 3; };
+  const bool whole = (g.W & 3) == 0 && (reinterpret_cast<uintptr_t>(labels) & 15) == 0;   // every row starts on a word
+  unsigned long long roots[PER];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int ly = row0 + STEP * j;
+    roots[j] = ly < h && 4 * q < w ? reinterpret_cast<const unsigned long long*>(lr + ly * TILE_W)[q] : 0ull;
+  }
+  if (!whole) {
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int ly = row0 + STEP * j;
+      if (q == WORDS - 1) fs.last[ly] = roots[j];
+      unsigned long long before = __shfl_up_sync(FULL, roots[j], 1);
+      if (WORDS > 32 && lane == 0 && q > 0 && ly < h && 4 * (q - 1) < w)
+        before = reinterpret_cast<const unsigned long long*>(lr + ly * TILE_W)[q - 1];
+      const int shift = shift_of(row_at(ly));
+      if (shift) roots[j] = roots[j] << (16 * shift) | before >> (64 - 16 * shift);
+    }
+  }
   uint32_t edge = 0u;
   if (threadIdx.x < TH * TILE_W / 32) edge = (uint32_t)__ldcg(ccl_edges<TH>(s, t) + threadIdx.x);
   if (threadIdx.x == 0) fs.n_edge = 0;
-  // 1. the table: own global indices
-  for (int k = threadIdx.x; k < h * (TILE_W / 4); k += FINAL_THREADS) {
+  // 2. the table: own global indices
+  for (int k = threadIdx.x; k < h * WORDS; k += FINAL_THREADS) {
     const int G = tile_global(4 * k, y0, x0, g.W);   // four local indices of a strip are four sites in a row
     *reinterpret_cast<int4*>(fs.table + 4 * k) = make_int4(G, G + 1, G + 2, G + 3);
   }
   __syncthreads();
-  // 2. edge roots listed, then their cluster roots
+  // 3. edge roots listed, then their cluster roots
   {
     const int cnt = __popc(edge);
     int incl = cnt;
@@ -271,29 +297,24 @@ __device__ __forceinline__ void final_labels_tile(int32_t* labels, const Grid& g
     const int r = fs.list[k];
     fs.table[r] = g_find(labels, fs.table[r], limit, s.err);
   }
-  copies_wait();
   __syncthreads();
-  // 3. every site takes its tile root's label: a warp per row, a lane per
-  //    aligned word of four labels
-  for (int ly = warp; ly < h; ly += FINAL_THREADS / 32) {
-    int32_t* row = labels + (int64_t)(y0 + ly) * g.W + x0;
-    const int shift = (int)(reinterpret_cast<uintptr_t>(row) >> 2) & 3;   // sites of the first word before the row
-    const uint16_t* rr = (FINAL_STAGED ? fs.roots : lr) + ly * TILE_W;
-    for (int q = lane; 4 * q < w + shift; q += 32) {
-      const int lx = 4 * q - shift;
-      if (lx >= 0 && lx + 4 <= w) {
-        int4 v;
-        if (shift == 0) {
-          const uint2 r = *reinterpret_cast<const uint2*>(rr + lx);
-          v = make_int4(fs.table[r.x & 0xFFFFu], fs.table[r.x >> 16], fs.table[r.y & 0xFFFFu], fs.table[r.y >> 16]);
-        } else {
-          v = make_int4(fs.table[rr[lx]], fs.table[rr[lx + 1]], fs.table[rr[lx + 2]], fs.table[rr[lx + 3]]);
-        }
-        *reinterpret_cast<int4*>(row + lx) = v;
-      } else {
-        for (int i = max(lx, 0); i < min(lx + 4, w); ++i) row[i] = fs.table[rr[i]];
-      }
+  // 4. every site takes its tile root's label
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int ly = row0 + STEP * j;
+    if (ly >= h) break;
+    int32_t* row = row_at(ly);
+    auto label = [&](int i) { return fs.table[(int)(roots[j] >> (16 * i)) & 0xFFFF]; };
+    const int shift = whole ? 0 : shift_of(row), lx = 4 * q - shift;
+    if (lx >= 0 && lx + 4 <= w) {
+      *reinterpret_cast<int4*>(row + lx) = make_int4(label(0), label(1), label(2), label(3));
+    } else if (!whole) {   // else w is a multiple of 4 too
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (lx + i >= 0 && lx + i < w) row[lx + i] = label(i);
     }
+    if (!whole && q == WORDS - 1)   // the word after the tile's last one
+      for (int i = TILE_W - shift; i < w; ++i) row[i] = fs.table[(int)(fs.last[ly] >> (16 * (i & 3))) & 0xFFFF];
   }
 }
 
