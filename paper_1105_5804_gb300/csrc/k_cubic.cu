@@ -127,15 +127,18 @@ __device__ __forceinline__ uint32_t eq_row(const uint32_t (&a)[4], const uint32_
 }
 
 // Local step of a brick.  Bound by instruction issue and by the latency of the
-// shared-memory walks: 16 draws per thread (about 45 instructions each, 18 % of
-// a warp's time), the engine (17 %), the +y joins (22 %), so eight CTAs per SM
+// shared-memory walks: 16 draws per thread (about 45 instructions each), the
+// engine and the +y joins take most of a warp's time, so eight CTAs per SM
 // (32 registers) beat six.  A lane has half a row: its spins and those at +y and
-// +z are three 16-byte loads (the neighbours' from L1), compared four per word,
-// and the bond bits are row words already.  With a thread per column (byte
-// loads, neighbours' spins through shared memory, bit-matrix transposes) and
-// the +y joins in three rounds between disjoint planes (plain stores, but one to
-// four warps of eight busy): 185 us at 256^3 and six CTAs, 172 with joins by
-// compare-and-swap all at once, 159 with rows, 153 with eight CTAs.
+// +z are three 16-byte loads (the neighbours' from L1), Ising spins packed one
+// bit per site, others compared four per word, and the bond bits are row words
+// already.  256^3, us: 185 with a thread per column (byte loads, neighbours' spins
+// through shared memory, bit-matrix transposes), six CTAs and the +y joins in
+// three rounds between disjoint planes (plain stores, but one to four warps of
+// eight busy); 172 with joins by compare-and-swap all at once, 159 with rows, 153
+// with eight CTAs, 142 with packed spins, 131 with the face roots looked up a lane
+// per face site (before: by the sites' owners, a few lanes per warp) and parent
+// entries written from the edge bits.
 __global__ void __launch_bounds__(B3_THREADS, 8)
 k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t* __restrict__ gpar,
          uint32_t* __restrict__ words, Box3 b, int q, uint64_t T, const __grid_constant__ PhiloxKeys keys,
@@ -170,24 +173,42 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
     load_row(spins, site0 + (z + 1 == b.Z ? -(uint32_t)z : 1u) * ((uint32_t)b.X * (uint32_t)b.Y), nv, whole, nz);
     const uint32_t next = nv > 0 ? (uint32_t)(uint8_t)spins[x1 == b.X ? row0 - k.x0 : row0 - k.x0 + x1] : 0u;
     const uint32_t mine = (1u << nv) - 1u;
+    uint32_t ones = 0u;
+    if (q == 2) {   // bytes 0 or 1, packed one bit per site
+      auto pack = [](const uint32_t (&v)[4]) {
+        return (v[0] * 0x01020408u) >> 24 | (v[1] * 0x01020408u) >> 24 << 4 | (v[2] * 0x01020408u) >> 24 << 8 |
+               (v[3] * 0x01020408u) >> 24 << 12;
+      };
+      ones = pack(c) & mine;
+      ex = ~(ones ^ ((ones | next << nv) >> 1)) & mine;
+      ey = ~(ones ^ pack(ny)) & mine;
+      ez = ~(ones ^ pack(nz)) & mine;
+    } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      n[j] = __funnelshift_r(c[j], j < 3 ? c[j + 1] : next, 8);
-      if (nv < 16 && (nv - 1) >> 2 == j) {
-        const int sh = 8 * ((nv - 1) & 3);
-        n[j] = (n[j] & ~(0xFFu << sh)) | next << sh;
+      for (int j = 0; j < 4; ++j) {
+        n[j] = __funnelshift_r(c[j], j < 3 ? c[j + 1] : next, 8);
+        if (nv < 16 && (nv - 1) >> 2 == j) {
+          const int sh = 8 * ((nv - 1) & 3);
+          n[j] = (n[j] & ~(0xFFu << sh)) | next << sh;
+        }
       }
+      ex = eq_row(c, n) & mine;
+      ey = eq_row(c, ny) & mine;
+      ez = eq_row(c, nz) & mine;
     }
-    ex = eq_row(c, n) & mine;
-    ey = eq_row(c, ny) & mine;
-    ez = eq_row(c, nz) & mine;
     if (do_obs) {
-      int cnt[QREG];
+      int cnt[QREG] = {};
+      if (q == 2) {
+        cnt[1] = __popc(ones);
+        cnt[0] = nv - cnt[1];
+      } else if (q <= QREG) {
 #pragma unroll
-      for (int s = 0; s < QREG; ++s) {
-        const uint32_t same = 0x01010101u * (uint32_t)s;
-        const uint32_t v[4] = {same, same, same, same};
-        cnt[s] = s < q && q <= QREG ? __popc(eq_row(c, v) & mine) : 0;
+        for (int s = 0; s < QREG; ++s) {
+          if (s >= q) break;
+          const uint32_t same = 0x01010101u * (uint32_t)s;
+          const uint32_t v[4] = {same, same, same, same};
+          cnt[s] = __popc(eq_row(c, v) & mine);
+        }
       }
       if (q > QREG) {
         __syncthreads();   // the histogram is cleared
@@ -353,29 +374,21 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
 
   // 7. brick roots of my plane's sites (site -> its plane's node -> that
   //    node's plane root -> the brick root), eight consecutive sites per
-  //    thread and step; roots on the brick's faces marked; bit 4j + i of mine
-  //    flags site 2i of step j as a root, bit 16 + 4j + i site 2i + 1
+  //    thread and step
   const int lx0 = 8 * (lane & 3);
   const int in = plane ? min(max(k.w - lx0, 0), 8) : 0;
-  uint32_t mine = 0;
   if (in > 0) {
-    const uint32_t in_mask = ((1u << ((in + 1) >> 1)) - 1u) | ((1u << (in >> 1)) - 1u) << 16;
-    auto mark = [&](uint32_t r) {
-      const uint32_t bit = 1u << (r & 31);
-      if (!(*reinterpret_cast<volatile uint32_t*>(&ls.edge[r >> 5]) & bit)) atomicOr(&ls.edge[r >> 5], bit);
-    };
 #pragma unroll
     for (int j = 0; j < B3Z / 8; ++j) {
-      const int lz = (lane >> 2) + 8 * j;
-      if (lz >= k.d) continue;
-      const int l0 = brick_local(lx0, ly, lz);
-      const uint4 v = *reinterpret_cast<const uint4*>(par + l0);
+      const int z = (lane >> 2) + 8 * j;
+      if (z >= k.d) continue;
+      const uint4 v = *reinterpret_cast<const uint4*>(par + brick_local(lx0, ly, z));
       auto two = [&](uint32_t w) {
         const int p0 = sm_at(par, w & 0xFFFFu), p1 = sm_at(par, w >> 16);
         return (uint32_t)sm_at(par, p0) >> 1 | (uint32_t)sm_at(par, p1) << 15;
       };
       const uint32_t wv[4] = {two(v.x), two(v.y), two(v.z), two(v.w)};
-      uint16_t* dst = lroot + site3(b, k.x0 + lx0, k.y0 + ly, k.z0 + lz);
+      uint16_t* dst = lroot + site3(b, k.x0 + lx0, k.y0 + ly, k.z0 + z);
       if ((b.X & 7) == 0) {   // then k.w is a multiple of 8 too
         *reinterpret_cast<uint4*>(dst) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
       } else {
@@ -383,29 +396,35 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
         for (int i = 0; i < 8; ++i)
           if (i < in) dst[i] = (uint16_t)(wv[i >> 1] >> (16 * (i & 1)));
       }
-      const uint32_t own = (uint32_t)l0 * 0x00010001u + 0x00010000u;   // (l0, l0 + 1)
-      uint32_t m = 0;
+    }
+  }
+  // 8. roots on the brick's faces marked, a lane per site: rows ly and ly + 8 of
+  //    the first and the last plane, the first and last row of my plane, its
+  //    first and last column (16 lanes each); of a run of equal roots the first
+  //    lane marks.  The lookups go in step.
+  {
+    constexpr int N = 7;
+    const int z_of[N] = {ly, ly + 8, ly, ly + 8, 0, k.d - 1, lane & 15};
+    const int y_of[N] = {0, 0, k.h - 1, k.h - 1, ly, ly, ly};
+    int r[N];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) m |= zero_halves(wv[i] ^ (own + (uint32_t)i * 0x00020002u)) >> (15 - i);
-      mine |= (m & in_mask) << (4 * j);
-      if (ly == 0 || y_last || lz == 0 || lz == k.d - 1) {
-        uint32_t left = 0xFFFFFFFFu;
+    for (int u = 0; u < N; ++u) {
+      const int x = u < N - 1 ? lane : lane < 16 ? 0 : k.w - 1;
+      const bool ok = x < k.w && z_of[u] < k.d && (u < 4 || plane);
+      r[u] = ok ? 2 * brick_local(x, y_of[u], z_of[u]) : -1;
+    }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const uint32_t r = (wv[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
-          if (i < in && r != left) mark(r);
-          left = r;
-        }
-      } else {
-        if (lx0 == 0) mark(wv[0] & 0xFFFFu);
-        if (lx0 + in == k.w) {
-          uint32_t last = wv[0];
+    for (int hop = 0; hop < 3; ++hop)   // site -> node -> plane root -> brick root
 #pragma unroll
-          for (int i = 1; i < 4; ++i)
-            if (2 * i < in) last = wv[i];
-          mark((last >> (16 * ((in - 1) & 1))) & 0xFFFFu);
-        }
-      }
+      for (int u = 0; u < N; ++u)
+        if (r[u] >= 0) r[u] = sm_at(par, r[u]);
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      const int left = __shfl_up_sync(FULL, r[u], 1);
+      const uint32_t bit = 1u << ((r[u] >> 1) & 31);
+      uint32_t* word = &ls.edge[r[u] >= 0 ? r[u] >> 6 : 0];
+      if (r[u] >= 0 && (lane == 0 || left != r[u]) && !(*reinterpret_cast<volatile uint32_t*>(word) & bit))
+        atomicOr(word, bit);
     }
   }
   if (do_obs) {
@@ -414,14 +433,15 @@ k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t
     observables_commit<B3_THREADS>(q, q <= QREG ? q : 0, oslot, ls.red, ls.hist);
   }
   __syncthreads();
-  // 8. parent entries of edge roots; the brick's edge bits for the flip
-  while (mine) {
-    const int bit = __ffs(mine) - 1;
-    mine &= mine - 1;
-    const int jk = bit & 15;
-    const int l = brick_local(lx0, ly, (lane >> 2) + 8 * (jk >> 2)) + 2 * (jk & 3) + (bit >> 4);
-    if ((ls.edge[l >> 5] >> (l & 31)) & 1u) {
-      const int32_t G = (int32_t)brick_global(b, k, l);
+  // 9. parent entries of edge roots, each by the owner of its site; the brick's
+  //    edge bits for the flip
+  if (in > 0) {
+    const uint8_t* eb = reinterpret_cast<const uint8_t*>(ls.edge) + (brick_local(lx0, ly, lane >> 2) >> 3);
+    const int32_t G0 = (int32_t)site3(b, k.x0 + lx0, k.y0 + ly, k.z0 + (lane >> 2));
+    static_assert(B3Z == 16, "two steps of eight rows");
+    for (uint32_t bits = eb[0] | (uint32_t)eb[TILE_W] << 8; bits; bits &= bits - 1) {
+      const int i = high_bit(bits & -bits);
+      const int32_t G = G0 + (i & 7) + (i & 8) * b.X * b.Y;
       gpar[G] = G;
     }
   }
