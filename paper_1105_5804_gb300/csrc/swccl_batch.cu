@@ -37,6 +37,7 @@ struct sw_batch {
   int* d_tile_rep = nullptr;
   BatchCtl* ctl = nullptr;
   std::vector<SwRep> reps;
+  std::vector<char> tables;       // host image of the tables at the start of the arena
   BatchView view{};
   LowBatch low{};                 // lower tiles for the phase schedule, if the batch has few
   int schedule = SW_BATCH_PHASES;
@@ -232,8 +233,11 @@ sw_batch* create_batch(int n, const int* L, const int* q, const double* beta, co
   int* err = reinterpret_cast<int*>(reinterpret_cast<char*>(b->ctl) + offsetof(BatchCtl, err));
   // the tables (control block, chains, tile map) lie together at the start of the
   // arena: one copy brings them, one kernel sets up every chain from them (eight
-  // chains of a served group: two calls where there were nineteen)
-  std::vector<char> tables(lay.chain[0], 0);
+  // chains of a served group: two calls where there were nineteen).  The copy is
+  // from pageable memory and nobody waits for it here, so the batch keeps the
+  // image: the runtime need not have read it when cudaMemcpyAsync returns.
+  std::vector<char>& tables = b->tables;
+  tables.assign(lay.chain[0], 0);
   static const BatchCtl init_ctl = {0ull, -1ll, 0, 0u, 0u, 0};
   memcpy(tables.data() + lay.ctl, &init_ctl, sizeof(BatchCtl));
   int* tile_rep = reinterpret_cast<int*>(tables.data() + lay.tile_rep);
@@ -275,8 +279,6 @@ sw_batch* create_batch(int n, const int* L, const int* q, const double* beta, co
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->blocks = std::max(1, batch_persistent_blocks_per_sm()) * std::max(1, sms);
-  // the host tables above are copied from pageable memory: the copy is
-  // staged before cudaMemcpyAsync returns, so no wait is needed here
   return b;
 }
 
