@@ -39,20 +39,20 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "d6bd4182c90a954a"
+SWEEP_COUNTER_HASH = "2a018925f18a42f6"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
-    "k_sw_label": ((88.904192 + 130.759680) * 1e6 / 67108864, 184289152 / 67108864),
-    "k_merge": ((56.311296 + 0.752896) * 1e6 / 67108864, 14601833 / 67108864),
-    "k_sw_flip": ((203.559168 + 48.247552) * 1e6 / 67108864, 71110591 / 67108864),
+    "k_sw_label": ((88.849408 + 130.423296) * 1e6 / 67108864, 184289423 / 67108864),
+    "k_merge": ((56.291072 + 0.763392) * 1e6 / 67108864, 14599000 / 67108864),
+    "k_sw_flip": ((203.587072 + 47.656448) * 1e6 / 67108864, 71101877 / 67108864),
 }
 # The stand-alone labeling call (k_ccl_tile, k_merge, k_ccl_final), one ncu
 # capture per kernel of a 4096^2 critical percolation mask: DRAM bytes per site,
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "659e35c098ba7572"
+CCL_COUNTER_HASH = "f1396811bb2420ef"
 CCL_COUNTER_TILE_W = 128
-CCL_TRAFFIC_BYTES_PER_SITE = ((6.701568 + 2.637824) + (16.643072 + 0.000000) + (53.529344 + 10.402304)) * 1e6 / 16777216
+CCL_TRAFFIC_BYTES_PER_SITE = ((6.649600 + 2.546176) + (16.568832 + 0.000000) + (53.476608 + 10.269184)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8
 # spins once (2 B, the minimum of any sweep); the kernel split adds the
 # 16-bit tile roots written by k_sw_label and read by k_sw_flip (6 B).

@@ -20,7 +20,7 @@ struct RowEqual {
   int cnt[QREG_MAX];        // sites per state (q <= 8)
 };
 
-__device__ __forceinline__ void row_equal(const int8_t* __restrict__ spins, int L, int y, int x, int nvalid, int q,
+__device__ __forceinline__ void row_equal(const int8_t* spins, int L, int y, int x, int nvalid, int q,
                                           RowEqual& rb) {
   const int yn = (y + 1 == L) ? 0 : y + 1;
   const int64_t row = (int64_t)y * L, rown = (int64_t)yn * L;
@@ -234,9 +234,9 @@ __device__ __forceinline__ void sw_label_tile(const SwRep& R, int t, uint64_t sw
   TileSmem& sm = ls.tile;
   unsigned* red = reinterpret_cast<unsigned*>(ls.red);
   int* hist = ls.hist;
-  const int8_t* __restrict__ spins = R.spins;
-  uint16_t* __restrict__ lroot = R.lroot;
-  int32_t* __restrict__ gpar = R.gpar;
+  const int8_t* spins = R.spins;
+  uint16_t* lroot = R.lroot;
+  int32_t* gpar = R.gpar;
   const Grid& g = R.g;
   const LabelScratch& s = R.s;
   const int q = R.q;
@@ -362,8 +362,8 @@ __device__ __forceinline__ void sw_flip_tile(const SwRep& R, int t, uint64_t swe
                                              const Keys& keys) {
   constexpr int PASSES = TH / 8, FLIP_LIST = FlipTileSmemT<TH>::LIST;
   uint8_t* ns = fs.ns;
-  int8_t* __restrict__ spins = R.spins;
-  int32_t* __restrict__ gpar = R.gpar;
+  int8_t* spins = R.spins;
+  int32_t* gpar = R.gpar;
   const int q = R.q;
   int* err = R.s.err;
   const int L = R.g.W;
@@ -549,10 +549,10 @@ struct FewFlipSmem {
 
 template <int TH, class Keys>
 __device__ __forceinline__ void sw_flip_few_tile(const SwRep& R, int t, uint64_t sweep, int limit, FewFlipSmem<TH>& fs,
-                                                 const Keys& keys, const uint32_t* __restrict__ sel, uint64_t P) {
+                                                 const Keys& keys, const uint32_t* sel, uint64_t P) {
   constexpr int LIST = FewFlipSmem<TH>::LIST, WORDS = TH * TILE_W / 32;
-  int8_t* __restrict__ spins = R.spins;
-  int32_t* __restrict__ gpar = R.gpar;
+  int8_t* spins = R.spins;
+  int32_t* gpar = R.gpar;
   const int q = R.q, L = R.g.W;
   int* err = R.s.err;
   const int ty = t / R.g.tiles_x, tx = t - ty * R.g.tiles_x;
@@ -611,7 +611,7 @@ __device__ __forceinline__ void sw_flip_few_tile(const SwRep& R, int t, uint64_t
       int G = tile_global(r, y0, x0, L);
       if (k < ne) {
         G = g_find(gpar, G, limit, err);
-        if (!((__ldg(sel + (G >> 5)) >> (G & 31)) & 1u)) continue;
+        if (!((sel[G >> 5] >> (G & 31)) & 1u)) continue;
       }
       const uint4 d = philox_draw(make_uint4((uint32_t)G, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_FLIP), keys);
       if ((uint64_t)d.y < P) {

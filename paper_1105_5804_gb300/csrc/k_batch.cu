@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(LABEL_THREADS) k_batch_init(BatchView b, int h
 
 // ---------------------------------------------------------------------------
 // Phase kernels: one CTA per global tile (merge: per few tiles).
-__global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_batch_label(BatchView b, const BatchCtl* __restrict__ ctl) {
+__global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM) k_batch_label(BatchView b, const BatchCtl* ctl) {
   __shared__ LabelTileSmem ls;
   wait_for_previous();
   const uint64_t sweep = ctl->sweep;
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(MERGE_PER_TILE) k_batch_merge(BatchView b, Bat
               b.limit);
 }
 
-__global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM) k_batch_flip(BatchView b, const BatchCtl* __restrict__ ctl) {
+__global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM) k_batch_flip(BatchView b, const BatchCtl* ctl) {
   __shared__ FlipTileSmem fs;
   wait_for_previous();
   const int gt = blockIdx.x;
@@ -156,7 +156,7 @@ __device__ __forceinline__ LowChain low_chain(const BatchView& b, const LowBatch
 
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS)
-k_batch_label_low(BatchView b, const __grid_constant__ LowBatch low, const BatchCtl* __restrict__ ctl) {
+k_batch_label_low(BatchView b, const __grid_constant__ LowBatch low, const BatchCtl* ctl) {
   __shared__ LowTileSmem<TH> ls;
   const LowChain c = low_chain<TH>(b, low, blockIdx.x);   // tables: not written by the kernels ahead
   wait_for_previous();
@@ -177,7 +177,7 @@ k_batch_merge_low(BatchView b, const __grid_constant__ LowBatch low, BatchCtl* c
 
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS)
-k_batch_flip_low(BatchView b, const __grid_constant__ LowBatch low, const BatchCtl* __restrict__ ctl) {
+k_batch_flip_low(BatchView b, const __grid_constant__ LowBatch low, const BatchCtl* ctl) {
   __shared__ FlipTileSmemT<TH> fs;
   const LowChain c = low_chain<TH>(b, low, blockIdx.x);
   wait_for_previous();

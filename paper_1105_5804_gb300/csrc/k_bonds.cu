@@ -110,7 +110,7 @@ cudaError_t launch_perc_mask(uint8_t* mask, int H, int W, uint64_t k, cudaStream
 
 // ---------------------------------------------------------------------------
 // Mask byte b of the image: four sites, one by one.
-__device__ __forceinline__ uint32_t pixel_bond_byte(const uint8_t* __restrict__ px, int64_t b, int H, int W, int periodic) {
+__device__ __forceinline__ uint32_t pixel_bond_byte(const uint8_t* px, int64_t b, int H, int W, int periodic) {
   const int64_t n = (int64_t)H * W;
   uint32_t out = 0;
 #pragma unroll
@@ -138,7 +138,7 @@ __device__ __forceinline__ uint32_t pixel_bond_byte(const uint8_t* __restrict__ 
 constexpr int PIXEL_THREADS = 256;
 
 __global__ void __launch_bounds__(PIXEL_THREADS)
-k_pixel_bonds(const uint8_t* __restrict__ px, uint8_t* __restrict__ mask, int H, int W, int periodic, int aligned) {
+k_pixel_bonds(const uint8_t* px, uint8_t* mask, int H, int W, int periodic, int aligned) {
   wait_for_previous();
   const uint32_t n = (uint32_t)H * (uint32_t)W;   // < 2^31
   const uint32_t t = blockIdx.x * (uint32_t)PIXEL_THREADS + threadIdx.x, i0 = 16u * t;

@@ -102,7 +102,7 @@ struct Local3Smem {
 // (the others are arbitrary).  whole: rows start 16-byte aligned and nv is 0 or
 // 16; otherwise aligned words are shifted into place (a word is read only if it
 // holds a wanted spin, so reads stay inside the array's last word).
-__device__ __forceinline__ void load_row(const int8_t* __restrict__ spins, uint32_t i, int nv, bool whole,
+__device__ __forceinline__ void load_row(const int8_t* spins, uint32_t i, int nv, bool whole,
                                          uint32_t (&c)[4]) {
   if (whole) {
     const uint4 v = nv > 0 ? *reinterpret_cast<const uint4*>(spins + i) : make_uint4(0u, 0u, 0u, 0u);
@@ -140,9 +140,8 @@ __device__ __forceinline__ uint32_t eq_row(const uint32_t (&a)[4], const uint32_
 // per face site (before: by the sites' owners, a few lanes per warp) and parent
 // entries written from the edge bits.
 __global__ void __launch_bounds__(B3_THREADS, 8)
-k3_local(const int8_t* __restrict__ spins, uint16_t* __restrict__ lroot, int32_t* __restrict__ gpar,
-         uint32_t* __restrict__ words, Box3 b, int q, uint64_t T, const __grid_constant__ PhiloxKeys keys,
-         const SwCtl* __restrict__ ctl, int64_t* obs, int obs_cap, int* err) {
+k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, Box3 b, int q, uint64_t T,
+         const __grid_constant__ PhiloxKeys keys, const SwCtl* ctl, int64_t* obs, int obs_cap, int* err) {
   __shared__ Local3Smem ls;
   TileSmemT<B3Z>& sm = ls.tile;
   uint16_t* par = sm.par;
@@ -459,7 +458,7 @@ constexpr int B3_MERGE_UNITS = B3Y + B3Z + B3Y / 2;
 constexpr int MERGE3_THREADS = 256;
 
 __global__ void __launch_bounds__(MERGE3_THREADS)
-k3_merge(const uint16_t* __restrict__ lroot, int32_t* gpar, const uint32_t* __restrict__ words, Box3 b, int limit,
+k3_merge(const uint16_t* lroot, int32_t* gpar, const uint32_t* words, Box3 b, int limit,
          SwCtl* ctl, int64_t* obs, int obs_cap, int q) {
   constexpr int WARPS = MERGE3_THREADS / 32, UNITS = (B3_MERGE_UNITS + WARPS - 1) / WARPS;
   __shared__ int2 pairs[B3_MERGE_UNITS * 32];
@@ -529,9 +528,9 @@ k3_merge(const uint16_t* __restrict__ lroot, int32_t* gpar, const uint32_t* __re
 // are in flight while the interior roots are drawn.  256^3: 54 us against 71 with
 // flags looked up root by root and walks and draws in turn.
 __global__ void __launch_bounds__(B3_THREADS, 6)
-k3_flip(int8_t* __restrict__ spins, const uint16_t* __restrict__ lroot, int32_t* gpar,
-        const uint32_t* __restrict__ words, Box3 b, int q, const __grid_constant__ PhiloxKeys keys,
-        const SwCtl* __restrict__ ctl, int limit, int* err) {
+k3_flip(int8_t* spins, const uint16_t* lroot, int32_t* gpar,
+        const uint32_t* words, Box3 b, int q, const __grid_constant__ PhiloxKeys keys,
+        const SwCtl* ctl, int limit, int* err) {
   __shared__ uint16_t rlist[B3_SITES];
   __shared__ uint8_t ns[B3_SITES];
   __shared__ int warp_cnt[B3_THREADS / 32];

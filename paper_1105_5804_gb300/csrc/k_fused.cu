@@ -48,7 +48,7 @@ __device__ __forceinline__ void clear_bits(const ClearBits& c) {
 
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
-k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys, ClearBits clear) {
+k_sw_label(SwRep R, const SwCtl* ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys, ClearBits clear) {
   __shared__ LabelTileSmem ls;
   wait_for_previous();
   clear_bits(clear);
@@ -60,7 +60,7 @@ k_sw_label(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_con
 // The same for a lattice cut into low tiles.
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS)
-k_sw_label_low(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys,
+k_sw_label_low(SwRep R, const SwCtl* ctl, int obs_cap, const __grid_constant__ PhiloxKeys keys,
                ClearBits clear) {
   __shared__ LowTileSmem<TH> ls;
   wait_for_previous();
@@ -73,7 +73,7 @@ k_sw_label_low(SwRep R, const SwCtl* __restrict__ ctl, int obs_cap, const __grid
 // The merge has advanced the counter.
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
-k_sw_flip(SwRep R, const SwCtl* __restrict__ ctl, int limit, const __grid_constant__ PhiloxKeys keys) {
+k_sw_flip(SwRep R, const SwCtl* ctl, int limit, const __grid_constant__ PhiloxKeys keys) {
   __shared__ FlipTileSmemT<TH> fs;
   wait_for_previous();
   sw_flip_tile<TH>(R, blockIdx.x, ctl->sweep - 1, limit, fs, keys);
@@ -81,7 +81,7 @@ k_sw_flip(SwRep R, const SwCtl* __restrict__ ctl, int limit, const __grid_consta
 
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, FLIP_CTAS_PER_SM)
-k_sw_flip_few(SwRep R, const SwCtl* __restrict__ ctl, int limit, const uint32_t* __restrict__ sel, uint64_t P,
+k_sw_flip_few(SwRep R, const SwCtl* ctl, int limit, const uint32_t* sel, uint64_t P,
               const __grid_constant__ PhiloxKeys keys) {
   __shared__ FewFlipSmem<TH> fs;
   wait_for_previous();
@@ -91,7 +91,7 @@ k_sw_flip_few(SwRep R, const SwCtl* __restrict__ ctl, int limit, const uint32_t*
 constexpr int SELECT_THREADS = 256;
 
 __global__ void __launch_bounds__(SELECT_THREADS)
-k_few_select(SwRep R, const SwCtl* __restrict__ ctl, int ell, uint32_t* sel, int limit) {
+k_few_select(SwRep R, const SwCtl* ctl, int ell, uint32_t* sel, int limit) {
   const int64_t b = blockIdx.x * (int64_t)SELECT_THREADS + threadIdx.x;   // one thread per seed
   wait_for_previous();
   if (b < (int64_t)ell * ell) few_select_seed(R, ell, b, ctl->sweep - 1, sel, limit);

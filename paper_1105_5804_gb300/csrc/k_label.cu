@@ -49,7 +49,7 @@ cudaError_t launch_tile_label(const uint8_t* mask, int32_t* labels, const Grid& 
 // the seam merge) the final labels of every tile in one pass.
 template <int TH>
 __global__ void __launch_bounds__(LABEL_THREADS, LABEL_CTAS_PER_SM)
-k_ccl_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels, Grid g, LabelScratch s) {
+k_ccl_tile(const uint8_t* mask, int32_t* labels, Grid g, LabelScratch s) {
   __shared__ CclTileSmemT<TH> sm;
   wait_for_previous();
   ccl_label_tile<true, TH>(mask, labels, g, s, blockIdx.x, sm);
@@ -84,7 +84,7 @@ int ccl_tile_rows(int64_t tiles8, int64_t tiles16) { return low_tile_rows(tiles8
 // Seam merge: one CTA per `per` consecutive tiles (merge_tiles).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(MERGE_PER_TILE)
-k_merge(int32_t* __restrict__ labels, const __grid_constant__ Grid g, LabelScratch s, int per, int limit, SwCtl* adv,
+k_merge(int32_t* labels, const __grid_constant__ Grid g, LabelScratch s, int per, int limit, SwCtl* adv,
         int64_t* obs, int obs_cap, int q) {
   __shared__ MergeSmem ms;
   wait_for_previous();

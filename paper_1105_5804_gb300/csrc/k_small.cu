@@ -67,8 +67,8 @@ static_assert(((SMALL_L + 31) / 32) * ((SMALL_L + 15) / 16) <= SMALL_UNITS, "one
 // ISING: q = 2, spins packed one bit per site.
 template <bool ISING, int SMALL_H>
 __global__ void __launch_bounds__(32 * SMALL_UNITS)
-k_sw_small(int8_t* __restrict__ spins_g, int L, int q, uint64_t T, const __grid_constant__ PhiloxKeys keys,
-           SwCtl* __restrict__ ctl, int64_t* __restrict__ obs, int obs_cap, int n) {
+k_sw_small(int8_t* spins_g, int L, int q, uint64_t T, const __grid_constant__ PhiloxKeys keys,
+           SwCtl* ctl, int64_t* obs, int obs_cap, int n) {
   extern __shared__ __align__(16) unsigned char small_smem[];
   SmallSmem& ss = *reinterpret_cast<SmallSmem*>(small_smem);
   uint16_t* par = reinterpret_cast<uint16_t*>(small_smem + sizeof(SmallSmem));

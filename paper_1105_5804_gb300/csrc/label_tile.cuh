@@ -24,7 +24,7 @@ __device__ __forceinline__ uint32_t even_bits(unsigned long long x) {
 // sites start on a 32-site word; else three 32-bit words shifted into place
 // (rows of any width start anywhere in a byte); single bytes only for a mask
 // that is not 4-byte aligned and in its last word.
-__device__ __forceinline__ unsigned long long mask_word(const uint8_t* __restrict__ mask, int64_t n_bytes,
+__device__ __forceinline__ unsigned long long mask_word(const uint8_t* mask, int64_t n_bytes,
                                                         int64_t site0, int nvalid) {
   const int64_t b0 = site0 >> 2;
   unsigned long long wd = 0ull;
@@ -79,7 +79,7 @@ using CclTileSmem = CclTileSmemT<TILE_H>;
 static_assert(TILE_SITES / 32 == LABEL_THREADS, "at most one edge word per thread");
 
 template <bool LOCAL = false, int TH = TILE_H>
-__device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask, int32_t* __restrict__ labels,
+__device__ __forceinline__ void ccl_label_tile(const uint8_t* mask, int32_t* labels,
                                                const Grid& g, const LabelScratch& s, int t, CclTileSmemT<TH>& cs) {
   TileSmemT<TH>& sm = cs.tile;
   const uint16_t* par = sm.par;
@@ -179,8 +179,8 @@ __device__ __forceinline__ void ccl_label_tile(const uint8_t* __restrict__ mask,
 
 // Tile t's roots: label = final root; in a Swendsen-Wang sweep (spins set)
 // final roots also draw their cluster's new state.  All threads call it.
-__device__ __forceinline__ void root_compress_tile(int32_t* __restrict__ labels, const LabelScratch& s, int t,
-                                                   int8_t* __restrict__ spins, int q, uint64_t seed, uint64_t sweep,
+__device__ __forceinline__ void root_compress_tile(int32_t* labels, const LabelScratch& s, int t,
+                                                   int8_t* spins, int q, uint64_t seed, uint64_t sweep,
                                                    int limit) {
   const int n = __ldcg(s.root_counts + t);
   const int32_t* list = s.roots + (int64_t)t * TILE_SITES;
@@ -195,7 +195,7 @@ __device__ __forceinline__ void root_compress_tile(int32_t* __restrict__ labels,
 // Site pass of tile t: every label of the tile points at a tile root whose
 // entry holds the final root after root compression; one jump makes the
 // label canonical.
-__device__ __forceinline__ void site_compress_tile(int32_t* __restrict__ labels, const Grid& g, int t) {
+__device__ __forceinline__ void site_compress_tile(int32_t* labels, const Grid& g, int t) {
   const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
   const int y0 = ty * TILE_H, x0 = tx * TILE_W;
   const int h = min(TILE_H, g.H - y0), w = min(TILE_W, g.W - x0);

@@ -28,7 +28,7 @@ __device__ __forceinline__ void sw_label_low_tile(const SwRep& R, int t, uint64_
                                                   LowTileSmem<TH>& ls, const Keys& keys) {
   constexpr int SP = TH;                 // 32 / TH lanes per row, SP sites per lane
   constexpr int NW = LABEL_THREADS / 32;
-  const int8_t* __restrict__ spins = R.spins;
+  const int8_t* spins = R.spins;
   const int q = R.q;
   const uint64_t T = R.T;
   const int L = R.g.W;

@@ -18,7 +18,11 @@ namespace swccl {
 // launched before the kernels ahead of it in the stream have ended, so that its
 // launch overlaps them.  Every thread of such a kernel calls wait_for_previous
 // first: it returns when the kernels ahead have completed and their writes are
-// visible (at once in a kernel launched plainly).  A sweep at L = 256 took 25.0
+// visible (at once in a kernel launched plainly).  Such a kernel, and the bodies
+// it inlines, read what a kernel ahead of them may write through plain pointers
+// or __ldcg: __restrict__ on a pointer that is only read, and __ldg, promise that
+// the data does not change while the kernel runs and allow a read-only load
+// ahead of the wait.  A sweep at L = 256 took 25.0
 // us instead of 27.4 with it, 17.5 instead of 20.2 on low tiles where it also
 // joins the sweeps.  The other half, a trigger that lets the next kernel's blocks
 // become resident while this one's run, made everything slower (they take issue
