@@ -45,7 +45,9 @@ inline cudaError_t launch_after_smem(void (*kernel)(P...), unsigned blocks, unsi
   cfg.stream = st;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  if (e != cudaSuccess) cudaGetLastError();   // returned here, not left pending for the caller's next check
+  return e;
 }
 template <class... P, class... A>
 inline cudaError_t launch_after(void (*kernel)(P...), unsigned blocks, unsigned threads, cudaStream_t st, A... args) {

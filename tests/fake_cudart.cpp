@@ -38,7 +38,7 @@ thread_local cudaError_t last = cudaSuccess;
 std::set<Stream*> streams;
 std::map<const void*, void*> symbols;
 long long launches = 0, captured = 0, graph_launches = 0;
-int fail_launches = 0;   // launches from now on that fail
+int fail_launch = 0;   // fails when it counts down to zero
 
 cudaError_t ret(cudaError_t e) {
   if (e != cudaSuccess) last = e;
@@ -60,10 +60,7 @@ cudaError_t enqueue(cudaStream_t st, bool needs_device, std::function<void()> f)
   return cudaSuccess;
 }
 cudaError_t launch(cudaStream_t st) {
-  if (fail_launches > 0) {
-    --fail_launches;
-    return ret(cudaErrorLaunchOutOfResources);
-  }
+  if (fail_launch > 0 && --fail_launch == 0) return ret(cudaErrorLaunchOutOfResources);
   const cudaError_t e = enqueue(st, true, [] {});
   if (e == cudaSuccess) ++launches;
   return e;
@@ -96,8 +93,7 @@ void fake_counts(long long* c) {
   c[1] = captured;
   c[2] = graph_launches;
 }
-int fake_last_error() { return (int)last; }
-void fake_fail_launches(int n) { fail_launches = n; }
+void fake_fail_launch(int nth) { fail_launch = nth; }
 
 // --- modules and launches
 void** __cudaRegisterFatBinary(void*) {

@@ -15,6 +15,12 @@ def fake(tmp_path_factory):
     return host_runtime.load(tmp_path_factory.mktemp("fake"))
 
 
+def _ptr(n):
+    """A device buffer of the fake runtime (kernels do not run)."""
+    a = np.zeros(n, np.uint8)
+    return a, a.ctypes.data_as(ctypes.c_void_p)
+
+
 def _batch(fake, L, stream):
     n = len(L)
     q, beta, seed = np.full(n, 3, np.int32), np.full(n, 0.7), np.arange(n, dtype=np.uint64)
@@ -47,3 +53,20 @@ def test_batch_tables_outlive_their_copy(fake, L):
     first_chain = at + -(-tile_map.nbytes // 256) * 256
     assert ws[256:264].view(np.uint64)[0] == ws.ctypes.data + first_chain   # chain 0: its spins
     fake.sw_batch_destroy(b)
+
+
+@pytest.mark.parametrize("failing", [1, 2, 3])
+def test_a_failed_launch_leaves_no_pending_error(fake, failing):
+    """A failed launch is the call's to report; the caller's next
+    cudaGetLastError does not find it again."""
+    st = fake.fake_stream(0)
+    mask, m = _ptr(1024)
+    lab, l = _ptr(4 * 4096)
+    h = fake.sw_create_threshold(256, 2, 1 << 31, 1, 1, st)
+    h3 = fake.sw3_create(40, 9, 20, 2, 1 << 31, 1, 1, st)
+    for call in (lambda: fake.ccl_label(m, l, 64, 64, 1, st), lambda: fake.sw_sweep(h, 1), lambda: fake.sw3_sweep(h3, 1)):
+        fake.fake_fail_launch(failing)
+        assert call() == SW_ERR_CUDA and fake.sw_last_error()
+        assert fake.cudaGetLastError() == 0
+    fake.sw_destroy(h)
+    fake.sw3_destroy(h3)
