@@ -129,7 +129,9 @@ int sw_destroy(sw_handle* h);
  * stream and return without waiting.  Sweep k of the chain (k = 0 for the
  * first sweep after create) draws its bonds and flips with sweep index k.
  * After each sweep the observables (n_eq, n_0..n_{q-1}) of the new spins
- * are stored in a device ring of the last 4096 sweeps. */
+ * are stored in a device ring of the last 4096 sweeps.  SW_ERR_CUDA while the
+ * stream is being captured (the sweeps would be counted without having run);
+ * nothing is enqueued then and the capture goes on. */
 int sw_sweep(sw_handle* h, int n);
 
 /* Wait for the handle's stream; report SW_ERR_STATE if a device check failed. */
@@ -170,7 +172,8 @@ int sw_set_spins(sw_handle* h, const int8_t* src, int is_device);
  *    sweeps.
  * Results are ready when the stream reaches the end of the call (an event
  * recorded on sw_stream(h), or sw_sync).  Returns SW_OK, or SW_ERR_ARG /
- * SW_ERR_CUDA for what the host can see when enqueueing. */
+ * SW_ERR_CUDA for what the host can see when enqueueing (with n > 0 also a
+ * stream that is being captured: nothing is enqueued then). */
 int sw_sweep_io(sw_handle* h, const int8_t* in, int n, int64_t* obs_out, int8_t* out);
 
 /* Copy the bond mask (ceil(L*L/4) bytes, packed as above) and the canonical
@@ -265,7 +268,8 @@ sw3_handle* sw3_create_ex(int X, int Y, int Z, int q, double beta, double J, int
                           int hot_start, void* stream);
 int sw3_destroy(sw3_handle* h);
 
-/* n sweeps, asynchronously on the handle's stream. */
+/* n sweeps, asynchronously on the handle's stream (SW_ERR_CUDA while it is being
+ * captured, as sw_sweep). */
 int sw3_sweep(sw3_handle* h, int n);
 
 /* Waits for the stream; reports device-side failures (SW_ERR_STATE). */
@@ -313,7 +317,10 @@ int sw3_phase_times(sw3_handle* h, double* ms, int64_t* n_sweeps);
  *     sw_batch_get_spins report it.  The chains are then invalid and the
  *     batch refuses further sweeps with SW_ERR_STATE: destroy it.
  * One sweep of either schedule is captured as a CUDA graph and replayed
- * (direct launches if capture is refused).  Both give, for every chain, the
+ * (direct launches if capture is refused, and into a capture of the caller's
+ * on the batch's stream: such sweeps count when they are enqueued, so launch
+ * the caller's graph once before the batch is read or swept again; SW_ERR_CUDA
+ * if this schedule already replays a graph).  Both give, for every chain, the
  * same result bit for bit as a single handle with the same arguments. */
 #define SW_BATCH_PHASES 0
 #define SW_BATCH_PERSISTENT 1

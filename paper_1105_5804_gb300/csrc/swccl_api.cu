@@ -217,6 +217,16 @@ int check_device_status(sw_handle* h) {
   return SW_OK;
 }
 
+// Sweeps on a stream that is being captured would not run but be counted, their
+// observables' rows with them, and their phase events could never be read: they
+// are refused before anything changes or is enqueued, and the capture goes on.
+int refuse_capture(const sw_handle* h, const char* who) {
+  cudaStreamCaptureStatus capture;
+  CK(cudaStreamIsCapturing(h->stream, &capture));
+  if (capture == cudaStreamCaptureStatusNone) return SW_OK;
+  return fail(SW_ERR_CUDA, std::string(who) + ": the stream is being captured");
+}
+
 double coupling_K(int q, double beta, double J, int conv) {
   if (conv == SW_CONV_AUTO) conv = (q == 2) ? SW_CONV_ISING : SW_CONV_POTTS;
   return conv == SW_CONV_ISING ? 2.0 * beta * J : beta * J;
@@ -363,11 +373,7 @@ int sw_sweep(sw_handle* h, int n) {
   if (n == 0) return SW_OK;
   const bool fused = h->mode == SW_MODE_FUSED;
   auto enqueue = fused ? enqueue_sweep_fused : enqueue_sweep;
-  if (fused && !h->timing) {   // a captured sweep would not be counted: refused
-    cudaStreamCaptureStatus capture;
-    CK(cudaStreamIsCapturing(h->stream, &capture));
-    if (capture != cudaStreamCaptureStatusNone) return fail(SW_ERR_CUDA, "sw_sweep: the stream is being captured");
-  }
+  if (const int rc = refuse_capture(h, "sw_sweep")) return rc;
   if (fused && !h->timing && h->update == SW_UPDATE_SW && h->L <= SMALL_L) {
     // all sweeps of the call by one block, which writes their observables too
     for (int done = 0; done < n; done += SMALL_SWEEPS) {
@@ -509,6 +515,8 @@ int sw_sweep_io(sw_handle* h, const int8_t* in, int n, int64_t* obs_out, int8_t*
   if (!h || n < 0 || n > OBS_CAP) return fail(SW_ERR_ARG, "sw_sweep_io: bad arguments");
   const int64_t N = (int64_t)h->L * h->L;
   const cudaStream_t st = h->stream;
+  if (n > 0)
+    if (const int rc = refuse_capture(h, "sw_sweep_io")) return rc;
   if (in) {
     // the observables still pending belong to the spins being replaced; the
     // input goes in only if every value is valid, else the code is noted in

@@ -357,8 +357,16 @@ int sw_batch_sweep(sw_batch* b, int n) {
                                             std::to_string(b->failed) + "); the chains are invalid, destroy the batch");
   if (n == 0) return SW_OK;
   const int k = b->schedule;
-  cudaError_t e;
-  if (b->use_graph && !b->exec[k] && !b->graph_failed[k]) {
+  // on a stream that is being captured the sweeps go into that capture as direct
+  // launches (and the batch's own graph is left for later); a graph cannot
+  cudaStreamCaptureStatus capture;
+  cudaError_t e = cudaStreamIsCapturing(b->stream, &capture);
+  if (e != cudaSuccess) return set_last_error(SW_ERR_CUDA, std::string("sw_batch_sweep: ") + cudaGetErrorString(e));
+  const bool capturing = capture != cudaStreamCaptureStatusNone;
+  if (capturing && b->use_graph && b->exec[k])
+    return set_last_error(SW_ERR_CUDA, "sw_batch_sweep: the stream is being captured and this batch's sweeps run from a "
+                                       "graph (sw_batch_set_graph)");
+  if (b->use_graph && !capturing && !b->exec[k] && !b->graph_failed[k]) {
     e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       cudaError_t e1 = enqueue_batch_sweep(b);

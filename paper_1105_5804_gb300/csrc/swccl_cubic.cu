@@ -154,6 +154,9 @@ int sw3_destroy(sw3_handle* h) {
 int sw3_sweep(sw3_handle* h, int n) {
   if (!h || n < 0) return fail3(SW_ERR_ARG, "sw3_sweep: bad arguments");
   if (n == 0) return SW_OK;
+  cudaStreamCaptureStatus capture;   // captured sweeps would be counted without having run: refused
+  CK3(cudaStreamIsCapturing(h->stream, &capture));
+  if (capture != cudaStreamCaptureStatusNone) return fail3(SW_ERR_CUDA, "sw3_sweep: the stream is being captured");
   if (h->timing) {
     for (int k = 0; k < n; ++k) {
       cudaEvent_t ev[SW3_N_PHASES + 1];
@@ -171,9 +174,6 @@ int sw3_sweep(sw3_handle* h, int n) {
       h->sweeps++;
     }
   } else {
-    cudaStreamCaptureStatus capture;   // a captured sweep would not be counted: refused
-    CK3(cudaStreamIsCapturing(h->stream, &capture));
-    if (capture != cudaStreamCaptureStatusNone) return fail3(SW_ERR_CUDA, "sw3_sweep: the stream is being captured");
     for (int k = 0; k < n; ++k) {
       CK3(launch_sweep3(h->spins, h->lroot, h->gpar, h->words, h->box, h->q, h->T, h->seed, h->ctl, h->obs, OBS3_CAP,
                         h->stream, nullptr));

@@ -70,3 +70,88 @@ def test_a_failed_launch_leaves_no_pending_error(fake, failing):
         assert fake.cudaGetLastError() == 0
     fake.sw_destroy(h)
     fake.sw3_destroy(h3)
+
+
+def _counts(fake):
+    c = (ctypes.c_longlong * 3)()
+    fake.fake_counts(c)
+    return list(c)
+
+
+def _sweeps(info, h, k):
+    v = (ctypes.c_int64 * 8)()
+    info(h, v)
+    return v[k]
+
+
+@pytest.mark.parametrize("L", [64, 256, 2048])
+@pytest.mark.parametrize("mode", ["fused", "staged", "few"])
+@pytest.mark.parametrize("timing", [0, 1])
+@pytest.mark.parametrize("call", ["sweep", "io"])
+def test_captured_sweeps_are_refused_before_anything_is_enqueued(fake, L, mode, timing, call):
+    st = fake.fake_stream(0)
+    h = fake.sw_create_threshold(L, 2, 1 << 31, 1, 1, st)
+    if mode == "staged":
+        fake.sw_set_mode(h, 0)
+    elif mode == "few":
+        fake.sw_set_update(h, 1, 4, 1 << 31)
+    fake.sw_set_timing(h, timing)
+    _, spins = _ptr(L * L)
+    run = (lambda: fake.sw_sweep(h, 3)) if call == "sweep" else (lambda: fake.sw_sweep_io(h, spins, 3, None, spins))
+    for warm in range(2):
+        before = _counts(fake)
+        fake.fake_capture(st, 1)
+        assert run() == SW_ERR_CUDA and b"captured" in fake.sw_last_error()
+        assert _counts(fake) == before and fake.fake_capture_valid(st)
+        fake.fake_capture(st, 0)
+        assert fake.cudaGetLastError() == 0
+        assert _sweeps(fake.sw_get_info, h, 4) == 3 * warm
+        assert run() == SW_OK
+    if mode == "fused" and L > 112:   # the sweeps' last observables are still to be counted when they are read
+        before = _counts(fake)[0]
+        fake.fake_capture(st, 1)
+        run()
+        fake.fake_capture(st, 0)
+        n, rows = ctypes.c_int(), (ctypes.c_int64 * 18)()
+        assert fake.sw_observables(h, rows, 6, ctypes.byref(n)) == SW_OK and n.value == 6
+        assert _counts(fake)[0] > before + 2   # counted, then read: status and rows
+    fake.sw_destroy(h)
+
+
+@pytest.mark.parametrize("timing", [0, 1])
+def test_captured_cubic_sweeps_are_refused(fake, timing):
+    st = fake.fake_stream(0)
+    h = fake.sw3_create(40, 9, 20, 2, 1 << 31, 1, 1, st)
+    fake.sw3_set_timing(h, timing)
+    for warm in range(2):
+        before = _counts(fake)
+        fake.fake_capture(st, 1)
+        assert fake.sw3_sweep(h, 2) == SW_ERR_CUDA
+        assert _counts(fake) == before and fake.fake_capture_valid(st)
+        fake.fake_capture(st, 0)
+        assert _sweeps(fake.sw3_get_info, h, 6) == 2 * warm
+        assert fake.sw3_sweep(h, 2) == SW_OK
+    fake.sw3_destroy(h)
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+def test_batch_sweeps_in_a_capture(fake, graph):
+    """They go into it as direct launches and leave the batch's own graph for
+    later; a batch that replays its graph already refuses, and the capture goes
+    on."""
+    st = fake.fake_stream(0)
+    b, ws = _batch(fake, [64, 300], st)
+    fake.sw_batch_set_graph(b, graph)
+    fake.fake_capture(st, 1)
+    before = _counts(fake)
+    assert fake.sw_batch_sweep(b, 2) == SW_OK
+    after = _counts(fake)
+    assert after[1] - before[1] == 6 and after[2] == before[2] and fake.fake_capture_valid(st)
+    fake.fake_capture(st, 0)
+    assert fake.sw_batch_sweep(b, 2) == SW_OK
+    assert _counts(fake)[2] - after[2] == 2 * graph and _sweeps(fake.sw_batch_info, b, 6) == graph
+    fake.fake_capture(st, 1)
+    assert fake.sw_batch_sweep(b, 1) == (SW_ERR_CUDA if graph else SW_OK)
+    assert fake.fake_capture_valid(st) and _sweeps(fake.sw_batch_info, b, 3) == (4 if graph else 5)
+    fake.fake_capture(st, 0)
+    fake.sw_batch_destroy(b)
