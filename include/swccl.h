@@ -131,7 +131,9 @@ int sw_destroy(sw_handle* h);
  * After each sweep the observables (n_eq, n_0..n_{q-1}) of the new spins
  * are stored in a device ring of the last 4096 sweeps.  SW_ERR_CUDA while the
  * stream is being captured (the sweeps would be counted without having run);
- * nothing is enqueued then and the capture goes on. */
+ * nothing is enqueued then and the capture goes on.  sw_sweep and sw3_sweep
+ * may be called whichever device is current (it stays current); other calls
+ * that launch kernels need the device the handle was made on. */
 int sw_sweep(sw_handle* h, int n);
 
 /* Wait for the handle's stream; report SW_ERR_STATE if a device check failed. */

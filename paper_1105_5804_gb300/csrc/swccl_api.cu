@@ -17,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "on_device.h"
 #include "swccl_shared.h"
 
 namespace swccl {
@@ -374,6 +375,8 @@ int sw_sweep(sw_handle* h, int n) {
   const bool fused = h->mode == SW_MODE_FUSED;
   auto enqueue = fused ? enqueue_sweep_fused : enqueue_sweep;
   if (const int rc = refuse_capture(h, "sw_sweep")) return rc;
+  const OnDevice on(h->device);
+  CK(on.error());
   if (fused && !h->timing && h->update == SW_UPDATE_SW && h->L <= SMALL_L) {
     // all sweeps of the call by one block, which writes their observables too
     for (int done = 0; done < n; done += SMALL_SWEEPS) {

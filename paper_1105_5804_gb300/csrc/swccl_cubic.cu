@@ -5,6 +5,7 @@
 #include <string>
 #include <vector>
 
+#include "on_device.h"
 #include "swccl_shared.h"
 
 using namespace swccl;
@@ -33,6 +34,7 @@ struct sw3_handle {
   uint64_t T = 0, seed = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
+  int device = 0;
   int8_t* spins = nullptr;
   uint16_t* lroot = nullptr;      // brick root of every site (16-bit local index)
   int32_t* gpar = nullptr;        // parents of edge roots; also staging for host spins
@@ -112,6 +114,7 @@ sw3_handle* sw3_create(int X, int Y, int Z, int q, uint64_t T, uint64_t seed, in
     free3(h);
     return nullptr;
   };
+  if (cudaGetDevice(&h->device) != cudaSuccess) return bail(SW_ERR_CUDA, "sw3_create: cudaGetDevice failed");
   if (stream) {
     h->stream = static_cast<cudaStream_t>(stream);
   } else {
@@ -157,6 +160,8 @@ int sw3_sweep(sw3_handle* h, int n) {
   cudaStreamCaptureStatus capture;   // captured sweeps would be counted without having run: refused
   CK3(cudaStreamIsCapturing(h->stream, &capture));
   if (capture != cudaStreamCaptureStatusNone) return fail3(SW_ERR_CUDA, "sw3_sweep: the stream is being captured");
+  const OnDevice on(h->device);
+  CK3(on.error());
   if (h->timing) {
     for (int k = 0; k < n; ++k) {
       cudaEvent_t ev[SW3_N_PHASES + 1];

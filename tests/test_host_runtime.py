@@ -155,3 +155,22 @@ def test_batch_sweeps_in_a_capture(fake, graph):
     assert fake.fake_capture_valid(st) and _sweeps(fake.sw_batch_info, b, 3) == (4 if graph else 5)
     fake.fake_capture(st, 0)
     fake.sw_batch_destroy(b)
+
+
+@pytest.mark.parametrize("L", [64, 256, 2048])
+@pytest.mark.parametrize("timing", [0, 1])
+def test_sweeps_enqueued_while_another_device_is_current(fake, L, timing):
+    st = fake.fake_stream(1)
+    fake.fake_set_device(1)
+    h = fake.sw_create_threshold(L, 2, 1 << 31, 1, 1, st)
+    h3 = fake.sw3_create(40, 9, 20, 2, 1 << 31, 1, 1, st)
+    fake.sw_set_timing(h, timing)
+    fake.sw3_set_timing(h3, timing)
+    for warm in range(2):
+        fake.fake_set_device(0)
+        assert fake.sw_sweep(h, 3) == SW_OK, fake.sw_last_error()
+        assert fake.sw3_sweep(h3, 3) == SW_OK, fake.sw_last_error()
+        assert fake.fake_device() == 0 and fake.cudaGetLastError() == 0
+    assert _sweeps(fake.sw_get_info, h, 4) == _sweeps(fake.sw3_get_info, h3, 6) == 6
+    fake.sw_destroy(h)
+    fake.sw3_destroy(h3)
