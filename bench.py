@@ -50,9 +50,9 @@ SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per si
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "733ea9b36de62752"
+CCL_COUNTER_HASH = "8c3cdb81a85acf83"
 CCL_COUNTER_TILE_W = 128
-CCL_TRAFFIC_BYTES_PER_SITE = ((6.649600 + 2.546176) + (16.568832 + 0.000000) + (53.476608 + 10.269184)) * 1e6 / 16777216
+CCL_TRAFFIC_BYTES_PER_SITE = ((6.633472 + 2.572032) + (16.572672 + 0.000000) + (53.475328 + 10.488320)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8
 # spins once (2 B, the minimum of any sweep); the kernel split adds the
 # 16-bit tile roots written by k_sw_label and read by k_sw_flip (6 B).
