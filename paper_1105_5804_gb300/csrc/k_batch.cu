@@ -16,6 +16,8 @@
 // Small lattices alone leave most SMs idle (L = 64 is two tiles); in one
 // batch their tiles fill the machine.  Every chain draws from its own seed,
 // so a chain's result is the same alone or in any batch.
+#include <algorithm>
+
 #include "low_tile.cuh"
 
 namespace swccl {
@@ -79,12 +81,17 @@ __device__ __forceinline__ bool grid_barrier(BatchCtl* ctl, unsigned nblocks, lo
 
 }  // namespace
 
-// Initial state of every chain: its tiles' blocks share its sites, four per
-// thread and step (L % 4 == 0), and the clearing of its observable ring.
+// Initial state of every chain: its tiles' blocks (blockIdx.y of them per tile)
+// share its sites, four per thread and step (L % 4 == 0), and the clearing of its
+// observable ring, 16 bytes per thread and step.  The ring of a chain with many
+// states is larger than a small lattice by far, so a batch of few tiles takes
+// more blocks per tile, as many as fill the GPU (one chain, L = 16, q = 127,
+// created in 37 us, 163 with one block for its 4 MB ring).
 __global__ void __launch_bounds__(LABEL_THREADS) k_batch_init(BatchView b, int hot) {
   const SwRep& R = b.reps[b.tile_rep[blockIdx.x]];
-  const int64_t i0 = (int64_t)(blockIdx.x - R.tile0) * LABEL_THREADS + threadIdx.x;
-  const int64_t stride = (int64_t)R.g.n_tiles() * LABEL_THREADS;
+  const int64_t tiles = R.g.n_tiles();
+  const int64_t i0 = (blockIdx.x - R.tile0 + tiles * blockIdx.y) * LABEL_THREADS + threadIdx.x;
+  const int64_t stride = tiles * gridDim.y * LABEL_THREADS;
   for (int64_t i = i0; i < R.g.n_sites() / 4; i += stride) {
     uint32_t w = 0u;
     if (hot) {
@@ -94,7 +101,8 @@ __global__ void __launch_bounds__(LABEL_THREADS) k_batch_init(BatchView b, int h
     }
     reinterpret_cast<uint32_t*>(R.spins)[i] = w;
   }
-  for (int64_t i = i0; i < (int64_t)b.obs_cap * (R.q + 1); i += stride) R.obs[i] = 0;
+  ulonglong2* ring = reinterpret_cast<ulonglong2*>(R.obs);   // 256-byte aligned, an even number of rows
+  for (int64_t i = i0; i < (int64_t)b.obs_cap / 2 * (R.q + 1); i += stride) ring[i] = make_ulonglong2(0ull, 0ull);
 }
 
 // ---------------------------------------------------------------------------
@@ -235,7 +243,9 @@ __global__ void __launch_bounds__(LABEL_THREADS, 4 * 256 / TILE_W) k_batch_persi
 
 // ---------------------------------------------------------------------------
 cudaError_t launch_batch_init(const BatchView& b, int hot, cudaStream_t st) {
-  k_batch_init<<<b.n_tiles, LABEL_THREADS, 0, st>>>(b, hot);
+  constexpr int BLOCKS = 152 * 8 * 256 / TILE_W, MAX_PER_TILE = 64 * 256 / TILE_W;
+  const int per_tile = std::max(1, std::min(MAX_PER_TILE, BLOCKS / b.n_tiles));
+  k_batch_init<<<dim3(b.n_tiles, per_tile), LABEL_THREADS, 0, st>>>(b, hot);
   return cudaGetLastError();
 }
 

@@ -37,7 +37,7 @@ thread_local int current = 0;
 thread_local cudaError_t last = cudaSuccess;
 std::set<Stream*> streams;
 std::map<const void*, void*> symbols;
-long long launches = 0, captured = 0, graph_launches = 0;
+long long launches = 0, captured = 0, graph_launches = 0, last_blocks = 0;   // last_blocks: of the last plain launch
 int fail_launch = 0;   // fails when it counts down to zero
 
 cudaError_t ret(cudaError_t e) {
@@ -92,6 +92,7 @@ void fake_counts(long long* c) {
   c[0] = launches;
   c[1] = captured;
   c[2] = graph_launches;
+  c[3] = last_blocks;
 }
 void fake_fail_launch(int nth) { fail_launch = nth; }
 
@@ -123,7 +124,10 @@ cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
   *k = reinterpret_cast<cudaKernel_t>(const_cast<void*>(f));
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void**, size_t, cudaStream_t st) { return launch(st); }
+cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3 g, dim3, void**, size_t, cudaStream_t st) {
+  last_blocks = (int64_t)g.x * g.y * g.z;
+  return launch(st);
+}
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**) { return launch(c->stream); }
 cudaError_t cudaLaunchCooperativeKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t st) { return launch(st); }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }

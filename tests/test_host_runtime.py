@@ -21,9 +21,9 @@ def _ptr(n):
     return a, a.ctypes.data_as(ctypes.c_void_p)
 
 
-def _batch(fake, L, stream):
+def _batch(fake, L, stream, q=3):
     n = len(L)
-    q, beta, seed = np.full(n, 3, np.int32), np.full(n, 0.7), np.arange(n, dtype=np.uint64)
+    q, beta, seed = np.full(n, q, np.int32), np.full(n, 0.7), np.arange(n, dtype=np.uint64)
     L = np.asarray(L, np.int32)
     p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
     need = fake.sw_batch_device_bytes(n, p(L), p(q))
@@ -72,10 +72,22 @@ def test_a_failed_launch_leaves_no_pending_error(fake, failing):
     fake.sw3_destroy(h3)
 
 
-def _counts(fake):
-    c = (ctypes.c_longlong * 3)()
+@pytest.mark.parametrize("L,tiles", [([16], 1), ([16, 100, 300], 24), ([2048] * 3, 1536)])
+def test_a_batch_is_set_up_by_many_blocks(fake, L, tiles):
+    """Its observable rings (4 MB a chain for q = 127) take more than a block
+    per tile if the tiles are few."""
+    st = fake.fake_stream(0)
+    b, ws = _batch(fake, L, st, q=127)
+    c = (ctypes.c_longlong * 4)()
     fake.fake_counts(c)
-    return list(c)
+    assert c[3] == tiles * max(1, min(64, 1216 // tiles))
+    fake.sw_batch_destroy(b)
+
+
+def _counts(fake):
+    c = (ctypes.c_longlong * 4)()
+    fake.fake_counts(c)
+    return list(c)[:3]
 
 
 def _sweeps(info, h, k):
