@@ -39,7 +39,7 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "306cdc17fe252ba2"
+SWEEP_COUNTER_HASH = "3bc044a4cb9f5605"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
     "k_sw_label": ((88.849408 + 130.423296) * 1e6 / 67108864, 184289423 / 67108864),
     "k_merge": ((56.291072 + 0.763392) * 1e6 / 67108864, 14599000 / 67108864),
@@ -50,7 +50,7 @@ SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per si
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "8c3cdb81a85acf83"
+CCL_COUNTER_HASH = "a095e4ee7057a80d"
 CCL_COUNTER_TILE_W = 128
 CCL_TRAFFIC_BYTES_PER_SITE = ((6.633472 + 2.572032) + (16.572672 + 0.000000) + (53.475328 + 10.488320)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8

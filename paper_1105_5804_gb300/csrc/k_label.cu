@@ -107,6 +107,23 @@ cudaError_t launch_merge(int32_t* labels, const Grid& g, const LabelScratch& s, 
                       adv, obs, obs_cap, q);
 }
 
+cudaError_t load_ccl_kernels() {
+  cudaError_t e = cudaSuccess;
+  auto load = [&](auto* kernel) {
+    cudaFuncAttributes attr;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&attr, kernel);
+  };
+  load(k_ccl_tile<8>);
+  load(k_ccl_tile<16>);
+  load(k_ccl_tile<TILE_H>);
+  load(k_merge);
+  load(k_ccl_final<8>);
+  load(k_ccl_final<16>);
+  load(k_ccl_final<TILE_H>);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // ---------------------------------------------------------------------------
 // Root compression (+ root draws for a Swendsen-Wang sweep).
 // ---------------------------------------------------------------------------

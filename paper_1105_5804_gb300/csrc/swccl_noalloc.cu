@@ -1,7 +1,7 @@
 // swccl_noalloc.cu -- connected-component labeling that allocates nothing.
 //
-// ccl_label takes its scratch (tile-root lists, root counts, seam records)
-// with cudaMallocAsync, and ccl_label_ws needs the caller to allocate it.
+// ccl_label takes its scratch (tile roots, edge-root bits, seam records) with
+// cudaMallocAsync, and ccl_label_ws needs the caller to allocate it.
 // Some callers can do neither when they label:
 //   * latency-bound loops (serving) that must not call cudaMalloc/cudaFree,
 //     since cudaFree synchronises the whole device and stalls other streams;
@@ -17,7 +17,9 @@
 // address; its device address is looked up once per device with
 // cudaGetSymbolAddress, with that device current, and handed to the kernels.
 // The first call on a device does this look-up (and that of the labeling
-// status word), so it should come before any stream capture.
+// status word), so it should come before any stream capture.  It also loads
+// the labeling kernels of every tile height: loaded at their first launch, a
+// later call with a larger grid would take device memory and wait for it.
 #include <mutex>
 #include <string>
 
@@ -26,8 +28,8 @@
 using namespace swccl;
 
 // Scratch of ccl_label_noalloc, shared by every call on this device.  Every
-// part the kernels read is written by the same call first (root counts,
-// root lists, seam records), so nothing needs clearing between calls.
+// part the kernels read is written by the same call first (tile roots,
+// edge-root bits, seam records), so nothing needs clearing between calls.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[CCL_NOALLOC_SCRATCH_BYTES];
 
 namespace {
@@ -57,6 +59,10 @@ void* scratch_address(std::string& msg) {
       msg = std::string("cudaGetSymbolAddress(scratch): ") + cudaGetErrorString(e);
       return nullptr;
     }
+    if ((e = load_ccl_kernels()) != cudaSuccess) {
+      msg = std::string("loading the labeling kernels: ") + cudaGetErrorString(e);
+      return nullptr;
+    }
     g_scratch_addr[dev] = p;
   }
   return g_scratch_addr[dev];
@@ -69,8 +75,9 @@ extern "C" int ccl_label_noalloc(const uint8_t* bond_mask, int32_t* labels, int 
   if (!bond_mask || !labels) return set_last_error(SW_ERR_ARG, "ccl_label_noalloc: null device pointer");
   if (H < 1 || W < 1 || (int64_t)H * W >= ((int64_t)1 << 31))
     return set_last_error(SW_ERR_ARG, "ccl_label_noalloc: need H, W >= 1 and H*W < 2^31");
-  const Grid g = make_grid(H, W, periodic);
-  const int64_t need = label_scratch_bytes(g);
+  // the documented limit is that of ccl_workspace_bytes; the kernels use less of
+  // the array (ccl_scratch_bytes)
+  const int64_t need = label_scratch_bytes(make_grid(H, W, periodic));
   if (need > (int64_t)CCL_NOALLOC_SCRATCH_BYTES)
     return set_last_error(SW_ERR_ARG, "ccl_label_noalloc: an " + std::to_string(H) + " x " + std::to_string(W) +
                                           " grid needs " + std::to_string(need) +

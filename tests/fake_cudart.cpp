@@ -38,6 +38,8 @@ thread_local cudaError_t last = cudaSuccess;
 std::set<Stream*> streams;
 std::map<const void*, void*> symbols;
 long long launches = 0, captured = 0, graph_launches = 0, last_blocks = 0;   // last_blocks: of the last plain launch
+std::set<const void*> loaded;   // kernels the runtime has been asked about or has launched
+long long cold_launches = 0;    // programmatic launches of kernels not loaded before
 int fail_launch = 0;   // fails when it counts down to zero
 
 cudaError_t ret(cudaError_t e) {
@@ -93,6 +95,7 @@ void fake_counts(long long* c) {
   c[1] = captured;
   c[2] = graph_launches;
   c[3] = last_blocks;
+  c[4] = cold_launches;
 }
 void fake_fail_launch(int nth) { fail_launch = nth; }
 
@@ -128,7 +131,14 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3 g, dim3, void**, size_t, cudaS
   last_blocks = (int64_t)g.x * g.y * g.z;
   return launch(st);
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**) { return launch(c->stream); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+  if (loaded.insert(f).second) ++cold_launches;
+  return launch(c->stream);
+}
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes*, const void* f) {
+  loaded.insert(f);
+  return cudaSuccess;
+}
 cudaError_t cudaLaunchCooperativeKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t st) { return launch(st); }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {

@@ -36,7 +36,7 @@ def load(out_dir):
             ("sw_phase_times", [vp, vp, vp], i32), ("sw_observables", [vp, vp, i32, vp], i32),
             ("sw_destroy", [vp], i32), ("sw3_destroy", [vp], i32), ("sw_batch_destroy", [vp], i32),
             ("cudaStreamSynchronize", [vp], i32), ("cudaGetLastError", [], i32),
-            ("ccl_label", [vp, vp, i32, i32, i32, vp], i32)]:
+            ("ccl_label_noalloc", [vp, vp, i32, i32, i32, vp], i32), ("ccl_label", [vp, vp, i32, i32, i32, vp], i32)]:
         f = getattr(L, name)
         f.argtypes, f.restype = args, res
     return L

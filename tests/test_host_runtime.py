@@ -78,14 +78,14 @@ def test_a_batch_is_set_up_by_many_blocks(fake, L, tiles):
     per tile if the tiles are few."""
     st = fake.fake_stream(0)
     b, ws = _batch(fake, L, st, q=127)
-    c = (ctypes.c_longlong * 4)()
+    c = (ctypes.c_longlong * 5)()
     fake.fake_counts(c)
     assert c[3] == tiles * max(1, min(64, 1216 // tiles))
     fake.sw_batch_destroy(b)
 
 
 def _counts(fake):
-    c = (ctypes.c_longlong * 4)()
+    c = (ctypes.c_longlong * 5)()
     fake.fake_counts(c)
     return list(c)[:3]
 
@@ -186,3 +186,18 @@ def test_sweeps_enqueued_while_another_device_is_current(fake, L, timing):
     assert _sweeps(fake.sw_get_info, h, 4) == _sweeps(fake.sw3_get_info, h3, 6) == 6
     fake.sw_destroy(h)
     fake.sw3_destroy(h3)
+
+
+def test_noalloc_loads_every_kernel_on_its_first_call(tmp_path):
+    """The first call on a device may take device memory and time; later ones,
+    of any size, launch only what is loaded."""
+    fake = host_runtime.load(tmp_path)   # a library of its own: nothing loaded yet
+    st = fake.fake_stream(0)
+    mask, m = _ptr(1 << 20)
+    lab, l = _ptr(1 << 24)
+    cold = lambda: (lambda c: (fake.fake_counts(c), c[4])[1])((ctypes.c_longlong * 5)())
+    assert fake.ccl_label_noalloc(m, l, 1, 1, 1, st) == SW_OK, fake.sw_last_error()
+    assert cold() == 0
+    for H, W in [(200, 300), (1000, 1200), (1500, 1500), (2000, 2000)]:
+        assert fake.ccl_label_noalloc(m, l, H, W, 0, st) == SW_OK, fake.sw_last_error()
+    assert cold() == 0
