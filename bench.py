@@ -39,20 +39,20 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "3bc044a4cb9f5605"
+SWEEP_COUNTER_HASH = "9e7d7f30a68f38ab"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
-    "k_sw_label": ((88.849408 + 130.423296) * 1e6 / 67108864, 184289423 / 67108864),
-    "k_merge": ((56.291072 + 0.763392) * 1e6 / 67108864, 14599000 / 67108864),
-    "k_sw_flip": ((203.587072 + 47.656448) * 1e6 / 67108864, 71101877 / 67108864),
+    "k_sw_label": ((88.882944 + 130.552576) * 1e6 / 67108864, 184289377 / 67108864),
+    "k_merge": ((56.290304 + 0.759040) * 1e6 / 67108864, 14597217 / 67108864),
+    "k_sw_flip": ((203.559680 + 47.665408) * 1e6 / 67108864, 71103822 / 67108864),
 }
 # The stand-alone labeling call (k_ccl_tile, k_merge, k_ccl_final), one ncu
 # capture per kernel of a 4096^2 critical percolation mask: DRAM bytes per site,
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "a095e4ee7057a80d"
+CCL_COUNTER_HASH = "9a133ef348ac4f70"
 CCL_COUNTER_TILE_W = 128
-CCL_TRAFFIC_BYTES_PER_SITE = ((6.633472 + 2.572032) + (16.572672 + 0.000000) + (53.475328 + 10.488320)) * 1e6 / 16777216
+CCL_TRAFFIC_BYTES_PER_SITE = ((6.647808 + 2.541824) + (16.571136 + 0.000000) + (53.475584 + 10.175232)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8
 # spins once (2 B, the minimum of any sweep); the kernel split adds the
 # 16-bit tile roots written by k_sw_label and read by k_sw_flip (6 B).

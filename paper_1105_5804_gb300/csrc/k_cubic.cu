@@ -29,6 +29,8 @@
 // HBM traffic per site: spins read 1 B and brick roots written 2 B (local),
 // brick roots read 2 B and spins written 1 B (flip), plus the face sites,
 // the edge-root and face bits (0.16 B) and the sparse parent entries.
+#include <type_traits>
+
 #include "fused_tile.cuh"
 
 namespace swccl {
@@ -126,6 +128,72 @@ __device__ __forceinline__ uint32_t eq_row(const uint32_t (&a)[4], const uint32_
   return eq4(a[0], b[0]) | eq4(a[1], b[1]) << 4 | eq4(a[2], b[2]) << 8 | eq4(a[3], b[3]) << 12;
 }
 
+// Open bonds of row `lane` of a plane (bit = site), zero past its rows.
+struct RowBonds {
+  uint32_t x, y, z;
+};
+
+// Bonds, and observables of the spins read, of a plane of a flat brick (at most
+// FLAT_D rows): the rows spread over all lanes, R consecutive sites of a row
+// each, R being the power of two from the number of rows on.  With two lanes per
+// row and sixteen sites per lane, as in a full brick, a brick of one row costs
+// what a full one does: a sweep of 1000 x 1000 x 1 took 126 us, 79 this way (the
+// 16 rows of the engine not swept and one-site axes not joined to themselves are
+// part of it), 1000 x 1000 x 2 138 and 98, x 4 153 and 123, x 8 176 and 169.
+constexpr int FLAT_D = B3Z / 2;
+__device__ __forceinline__ RowBonds flat_bonds(const int8_t* spins, const Box3& b, const Brick& k, int q, uint64_t T,
+                                               const PhiloxKeys& keys, uint64_t sweep, bool do_obs, unsigned* red,
+                                               int* hist) {
+  const int lane = threadIdx.x & 31, ly = threadIdx.x >> 5;
+  const int R = k.d <= 1 ? 1 : k.d <= 2 ? 2 : k.d <= 4 ? 4 : 8;
+  const int lz = lane & (R - 1), x0 = lane & ~(R - 1);   // my row, my first column
+  const int y = k.y0 + ly, z = k.z0 + lz;
+  const int n = ly < k.h && lz < k.d ? min(k.w - x0, R) : 0;
+  const uint32_t first = (uint32_t)site3(b, k.x0 + x0, y, z);
+  const uint32_t to_y = (y + 1 == b.Y ? -(uint32_t)y : 1u) * (uint32_t)b.X;
+  const uint32_t to_z = (z + 1 == b.Z ? -(uint32_t)z : 1u) * ((uint32_t)b.X * (uint32_t)b.Y);
+  const uint32_t thr = (uint32_t)T;
+  RowBonds o = {0u, 0u, 0u};
+  unsigned n_eq = 0u;
+  unsigned long long states = 0ull;   // sites per state, 8 bits each (q <= QREG)
+  if (do_obs && q > QREG) __syncthreads();   // the histogram is cleared
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    const uint32_t site = first + (uint32_t)i, bit = 1u << (x0 + i);
+    const int x = k.x0 + x0 + i;
+    const int s = spins[site];
+    const bool ex = spins[x + 1 == b.X ? site - (uint32_t)x : site + 1u] == s, ey = spins[site + to_y] == s,
+               ez = spins[site + to_z] == s;
+    if (do_obs) {
+      n_eq += (unsigned)ex + (unsigned)ey + (unsigned)ez;
+      if (q <= QREG) states += 1ull << (8 * s);
+      else atomicAdd(&hist[s], 1);
+    }
+    if (T == 0) continue;
+    uint4 r = make_uint4(0u, 0u, 0u, 0u);
+    if (T < (1ull << 32))
+      r = philox_draw(make_uint4(site, (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_BOND3), keys);
+    const bool all = T >= (1ull << 32);
+    if (ex && (all || r.x < thr)) o.x |= bit;
+    if (ey && (all || r.y < thr)) o.y |= bit;
+    if (ez && (all || r.z < thr)) o.z |= bit;
+  }
+  __syncwarp();
+  for (int u = R; u < 32; u *= 2) {
+    o.x |= __shfl_xor_sync(FULL, o.x, u);
+    o.y |= __shfl_xor_sync(FULL, o.y, u);
+    o.z |= __shfl_xor_sync(FULL, o.z, u);
+  }
+  if (lane >= k.d) o = {0u, 0u, 0u};
+  if (do_obs) {
+    int cnt[QREG];
+#pragma unroll
+    for (int s = 0; s < QREG; ++s) cnt[s] = (int)(states >> (8 * s) & 0xFFu);
+    observables_warp_sums<B3_THREADS>(n_eq, cnt, q <= QREG ? q : 0, red);
+  }
+  return o;
+}
+
 // Local step of a brick.  Bound by instruction issue and by the latency of the
 // shared-memory walks: 16 draws per thread (about 45 instructions each), the
 // engine and the +y joins take most of a warp's time, so eight CTAs per SM
@@ -139,6 +207,10 @@ __device__ __forceinline__ uint32_t eq_row(const uint32_t (&a)[4], const uint32_
 // with eight CTAs, 142 with packed spins, 131 with the face roots looked up a lane
 // per face site (before: by the sites' owners, a few lanes per warp) and parent
 // entries written from the edge bits.
+// FLAT: for boxes whose last layer of bricks has at most FLAT_D planes of rows (its
+// bricks, not the others, go by flat_bonds; the engine's sweep is a loop over the
+// brick's rows instead of unrolled: 256 x 256 x 17 43.2 us a sweep against 42.2).
+template <bool FLAT>
 __global__ void __launch_bounds__(B3_THREADS, 8)
 k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, Box3 b, int q, uint64_t T,
          const __grid_constant__ PhiloxKeys keys, const SwCtl* ctl, int64_t* obs, int obs_cap, int* err) {
@@ -162,101 +234,110 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
   const int nv = plane && lz < k.d ? min(max(k.w - 16 * half, 0), 16) : 0;
   const uint32_t row0 = (uint32_t)site3(b, k.x0, k.y0 + ly, k.z0 + lz);   // my row's first site; past the box without sites
   const uint32_t site0 = row0 + 16 * half;
-  uint32_t ex = 0u, ey = 0u, ez = 0u;
-  {
-    const bool whole = (b.X & 15) == 0;
-    const int y = k.y0 + ly, z = k.z0 + lz, x1 = k.x0 + 16 * half + nv;
-    uint32_t c[4], n[4], ny[4], nz[4];
-    load_row(spins, site0, nv, whole, c);
-    load_row(spins, site0 + (y + 1 == b.Y ? -(uint32_t)y : 1u) * (uint32_t)b.X, nv, whole, ny);
-    load_row(spins, site0 + (z + 1 == b.Z ? -(uint32_t)z : 1u) * ((uint32_t)b.X * (uint32_t)b.Y), nv, whole, nz);
-    const uint32_t next = nv > 0 ? (uint32_t)(uint8_t)spins[x1 == b.X ? row0 - k.x0 : row0 - k.x0 + x1] : 0u;
-    const uint32_t mine = (1u << nv) - 1u;
-    uint32_t ones = 0u;
-    if (q == 2) {   // bytes 0 or 1, packed one bit per site
-      auto pack = [](const uint32_t (&v)[4]) {
-        return (v[0] * 0x01020408u) >> 24 | (v[1] * 0x01020408u) >> 24 << 4 | (v[2] * 0x01020408u) >> 24 << 8 |
-               (v[3] * 0x01020408u) >> 24 << 12;
-      };
-      ones = pack(c) & mine;
-      ex = ~(ones ^ ((ones | next << nv) >> 1)) & mine;
-      ey = ~(ones ^ pack(ny)) & mine;
-      ez = ~(ones ^ pack(nz)) & mine;
-    } else {
+  const bool flat = FLAT && k.d <= FLAT_D;
+  RowBonds row = {0u, 0u, 0u};
+  if (flat) {
+    row = flat_bonds(spins, b, k, q, T, keys, sweep, do_obs, ls.red, ls.hist);
+  } else {
+    uint32_t ex = 0u, ey = 0u, ez = 0u;
+    {
+      const bool whole = (b.X & 15) == 0;
+      const int y = k.y0 + ly, z = k.z0 + lz, x1 = k.x0 + 16 * half + nv;
+      uint32_t c[4], n[4], ny[4], nz[4];
+      load_row(spins, site0, nv, whole, c);
+      load_row(spins, site0 + (y + 1 == b.Y ? -(uint32_t)y : 1u) * (uint32_t)b.X, nv, whole, ny);
+      load_row(spins, site0 + (z + 1 == b.Z ? -(uint32_t)z : 1u) * ((uint32_t)b.X * (uint32_t)b.Y), nv, whole, nz);
+      const uint32_t next = nv > 0 ? (uint32_t)(uint8_t)spins[x1 == b.X ? row0 - k.x0 : row0 - k.x0 + x1] : 0u;
+      const uint32_t mine = (1u << nv) - 1u;
+      uint32_t ones = 0u;
+      if (q == 2) {   // bytes 0 or 1, packed one bit per site
+        auto pack = [](const uint32_t (&v)[4]) {
+          return (v[0] * 0x01020408u) >> 24 | (v[1] * 0x01020408u) >> 24 << 4 | (v[2] * 0x01020408u) >> 24 << 8 |
+                 (v[3] * 0x01020408u) >> 24 << 12;
+        };
+        ones = pack(c) & mine;
+        ex = ~(ones ^ ((ones | next << nv) >> 1)) & mine;
+        ey = ~(ones ^ pack(ny)) & mine;
+        ez = ~(ones ^ pack(nz)) & mine;
+      } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        n[j] = __funnelshift_r(c[j], j < 3 ? c[j + 1] : next, 8);
-        if (nv < 16 && (nv - 1) >> 2 == j) {
-          const int sh = 8 * ((nv - 1) & 3);
-          n[j] = (n[j] & ~(0xFFu << sh)) | next << sh;
+        for (int j = 0; j < 4; ++j) {
+          n[j] = __funnelshift_r(c[j], j < 3 ? c[j + 1] : next, 8);
+          if (nv < 16 && (nv - 1) >> 2 == j) {
+            const int sh = 8 * ((nv - 1) & 3);
+            n[j] = (n[j] & ~(0xFFu << sh)) | next << sh;
+          }
         }
+        ex = eq_row(c, n) & mine;
+        ey = eq_row(c, ny) & mine;
+        ez = eq_row(c, nz) & mine;
       }
-      ex = eq_row(c, n) & mine;
-      ey = eq_row(c, ny) & mine;
-      ez = eq_row(c, nz) & mine;
-    }
-    if (do_obs) {
-      int cnt[QREG] = {};
-      if (q == 2) {
-        cnt[1] = __popc(ones);
-        cnt[0] = nv - cnt[1];
-      } else if (q <= QREG) {
+      if (do_obs) {
+        int cnt[QREG] = {};
+        if (q == 2) {
+          cnt[1] = __popc(ones);
+          cnt[0] = nv - cnt[1];
+        } else if (q <= QREG) {
 #pragma unroll
-        for (int s = 0; s < QREG; ++s) {
-          if (s >= q) break;
-          const uint32_t same = 0x01010101u * (uint32_t)s;
-          const uint32_t v[4] = {same, same, same, same};
-          cnt[s] = __popc(eq_row(c, v) & mine);
+          for (int s = 0; s < QREG; ++s) {
+            if (s >= q) break;
+            const uint32_t same = 0x01010101u * (uint32_t)s;
+            const uint32_t v[4] = {same, same, same, same};
+            cnt[s] = __popc(eq_row(c, v) & mine);
+          }
         }
+        if (q > QREG) {
+          __syncthreads();   // the histogram is cleared
+          for (int i = 0; i < nv; ++i) atomicAdd(&ls.hist[(uint8_t)spins[site0 + i]], 1);
+        }
+        observables_warp_sums<B3_THREADS>((unsigned)(__popc(ex) + __popc(ey) + __popc(ez)), cnt, q <= QREG ? q : 0,
+                                          ls.red);
       }
-      if (q > QREG) {
-        __syncthreads();   // the histogram is cleared
-        for (int i = 0; i < nv; ++i) atomicAdd(&ls.hist[(uint8_t)spins[site0 + i]], 1);
-      }
-      observables_warp_sums<B3_THREADS>((unsigned)(__popc(ex) + __popc(ey) + __popc(ez)), cnt, q <= QREG ? q : 0,
-                                        ls.red);
     }
-  }
 
-  // 2. open bonds of my sites
-  if (T == 0) {
-    ex = ey = ez = 0u;
-  } else if (T < (1ull << 32) && plane) {
-    const uint32_t thr = (uint32_t)T;
-    uint32_t ox = 0u, oy = 0u, oz = 0u;
-    constexpr int U = 8;
+    // 2. open bonds of my sites
+    if (T == 0) {
+      ex = ey = ez = 0u;
+    } else if (T < (1ull << 32) && plane) {
+      const uint32_t thr = (uint32_t)T;
+      uint32_t ox = 0u, oy = 0u, oz = 0u;
+      constexpr int U = 8;
 #pragma unroll 1
-    for (int i0 = 0; i0 < min(k.w, 16); i0 += U) {
-      uint32_t bx = 0u, by = 0u, bz = 0u;
+      for (int i0 = 0; i0 < min(k.w, 16); i0 += U) {
+        uint32_t bx = 0u, by = 0u, bz = 0u;
 #pragma unroll
-      for (int i = 0; i < U; ++i) {
-        const uint4 r = philox_draw(
-            make_uint4(site0 + (uint32_t)(i0 + i), (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_BOND3), keys);
-        set_if_below(bx, r.x, thr, 1u << i);
-        set_if_below(by, r.y, thr, 1u << i);
-        set_if_below(bz, r.z, thr, 1u << i);
+        for (int i = 0; i < U; ++i) {
+          const uint4 r = philox_draw(
+              make_uint4(site0 + (uint32_t)(i0 + i), (uint32_t)sweep, (uint32_t)(sweep >> 32), TAG_BOND3), keys);
+          set_if_below(bx, r.x, thr, 1u << i);
+          set_if_below(by, r.y, thr, 1u << i);
+          set_if_below(bz, r.z, thr, 1u << i);
+        }
+        ox |= bx << i0;
+        oy |= by << i0;
+        oz |= bz << i0;
       }
-      ox |= bx << i0;
-      oy |= by << i0;
-      oz |= bz << i0;
+      ex &= ox;
+      ey &= oy;
+      ez &= oz;
     }
-    ex &= ox;
-    ey &= oy;
-    ez &= oz;
+
+    // row words (lane = row lz)
+    auto row_word = [&](uint32_t e) {
+      e <<= 16 * half;
+      e |= __shfl_xor_sync(FULL, e, 1);
+      e = __shfl_sync(FULL, e, 2 * (lane & 15));
+      return lane < B3Z ? e : 0u;
+    };
+    row = {row_word(ex), row_word(ey), row_word(ez)};
   }
 
-  // 3. row words (lane = row lz) of the plane's bonds: inside the brick for
-  //    the engine and the +y joins, leaving it for the merge, wrapping inside
-  //    it where the axis is one brick long
-  auto row_word = [&](uint32_t e) {
-    e <<= 16 * half;
-    e |= __shfl_xor_sync(FULL, e, 1);
-    e = __shfl_sync(FULL, e, 2 * (lane & 15));
-    return lane < B3Z ? e : 0u;
-  };
-  uint32_t we = row_word(ex);
-  uint32_t wn = row_word(ez);
-  const uint32_t yb = row_word(ey);
+  // 3. the plane's bonds: inside the brick for the engine and the +y joins,
+  //    leaving it for the merge, wrapping inside it where the axis is one brick
+  //    long
+  uint32_t we = row.x;
+  uint32_t wn = row.z;
+  const uint32_t yb = row.y;
   const uint32_t last_x = 1u << (k.w - 1);
   const uint32_t x_out = __ballot_sync(FULL, (we & last_x) != 0u);  // bit = lz
   const uint32_t z_out = __shfl_sync(FULL, wn, k.d - 1);            // bit = lx
@@ -271,7 +352,7 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
   if (y_last && lane < B3Z) out[B3_FACE_Y + lane] = b.by > 1 ? yb : 0u;
 
   // 4. the engine labels the planes (no bond joins two of its strips)
-  tile_engine(sm, we, wn, k.d, B3X * k.h, err);
+  tile_engine<!FLAT>(sm, we, wn, k.d, B3X * k.h, err);
   __syncthreads();
 
   // 5. +y bonds between planes ly and ly + 1.  One contact per overlap of an
@@ -321,22 +402,23 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
     }
     __syncthreads();
   }
-  // wraps of an axis one brick long
-  const bool wraps = b.bx == 1 || b.by == 1 || b.bz == 1;
+  // wraps of an axis one brick long (of one site: its own neighbour)
+  const bool wrap_x = b.bx == 1 && b.X > 1, wrap_y = b.by == 1 && b.Y > 1, wrap_z = b.bz == 1 && b.Z > 1;
+  const bool wraps = wrap_x || wrap_y || wrap_z;
   if (wraps) {
     if (plane) {
       const int self = 2 * brick_local(0, ly, 0);
-      if (b.bx == 1) {
+      if (wrap_x) {
         const bool on = lane < k.d && ((x_out >> lane) & 1u);
         sm_union_tile(par, on ? 2 * brick_local(k.w - 1, ly, lane) : self, on ? 2 * brick_local(0, ly, lane) : self,
                       err);
       }
-      if (b.bz == 1) {
+      if (wrap_z) {
         const bool on = (z_out >> lane) & 1u;
         sm_union_tile(par, on ? 2 * brick_local(lane, ly, k.d - 1) : self, on ? 2 * brick_local(lane, ly, 0) : self,
                       err);
       }
-      if (b.by == 1 && y_last) {
+      if (wrap_y && y_last) {
         for (int lz = 0; lz < k.d; ++lz) {
           const bool on = (__shfl_sync(FULL, yb, lz) >> lane) & 1u;
           sm_union_tile(par, on ? 2 * brick_local(lane, ly, lz) : self, on ? 2 * brick_local(lane, 0, lz) : self, err);
@@ -397,19 +479,19 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
       }
     }
   }
-  // 8. roots on the brick's faces marked, a lane per site: rows ly and ly + 8 of
-  //    the first and the last plane, the first and last row of my plane, its
-  //    first and last column (16 lanes each); of a run of equal roots the first
-  //    lane marks.  The lookups go in step.
-  {
-    constexpr int N = 7;
-    const int z_of[N] = {ly, ly + 8, ly, ly + 8, 0, k.d - 1, lane & 15};
-    const int y_of[N] = {0, 0, k.h - 1, k.h - 1, ly, ly, ly};
+  // 8. roots on the brick's faces marked, a lane per site: the first and last row
+  //    of my plane, its first and last column (16 lanes each), rows ly and ly + 8
+  //    of the first and the last plane (a flat brick has no row ly + 8); of a run
+  //    of equal roots the first lane marks.  The lookups go in step.
+  auto mark_faces = [&](auto n) {
+    constexpr int N = decltype(n)::value;
+    const int z_of[7] = {0, k.d - 1, lane & 15, ly, ly, ly + 8, ly + 8};
+    const int y_of[7] = {ly, ly, ly, 0, k.h - 1, 0, k.h - 1};
     int r[N];
 #pragma unroll
     for (int u = 0; u < N; ++u) {
-      const int x = u < N - 1 ? lane : lane < 16 ? 0 : k.w - 1;
-      const bool ok = x < k.w && z_of[u] < k.d && (u < 4 || plane);
+      const int x = u != 2 ? lane : lane < 16 ? 0 : k.w - 1;
+      const bool ok = x < k.w && z_of[u] < k.d && (u > 2 || plane);
       r[u] = ok ? 2 * brick_local(x, y_of[u], z_of[u]) : -1;
     }
 #pragma unroll
@@ -425,7 +507,9 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
       if (r[u] >= 0 && (lane == 0 || left != r[u]) && !(*reinterpret_cast<volatile uint32_t*>(word) & bit))
         atomicOr(word, bit);
     }
-  }
+  };
+  if (!flat) mark_faces(std::integral_constant<int, 7>());
+  else mark_faces(std::integral_constant<int, 5>());
   if (do_obs) {
     unsigned long long* oslot =
         reinterpret_cast<unsigned long long*>(obs + (int64_t)((sweep - 1) % (uint64_t)obs_cap) * (q + 1));
@@ -453,10 +537,12 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
 // the union; the others' pairs are listed and joined with all lanes busy (see
 // merge_tiles).  Bound by the latency of the root loads and parent walks;
 // 256^3: 37 us against 61 with a union per lane where its bond stands (blocks of
-// 128 threads 40 us, of 448 45).
+// 128 threads 40 us, of 448 45).  Flat bricks have few face bonds, and there what
+// counts is bricks in flight: with more of them than blocks of 256 threads fit
+// the GPU at once, blocks of 64 (2000 x 2000 x 1, 15750 bricks: 28.8 us against
+// 35.9; 300 x 300 x 3, 380 bricks: 9.9 against 8.3).
 constexpr int B3_MERGE_UNITS = B3Y + B3Z + B3Y / 2;
-constexpr int MERGE3_THREADS = 256;
-
+template <int MERGE3_THREADS>
 __global__ void __launch_bounds__(MERGE3_THREADS)
 k3_merge(const uint16_t* lroot, int32_t* gpar, const uint32_t* words, Box3 b, int limit,
          SwCtl* ctl, int64_t* obs, int obs_cap, int q) {
@@ -467,7 +553,7 @@ k3_merge(const uint16_t* lroot, int32_t* gpar, const uint32_t* words, Box3 b, in
   int* err = &ctl->err;
   if (blockIdx.x == 0) {   // the next sweep's local step fills this sweep's observable slot
     const uint64_t s = ctl->sweep;
-    if ((int)threadIdx.x <= q) obs[(int64_t)(s % (uint64_t)obs_cap) * (q + 1) + threadIdx.x] = 0;
+    for (int j = threadIdx.x; j <= q; j += MERGE3_THREADS) obs[(int64_t)(s % (uint64_t)obs_cap) * (q + 1) + j] = 0;
     __syncthreads();
     if (threadIdx.x == 0) ctl->sweep = s + 1;
   }
@@ -752,14 +838,17 @@ cudaError_t launch_sweep3(int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_
   int* err = &ctl->err;
   if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
   const PhiloxKeys keys = philox_keys(seed);
-  e = launch_after(k3_local, (unsigned)b.n_bricks(), B3_THREADS, st, spins, lroot, gpar, words, b, q, T, keys, ctl, obs,
+  const int last_d = b.Z - (b.bz - 1) * B3Z;   // planes of the last layer of bricks
+  e = launch_after(last_d <= FLAT_D ? k3_local<true> : k3_local<false>, (unsigned)b.n_bricks(), B3_THREADS, st, spins, lroot, gpar, words, b, q, T, keys, ctl, obs,
                    obs_cap, err);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
   // a box of one brick has no face bonds: one block only advances the counter
   const bool faces = b.bx > 1 || b.by > 1 || b.bz > 1;
   const int64_t blocks = faces ? b.n_bricks() : 1;
-  e = launch_after(k3_merge, (unsigned)blocks, MERGE3_THREADS, st, lroot, gpar, words, b, limit3(b), ctl, obs, obs_cap, q);
+  const bool narrow = b.Z <= FLAT_D && blocks > 152 * 8;
+  e = launch_after(narrow ? k3_merge<64> : k3_merge<256>, (unsigned)blocks, narrow ? 64u : 256u, st, lroot, gpar, words,
+                   b, limit3(b), ctl, obs, obs_cap, q);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   e = launch_after(k3_flip, (unsigned)b.n_bricks(), B3_THREADS, st, spins, lroot, gpar, words, b, q, keys, ctl, limit3(b),

@@ -162,10 +162,12 @@ __device__ __forceinline__ uint32_t run_words(uint32_t we, uint32_t wn, int h, u
 
 // Runs the engine.  we, wn: the calling thread's row word (row = lane, strip =
 // warp), zero for rows >= h; w: columns of the tile (strips past them hold no
-// sites and are skipped); rows past h are swept as rows of single sites.  All
-// threads call it.  On return the calling warp's strip is
-// resolved: other strips' roots may be read after a __syncthreads().
-template <int ROWS>
+// sites and are skipped); rows past h are swept as rows of single sites, or with
+// ALL_ROWS false not at all, their entries left unwritten (a rolled loop, for
+// tiles of which h is a small part).  All threads call it.  On return the calling
+// warp's strip is resolved: other strips' roots may be read after a
+// __syncthreads().
+template <bool ALL_ROWS = true, int ROWS>
 __device__ __forceinline__ void tile_engine(TileSmemT<ROWS>& sm, uint32_t we, uint32_t wn, int h, int w, int* err) {
   constexpr int LIST_CAP = TileSmemT<ROWS>::LIST_CAP;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -193,8 +195,7 @@ __device__ __forceinline__ void tile_engine(TileSmemT<ROWS>& sm, uint32_t we, ui
     const uint32_t upto = FULL >> lane;          // bits 0..col
     const uint32_t me = 1u << col;
     int lab_below = 0;
-#pragma unroll SWEEP_UNROLL
-    for (int ly = 0; ly < ROWS; ++ly) {
+    auto sweep_row = [&](int ly) {
       const uint4 ri = sm.rowinfo[warp * ROWS + ly];
       const int start = high_bit(ri.x & upto);
       const int from = high_bit(ri.y & (FULL >> start));
@@ -203,6 +204,13 @@ __device__ __forceinline__ void tile_engine(TileSmemT<ROWS>& sm, uint32_t we, ui
       const int label = __shfl_sync(FULL, cand, from);
       par[site] = (uint16_t)label;
       lab_below = label;
+    };
+    if (ALL_ROWS) {
+#pragma unroll SWEEP_UNROLL
+      for (int ly = 0; ly < ROWS; ++ly) sweep_row(ly);
+    } else {
+#pragma unroll 1
+      for (int ly = 0; ly < h; ++ly) sweep_row(ly);
     }
   }
   __syncwarp();
