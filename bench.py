@@ -39,7 +39,7 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "9e7d7f30a68f38ab"
+SWEEP_COUNTER_HASH = "2daed6bc6724d9fa"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
     "k_sw_label": ((88.882944 + 130.552576) * 1e6 / 67108864, 184289377 / 67108864),
     "k_merge": ((56.290304 + 0.759040) * 1e6 / 67108864, 14597217 / 67108864),
@@ -50,7 +50,7 @@ SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per si
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "9a133ef348ac4f70"
+CCL_COUNTER_HASH = "19e1c8599320473d"
 CCL_COUNTER_TILE_W = 128
 CCL_TRAFFIC_BYTES_PER_SITE = ((6.647808 + 2.541824) + (16.571136 + 0.000000) + (53.475584 + 10.175232)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8

@@ -23,11 +23,17 @@
 //     the root) into their own spins;
 //  5. after a barrier, every site takes its root's spin.
 // Bound by the latency of its chains up to about L = 80 (an instruction every
-// five cycles in a warp, 4 warps per scheduler) and by issue above.  Critical
-// Ising, us per sweep here / as three kernels on low tiles: L = 16 4.8 / 11.4, 64
-// 7.8 / 14.3, 96 12.1 / 15.2, 100 15.1 / 15.5, 112 15.3 / 16.6, 116 16.8 / 17.0,
-// 124 19.8 / 16.9 (q = 3: 112 16.2 / 16.6, 116 17.7 / 16.8); the line lies where
-// one SM no longer keeps up with tiles spread over the GPU.
+// five cycles in a warp, 4 warps per scheduler) and by issue above; the line
+// (small_line) lies where one SM no longer keeps up with tiles spread over the
+// GPU.  At the critical point, us per sweep here / as three kernels on low tiles:
+// q = 2: L = 16 4.8 / 11.4, 64 7.8 / 14.3, 96 12.1 / 15.2, 100 15.1 / 15.5, 112
+// 15.3 / 16.6, 116 16.8 / 17.0, 124 19.8 / 16.9; q = 3: 96 12.7 / 15.8, 112 16.2 /
+// 16.6, 116 17.7 / 16.8.  More states mean more clusters, all drawn by one block,
+// and past 8 their counts go by shared atomics: times as three kernels over times
+// here at L = 96, 104, 112: q = 4 1.23, 0.98, 0.95; q = 6 1.03, 0.84, 0.87; q = 9
+// 1.04, 0.88, 0.85; q = 20 0.83, 0.80, 0.80; q = 127 0.73, 0.66, 0.64 (L = 84: 1.29,
+// 1.19, 1.35, 1.12, 0.99).  At 0.8 of the critical coupling the lines lie lower:
+// q = 2 1.05, 0.88, 0.86; q = 3 0.96, 0.81, 0.78.
 #include "fused_tile.cuh"
 
 namespace swccl {

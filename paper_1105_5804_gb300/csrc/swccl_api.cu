@@ -48,7 +48,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 constexpr int OBS_CAP = 4096;
 constexpr size_t READBACK_BYTES = 64 << 10;
-constexpr int SMALL_SWEEPS = 1024;   // sweeps per launch of the small-lattice kernel (a few ms at L = 128)
+constexpr int SMALL_SWEEPS = 1024;   // sweeps per launch of the small-lattice kernel (16 ms at L = 112)
 
 }  // namespace
 
@@ -334,7 +334,7 @@ sw_handle* sw_create_threshold(int L, int q, uint64_t T, uint64_t seed, int hot_
   if ((e = cudaHostAlloc(&h->readback, READBACK_BYTES, cudaHostAllocMapped))) return bad(e, "read-back buffer");
   if ((e = cudaMalloc(&h->obs, (int64_t)OBS_CAP * (q + 1) * 8))) return bad(e, "observable ring");
   if ((e = cudaMalloc(&h->lroot, (N * 2 + 15) & ~15LL))) return bad(e, "tile roots");
-  if (L <= SMALL_L && (e = small_prepare())) return bad(e, "small-lattice kernel");
+  if (L <= small_line(q) && (e = small_prepare())) return bad(e, "small-lattice kernel");
   h->ls = carve_label_scratch(h->grid, h->scratch,
                               reinterpret_cast<int*>(reinterpret_cast<char*>(h->ctl) + offsetof(SwCtl, err)));
   h->ls_f = sweep_scratch(h->grid_f, h->ls);
@@ -377,7 +377,7 @@ int sw_sweep(sw_handle* h, int n) {
   if (const int rc = refuse_capture(h, "sw_sweep")) return rc;
   const OnDevice on(h->device);
   CK(on.error());
-  if (fused && !h->timing && h->update == SW_UPDATE_SW && h->L <= SMALL_L) {
+  if (fused && !h->timing && h->update == SW_UPDATE_SW && h->L <= small_line(h->q)) {
     // all sweeps of the call by one block, which writes their observables too
     for (int done = 0; done < n; done += SMALL_SWEEPS) {
       const int m = std::min(n - done, SMALL_SWEEPS);

@@ -253,11 +253,12 @@ cudaError_t launch_sw_flip_few(int8_t* spins, const uint16_t* lroot, int32_t* gp
                                const LabelScratch& s, int q, uint64_t seed, const uint32_t* sel, uint64_t P,
                                const SwCtl* ctl, cudaStream_t st);
 
-// Whole sweeps of a lattice with L <= SMALL_L by one block (k_small.cu): n sweeps
+// Whole sweeps of a lattice with L <= small_line(q) by one block (k_small.cu): n sweeps
 // in one launch, their observables (and the pending ones of the sweep before)
 // written to the ring, ctl advanced.  small_prepare: once per device before the
 // first launch.
 constexpr int SMALL_L = 112;
+inline int small_line(int q) { return q <= 3 ? SMALL_L : 96; }
 cudaError_t small_prepare();
 cudaError_t launch_sw_small(int8_t* spins, int L, int q, uint64_t T, uint64_t seed, SwCtl* ctl, int64_t* obs,
                             int obs_cap, int n, cudaStream_t st);

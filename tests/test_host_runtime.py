@@ -201,3 +201,15 @@ def test_noalloc_loads_every_kernel_on_its_first_call(tmp_path):
     for H, W in [(200, 300), (1000, 1200), (1500, 1500), (2000, 2000)]:
         assert fake.ccl_label_noalloc(m, l, H, W, 0, st) == SW_OK, fake.sw_last_error()
     assert cold() == 0
+
+
+@pytest.mark.parametrize("q,line", [(2, 112), (3, 112), (4, 96), (8, 96), (9, 96), (127, 96)])
+def test_where_the_one_block_kernel_ends(fake, q, line):
+    """Up to the line all sweeps of a call are one launch, past it three each."""
+    st = fake.fake_stream(0)
+    for L, launches in ((4, 1), (line, 1), (line + 4, 30)):
+        h = fake.sw_create_threshold(L, q, 1 << 31, 1, 1, st)
+        before = _counts(fake)[0]
+        assert fake.sw_sweep(h, 10) == SW_OK
+        assert _counts(fake)[0] - before == launches, L
+        fake.sw_destroy(h)
