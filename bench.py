@@ -39,20 +39,20 @@ WORKLOAD = "sw_ising_q2_L%d_beta_c_hot_start_seed7"
 # reports null.
 SWEEP_COUNTER_SOURCES = ("fused_tile.cuh", "tile_engine.cuh", "k_fused.cu", "k_label.cu", "swccl_device.cuh",
                          "swccl_shared.h")
-SWEEP_COUNTER_HASH = "2daed6bc6724d9fa"
+SWEEP_COUNTER_HASH = "70983702d6fd20d9"
 SWEEP_COUNTERS = {      # kernel: (DRAM bytes per site, warp instructions per site)
-    "k_sw_label": ((88.882944 + 130.552576) * 1e6 / 67108864, 184289377 / 67108864),
-    "k_merge": ((56.290304 + 0.759040) * 1e6 / 67108864, 14597217 / 67108864),
-    "k_sw_flip": ((203.559680 + 47.665408) * 1e6 / 67108864, 71103822 / 67108864),
+    "k_sw_label": ((88.854016 + 130.508032) * 1e6 / 67108864, 184287485 / 67108864),
+    "k_merge": ((56.306432 + 0.800256) * 1e6 / 67108864, 14605302 / 67108864),
+    "k_sw_flip": ((203.560960 + 47.639552) * 1e6 / 67108864, 71106685 / 67108864),
 }
 # The stand-alone labeling call (k_ccl_tile, k_merge, k_ccl_final), one ncu
 # capture per kernel of a 4096^2 critical percolation mask: DRAM bytes per site,
 # for the build with CCL_COUNTER_TILE_W-wide tiles, to which the binding routes
 # labeling.
 CCL_COUNTER_SOURCES = ("label_tile.cuh", "tile_engine.cuh", "k_label.cu", "swccl_device.cuh", "swccl_shared.h")
-CCL_COUNTER_HASH = "19e1c8599320473d"
+CCL_COUNTER_HASH = "b08f7044266b5cef"
 CCL_COUNTER_TILE_W = 128
-CCL_TRAFFIC_BYTES_PER_SITE = ((6.647808 + 2.541824) + (16.571136 + 0.000000) + (53.475584 + 10.175232)) * 1e6 / 16777216
+CCL_TRAFFIC_BYTES_PER_SITE = ((6.660096 + 2.575872) + (16.570112 + 0.000000) + (53.475328 + 10.458624)) * 1e6 / 16777216
 # Algorithmic HBM bytes per site: the fused sweep reads and writes the int8
 # spins once (2 B, the minimum of any sweep); the kernel split adds the
 # 16-bit tile roots written by k_sw_label and read by k_sw_flip (6 B).

@@ -257,8 +257,9 @@ uint64_t sw_prob_threshold(double p);
  * F_q of word 0) and the observables (n_eq over the 3N bonds, then n_k) are
  * as on the square lattice.  Hot start: INIT draw of site i as in 2D.
  * Requires X, Y, Z >= 1 with X*Y*Z <= 2^30, 2 <= q <= 127, T <= 2^32.  The
- * library owns the device memory: about 7.2 bytes per site (spins, brick
- * roots, parent array, edge and face bits) plus the observable ring.  NULL on failure (see sw_last_error).  Each sweep is
+ * library owns the device memory: 7 bytes per site (spins, brick roots,
+ * parent array) and 640 per brick of 32 x 8 x 16 sites (edge and face bits;
+ * 0.16 per site where bricks are full) plus the observable ring.  NULL on failure (see sw_last_error).  Each sweep is
  * three kernels (brick-local union-find with the previous sweep's
  * observables, face merge and counter advance, flip), launched so that each
  * launch overlaps the kernel before it. */
@@ -416,8 +417,10 @@ void* sw_batch_stream(sw_batch* b);
  * periodic == 0: those bonds are ignored (image segmentation).
  * Requires H, W >= 1 and H*W < 2^31.  Enqueued on `stream` (a
  * cudaStream_t, NULL = legacy default stream); returns without waiting.
- * Scratch memory (2.4 to 3.4 bytes per site) is taken with cudaMallocAsync
- * on the same stream and released in stream order. */
+ * Scratch memory (2.4 to 3.4 bytes per site of whole tiles: 128 columns by 8,
+ * 16 or 32 rows as the Python binding routes the call, a thin grid's tiles
+ * counting whole) is taken with cudaMallocAsync on the same stream and
+ * released in stream order. */
 int ccl_label(const uint8_t* bond_mask, int32_t* labels, int H, int W, int periodic, void* stream);
 
 /* Bytes of scratch ccl_label_ws needs for an H x W grid (-1 if invalid). */
@@ -473,8 +476,9 @@ int ccl_perc_mask(uint64_t k, uint8_t* mask, int H, int W, void* stream);
  * wrong labels: order them.  The first call on each device looks up the
  * array's device address and that of the labeling status word (the latter
  * also by the first call of any other ccl_* entry point), with that device
- * current (with lazy module loading the driver places the array in device
- * memory then); make that first call before any stream capture.  Grids whose
+ * current, and loads every kernel that later calls may launch (with lazy module
+ * loading the driver places the array and the kernels in device memory then);
+ * make that first call before any stream capture.  Grids whose
  * scratch exceeds CCL_NOALLOC_SCRATCH_BYTES are rejected with SW_ERR_ARG
  * before anything is launched.  Device-side failures are reported by
  * ccl_status(). */

@@ -202,10 +202,6 @@ using namespace fused;
 constexpr int EDGE_WORDS = TILE_SITES / 32;
 __device__ __forceinline__ int32_t* sweep_edges(const LabelScratch& s, int t) { return s.roots + (int64_t)t * EDGE_WORDS; }
 static_assert(EDGE_WORDS == LABEL_THREADS, "one edge word per thread");
-// Flag on a root-list entry (local indices are below TILE_SITES).
-constexpr uint16_t EDGE_ROOT = 0x8000u;
-constexpr uint16_t ROOT_MASK = 0x7FFFu;
-static_assert(TILE_SITES <= ROOT_MASK + 1, "local index fits below the flag");
 
 struct LabelTileSmem {
   TileSmem tile;

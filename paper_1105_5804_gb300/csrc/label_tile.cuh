@@ -183,24 +183,6 @@ __device__ __forceinline__ void root_compress_tile(int32_t* labels, const LabelS
   }
 }
 
-// Site pass of tile t: every label of the tile points at a tile root whose
-// entry holds the final root after root compression; one jump makes the
-// label canonical.
-__device__ __forceinline__ void site_compress_tile(int32_t* labels, const Grid& g, int t) {
-  const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-  const int y0 = ty * TILE_H, x0 = tx * TILE_W;
-  const int h = min(TILE_H, g.H - y0), w = min(TILE_W, g.W - x0);
-  for (int k = threadIdx.x; k < TILE_SITES; k += blockDim.x) {
-    const int ly = k >> TILE_W_LOG2, lx = k & (TILE_W - 1);
-    if (ly < h && lx < w) {
-      int32_t* p = labels + (int64_t)(y0 + ly) * g.W + x0 + lx;
-      const int r = __ldcg(p);
-      const int R = __ldcg(labels + r);
-      if (R != r) *p = R;
-    }
-  }
-}
-
 // Final labels of tile t for the stand-alone path (after the seam merge, on
 // what ccl_label_tile<true> wrote): `table` holds every local index's label --
 // first its own global index, the label of a component that stays in the tile;
@@ -208,8 +190,8 @@ __device__ __forceinline__ void site_compress_tile(int32_t* labels, const Grid& 
 // site takes table[its tile root].  A walk compresses the entries it passes to
 // smaller ones of the same tree, so walks of other tiles stay valid.  The tile
 // roots of a thread's sites wait in registers while the table is filled and the
-// edge roots walk; an edge root is on the tile's perimeter, so a thread has at
-// most five walks.  Labels go out as 16-byte words wherever the rows start (a row
+// edge roots walk; a tile has at most as many edge roots as sites on its
+// perimeter, three per thread.  Labels go out as 16-byte words wherever the rows start (a row
 // of any width, its roots shifted by up to three sites against the words they
 // come in).  Bound by the latency of the walks, so what counts is tiles in
 // flight: ten per SM, with a thread per column and no roots in shared memory,

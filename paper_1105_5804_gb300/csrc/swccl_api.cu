@@ -379,8 +379,8 @@ int sw_sweep(sw_handle* h, int n) {
   CK(on.error());
   if (fused && !h->timing && h->update == SW_UPDATE_SW && h->L <= small_line(h->q)) {
     // all sweeps of the call by one block, which writes their observables too
-    for (int done = 0; done < n; done += SMALL_SWEEPS) {
-      const int m = std::min(n - done, SMALL_SWEEPS);
+    for (int left = n; left > 0; left -= SMALL_SWEEPS) {
+      const int m = std::min(left, SMALL_SWEEPS);
       CK(launch_sw_small(h->spins, h->L, h->q, h->T, h->seed, h->ctl, h->obs, OBS_CAP, m, h->stream));
       h->sweeps += m;
     }

@@ -79,7 +79,7 @@ inline Grid make_grid(int H, int W, int periodic, int th = TILE_H) {
 // Scratch of one labeling problem.
 struct LabelScratch {
   int32_t* roots;        // n_tiles * TILE_H * TILE_W: tile-root lists (fused sweeps: TILE_SITES / 32 edge-root words per tile)
-  int32_t* work;         // n_tiles * TILE_H * TILE_W: unused by sweeps (stand-alone labeling: 16-bit tile roots)
+  int32_t* work;         // n_tiles * TILE_H * TILE_W: sweeps on low tiles: their seam records; stand-alone labeling: 16-bit tile roots
   int32_t* root_counts;  // n_tiles
   int32_t* seams;        // n_tiles * SeamLayout::INTS
   int* err;              // device status word
