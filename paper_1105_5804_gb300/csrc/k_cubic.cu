@@ -29,8 +29,6 @@
 // HBM traffic per site: spins read 1 B and brick roots written 2 B (local),
 // brick roots read 2 B and spins written 1 B (flip), plus the face sites,
 // the edge-root and face bits (0.16 B) and the sparse parent entries.
-#include <type_traits>
-
 #include "fused_tile.cuh"
 
 namespace swccl {
@@ -137,15 +135,16 @@ struct RowBonds {
 // FLAT_D rows): the rows spread over all lanes, R consecutive sites of a row
 // each, R being the power of two from the number of rows on.  With two lanes per
 // row and sixteen sites per lane, as in a full brick, a brick of one row costs
-// what a full one does: a sweep of 1000 x 1000 x 1 took 126 us, 79 this way (the
+// what a full one does: a sweep of 1000 x 1000 x 1 took 126 us, 78 this way (the
 // 16 rows of the engine not swept and one-site axes not joined to themselves are
-// part of it), 1000 x 1000 x 2 138 and 98, x 4 153 and 123, x 8 176 and 169.
-constexpr int FLAT_D = B3Z / 2;
+// part of it), x 2 138 and 97, x 4 153 and 122 (x 8 176 and 169, but 256 x 8 x 8
+// without draws 16.1 and 17.4: bytes are loaded one by one here).
+constexpr int FLAT_D = 4;
 __device__ __forceinline__ RowBonds flat_bonds(const int8_t* spins, const Box3& b, const Brick& k, int q, uint64_t T,
                                                const PhiloxKeys& keys, uint64_t sweep, bool do_obs, unsigned* red,
                                                int* hist) {
   const int lane = threadIdx.x & 31, ly = threadIdx.x >> 5;
-  const int R = k.d <= 1 ? 1 : k.d <= 2 ? 2 : k.d <= 4 ? 4 : 8;
+  const int R = k.d <= 2 ? k.d : 4;
   const int lz = lane & (R - 1), x0 = lane & ~(R - 1);   // my row, my first column
   const int y = k.y0 + ly, z = k.z0 + lz;
   const int n = ly < k.h && lz < k.d ? min(k.w - x0, R) : 0;
@@ -207,9 +206,11 @@ __device__ __forceinline__ RowBonds flat_bonds(const int8_t* spins, const Box3& 
 // with eight CTAs, 142 with packed spins, 131 with the face roots looked up a lane
 // per face site (before: by the sites' owners, a few lanes per warp) and parent
 // entries written from the edge bits.
-// FLAT: for boxes whose last layer of bricks has at most FLAT_D planes of rows (its
-// bricks, not the others, go by flat_bonds; the engine's sweep is a loop over the
-// brick's rows instead of unrolled: 256 x 256 x 17 43.2 us a sweep against 42.2).
+// FLAT: for boxes of at most FLAT_D rows in z, all of whose bricks are flat.  With
+// a flat last layer behind full ones the other kernel is as fast or faster, since
+// here the engine's sweep is a loop over the brick's rows instead of unrolled
+// (256 x 256 x 17 42.2 us a sweep against 43.2 with the flat bricks told apart, x 24
+// 42.8 against 44.3).
 template <bool FLAT>
 __global__ void __launch_bounds__(B3_THREADS, 8)
 k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, Box3 b, int q, uint64_t T,
@@ -234,9 +235,8 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
   const int nv = plane && lz < k.d ? min(max(k.w - 16 * half, 0), 16) : 0;
   const uint32_t row0 = (uint32_t)site3(b, k.x0, k.y0 + ly, k.z0 + lz);   // my row's first site; past the box without sites
   const uint32_t site0 = row0 + 16 * half;
-  const bool flat = FLAT && k.d <= FLAT_D;
   RowBonds row = {0u, 0u, 0u};
-  if (flat) {
+  if (FLAT) {
     row = flat_bonds(spins, b, k, q, T, keys, sweep, do_obs, ls.red, ls.hist);
   } else {
     uint32_t ex = 0u, ey = 0u, ez = 0u;
@@ -483,8 +483,8 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
   //    of my plane, its first and last column (16 lanes each), rows ly and ly + 8
   //    of the first and the last plane (a flat brick has no row ly + 8); of a run
   //    of equal roots the first lane marks.  The lookups go in step.
-  auto mark_faces = [&](auto n) {
-    constexpr int N = decltype(n)::value;
+  {
+    constexpr int N = FLAT ? 5 : 7;
     const int z_of[7] = {0, k.d - 1, lane & 15, ly, ly, ly + 8, ly + 8};
     const int y_of[7] = {ly, ly, ly, 0, k.h - 1, 0, k.h - 1};
     int r[N];
@@ -507,9 +507,7 @@ k3_local(const int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_t* words, B
       if (r[u] >= 0 && (lane == 0 || left != r[u]) && !(*reinterpret_cast<volatile uint32_t*>(word) & bit))
         atomicOr(word, bit);
     }
-  };
-  if (!flat) mark_faces(std::integral_constant<int, 7>());
-  else mark_faces(std::integral_constant<int, 5>());
+  }
   if (do_obs) {
     unsigned long long* oslot =
         reinterpret_cast<unsigned long long*>(obs + (int64_t)((sweep - 1) % (uint64_t)obs_cap) * (q + 1));
@@ -838,15 +836,15 @@ cudaError_t launch_sweep3(int8_t* spins, uint16_t* lroot, int32_t* gpar, uint32_
   int* err = &ctl->err;
   if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return e;
   const PhiloxKeys keys = philox_keys(seed);
-  const int last_d = b.Z - (b.bz - 1) * B3Z;   // planes of the last layer of bricks
-  e = launch_after(last_d <= FLAT_D ? k3_local<true> : k3_local<false>, (unsigned)b.n_bricks(), B3_THREADS, st, spins, lroot, gpar, words, b, q, T, keys, ctl, obs,
-                   obs_cap, err);
+  const bool flat = b.Z <= FLAT_D;
+  e = launch_after(flat ? k3_local<true> : k3_local<false>, (unsigned)b.n_bricks(), B3_THREADS, st, spins, lroot, gpar,
+                   words, b, q, T, keys, ctl, obs, obs_cap, err);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
   // a box of one brick has no face bonds: one block only advances the counter
   const bool faces = b.bx > 1 || b.by > 1 || b.bz > 1;
   const int64_t blocks = faces ? b.n_bricks() : 1;
-  const bool narrow = b.Z <= FLAT_D && blocks > 152 * 8;
+  const bool narrow = flat && blocks > 152 * 8;
   e = launch_after(narrow ? k3_merge<64> : k3_merge<256>, (unsigned)blocks, narrow ? 64u : 256u, st, lroot, gpar, words,
                    b, limit3(b), ctl, obs, obs_cap, q);
   if (e != cudaSuccess) return e;
